@@ -163,6 +163,83 @@ def run(state):
     return out
 
 
+# ---------------------------------------------------------------- the same results in 64 bits, plain torch
+def exact(case, seed):
+    """What `run` returns on its first pass over these inputs, in float64 from the definitions.  Index lists, lengths,
+    and values that are only copied or picked (page summaries, codes) have no such value: None."""
+    if case["op"] == "ingest":
+        return None
+    cfg, op = _config(case), case["op"]
+    out = []
+    for i in range(case["layers"]):
+        w = wl.DeviceWorkload(cfg, replica=seed, layer=i)
+        xs = [w.start_block()] + [w.next_step() for _ in range({"steps": 1, "first": 0}.get(op, cfg.steps - 1))]
+        shape = tuple(xs[0].q.shape)
+        st = {"o": torch.zeros(shape, dtype=torch.float64, device="cuda"), "merged": None,
+              "l": torch.zeros(shape[:3], dtype=torch.float64, device="cuda"), "q": None}
+        caches = [_exact_cache(case, w, s) for s in range(cfg.batch)]
+        for x in xs + (xs[:1] if op == "steps" else []):
+            _exact_step(case, cfg, caches, x, st)
+        if op == "block":
+            out += [None, None, None]
+        out.append((*st["merged"], st["o"], st["l"], st["q"], None, None, None, None))
+    return out
+
+
+def _exact_cache(case, w, s):
+    """Keys and values [P, g, H_kv, d] of a prefix (zero past its end), the valid tokens, and each page's min / max keys."""
+    L, g = int(w.kv_len[s]), case["page"]
+    P = -(-L // g)
+    phys = w.page_table[s, :P].long()
+    valid = (torch.arange(P * g, device="cuda") < L).view(P, g)
+    kv = [t[phys].double().transpose(1, 2).masked_fill(~valid[:, :, None, None], 0.0) for t in (w.k_pages, w.v_pages)]
+    if case["kv"] == "fp8":            # E4M3 codes under one power-of-two scale per (page, KV head)
+        for j, t in enumerate(kv):
+            amax = t.abs().amax((1, 3), keepdim=True)
+            scale = 2.0 ** torch.ceil(torch.log2(amax.clamp_min(1e-30) / 448.0)).clamp(-6, 7)
+            kv[j] = (t / scale).clamp(-448, 448).to(torch.float8_e4m3fn).double() * scale
+    no = ~valid[:, :, None, None]
+    return kv[0], kv[1], valid, kv[0].masked_fill(no, math.inf).amin(1), kv[0].masked_fill(no, -math.inf).amax(1)
+
+
+def _exact_attend(q, k, v, scale):
+    """Softmax attention of q [.., n, d] over k, v [t, d]: output and log of the exponentials' sum."""
+    sc = q @ k.T * scale
+    lse = torch.logsumexp(sc, -1)
+    return torch.exp(sc - lse[..., None]) @ v, lse
+
+
+def _exact_step(case, cfg, caches, x, st):
+    G, B = cfg.group, cfg.block_size
+    q, kb, vb = x.q.double(), x.k_blk.double(), x.v_blk.double()
+    out, lse = torch.empty_like(q), torch.empty_like(st["l"])
+    for s, (k, v, valid, kmin, kmax) in enumerate(caches):
+        P = k.shape[0]
+        if st["q"] is None:
+            act = torch.arange(B, device="cuda")
+        else:
+            delta = (q[s] - st["q"][s]).square().mean((1, 2))
+            act = torch.argsort(delta, descending=True, stable=True)[:case["active"]].sort().values
+        for h in range(cfg.n_kv_heads):
+            heads = slice(h * G, (h + 1) * G)
+            qa = q[s, act, heads]
+            pages = torch.arange(P, device="cuda")
+            if st["q"] is not None:
+                u = qa.clamp_min(0) @ kmax[:, h].T + qa.clamp_max(0) @ kmin[:, h].T
+                if case["selector"] == "pooled":
+                    u = u.amax(1)
+                top = torch.argsort(u, dim=-1, descending=True, stable=True)[..., :min(case["topk"], P)]
+                pages = torch.unique(top)
+            t = valid[pages]
+            o, l = _exact_attend(qa, k[pages, :, h][t], v[pages, :, h][t], cfg.sm_scale)
+            st["o"][s, act, heads], st["l"][s, act, heads] = o, l
+            ob, lb = _exact_attend(q[s, :, heads], kb[s, :, h], vb[s, :, h], cfg.sm_scale)
+            lse[s, :, heads] = torch.logaddexp(lb, st["l"][s, :, heads])
+            wp = torch.exp(st["l"][s, :, heads] - lse[s, :, heads])[..., None]
+            out[s, :, heads] = wp * st["o"][s, :, heads] + torch.exp(lb - lse[s, :, heads])[..., None] * ob
+    st["q"], st["merged"] = q, (out, lse)
+
+
 # Share of the independent draws that a block's selections are worth: the queries of a block share a
 # direction, so the distinct pages of n lists of k pages out of P are P (1 - (1 - k/P)^(f n)) with f
 # as measured on these inputs (per-head lists, lists pooled over a KV head's heads, heavy-hitter keys).
