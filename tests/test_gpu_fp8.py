@@ -71,6 +71,34 @@ def test_fp8_cache_appends_blocks_and_requantises_touched_pages():
         run_fp8_blocks(cfg, n_blocks=3, fused=True)
 
 
+@pytest.mark.parametrize("g,d", [(16, 64), (32, 64), (64, 64), (16, 128), (32, 128), (64, 128)])
+def test_fp8_pages_zero_codes_and_a_block_off_its_alignment(g, d):
+    """Every (page size, d) of the page kernels: columns that round to zero codes of both signs, pages of one token,
+    odd heads (warps past the last page), and a block whose rows are not 16-byte aligned when it is appended."""
+    import torch
+    from paper_2604_12056_b200.layer import LosaLayer, to_device
+    cfg = wl.config("c5", page_size=g, head_dim=d, n_q_heads=6, n_kv_heads=3, kv_lens=(3 * g + 1, 2 * g, 5), steps=1, topk=2,
+                    block_size=min(g + 3, 61), n_blocks=2)
+    w = wl.Workload(cfg)
+    k = wl.bf16_bits_to_f32(w.k_pages)
+    k[..., 3::5] = np.sign(k[..., 3::5]) * 1e-6
+    w.k_pages[...] = wl.f32_to_bf16_bits(k)
+    gl = LosaLayer(cfg, w.k_pages, w.v_pages, w.page_table, w.kv_len, fp8_kv=True)
+    o = OracleFp8Layer(w)
+    assert_cache_equal(gl, o, cfg)
+    inp = w.block_steps()[0]
+    gl.run_step(to_device(inp.q), to_device(inp.k_blk), to_device(inp.v_blk), to_device(inp.m_per_seq))
+    o.run_step(inp, finalize=True)
+    off = []
+    for a in (inp.k_blk, inp.v_blk):
+        buf = torch.empty(a.size + 1, dtype=torch.bfloat16, device="cuda")
+        buf[1:] = to_device(a).flatten()
+        off.append(buf[1:].view(a.shape))
+    gl.finalize_block(*off)
+    assert gl.ctx.poll_status() == 0
+    assert_cache_equal(gl, o, cfg)
+
+
 def test_fp8_cache_dense_mode_and_two_row_groups():
     cfg = wl.config("c4", kv_lens=(64 * 40 + 17,), steps=2, topk=8, m_active=40, heavy_frac=0.0)
     run_fp8_blocks(cfg)
