@@ -525,7 +525,7 @@ int32_t ensure_tensor_maps(losa_ctx* c, const losa_kv_t* kv) {
 
 template <int D, int GP, bool FP8>
 int32_t launch_tc5(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool with_combine) {
-  constexpr int smem = tc5_smem_bytes<D, FP8>();
+  constexpr int smem = tc5_smem_bytes<D, GP, FP8>();
   static_assert(smem <= kSmemBudget, "shared memory of the stage-4 kernel");
   constexpr int bit = FP8 ? 2 : 1;  // a context has one shape on one device: one instantiation per cache format
   if (!(c->attn_attr_set & bit)) {
@@ -536,7 +536,7 @@ int32_t launch_tc5(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool with
   memcpy(&mk, c->tmap_k, sizeof(mk));
   memcpy(&mv, c->tmap_v, sizeof(mv));
   if (c->profile) LOSA_CUDA_TRY(c, cudaEventRecord(c->ev_begin, st));
-  launch_k(attn_tc5_kernel<D, GP, FP8>, ap.n_ctas, kTc5Threads, smem, st, mk, mv, ap);
+  launch_k(attn_tc5_kernel<D, GP, FP8>, ap.n_ctas, tc5_threads<FP8>(), smem, st, mk, mv, ap);
   if (c->profile) LOSA_CUDA_TRY(c, cudaEventRecord(c->ev_end, st));
   int32_t rc = after_launch(c);
   if (rc != LOSA_OK || !with_combine) return rc;

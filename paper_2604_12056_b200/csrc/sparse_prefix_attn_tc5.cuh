@@ -23,25 +23,31 @@
 
 constexpr int kTc5SoftmaxWarps = 8;              // two sets of four: set h takes columns 64h .. 64h+63 of every group
 constexpr int kTc5QkWarp = 8, kTc5PvWarp = 9, kTc5KWarp = 10, kTc5VWarp = 11;
-constexpr int kTc5Threads = 384;
+constexpr int kTc5CvtWarp = 12;                  // FP8 pages: four converting warps, two for K and two for V
+template <bool FP8> constexpr int tc5_threads() { return FP8 ? 512 : 384; }
 constexpr int kTc5Tok = 128;                     // tokens per group = N of Q K^T = columns of one S buffer
 constexpr int kTc5PgMax = 8;                     // pages per group at the smallest page size (16)
 constexpr int kTc5MetaRing = 16;                 // groups whose per-page token counts are kept (producer lead < 16)
 constexpr float kTc5Tau = 8.0f;                  // reference maximum moves only when it would grow by more than this (log2 units)
 constexpr int kTc5XchgBytes = (2 * 2 + 1) * kRowsPerGroup * 4;   // row maxima [group parity][set][row], row sums [row]
-constexpr int kTc5ScaleBytes = 2 * kTc5MetaRing * (kTc5PgMax + 1) * 4;   // FP8 pages: per-page scales and page counts of the groups in flight, K and V
-constexpr int kTc5TailBytes = kTailBytes + 512 + kTc5XchgBytes + kTc5ScaleBytes + (kMaxSegments + 1) * 4;  // 1024 bytes of barriers + page meta, the segment prefix and index cache, the exchange arrays, the scales
-constexpr int kTc5Stg = 2;                       // FP8 pages: staging slots (bytes as they lie in memory) per tensor
+constexpr int kTc5StgMax = 20;                   // FP8 pages: staging slots per tensor, one page each, at most
+constexpr int kTc5StgTail = kTc5StgMax * 2 * (8 + 8) + 2 * kTc5MetaRing * kTc5PgMax * 4;   // ... their barriers (landed, emptied), K and V; the page scales of the groups in flight
+constexpr int kTc5TailBytes = kTailBytes + 512 + kTc5XchgBytes + kTc5StgTail + (kMaxSegments + 2) * 4;  // 1024 bytes of barriers + page meta, the segment prefix and index cache, the exchange arrays, the scales
 
 template <int D> constexpr int tc5_slot_bytes() { return kTc5Tok * D * 2; }
-template <int D> constexpr int tc5_stg_bytes() { return kTc5Tok * D; }
 template <int D, bool FP8> constexpr int tc5_ring_slots() {     // per ring (K and V have one each)
   if (FP8) return 2;                                            // the staging slots take the rest
   const int n = (kSmemBudget - 1024 - kTc5TailBytes) / tc5_slot_bytes<D>() / 2;
   return n > 6 ? 6 : n;
 }
-template <int D, bool FP8> constexpr int tc5_smem_bytes() {
-  return 1024 + 2 * tc5_ring_slots<D, FP8>() * tc5_slot_bytes<D>() + (FP8 ? 2 * kTc5Stg * tc5_stg_bytes<D>() : 0) + kTc5TailBytes;
+// FP8: pages per staging ring (one for K, one for V): what the ring slots leave, up to five groups
+template <int D, int GP> constexpr int tc5_stg_slots() {
+  const int fit = (kSmemBudget - 1024 - kTc5TailBytes - 4 * tc5_slot_bytes<D>()) / 2 / (GP * D), five = 5 * (kTc5Tok / GP);
+  const int n = fit < five ? fit : five;
+  return n < kTc5StgMax ? n : kTc5StgMax;
+}
+template <int D, int GP, bool FP8> constexpr int tc5_smem_bytes() {
+  return 1024 + 2 * tc5_ring_slots<D, FP8>() * tc5_slot_bytes<D>() + (FP8 ? 2 * tc5_stg_slots<D, GP>() * GP * D : 0) + kTc5TailBytes;
 }
 
 // Shared-memory matrix descriptor: 128-byte swizzle, 8-row groups 1024 bytes apart; lbo = distance
@@ -117,15 +123,27 @@ __device__ __forceinline__ void tc5_wait_st() { asm volatile("tcgen05.wait::st.s
 __device__ __forceinline__ uint32_t tc5_sw(int t, int c) { return static_cast<uint32_t>(t * 128 + ((c ^ (t & 7)) << 4)); }
 
 // FP8: the K / V pools hold E4M3 bytes with one power-of-two scale per (page, KV head).  The page
-// copies land in staging slots as they lie in memory (half the bytes); the producer warp that issued
-// them converts a landed group to fp16 times its page's scale (exact) into the ring slot, in the
-// layout the tensor maps of the bf16 path produce, and every MMA runs on fp16 operands (Q and P are
-// converted to fp16 instead of bf16); nothing else changes.
+// copies land in staging rings as they lie in memory (half the bytes); four converting warps, one
+// per scheduler, turn a landed page's codes into fp16 (exact) in the group's ring slot, in the layout
+// the tensor maps of the bf16 path produce, and every MMA runs on fp16 operands (Q and P are
+// converted to fp16 instead of bf16).  The scales stay out of the conversion, which is bound by its
+// instruction count: the key scale joins the softmax scale of the page's columns, and the value
+// scale 2^e is added to their exponent, so that P' = p 2^e multiplies the codes of V and the row sum
+// takes its columns back by 2^-e.  The reference maximum is that of the shifted exponents: every P'
+// has the same headroom, and with equal scales the bits are those of scaled operands.  A group is 2 x 16 KiB of codes:
+// one warp needs about 3.8 us for 16 KiB, and while the two producing warps did this work it set the
+// pace (eight 32K prompts: dense step 372 us, sparse step at three active tokens 120 us).  Now 224 and
+// 81 us (scaling in the converters: 245 and 87; bit moves instead of the conversion instruction: 306
+// and 105; no conversion at all: 207 and 77).  Staging slots are single pages, so that one is refilled
+// while its neighbours are converted.  The
+// CTA's 512 threads start with 128 registers each; the softmax warps take 168 and the other eight
+// give theirs up to 88 (2 x 128 x 168 + 2 x 128 x 88 = 512 x 128).
 template <int D, int GP, bool FP8>
-__global__ void __launch_bounds__(kTc5Threads, 1)
+__global__ void __launch_bounds__(tc5_threads<FP8>(), 1)
 attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, AttnParams p) {
   constexpr int NR = tc5_ring_slots<D, FP8>();  // slots per ring
-  constexpr int NSTG = kTc5Stg, STG = tc5_stg_bytes<D>();
+  constexpr int NSP = FP8 ? tc5_stg_slots<D, GP>() : 1, STG = GP * D;   // FP8: staging slots per tensor, bytes of a slot (one page of codes)
+  constexpr int NT = tc5_threads<FP8>();
   constexpr uint32_t FMT = FP8 ? 0u : 1u;       // operand format of the MMAs: fp16 / bf16
   constexpr int SLOT = tc5_slot_bytes<D>();
   constexpr int PG = kTc5Tok / GP;              // pages per group
@@ -137,22 +155,22 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   static_assert(D == 64 || D == 128, "head dimensions of the tensor-core path");
   static_assert(GP == 16 || GP == 32 || GP == 64, "page sizes of the tensor-core path");
   static_assert(NR >= 2 && PG <= kTc5PgMax, "ring too shallow / group too long");
-  static_assert(8 * (4 * 6 + 14 + 2 * kTc5Stg) + 4 * kTc5MetaRing * kTc5PgMax + 16 <= 1024, "tail layout");
+  static_assert(!FP8 || (NSP >= PG && NSP <= kTc5StgMax), "staging ring");
+  static_assert(8 * (4 * 6 + 14) + 4 * kTc5MetaRing * kTc5PgMax + 16 <= 1024, "tail layout");
 
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* gen = smem_raw + (base - raw);
   const uint32_t kring = base, vring = base + NR * SLOT;
-  constexpr int STG_ALL = FP8 ? 2 * NSTG * STG : 0;
-  const uint32_t kstg = base + 2 * NR * SLOT, vstg = kstg + NSTG * STG;          // FP8 only
+  constexpr int STG_ALL = FP8 ? 2 * NSP * STG : 0;
+  const uint32_t kstg = base + 2 * NR * SLOT, vstg = kstg + NSP * STG;          // FP8 only
   uint8_t* tail = gen + 2 * NR * SLOT + STG_ALL;
   const uint32_t tail_s = base + 2 * NR * SLOT + STG_ALL;
   const uint32_t kfull = tail_s, kfree = kfull + 8 * NR, vfull = kfree + 8 * NR, vfree = vfull + 8 * NR;
   const uint32_t s_full = vfree + 8 * NR, s_free = s_full + 16, p_full = s_free + 16, q_full = p_full + 16, q_free = q_full + 8, xbar = q_free + 8;
   const uint32_t drain_bar = xbar + 32;            // two barriers: the issuing threads' last commit when the CTA gives up
-  const uint32_t kstg_full = drain_bar + 16, vstg_full = kstg_full + 8 * NSTG;   // FP8: a staging slot's copies have landed
-  volatile int* meta = reinterpret_cast<volatile int*>(tail + 8 * (4 * 6 + 14 + 2 * kTc5Stg));   // [kTc5MetaRing][kTc5PgMax] valid tokens per page
+  volatile int* meta = reinterpret_cast<volatile int*>(tail + 8 * (4 * 6 + 14));   // [kTc5MetaRing][kTc5PgMax] valid tokens per page
   volatile int* abort_flag = meta + kTc5MetaRing * kTc5PgMax;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(const_cast<int*>(abort_flag) + 1);
   int* pre = reinterpret_cast<int*>(tail + 1024);
@@ -161,17 +179,20 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   int* len_s = na_s + kStageSeq;
   float* xmax = reinterpret_cast<float*>(len_s + kStageSeq);   // [2][2][128]
   float* xsum = xmax + 4 * kRowsPerGroup;                        // [128]
-  volatile float* scale_meta = xsum + kRowsPerGroup;             // FP8: [2 (K, V)][kTc5MetaRing][kTc5PgMax] page scales,
-  volatile int* ng_meta = reinterpret_cast<volatile int*>(const_cast<float*>(scale_meta) + 2 * kTc5MetaRing * kTc5PgMax);   // [2][kTc5MetaRing] pages per group
-  int* vpre = const_cast<int*>(ng_meta) + 2 * kTc5MetaRing;       // prefix of the charged segment lengths (pages + pad)
+  int* vpre = reinterpret_cast<int*>(xsum + kRowsPerGroup);      // prefix of the charged segment lengths (pages + pad)
+  // FP8: per tensor, a staging slot's page has landed / has been converted; the scales of the groups' pages
+  const uint32_t stg_bars = smem_u32(vpre + kMaxSegments + 1) + 4;   // (kMaxSegments + 1 is odd)
+  const uint32_t kstg_full = stg_bars, vstg_full = kstg_full + 8 * kTc5StgMax, kstg_free = vstg_full + 8 * kTc5StgMax, vstg_free = kstg_free + 8 * kTc5StgMax;
+  volatile float* kscale_meta = reinterpret_cast<volatile float*>(vpre + kMaxSegments + 2 + 8 * kTc5StgMax);   // [kTc5MetaRing][kTc5PgMax]
+  volatile float* vscale_meta = kscale_meta + kTc5MetaRing * kTc5PgMax;
   const bool staged = p.N * p.B <= kStageIdx && p.N <= kStageSeq;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) {
     for (int i = 0; i < NR; ++i) {
-      mbar_init(kfull + 8 * i, 1);
+      mbar_init(kfull + 8 * i, FP8 ? 2 : 1);         // the copies' bytes / the two converting warps
       mbar_init(kfree + 8 * i, 1);
-      mbar_init(vfull + 8 * i, 1);
+      mbar_init(vfull + 8 * i, FP8 ? 2 : 1);
       mbar_init(vfree + 8 * i, 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -185,9 +206,11 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     mbar_init(drain_bar, 1);
     mbar_init(drain_bar + 8, 1);
     if (FP8)
-      for (int i = 0; i < NSTG; ++i) {
+      for (int i = 0; i < NSP; ++i) {
         mbar_init(kstg_full + 8 * i, 1);
         mbar_init(vstg_full + 8 * i, 1);
+        mbar_init(kstg_free + 8 * i, 2);
+        mbar_init(vstg_free + 8 * i, 2);
       }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -202,8 +225,8 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   if (warp == 0) {
     segment_prefix(pre, p.n_seg, p.n_rg, p.Hkv, p.G, p.n_active, p.union_count, p.B, lane, vpre);
   } else if (staged) {
-    for (int i = tid - 32; i < p.N * p.B; i += kTc5Threads - 32) tok_s[i] = p.active_idx[i];
-    for (int i = tid - 32; i < p.N; i += kTc5Threads - 32) {
+    for (int i = tid - 32; i < p.N * p.B; i += NT - 32) tok_s[i] = p.active_idx[i];
+    for (int i = tid - 32; i < p.N; i += NT - 32) {
       na_s[i] = clamp_active(p.n_active[i], p.B);
       len_s[i] = p.kv_len[i];
     }
@@ -213,7 +236,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   tc5_fence_after();
   const uint32_t tmem = *tmem_slot;
   if (blockIdx.x == 0)                             // the combine kernel reads the prefix instead of recomputing it
-    for (int i = tid; i <= p.n_seg; i += kTc5Threads) p.seg_prefix[i] = vpre[i];
+    for (int i = tid; i <= p.n_seg; i += NT) p.seg_prefix[i] = vpre[i];
   // this CTA's share of the charged list, mapped back to pages: the first page at or after a charged position
   const long long V_all = vpre[p.n_seg];
   auto page_at = [&](long long v) {
@@ -239,7 +262,9 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   auto kv_len_of = [&](int s) { return staged ? len_s[s] : p.kv_len[s]; };
   auto token_of = [&](int s, int a) { return staged ? tok_s[s * p.B + a] : p.active_idx[s * p.B + a]; };
 
-  int issued = -1;                                   // producer warps: newest group whose copies have been issued
+  int issued = -1;                                   // producer warps: newest group (FP8: page) whose copies have been issued
+  if (warp >= kTc5SoftmaxWarps) {
+  if constexpr (FP8) asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");    // whole warpgroups
   if (warp == kTc5KWarp || warp == kTc5VWarp) {
     // ------------------------------------------------------------------ producer warps: one for K, one for V
     // Lane j of a batch of 32 consecutive items resolves item -> logical page -> physical page (a
@@ -251,9 +276,10 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     const unsigned long long policy = l2_evict_first_policy();
     const CUtensorMap* map = is_v ? &tmV : &tmK;
     const uint32_t ring = is_v ? vring : kring, full0 = is_v ? vfull : kfull, free0 = is_v ? vfree : kfree;
+    const uint32_t stg = is_v ? vstg : kstg, landed = is_v ? vstg_full : kstg_full, emptied = is_v ? vstg_free : kstg_free;
     int cursor = sg0, gbase = 0, pstart = lo;       // segment of the lane's newest item, groups before its piece, the piece's first item
     struct Item { int page, sk, grp, j, ng; };
-    struct Ready { int phys, kh, valid, grp, j, ng; };
+    struct Ready { int phys, kh, valid, grp, j, ng; float ks, vs; };
     auto stage_a = [&](int i) {
       Item it{-1, 0, 0, 0, 0};
       if (i < hi) {
@@ -272,7 +298,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       return it;
     };
     auto stage_b = [&](int i, const Item& it) {
-      Ready r{0, 0, 0, it.grp, it.j, it.ng};
+      Ready r{0, 0, 0, it.grp, it.j, it.ng, 1.f, 1.f};
       if (i < hi) {
         const int s = it.sk / p.Hkv;
         r.kh = it.sk % p.Hkv;
@@ -282,139 +308,44 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       }
       return r;
     };
-    if constexpr (FP8) {
-      // ---- FP8 pages.  The copies go to staging slots (NSTG groups in flight); before a staging slot
-      // is reused, and at the end, this warp converts the groups that have landed: bytes -> fp16
-      // times the page's scale, written where the tensor maps of the bf16 path would have put them
-      // (two 128-byte-swizzled blocks per row), then announced to the MMA warps.
-      const uint32_t stg = is_v ? vstg : kstg, stg_full0 = is_v ? vstg_full : kstg_full;
-      uint8_t* stg_gen = gen + (stg - base);
-      uint8_t* ring_gen = gen + (ring - base);
-      volatile float* sc_meta = scale_meta + (is_v ? kTc5MetaRing * kTc5PgMax : 0);
-      volatile int* ngs = ng_meta + (is_v ? kTc5MetaRing : 0);
-      const float* scale_g = is_v ? p.v_scale : p.k_scale;
-      constexpr int CPRW = D / 16;                    // 16-byte chunks of a row of bytes
-      int conv = 0;                                   // groups converted so far
-      bool go = true;
-      auto convert = [&](int gc) {
-        const int ss = gc % NSTG, sr = gc % NR;
-        int ok = 1;
-        if (lane == 0) {
-          ok = mbar_wait(stg_full0 + 8 * ss, (gc / NSTG) & 1, abort_flag, p.status, p.wait_cycles);
-          if (ok && gc >= NR) ok = mbar_wait(free0 + 8 * sr, (gc / NR - 1) & 1, abort_flag, p.status, p.wait_cycles);
+    auto stage_c = [&](int i, Ready& r) {             // bounds; FP8, K warp: the page's scales (their address needs the physical page)
+      if (i < hi) {
+        if (r.phys < 0 || r.phys >= p.n_phys || r.valid <= 0) {
+          set_status(p.status, LOSA_ERR_BOUNDS);
+          r.phys = 0;
+          r.valid = 0;
         }
-        if (__shfl_sync(0xffffffffu, ok, 0) == 0) return false;
-        // Lane = (token within a batch of TPI, 16-byte chunk of the row); U batches are loaded before
-        // any is converted, so that the warp - alone with this work - has independent chains in flight.
-        // A byte s.eeee.mmm becomes the fp16 s.0eeee.mmm0000000 = its value / 256 (E4M3 subnormals land on
-        // fp16 subnormals), then one packed multiply by 256 * scale, exact; the quantiser never writes
-        // the NaN code.
-        constexpr int TPI = 32 / CPRW, U = (GP / TPI) < 4 ? (GP / TPI) : 4;
-        const int npg = ngs[gc % kTc5MetaRing];
-        const int tl = lane / CPRW, c8 = lane % CPRW, c = 2 * (c8 & 3);
-        const uint8_t* src = stg_gen + ss * STG + tl * D + c8 * 16;
-        uint8_t* row = ring_gen + sr * SLOT + (c8 >> 2) * HS;
-        for (int pg = 0; pg < npg; ++pg) {
-          const __half2 sc2 = __float2half2_rn(256.f * sc_meta[(gc % kTc5MetaRing) * kTc5PgMax + pg]);
-          for (int t0 = pg * GP; t0 < (pg + 1) * GP; t0 += TPI * U) {
-            uint4 rawb[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) rawb[u] = *reinterpret_cast<const uint4*>(src + (t0 + u * TPI) * D);
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-              const uint32_t w[4] = {rawb[u].x, rawb[u].y, rawb[u].z, rawb[u].w};
-              uint32_t h[8];
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-#pragma unroll
-                for (int hf = 0; hf < 2; ++hf) {
-                  const uint32_t x = __byte_perm(w[e], 0u, hf ? 0x3424u : 0x1404u);      // two bytes, each in the high byte of a half
-                  const uint32_t bits = ((x >> 1) & 0x3f803f80u) | (x & 0x80008000u);
-                  const __half2 v = __hmul2(*reinterpret_cast<const __half2*>(&bits), sc2);
-                  h[2 * e + hf] = *reinterpret_cast<const uint32_t*>(&v);
-                }
+        if (FP8 && !is_v) {
+          r.ks = __ldg(p.k_scale + static_cast<size_t>(r.phys) * p.Hkv + r.kh);
+          r.vs = __ldg(p.v_scale + static_cast<size_t>(r.phys) * p.Hkv + r.kh);
+        }
+      }
+    };
+    // copies of the batch of items b0 .. b0 + 31 (one per lane); false when a wait has run out
+    auto issue = [&](int b0, const Ready& b) {
+      const int nb = min(32, hi - b0);
+      if constexpr (FP8) {                            // page by page: every lane handles its own staging slot
+        for (int pos = 0; pos < nb; ++pos) {
+          int ok = 1;
+          if (lane == pos) {
+            const int x = b0 + pos - lo, slot = x % NSP, round = x / NSP;
+            if (round > 0) ok = mbar_wait(emptied + 8 * slot, (round - 1) & 1, abort_flag, p.status, p.wait_cycles);
+            if (ok) {
+              if (!is_v) {
+                const int at = (b.grp % kTc5MetaRing) * kTc5PgMax + b.j;
+                meta[at] = b.valid;
+                kscale_meta[at] = b.ks;
+                vscale_meta[at] = b.vs;
               }
-              const int t = t0 + u * TPI + tl;
-              *reinterpret_cast<uint4*>(row + tc5_sw(t, c)) = make_uint4(h[0], h[1], h[2], h[3]);
-              *reinterpret_cast<uint4*>(row + tc5_sw(t, c + 1)) = make_uint4(h[4], h[5], h[6], h[7]);
+              mbar_expect_tx(landed + 8 * slot, STG);
+              tma_load_4d(stg + slot * STG, map, landed + 8 * slot, 0, 0, b.kh, b.phys, policy);
             }
           }
+          if (__shfl_sync(0xffffffffu, ok, pos) == 0) return false;
+          issued = b0 + pos - lo;
         }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs read the slot through the async proxy; the next copies overwrite the staging slot through it
-        __syncwarp();
-        if (lane == 0) mbar_arrive(full0 + 8 * sr, 1);
         return true;
-      };
-      struct Ready8 { int phys, kh, valid, grp, j, ng; float scale; };
-      auto stage_b8 = [&](int i, const Item& it) {
-        const Ready r = stage_b(i, it);
-        return Ready8{r.phys, r.kh, r.valid, r.grp, r.j, r.ng, 1.f};
-      };
-      auto stage_c = [&](int i, Ready8& r) {          // the page's scale (its address needs the physical page)
-        if (i < hi) {
-          if (r.phys < 0 || r.phys >= p.n_phys || r.valid <= 0) {
-            set_status(p.status, LOSA_ERR_BOUNDS);
-            r.phys = 0;
-            r.valid = 0;
-          }
-          r.scale = __ldg(scale_g + static_cast<size_t>(r.phys) * p.Hkv + r.kh);
-        }
-      };
-      Item a = stage_a(lo + lane);
-      Ready8 b = stage_b8(lo + lane, a);
-      a = stage_a(lo + lane + 32);
-      stage_c(lo + lane, b);
-      Ready8 b1 = stage_b8(lo + lane + 32, a);
-      a = stage_a(lo + lane + 64);
-      int n_groups = 0;
-      for (int b0 = lo; b0 < hi && go; b0 += 32) {
-        const Item a_next = stage_a(b0 + lane + 96);
-        const Ready8 b2 = stage_b8(b0 + lane + 64, a);
-        stage_c(b0 + lane + 32, b1);
-        const int nb = min(32, hi - b0);
-        int pos = 0;
-        while (pos < nb && go) {
-          const int grp = __shfl_sync(0xffffffffu, b.grp, pos), j0 = __shfl_sync(0xffffffffu, b.j, pos);
-          const int ng = __shfl_sync(0xffffffffu, b.ng, pos);
-          const int cnt = min(ng - j0, nb - pos);
-          const int ss = grp % NSTG;
-          if (j0 == 0) {
-            while (go && conv + NSTG <= grp) go = convert(conv++);          // the staging slot must have been emptied
-            if (!go) break;
-          }
-          const bool mine = lane >= pos && lane < pos + cnt;
-          if (mine) {
-            if (!is_v) meta[(grp % kTc5MetaRing) * kTc5PgMax + b.j] = b.valid;
-            sc_meta[(grp % kTc5MetaRing) * kTc5PgMax + b.j] = b.scale;
-          }
-          if (j0 == 0 && lane == 0) ngs[grp % kTc5MetaRing] = ng;
-          __syncwarp();
-          if (j0 == 0 && lane == 0) mbar_expect_tx(stg_full0 + 8 * ss, ng * GP * D);
-          __syncwarp();
-          if (mine) tma_load_4d(stg + ss * STG + b.j * (GP * D), map, stg_full0 + 8 * ss, 0, 0, b.kh, b.phys, policy);
-          issued = grp;
-          n_groups = grp + 1;
-          pos += cnt;
-        }
-        a = a_next;
-        b = b1;
-        b1 = b2;
       }
-      while (go && conv < n_groups) go = convert(conv++);
-    } else {
-    Item a = stage_a(lo + lane);
-    Ready b = stage_b(lo + lane, a);
-    a = stage_a(lo + lane + 32);
-    bool go = true;
-    for (int b0 = lo; b0 < hi && go; b0 += 32) {
-      const Item a_next = stage_a(b0 + lane + 64);
-      const Ready b_next = stage_b(b0 + lane + 32, a);
-      if (b0 + lane < hi && (b.phys < 0 || b.phys >= p.n_phys || b.valid <= 0)) {
-        set_status(p.status, LOSA_ERR_BOUNDS);
-        b.phys = 0;
-        b.valid = 0;
-      }
-      const int nb = min(32, hi - b0);
       int pos = 0;
       while (pos < nb) {
         const int grp = __shfl_sync(0xffffffffu, b.grp, pos), j0 = __shfl_sync(0xffffffffu, b.j, pos);
@@ -424,8 +355,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         if (j0 == 0) {
           int ok = 1;
           if (lane == 0 && round > 0) ok = mbar_wait(free0 + 8 * slot, (round - 1) & 1, abort_flag, p.status, p.wait_cycles);
-          go = __shfl_sync(0xffffffffu, ok, 0) != 0;
-          if (!go) break;
+          if (__shfl_sync(0xffffffffu, ok, 0) == 0) return false;
         }
         const bool mine = lane >= pos && lane < pos + cnt;
         if (!is_v && mine) meta[(grp % kTc5MetaRing) * kTc5PgMax + b.j] = b.valid;
@@ -440,9 +370,97 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         issued = grp;
         pos += cnt;
       }
-      a = a_next;
-      b = b_next;
+      return true;
+    };
+    Item a = stage_a(lo + lane);
+    Ready b = stage_b(lo + lane, a);
+    a = stage_a(lo + lane + 32);
+    if constexpr (FP8) {                              // one stage deeper: the scales of a batch are requested a batch ahead
+      stage_c(lo + lane, b);
+      Ready b1 = stage_b(lo + lane + 32, a);
+      a = stage_a(lo + lane + 64);
+      bool go = true;
+      for (int b0 = lo; b0 < hi && go; b0 += 32) {
+        const Item a_next = stage_a(b0 + lane + 96);
+        const Ready b2 = stage_b(b0 + lane + 64, a);
+        stage_c(b0 + lane + 32, b1);
+        go = issue(b0, b);
+        a = a_next;
+        b = b1;
+        b1 = b2;
+      }
+    } else {
+      bool go = true;
+      for (int b0 = lo; b0 < hi && go; b0 += 32) {
+        const Item a_next = stage_a(b0 + lane + 64);
+        const Ready b_next = stage_b(b0 + lane + 32, a);
+        stage_c(b0 + lane, b);
+        go = issue(b0, b);
+        a = a_next;
+        b = b_next;
+      }
     }
+  } else if (FP8 && warp >= kTc5CvtWarp) {
+    // ------------------------------------------------------------------ converting warps (FP8 pages)
+    // Two warps per tensor, each half of every page's tokens.  A lane takes eight codes at a time (one
+    // 16-byte chunk of fp16): 8-byte reads of consecutive codes and 16-byte stores of consecutive
+    // swizzled chunks, both without bank conflicts; up to eight are requested before any is converted.
+    const bool is_v = warp >= kTc5CvtWarp + 2;
+    const int half = warp & 1;
+    const uint8_t* stg_gen = gen + ((is_v ? vstg : kstg) - base);
+    uint8_t* ring_gen = gen + ((is_v ? vring : kring) - base);
+    const uint32_t landed = is_v ? vstg_full : kstg_full, emptied = is_v ? vstg_free : kstg_free;
+    const uint32_t full0 = is_v ? vfull : kfull, free0 = is_v ? vfree : kfree;
+    constexpr int CPR = D / 8, TPI = 32 / CPR;        // chunks of a row, tokens per warp access
+    constexpr int NU = GP / 2 / TPI, U = NU < 8 ? NU : 8;   // accesses per page and warp, in flight
+    const int tl = half * (GP / 2) + lane / CPR, c = lane % CPR;
+    auto wait = [&](uint32_t bar, uint32_t parity) {
+      int ok = 1;
+      if (lane == 0) ok = mbar_wait(bar, parity, abort_flag, p.status, p.wait_cycles);
+      ok = __shfl_sync(0xffffffffu, ok, 0);
+      return ok != 0 && mbar_try_wait(bar, parity);   // (every lane observes the phase it was told of)
+    };
+    int sg = sg0, item = lo, g = 0;
+    bool ok = true;
+    while (item < hi && ok) {
+      const int seg_end = min(hi, pre[sg + 1]);
+      for (int first = item; first < seg_end && ok; first += PG, ++g) {
+        const int ng = min(PG, seg_end - first), sr = g % NR;
+        if (g >= NR) ok = wait(free0 + 8 * sr, (g / NR - 1) & 1);
+        for (int pg = 0; pg < ng; ++pg) {
+          const int x = first + pg - lo, ss = x % NSP;
+          ok = ok && wait(landed + 8 * ss, (x / NSP) & 1);
+          if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+          const uint8_t* src = stg_gen + ss * STG + tl * D + c * 8;
+          uint8_t* dst = ring_gen + sr * SLOT + (c >> 3) * HS;
+#pragma unroll
+          for (int u0 = 0; u0 < NU; u0 += U) {
+            uint2 w[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) w[u] = *reinterpret_cast<const uint2*>(src + (u0 + u) * TPI * D);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const uint32_t x4[4] = {w[u].x & 0xffffu, w[u].x >> 16, w[u].y & 0xffffu, w[u].y >> 16};
+              uint32_t h[4];
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const __half2_raw v = __nv_cvt_fp8x2_to_halfraw2(static_cast<__nv_fp8x2_storage_t>(x4[e]), __NV_E4M3);
+                h[e] = *reinterpret_cast<const uint32_t*>(&v);
+              }
+              *reinterpret_cast<uint4*>(dst + tc5_sw(pg * GP + tl + (u0 + u) * TPI, c & 7)) = make_uint4(h[0], h[1], h[2], h[3]);
+            }
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(emptied + 8 * ss, 1);
+        }
+        if (!ok) break;
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs read the slot through the async proxy
+        __syncwarp();
+        if (lane == 0) mbar_arrive(full0 + 8 * sr, 1);
+      }
+      item = seg_end;
+      ++sg;
+      while (item < hi && pre[sg + 1] <= item) ++sg;
     }
   } else if (warp == kTc5QkWarp) {
     // ------------------------------------------------------------------ Q K^T issuer (one thread)
@@ -499,8 +517,10 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         while (item < hi && pre[sg + 1] <= item) ++sg;
       }
     }
+  }
   } else {
     // ------------------------------------------------------------------ softmax / epilogue warps
+    if constexpr (FP8) asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
     // Thread = query row (tensor-memory lane 32 * (warp % 4) + lane) and one half of the columns:
     // set h = warp / 4 takes columns 64h .. 64h+63 of every group (and half of Q, of O when it is
     // rescaled or read out).  The exponentials are the bottleneck of this path (one special-function
@@ -602,17 +622,36 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
               }
           }
           // ---- pass 1: the row's maximum over the group (own columns, then the partner's)
+          // (FP8: of the shifted exponents; NP page runs of PW columns per 32, each with its scales)
+          constexpr int PW = (FP8 && GP == 16) ? 16 : 32, NP = 32 / PW;
+          float kmul[2 * NP], vexp[2 * NP];
+          if constexpr (FP8) {
+#pragma unroll
+            for (int x = 0; x < 2 * NP; ++x) {
+              const int j = (col0 + x * PW) / GP, at = (g % kTc5MetaRing) * kTc5PgMax + j;
+              kmul[x] = j < ng ? scale2 * kscale_meta[at] : 1.f;
+              vexp[x] = j < ng ? static_cast<float>((__float_as_int(vscale_meta[at]) >> 23) - 127) : 0.f;
+            }
+          }
+          float mx_own = -INFINITY;
           float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
           for (int c = 0; c < 2; ++c)
             if (col0 + c * 32 < ncol) {
 #pragma unroll
-              for (int e = 0; e < 32; ++e) mx[e & 3] = fmaxf(mx[e & 3], __uint_as_float(sraw[32 * c + e]));
+              for (int e = 0; e < 32; ++e) {
+                mx[e & 3] = fmaxf(mx[e & 3], __uint_as_float(sraw[32 * c + e]));
+                if (FP8 && (e + 1) % PW == 0) {
+                  const int x = c * NP + e / PW;
+                  mx_own = fmaxf(mx_own, fmaf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])), kmul[x], vexp[x]));
+                  mx[0] = mx[1] = mx[2] = mx[3] = -INFINITY;
+                }
+              }
             }
-          const float mx_own = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+          if (!FP8) mx_own = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
           xmax[(b * 2 + h) * kRowsPerGroup + r] = mx_own;
           ok = pair_sync();
-          const float m_new = fmaxf(mx_own, xmax[(b * 2 + (h ^ 1)) * kRowsPerGroup + r]) * scale2;
+          const float m_new = fmaxf(mx_own, xmax[(b * 2 + (h ^ 1)) * kRowsPerGroup + r]) * (FP8 ? 1.f : scale2);
           float corr = 1.f;
           if (m_new > m_ref + kTc5Tau || (m_ref == -INFINITY && m_new > -INFINITY)) {
             corr = (m_ref == -INFINITY) ? 0.f : ex2(m_ref - m_new);
@@ -649,16 +688,22 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                 uint32_t w[16];
 #pragma unroll
                 for (int e = 0; e < 16; ++e) {
-                  const float p0 = ex2(fmaf(__uint_as_float(sraw[32 * c + 2 * e]), scale2, -ms));
-                  const float p1 = ex2(fmaf(__uint_as_float(sraw[32 * c + 2 * e + 1]), scale2, -ms));
+                  const int x = c * NP + 2 * e / PW;
+                  const float mul = FP8 ? kmul[x] : scale2, add = FP8 ? vexp[x] - ms : -ms;
+                  const float p0 = ex2(fmaf(__uint_as_float(sraw[32 * c + 2 * e]), mul, add));
+                  const float p1 = ex2(fmaf(__uint_as_float(sraw[32 * c + 2 * e + 1]), mul, add));
                   sum[e & 3] += p0 + p1;
                   w[e] = FP8 ? pack_f16(p0, p1) : pack_bf16(p0, p1);
+                  if (FP8 && (2 * e + 2) % PW == 0) {     // the page run's sum, without the value scale
+                    l = fmaf((sum[0] + sum[1]) + (sum[2] + sum[3]), __int_as_float((127 - static_cast<int>(vexp[x])) << 23), l);
+                    sum[0] = sum[1] = sum[2] = sum[3] = 0.f;
+                  }
                 }
                 tc5_st16(s_addr + col0 / 2 + 16 * c, w);
               }
             }
             tc5_wait_st();
-            l += (sum[0] + sum[1]) + (sum[2] + sum[3]);
+            if (!FP8) l += (sum[0] + sum[1]) + (sum[2] + sum[3]);
           }
         }
         if (!ok) break;
@@ -729,7 +774,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     if ((warp == kTc5KWarp || warp == kTc5VWarp) && lane == 0) {
       // (FP8 pages: the copies land in the staging slots)
       const uint32_t full0 = FP8 ? (warp == kTc5VWarp ? vstg_full : kstg_full) : (warp == kTc5VWarp ? vfull : kfull);
-      constexpr int NSL = FP8 ? NSTG : NR;
+      constexpr int NSL = FP8 ? NSP : NR;
       for (int sl = 0; sl < NSL; ++sl) {
         if (issued < sl) continue;
         const int gl = issued - (issued - sl) % NSL;

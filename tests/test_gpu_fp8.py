@@ -99,6 +99,35 @@ def test_fp8_pages_zero_codes_and_a_block_off_its_alignment(g, d):
     assert_cache_equal(gl, o, cfg)
 
 
+@pytest.mark.parametrize("g,d", [(16, 64), (32, 64), (64, 64), (16, 128), (32, 128), (64, 128)])
+def test_fp8_pages_of_very_different_scales(g, d):
+    """Neighbouring pages whose key and value scales differ (2^-6 .. 2^2 and 2^-6 .. 2^5), more pages than the staging
+    rings hold, groups that end inside a run of 32 columns."""
+    from paper_2604_12056_b200.layer import LosaLayer, to_device
+    cfg = wl.config("c2", page_size=g, head_dim=d, n_q_heads=8, n_kv_heads=2, kv_lens=(61 * g - 3, 7 * g), steps=2, topk=3,
+                    block_size=16, m_active=3)
+    w = wl.Workload(cfg)
+    rng = np.random.default_rng(5)
+    for pool, factors in ((w.k_pages, (0.25, 1.0, 4.0)), (w.v_pages, (0.03, 1.0, 30.0, 1000.0))):
+        f = rng.choice(factors, size=pool.shape[:2]).astype(np.float32)
+        pool[...] = wl.f32_to_bf16_bits(wl.bf16_bits_to_f32(pool) * f[:, :, None, None])
+    gl = LosaLayer(cfg, w.k_pages, w.v_pages, w.page_table, w.kv_len, fp8_kv=True)
+    o = OracleFp8Layer(w)
+    assert_cache_equal(gl, o, cfg)
+    assert len(np.unique(o.k_scale)) > 2 and len(np.unique(o.v_scale)) > 3
+    for inp in w.block_steps():
+        gl.run_step(to_device(inp.q), to_device(inp.k_blk), to_device(inp.v_blk), to_device(inp.m_per_seq))
+        snap, ref = gl.snapshot(), o.run_step(inp)
+        assert gl.ctx.poll_status() == 0
+        for key in ("act", "na", "topk", "up", "uc"):
+            assert (snap[key] == ref[key]).all(), key
+        # P is rounded to 11 significant bits, numerator only: an error of at most 2^-11 of the weighted mean of |v|
+        # (fp32 sums and 2^x add far less); the reused rows of the second step carry that of the first
+        vmax = np.nanmax(np.abs(wl.bf16_bits_to_f32(w.v_pages)))
+        assert (np.abs(snap["o_p"] - ref["o_p"]) <= 2.0 ** -11 * vmax + 1e-4 * np.abs(ref["o_p"])).all()
+        assert (np.abs(snap["lse_p"] - ref["lse_p"]) <= 1e-3).all()
+
+
 def test_fp8_cache_dense_mode_and_two_row_groups():
     cfg = wl.config("c4", kv_lens=(64 * 40 + 17,), steps=2, topk=8, m_active=40, heavy_frac=0.0)
     run_fp8_blocks(cfg)
