@@ -46,7 +46,7 @@ struct AttnParams {
   int32_t* status;
   const float* k_scale;   // FP8 pages: [n_phys, H_kv] power-of-two scales (else null)
   const float* v_scale;
-  int N, B, Hq, Hkv, G, Pmax, n_phys, n_rg, n_seg, n_ctas;
+  int N, B, Hq, Hkv, G, Pmax, page, n_phys, n_rg, n_seg, n_ctas;
   float sm_scale;
   long long wait_cycles;  // bound of every mbarrier wait of the bf16 main kernel, in SM clock cycles
 };
@@ -114,129 +114,7 @@ template <int C> __device__ __forceinline__ void st_state(void* base, int bf16, 
   }
 }
 
-// ===================================================================== fp32 / CUDA-core kernel
-template <typename T, int D, int GP>
-__global__ void __launch_bounds__(256, 1) attn_simt_kernel(AttnParams p) {
-  grid_dep_wait();
-  extern __shared__ __align__(16) float sm[];
-  float* Ks = sm;                         // [GP][D]
-  float* Vs = Ks + GP * D;                // [GP][D]
-  float* Qs = Vs + GP * D;                // [128][D]
-  float* Os = Qs + kRowsPerGroup * D;     // [128][D]
-  float* Ms = Os + kRowsPerGroup * D;     // [128]
-  float* Ls = Ms + kRowsPerGroup;         // [128]
-  int* pre = reinterpret_cast<int*>(Ls + kRowsPerGroup);   // [n_seg + 1]
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (warp == 0) segment_prefix(pre, p.n_seg, p.n_rg, p.Hkv, p.G, p.n_active, p.union_count, p.B, lane);
-  __syncthreads();
-  const long long T_all = pre[p.n_seg];
-  const int lo = static_cast<int>(cta_lo(T_all, blockIdx.x, p.n_ctas));
-  const int hi = static_cast<int>(cta_lo(T_all, blockIdx.x + 1, p.n_ctas));
-  if (lo >= hi) return;
-  int sg = 0;
-  while (pre[sg + 1] <= lo) ++sg;
-  const T* q = static_cast<const T*>(p.q);
-  const T* kp = static_cast<const T*>(p.k_pages);
-  const T* vp = static_cast<const T*>(p.v_pages);
-  int item = lo;
-  while (item < hi) {
-    const int seg_end = min(hi, pre[sg + 1]);
-    const int n_sk = p.n_seg / p.n_rg, rg = sg / n_sk, sk = sg % n_sk, s = sk / p.Hkv, kh = sk % p.Hkv;
-    const int rows = rows_in_group(clamp_active(p.n_active[s], p.B), p.G, rg);
-    const int len = p.kv_len[s];
-    __syncthreads();
-    for (int idx = tid * 8; idx < rows * D; idx += 256 * 8) {
-      const int r = idx / D, j = idx % D;
-      const int row = rg * kRowsPerGroup + r, a = row / p.G, gi = row % p.G;
-      int tok = p.active_idx[s * p.B + a];
-      if (tok < 0 || tok >= p.B) { set_status(p.status, LOSA_ERR_BOUNDS); tok = 0; }
-      float v[8];
-      load8(q + ((static_cast<size_t>(s) * p.B + tok) * p.Hq + kh * p.G + gi) * D + j, v);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) { Qs[idx + e] = v[e]; Os[idx + e] = 0.f; }
-    }
-    for (int r = tid; r < rows; r += 256) { Ms[r] = -INFINITY; Ls[r] = 0.f; }
-    for (int u = item - pre[sg]; u < seg_end - pre[sg]; ++u) {
-      int page = p.union_pages[static_cast<size_t>(sk) * p.Pmax + u];
-      bool ok = page >= 0 && page < p.Pmax;
-      int phys = ok ? p.page_table[static_cast<size_t>(s) * p.Pmax + page] : 0;
-      ok = ok && phys >= 0 && phys < p.n_phys;
-      const int valid = ok ? min(GP, len - page * GP) : 0;
-      if (!ok || valid <= 0) { set_status(p.status, LOSA_ERR_BOUNDS); continue; }
-      __syncthreads();
-      const size_t off = static_cast<size_t>(phys) * p.stride_page + static_cast<size_t>(kh) * p.stride_head;
-      for (int idx = tid * 8; idx < GP * D; idx += 256 * 8) {
-        const int t = idx / D, j = idx % D;
-        float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, b[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        if (t < valid) {
-          load8(kp + off + static_cast<size_t>(t) * p.stride_tok + j, a);
-          load8(vp + off + static_cast<size_t>(t) * p.stride_tok + j, b);
-        }
-#pragma unroll
-        for (int e = 0; e < 8; ++e) { Ks[idx + e] = a[e]; Vs[idx + e] = b[e]; }
-      }
-      __syncthreads();
-      for (int r = warp; r < rows; r += 8) {
-        constexpr int TPL = (GP + 31) / 32;
-        float sc[TPL];
-#pragma unroll
-        for (int w = 0; w < TPL; ++w) {
-          const int t = lane + 32 * w;
-          float dot = 0.f;
-          if (t < valid) {
-            const float* kr = Ks + t * D;
-            const float* qr = Qs + r * D;
-#pragma unroll 8
-            for (int j = 0; j < D; ++j) {
-              const int jj = (j + lane) & (D - 1);
-              dot = fmaf(qr[jj], kr[jj], dot);
-            }
-          }
-          sc[w] = (t < valid) ? dot * p.sm_scale : -INFINITY;
-        }
-        float mx = sc[0];
-#pragma unroll
-        for (int w = 1; w < TPL; ++w) mx = fmaxf(mx, sc[w]);
-        mx = warp_max(mx);
-        const float m_old = Ms[r], m_new = fmaxf(m_old, mx);
-        const float corr = expf(m_old - m_new);
-        float pw[TPL], ps = 0.f;
-#pragma unroll
-        for (int w = 0; w < TPL; ++w) { pw[w] = expf(sc[w] - m_new); ps += pw[w]; }
-        ps = warp_sum(ps);
-        float acc[D / 32];
-#pragma unroll
-        for (int c = 0; c < D / 32; ++c) acc[c] = Os[r * D + lane + 32 * c] * corr;
-        for (int t = 0; t < valid; ++t) {
-          float pt = pw[0];
-#pragma unroll
-          for (int w = 1; w < TPL; ++w) pt = (t >= 32 * w) ? pw[w] : pt;
-          pt = __shfl_sync(0xffffffffu, pt, t & 31);
-#pragma unroll
-          for (int c = 0; c < D / 32; ++c) acc[c] = fmaf(pt, Vs[t * D + lane + 32 * c], acc[c]);
-        }
-#pragma unroll
-        for (int c = 0; c < D / 32; ++c) Os[r * D + lane + 32 * c] = acc[c];
-        __syncwarp();
-        if (lane == 0) { Ms[r] = m_new; Ls[r] = Ls[r] * corr + ps; }
-        __syncwarp();
-      }
-    }
-    __syncthreads();
-    for (int r = tid; r < rows; r += 256) {
-      float* rec = record_base(p.partials, blockIdx.x + sg, r / kTileRows, D);
-      rec[r % kTileRows] = Ms[r];
-      rec[kTileRows + r % kTileRows] = Ls[r];
-    }
-    for (int idx = tid; idx < rows * D; idx += 256) {
-      const int r = idx / D;
-      record_base(p.partials, blockIdx.x + sg, r / kTileRows, D)[2 * kTileRows + (r % kTileRows) * D + idx % D] = Os[idx];
-    }
-    item = seg_end;
-    ++sg;
-    while (item < hi && pre[sg + 1] <= item) ++sg;
-  }
-}
+#include "sparse_prefix_attn_f32.cuh"
 
 // ===================================================================== combine kernel
 // grid (n_seg, 8): warp = one query row of the segment's row group at a time.  The CTAs whose item range
@@ -247,7 +125,7 @@ __global__ void __launch_bounds__(256, 1) attn_simt_kernel(AttnParams p) {
 // Merge of the partial records of row r of segment sg by one warp: returns the un-normalised
 // output columns lane * C + c in acc, the reference maximum M and the sum of weights Lsum.
 template <int D, bool LOG2>
-__device__ __forceinline__ void merge_records(const AttnParams& p, int sg, int r, int start, int end, long long T_all,
+__device__ __forceinline__ void merge_records(const AttnParams& p, int n_ctas, int sg, int r, int start, int end, long long T_all,
                                               int lane, float (&acc)[D / 32], float& M, float& Lsum) {
   constexpr int C = D / 32;
   const int tile = r / kTileRows, rr = r % kTileRows;
@@ -256,17 +134,17 @@ __device__ __forceinline__ void merge_records(const AttnParams& p, int sg, int r
   M = -INFINITY;
   Lsum = 0.f;
   if (end <= start) return;
-  int b0 = static_cast<int>((static_cast<long long>(start) * p.n_ctas) / T_all);
-  while (b0 + 1 < p.n_ctas && cta_lo(T_all, b0 + 1, p.n_ctas) <= start) ++b0;
-  int b1 = static_cast<int>((static_cast<long long>(end - 1) * p.n_ctas) / T_all);   // last CTA that can meet it
-  while (b1 + 1 < p.n_ctas && cta_lo(T_all, b1 + 1, p.n_ctas) < end) ++b1;
+  int b0 = static_cast<int>((static_cast<long long>(start) * n_ctas) / T_all);
+  while (b0 + 1 < n_ctas && cta_lo(T_all, b0 + 1, n_ctas) <= start) ++b0;
+  int b1 = static_cast<int>((static_cast<long long>(end - 1) * n_ctas) / T_all);   // last CTA that can meet it
+  while (b1 + 1 < n_ctas && cta_lo(T_all, b1 + 1, n_ctas) < end) ++b1;
   const int n_pairs = b1 - b0 + 1;
   // record of piece x, or null when CTA b0 + x has no page of this segment
   auto record_of = [&](int x) -> const float* {
     if (x >= n_pairs) return nullptr;
     const int b = b0 + x;
-    const long long lo = max(cta_lo(T_all, b, p.n_ctas), static_cast<long long>(start));
-    const long long hi = min(cta_lo(T_all, b + 1, p.n_ctas), static_cast<long long>(end));
+    const long long lo = max(cta_lo(T_all, b, n_ctas), static_cast<long long>(start));
+    const long long hi = min(cta_lo(T_all, b + 1, n_ctas), static_cast<long long>(end));
     if (hi <= lo) return nullptr;
     return record_base(p.partials, b + sg, tile, D);
   };
@@ -321,6 +199,7 @@ __global__ void __launch_bounds__(256) attn_combine_kernel(AttnParams p) {
   }
   __syncthreads();
   constexpr int C = D / 32;
+  const int n_ctas = LOG2 ? p.n_ctas : f32_ctas(pre[p.n_seg], p.n_ctas, p.page);   // CTAs of the main kernel that share the list
   for (int r = blockIdx.y * 8 + warp; r < rows; r += gridDim.y * 8) {   // few CTAs per segment: most row blocks are empty on most steps
     const int row = rg * kRowsPerGroup + r, a = row / p.G, gi = row % p.G;
     const int tok = p.active_idx[s * p.B + a];
@@ -329,7 +208,7 @@ __global__ void __launch_bounds__(256) attn_combine_kernel(AttnParams p) {
     float acc[C], M, Lsum;
     // (PRE: the prefix left by the tensor-core kernel is that of the charged list; a segment's pages follow its pad)
     const int pad = (PRE && pre[sg + 1] > pre[sg]) ? segment_pad(rows) : 0;
-    merge_records<D, LOG2>(p, sg, r, pre[sg] + pad, pre[sg + 1], pre[p.n_seg], lane, acc, M, Lsum);
+    merge_records<D, LOG2>(p, n_ctas, sg, r, pre[sg] + pad, pre[sg + 1], pre[p.n_seg], lane, acc, M, Lsum);
     const bool empty = !(Lsum > 0.f);
     const float inv = empty ? 0.f : 1.f / Lsum;
 #pragma unroll
@@ -401,7 +280,7 @@ __global__ void __launch_bounds__(kFinishThreads) attn_finish_kernel(AttnParams 
     float acc[C], M, Lsum;
     const int v0 = p.seg_prefix[sg], v1 = p.seg_prefix[sg + 1];      // of the charged list: the segment's pages follow its pad
     const int pad = v1 > v0 ? segment_pad(rows_in_group(clamp_active(p.n_active[s], p.B), p.G, rg)) : 0;
-    merge_records<D, true>(p, sg, r, v0 + pad, v1, p.seg_prefix[p.n_seg], lane, acc, M, Lsum);
+    merge_records<D, true>(p, p.n_ctas, sg, r, v0 + pad, v1, p.seg_prefix[p.n_seg], lane, acc, M, Lsum);
     const bool empty = !(Lsum > 0.f);
     const float inv = empty ? 0.f : 1.f / Lsum;
     Lp = empty ? -INFINITY : (M + log2f(Lsum)) * kLn2;
@@ -544,16 +423,16 @@ int32_t launch_tc5(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool with
   return after_launch(c);
 }
 
-template <typename T, int D, int GP>
-int32_t launch_simt(losa_ctx* c, const AttnParams& ap, cudaStream_t st) {
-  const size_t smem = (static_cast<size_t>(2) * GP * D + 2 * kRowsPerGroup * D + 2 * kRowsPerGroup) * sizeof(float) +
-                      (ap.n_seg + 1) * sizeof(int);
+template <int D, int GP>
+int32_t launch_f32(losa_ctx* c, const AttnParams& ap, cudaStream_t st) {
+  constexpr int smem = sizeof(F32Smem<D>);
+  static_assert(smem <= kSmemBudget, "shared memory of the fp32 stage-4 kernel");
   if (!(c->attn_attr_set & 1)) {
-    LOSA_CUDA_TRY(c, cudaFuncSetAttribute(attn_simt_kernel<T, D, GP>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    LOSA_CUDA_TRY(c, cudaFuncSetAttribute(attn_f32_kernel<D, GP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     c->attn_attr_set |= 1;
   }
   if (c->profile) LOSA_CUDA_TRY(c, cudaEventRecord(c->ev_begin, st));
-  launch_k(attn_simt_kernel<T, D, GP>, ap.n_ctas, 256, smem, st, ap);
+  launch_k(attn_f32_kernel<D, GP>, ap.n_ctas, kF32Threads, smem, st, ap);
   if (c->profile) LOSA_CUDA_TRY(c, cudaEventRecord(c->ev_end, st));
   int32_t rc = after_launch(c);
   if (rc != LOSA_OK) return rc;
@@ -572,9 +451,9 @@ int32_t dispatch_page(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool w
     }
   }
   switch (c->shape.page_size) {
-    case 16: return bf ? launch_tc5<D, 16, false>(c, ap, st, with_combine) : launch_simt<float, D, 16>(c, ap, st);
-    case 32: return bf ? launch_tc5<D, 32, false>(c, ap, st, with_combine) : launch_simt<float, D, 32>(c, ap, st);
-    default: return bf ? launch_tc5<D, 64, false>(c, ap, st, with_combine) : launch_simt<float, D, 64>(c, ap, st);
+    case 16: return bf ? launch_tc5<D, 16, false>(c, ap, st, with_combine) : launch_f32<D, 16>(c, ap, st);
+    case 32: return bf ? launch_tc5<D, 32, false>(c, ap, st, with_combine) : launch_f32<D, 32>(c, ap, st);
+    default: return bf ? launch_tc5<D, 64, false>(c, ap, st, with_combine) : launch_f32<D, 64>(c, ap, st);
   }
 }
 
@@ -618,6 +497,7 @@ int32_t launch_sparse_prefix_attn(losa_ctx* c, const void* q, const losa_kv_t* k
   ap.Hkv = sh.n_kv_heads;
   ap.G = sh.n_q_heads / sh.n_kv_heads;
   ap.Pmax = sh.max_pages_per_seq;
+  ap.page = sh.page_size;
   ap.n_phys = kv->n_phys_pages;
   ap.n_rg = c->lay.n_row_groups;
   ap.n_seg = c->lay.n_segments;

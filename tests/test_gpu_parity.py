@@ -356,6 +356,40 @@ def test_many_rows_per_kv_head_fp32():
     run_blocks(cfg, modes=("losa",))
 
 
+@pytest.mark.parametrize("g,d,m,G", [(16, 64, 1, 1), (32, 128, 4, 4), (64, 64, 5, 4), (16, 128, 8, 4), (32, 64, 11, 3), (64, 128, 16, 4), (32, 128, 13, 5), (16, 64, 16, 8)])
+def test_fp32_attention_by_rows_per_kv_head(g, d, m, G):
+    """The fp32 stage-4 kernel at 1, 16, 20, 32, 33, 64, 65 and 128 query rows, odd page counts, empty and one-token prefixes."""
+    cfg = wl.config("c1", n_q_heads=2 * G, n_kv_heads=2, head_dim=d, page_size=g, kv_lens=(23 * g + 5, 0, 1, 3 * g), block_size=16,
+                    steps=3, topk=7, m_active=m, hidden_width=0)
+    run_blocks(cfg)
+
+
+def test_fp32_attention_over_more_pages_than_a_cta_resolves_at_once():
+    """48,000 pages: more than 256 for every CTA; compared with softmax in float64."""
+    import torch
+    from paper_2604_12056_b200.layer import LosaLayer
+    g, d, P, N = 16, 64, 16000, 3
+    cfg = wl.config("c1", n_q_heads=4, n_kv_heads=1, head_dim=d, page_size=g, kv_lens=(P * g - 7,) * N, block_size=2, steps=1,
+                    topk=4, m_active=1, hidden_width=0)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(3)
+    kp, vp = (torch.randn(N * P, 1, g, d, generator=gen, device="cuda") for _ in range(2))
+    q = torch.randn(N, 2, 4, d, generator=gen, device="cuda")
+    kb, vb = (torch.randn(N, 2, 1, d, generator=gen, device="cuda") for _ in range(2))
+    table = torch.randperm(N * P, generator=gen, device="cuda").to(torch.int32).reshape(N, P).contiguous()
+    kv_len = torch.full((N,), P * g - 7, dtype=torch.int32, device="cuda")
+    layer = LosaLayer(cfg, kp, vp, table, kv_len)
+    layer.run_step(q, kb, vb, torch.ones(N, dtype=torch.int32, device="cuda"))
+    assert layer.ctx.poll_status() == 0
+    for s in range(N):
+        k, v = (t[table[s].long()].reshape(-1, d)[:P * g - 7].double() for t in (kp, vp))
+        sc = q[s].double() @ k.T * cfg.sm_scale
+        want = torch.softmax(sc, -1) @ v
+        # 256,000 terms of weight about 1e-6 that cancel: fp32 sums of n terms of size 1e-6, n^0.5 roundings of 2^-24 relative to sum |p v|
+        assert (layer.o_p[s] - want).abs().max() < 1e-6
+        assert (layer.lse_p[s] - torch.logsumexp(sc, -1)).abs().max() < 1e-5
+
+
 def test_multi_block_append():
     cfg = wl.config("c5", kv_lens=(200, 90, 64), n_blocks=3, steps=3, topk=4)
     run_blocks(cfg, n_blocks=3)
