@@ -318,33 +318,38 @@ int32_t losa_denoise_step(losa_ctx* ctx, const void* q, const void* k_blk, const
   if (!aligned16(q) || !aligned16(k_blk) || !aligned16(v_blk) || !aligned16(out) || !aligned16(state->q_prev) ||
       !aligned16(state->o_p))
     return LOSA_ERR_UNSUPPORTED;
-  if (!ctx->side_stream) {
-    // lowest priority: when CTAs of both streams are pending, those of stages 1-4 go first
-    int prio_lo = 0, prio_hi = 0;
-    LOSA_CUDA_TRY(ctx, cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi));
-    LOSA_CUDA_TRY(ctx, cudaStreamCreateWithPriority(&ctx->side_stream, cudaStreamNonBlocking, prio_lo));
-    LOSA_CUDA_TRY(ctx, cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
-    LOSA_CUDA_TRY(ctx, cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming));
-  }
   cudaStream_t st = as_stream(stream);
   const losa_shape_t& sh = ctx->shape;
-  // fork: the in-block attention needs nothing from stages 1-4
-  LOSA_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_fork, st));
-  LOSA_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->side_stream, ctx->ev_fork, 0));
-  rc = launch_block_attn(ctx, q, k_blk, v_blk, ctx->side_stream);
-  if (rc != LOSA_OK) return rc;
-  LOSA_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_join, ctx->side_stream));
   int32_t* slot_map = reinterpret_cast<int32_t*>(ctx->ws + ctx->lay.slot_map);
+  // The in-block attention needs nothing from stages 1-4.  Where the selection ends in the candidate
+  // refinement, that kernel's grid carries it; elsewhere (fp32, long lists) it runs on a second stream.
+  const BlockInputs blk = {q, k_blk, v_blk};
+  const bool fork = !selects_by_refinement(ctx, k, ctx->pooled_selection);
+  if (fork) {
+    if (!ctx->side_stream) {
+      // lowest priority: when CTAs of both streams are pending, those of stages 1-4 go first
+      int prio_lo = 0, prio_hi = 0;
+      LOSA_CUDA_TRY(ctx, cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi));
+      LOSA_CUDA_TRY(ctx, cudaStreamCreateWithPriority(&ctx->side_stream, cudaStreamNonBlocking, prio_lo));
+      LOSA_CUDA_TRY(ctx, cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
+      LOSA_CUDA_TRY(ctx, cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming));
+    }
+    LOSA_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_fork, st));
+    LOSA_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->side_stream, ctx->ev_fork, 0));
+    rc = launch_block_attn(ctx, q, k_blk, v_blk, ctx->side_stream);
+    if (rc != LOSA_OK) return rc;
+    LOSA_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_join, ctx->side_stream));
+  }
   rc = launch_select_active(ctx, q, state->q_prev, sh.n_q_heads * sh.head_dim, m_per_seq, state->step,
                             buf->active_idx, buf->n_active, nullptr, st, 0.0, slot_map);
   bool union_done = false;                              // stage 3 written by the selection kernel itself
-  if (rc == LOSA_OK) rc = launch_page_scores_topk(ctx, q, kv, buf->active_idx, buf->n_active, state->step, k, buf->topk_pages, nullptr, st, ctx->pooled_selection, true, buf->union_pages, buf->union_count, &union_done);
+  if (rc == LOSA_OK) rc = launch_page_scores_topk(ctx, q, kv, buf->active_idx, buf->n_active, state->step, k, buf->topk_pages, nullptr, st, ctx->pooled_selection, true, buf->union_pages, buf->union_count, &union_done, fork ? nullptr : &blk);
   if (rc == LOSA_OK && !union_done) rc = launch_page_union(ctx, buf->topk_pages, buf->active_idx, buf->n_active, k, kv->kv_len, state->step, buf->union_pages, buf->union_count, st);
   if (rc == LOSA_OK) rc = launch_sparse_prefix_attn(ctx, q, kv, buf->active_idx, buf->n_active, buf->union_pages, buf->union_count, state, st, true);
-  // join (also when a launch above failed: the forked kernel must not be left reading the caller's
-  // buffers, nor a capture be left with an unjoined branch), then one pass over the rows: (merge of
+  // (join, also when a launch above failed: the forked kernel must not be left reading the caller's
+  // buffers, nor a capture be left with an unjoined branch;) then one pass over the rows: (merge of
   // the partial records,) merge with the block part, commit
-  const cudaError_t joined = cudaStreamWaitEvent(st, ctx->ev_join, 0);
+  const cudaError_t joined = fork ? cudaStreamWaitEvent(st, ctx->ev_join, 0) : cudaSuccess;
   if (rc != LOSA_OK) return rc;
   LOSA_CUDA_TRY(ctx, joined);
   if (finish_fuses_combine(ctx)) return launch_attn_finish(ctx, q, buf->active_idx, buf->n_active, slot_map, state, out, lse_out_opt, st);

@@ -112,11 +112,16 @@ inline void launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sme
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  // one shared-memory / L1 split for all kernels: an SM changes its split only when it is empty, so a
+  // kernel that asks for much shared memory could not start beside a predecessor that asks for little
+  // (the page-bound kernel's last CTA came in 5 us later)
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  attr[1].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);   // the error, if any, is read by after_launch()
 }
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -125,6 +130,15 @@ __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.w
 // grid has completed and its writes are visible.  Only for kernels whose whole grid is resident at
 // once and whose successor has a prologue worth hiding.
 __device__ __forceinline__ void grid_dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Ticket of a "last one finishes" scheme: releases what this thread, and what the threads it has met
+// at a CTA barrier, wrote before, and acquires what the earlier tickets released (__threadfence on
+// both sides is the stronger and slower sequentially consistent fence).
+__device__ __forceinline__ unsigned int atomic_inc_acq_rel(unsigned int* p, unsigned int wrap) {
+  unsigned int old;
+  asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(wrap) : "memory");
+  return old;
+}
 
 __device__ __forceinline__ void set_status(int32_t* status, int32_t code) { atomicCAS(status, 0, code); }
 
@@ -224,7 +238,21 @@ __device__ __forceinline__ int rows_in_group(int n_active, int G, int rg) {
   const int r = n_active * G - rg * kRowsPerGroup;
   return r < 0 ? 0 : (r > kRowsPerGroup ? kRowsPerGroup : r);
 }
-__device__ __forceinline__ long long cta_lo(long long T, int b, int n) { return (T * b) / n; }
+// floor(T * b / n); in 32 bits where the product fits (a 64-bit division is some 100 dependent instructions)
+__device__ __forceinline__ long long cta_lo(long long T, int b, int n) {
+  if (T < (1 << 22) && b <= 512) return static_cast<uint32_t>(T) * static_cast<uint32_t>(b) / static_cast<uint32_t>(n);
+  return (T * b) / n;
+}
+
+// CTAs of the tensor-core kernel that share a charged list of length V (page: tokens per page).  It takes
+// pages in groups of 128 tokens, and a group costs the same whatever it holds: short shares are
+// rounded up to whole groups, which costs the main kernel nothing and leaves the merge fewer records.
+__device__ __forceinline__ int tc5_ctas(long long V, int n_ctas, int page) {
+  const int pg = 128 / page, per = static_cast<int>((V + n_ctas - 1) / n_ctas);
+  if (per >= 8 * pg || per < 1) return n_ctas;
+  const int whole = (per + pg - 1) / pg * pg;
+  return static_cast<int>((V + whole - 1) / whole);
+}
 
 // The tensor-core kernel cuts a list in which every non-empty segment is charged segment_pad(rows)
 // items on top of its pages (placed before them): entering a segment costs a CTA about as much as

@@ -14,7 +14,13 @@ int32_t launch_page_scores_topk(losa_ctx* c, const void* q, const losa_kv_t* kv,
                                 const int32_t* active_idx, const int32_t* n_active,
                                 const int32_t* step, int32_t k, int32_t* topk_pages,
                                 float* topk_scores_opt, cudaStream_t st, int selector = 0, bool after_stage1 = false,
-                                int32_t* union_pages = nullptr, int32_t* union_count = nullptr, bool* union_done = nullptr);
+                                int32_t* union_pages = nullptr, int32_t* union_count = nullptr, bool* union_done = nullptr,
+                                const struct BlockInputs* blk = nullptr);
+// blk (whole-step call, only where selects_by_refinement): the selection's launch also computes the
+// in-block attention of these inputs into the workspace.
+struct BlockInputs { const void* q; const void* k_blk; const void* v_blk; };
+// bf16, lists of at most 512 pages, exact or pooled: bounds from the tensor cores, then the candidate refinement.
+bool selects_by_refinement(const losa_ctx* c, int32_t k, int selector);
 // union_pages / union_count / union_done (all three or none): where the selection can also write stage 3's
 // union (the bf16 candidate refinement, bitmaps of at most 256 words), it does so and sets *union_done;
 // otherwise *union_done is false and the caller launches stage 3 itself.

@@ -12,6 +12,7 @@
 //                        emits the set bits in ascending order with a popcount scan.
 #include <algorithm>
 
+#include "block_attn_mma.cuh"
 #include "kernels.h"
 
 namespace losa {
@@ -324,6 +325,8 @@ struct RefineParams {
   int32_t* union_pages;
   int32_t* union_count;
   int W;                          // words per bitmap, ceil(Pmax / 32) <= kSelBins
+  int slots;                      // CTAs per (sequence, head or KV head): active slots are dealt out round-robin
+  int blk_tiles;                  // row tiles of the in-block attention per (sequence, KV head)
 };
 
 // The set bits of a bitmap in shared memory, ascending, then -1 up to Pmax; the count.  All NT threads
@@ -369,7 +372,7 @@ __device__ __forceinline__ uint32_t prefix_word(int w, int P) {   // word w of t
   return (P >= lo + 32) ? 0xffffffffu : (P > lo ? ((1u << (P - lo)) - 1u) : 0u);
 }
 
-// One CTA of kSelThreads per (sequence, head, 1/8 of the active slots).  Per query: tau = lower edge
+// One CTA of kSelThreads per (sequence, head, share of the active slots).  Per query: tau = lower edge
 // of the histogram bin that holds the k-th largest LOWER bound; every page whose UPPER bound reaches
 // tau is a candidate (a superset of the exact top-k, ties included: the exact score lies between the
 // bounds); exact scores in the fixed order for the candidates (four lanes each), sort, emit.  More
@@ -382,9 +385,33 @@ __device__ __forceinline__ uint32_t prefix_word(int w, int P) {   // word w of t
 constexpr int kMaxPool = 16;     // heads per KV head the interface admits
 
 template <int D, bool POOLED>
+struct RefineSmem {
+  float qs[(POOLED ? kMaxPool : 1) * 2 * D];
+  unsigned long long ckey[kSelCap];
+  int cpage[kSelCap];
+  int hist[kSelBins];
+  uint32_t red[2][kSelThreads / 32];
+  int ncand, bstar;
+};
+
+// In a whole step the grid ends with the row tiles of the in-block attention (BK: its padded key
+// count).  It needs only the step's inputs, and these CTAs fill the gaps of a kernel that is bound by
+// latency.  On a second stream it was hidden as well, but the join in front of the step's last kernel
+// cost that kernel its early launch (4 us of idle GPU per step); in stage 1's launch it delayed stage
+// 2 (eight sequences: bounds from 12 us on instead of 7).
+template <int D, bool POOLED, int BK>
 __global__ void __launch_bounds__(kSelThreads, POOLED ? 4 : 6)
-topk_refine_kernel(RefineParams p) {
-  const int qid = blockIdx.x;
+topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
+  static_assert(kSelThreads == kMmaThreads, "one CTA size");
+  __shared__ __align__(16) union { RefineSmem<D, POOLED> r; BlockAttnSmem<D, BK> b; } sm;
+  const int qid = blockIdx.x, n_refine = p.N * (POOLED ? p.Hkv : p.Hq) * p.slots;
+  if (qid >= n_refine) {
+    const int t = qid - n_refine, sk = t / p.blk_tiles;
+    if (!(p.step && __ldcg(p.step + sk / p.Hkv) == 0)) grid_dep_trigger();      // (as below)
+    grid_dep_wait();
+    block_attn_mma_cta<D, BK, false>(bp, sm.b, t % p.blk_tiles, sk % p.Hkv, sk / p.Hkv);
+    return;
+  }
   const int pool = POOLED ? p.Hq / p.Hkv : 1, Hl = p.Hq / pool;
   const int h = (qid % Hl) * pool, s = (qid / Hl) % p.N, j0 = qid / (Hl * p.N);   // pooled: h = the group's first head
   // With stage 3 inside (whole-step call) the next kernel is stage 4, and the chain of launches
@@ -400,12 +427,13 @@ topk_refine_kernel(RefineParams p) {
   }
   grid_dep_wait();
   if (!p.union_bits) first_step = p.step && p.step[s] == 0;
-  __shared__ __align__(16) float qs[(POOLED ? kMaxPool : 1) * 2 * D];
-  __shared__ __align__(16) unsigned long long ckey[kSelCap];
-  __shared__ int cpage[kSelCap];
-  __shared__ int hist[kSelBins];
-  __shared__ uint32_t s_red[2][kSelThreads / 32];
-  __shared__ int s_ncand, s_bstar;
+  float* qs = sm.r.qs;
+  unsigned long long* ckey = sm.r.ckey;
+  int* cpage = sm.r.cpage;
+  int* hist = sm.r.hist;
+  uint32_t (&s_red)[2][kSelThreads / 32] = sm.r.red;
+  int& s_ncand = sm.r.ncand;
+  int& s_bstar = sm.r.bstar;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int kh = h / (p.Hq / p.Hkv);
   int na = first_step ? 0 : p.n_active[s];
@@ -431,7 +459,7 @@ topk_refine_kernel(RefineParams p) {
   const __nv_bfloat16* lo_base = p.kmin + static_cast<size_t>(kh) * D;
   const __nv_bfloat16* hi_base = p.kmax + static_cast<size_t>(kh) * D;
   const int u = lane & 3;
-  for (int a = j0; a < na; a += kSelSlots) {
+  for (int a = j0; a < na; a += p.slots) {
     const int tok = p.active_idx[s * p.B + a];
     if (tok < 0 || tok >= p.B) { if (tid == 0) set_status(p.status, LOSA_ERR_BOUNDS); continue; }
     float2* row2 = p.bounds + ((static_cast<size_t>(s) * p.B + a) * p.Hq + h) * p.score_stride;
@@ -676,15 +704,13 @@ topk_refine_kernel(RefineParams p) {
   if (!bits) return;
   // ---- stage 3: the last CTA of this (sequence, KV head) writes the union
   __syncthreads();                                 // every thread's marks precede ...
-  if (tid == 0) {
-    __threadfence();                               // ... this fence (cumulative), which precedes the ticket
+  if (tid == 0) {                                  // ... this thread's ticket, a release of all of them (cumulative)
     // CTAs of this (sequence, KV head) that hold a slot: all of them arrive here
-    const unsigned int n_grp = static_cast<unsigned int>((p.Hq / p.Hkv / pool) * min(na, static_cast<int>(gridDim.x) / (Hl * p.N)));
-    s_bstar = atomicInc(&p.union_tickets[s * p.Hkv + kh], n_grp - 1) == n_grp - 1 ? 1 : 0;
+    const unsigned int n_grp = static_cast<unsigned int>((p.Hq / p.Hkv / pool) * min(na, p.slots));
+    s_bstar = atomic_inc_acq_rel(&p.union_tickets[s * p.Hkv + kh], n_grp - 1) == n_grp - 1 ? 1 : 0;
   }
   __syncthreads();
   if (!s_bstar) return;
-  __threadfence();
   uint32_t* bm = reinterpret_cast<uint32_t*>(hist);
   for (int w = tid; w < p.W; w += kSelThreads) {
     bm[w] = atomicExch(bits + w, 0u);              // the marks were made in L2; all zero again for the next launch
@@ -815,18 +841,22 @@ int32_t topk_max_sortable(const losa_ctx* c) {
   return n;
 }
 
+bool selects_by_refinement(const losa_ctx* c, int32_t k, int selector) {
+  return c->shape.dtype == LOSA_BF16 && (selector == kSelectorExact || selector == kSelectorPooled) && k <= kSelCap &&
+         c->shape.max_pages_per_seq > 0;
+}
+
 int32_t launch_page_scores_topk(losa_ctx* c, const void* q, const losa_kv_t* kv,
                                 const int32_t* active_idx, const int32_t* n_active,
                                 const int32_t* step, int32_t k, int32_t* topk_pages,
                                 float* topk_scores_opt, cudaStream_t st, int selector, bool after_stage1,
-                                int32_t* union_pages, int32_t* union_count, bool* union_done) {
+                                int32_t* union_pages, int32_t* union_count, bool* union_done, const BlockInputs* blk) {
   if (union_done) *union_done = false;
   const losa_shape_t& sh = c->shape;
   if (sh.max_pages_per_seq == 0) return LOSA_OK;
   const bool pooled = selector == kSelectorPooled;
   const int pool = pooled ? sh.n_q_heads / sh.n_kv_heads : 1;
-  const bool bf = sh.dtype == LOSA_BF16;
-  if (bf && (selector == kSelectorExact || pooled) && k <= kSelCap) {
+  if (selects_by_refinement(c, k, selector)) {
     // bf16, exact lists (per query head, or per KV head from the group's maximum): bounds from the
     // tensor cores, exact scores for the candidates only
     int32_t rc = launch_page_bounds(c, q, kv, active_idx, n_active, step, st, false, after_stage1);
@@ -853,14 +883,20 @@ int32_t launch_page_scores_topk(losa_ctx* c, const void* q, const losa_kv_t* kv,
     rp.union_pages = union_pages;
     rp.union_count = union_count;
     if (with_union) *union_done = true;
-    const int queries = sh.batch * std::min<int>(sh.block_size, kSelSlots) * (sh.n_q_heads / pool);
-    if (pool > 1) {
-      if (sh.head_dim == 128) launch_k(topk_refine_kernel<128, true>, queries, kSelThreads, 0, st, rp);
-      else launch_k(topk_refine_kernel<64, true>, queries, kSelThreads, 0, st, rp);
-    } else {
-      if (sh.head_dim == 128) launch_k(topk_refine_kernel<128, false>, queries, kSelThreads, 0, st, rp);
-      else launch_k(topk_refine_kernel<64, false>, queries, kSelThreads, 0, st, rp);
-    }
+    // CTAs per (sequence, head): up to eight, but no more than are resident together - most slots are
+    // idle on most steps, and an idle CTA costs its dispatch (eight sequences of 32 heads: 2,048 CTAs for
+    // 768 busy ones kept the grid's tail waiting)
+    const int lists = sh.batch * (sh.n_q_heads / pool), resident = c->n_sms * (pool > 1 ? 4 : 6);
+    rp.slots = std::max(1, std::min({kSelSlots, sh.block_size, (resident + lists - 1) / lists}));
+    rp.blk_tiles = block_attn_tiles(sh);
+    const bool with_block = blk && blk->q;
+    const BlockAttnParams bp = with_block ? block_attn_params(c, blk->q, blk->k_blk, blk->v_blk) : BlockAttnParams{};
+    const int grid = lists * rp.slots + (with_block ? rp.blk_tiles * sh.n_kv_heads * sh.batch : 0);
+    with_block_attn_shape(sh, [&](auto d, auto bk) {
+      constexpr int D = decltype(d)::value, BK = decltype(bk)::value;
+      if (pool > 1) launch_k(topk_refine_kernel<D, true, BK>, grid, kSelThreads, 0, st, rp, bp);
+      else launch_k(topk_refine_kernel<D, false, BK>, grid, kSelThreads, 0, st, rp, bp);
+    });
     return after_launch(c);
   }
   int32_t rc = selector == kSelectorMma ? launch_page_bounds(c, q, kv, active_idx, n_active, step, st, true, after_stage1)

@@ -73,13 +73,11 @@ select_active_kernel(const T* __restrict__ x_cur, const T* __restrict__ x_prev, 
     t /= static_cast<double>(row_width);
     delta_ws[s * B + i] = t;
     if (delta_opt) delta_opt[s * B + i] = static_cast<float>(t);
-    __threadfence();
-    const unsigned int ticket = atomicInc(&counters[s], static_cast<unsigned int>(B - 1));
+    const unsigned int ticket = atomic_inc_acq_rel(&counters[s], static_cast<unsigned int>(B - 1));
     s_last = (ticket == static_cast<unsigned int>(B - 1));
   }
   __syncthreads();
   if (!s_last) return;
-  __threadfence();
   if (tid < B) {
     const double dv = *(reinterpret_cast<volatile double*>(delta_ws) + s * B + tid);
     s_delta[tid] = dv != dv ? static_cast<double>(INFINITY) : dv;    // NaN ranks as +inf: the order below stays total

@@ -118,10 +118,11 @@ template <int C> __device__ __forceinline__ void st_state(void* base, int bf16, 
 
 // ===================================================================== combine kernel
 // grid (n_seg, 8): warp = one query row of the segment's row group at a time.  The CTAs whose item range
-// meets the segment are consecutive; each of them left one record for the row's 16-row tile.  Lanes
-// take one piece each for the row maxima and sums, then the warp walks the pieces with the loads of
-// eight records issued together.  LOG2: partial maxima in base-2 units (tensor-core kernel) or
-// natural units (fp32 kernel).
+// meets the segment are consecutive; each of them left one record for the row's 16-row tile.  The
+// merge is a chain of dependent reads (latency bounds it), so lanes take one record's maximum and sum
+// each while the outputs of the first eight records are already on their way, and eight more are
+// requested at a time.  LOG2: partial maxima in base-2 units (tensor-core kernel) or natural units
+// (fp32 kernel).
 // Merge of the partial records of row r of segment sg by one warp: returns the un-normalised
 // output columns lane * C + c in acc, the reference maximum M and the sum of weights Lsum.
 template <int D, bool LOG2>
@@ -134,51 +135,56 @@ __device__ __forceinline__ void merge_records(const AttnParams& p, int n_ctas, i
   M = -INFINITY;
   Lsum = 0.f;
   if (end <= start) return;
-  int b0 = static_cast<int>((static_cast<long long>(start) * n_ctas) / T_all);
-  while (b0 + 1 < n_ctas && cta_lo(T_all, b0 + 1, n_ctas) <= start) ++b0;
-  int b1 = static_cast<int>((static_cast<long long>(end - 1) * n_ctas) / T_all);   // last CTA that can meet it
-  while (b1 + 1 < n_ctas && cta_lo(T_all, b1 + 1, n_ctas) < end) ++b1;
-  const int n_pairs = b1 - b0 + 1;
-  // record of piece x, or null when CTA b0 + x has no page of this segment
-  auto record_of = [&](int x) -> const float* {
-    if (x >= n_pairs) return nullptr;
-    const int b = b0 + x;
-    const long long lo = max(cta_lo(T_all, b, n_ctas), static_cast<long long>(start));
-    const long long hi = min(cta_lo(T_all, b + 1, n_ctas), static_cast<long long>(end));
-    if (hi <= lo) return nullptr;
-    return record_base(p.partials, b + sg, tile, D);
+  // the first and the last CTA whose range can meet start .. end - 1
+  auto cta_of = [&](int v) {
+    int b = T_all < (1 << 22) && n_ctas <= 512 ? static_cast<int>(static_cast<uint32_t>(v) * static_cast<uint32_t>(n_ctas) / static_cast<uint32_t>(T_all))
+                                              : static_cast<int>((static_cast<long long>(v) * n_ctas) / T_all);
+    while (b + 1 < n_ctas && cta_lo(T_all, b + 1, n_ctas) <= v) ++b;
+    return b;
   };
+  const int b0 = cta_of(start), n_pairs = cta_of(end - 1) - b0 + 1;
   for (int base = 0; base < n_pairs; base += 32) {
-    const float* rec = record_of(base + lane);
-    M = fmaxf(M, warp_max(rec ? rec[rr] : -INFINITY));
-  }
-  for (int base = 0; base < n_pairs; base += 32) {
-    const float* rec = record_of(base + lane);
-    float wj = 0.f, lj = 0.f;
-    if (rec) {
-      const float mj = rec[rr];
-      wj = (mj == -INFINITY) ? 0.f : (LOG2 ? exp2f(mj - M) : expf(mj - M));
-      lj = rec[kTileRows + rr];
+    // record of piece base + lane, or null when that CTA has no page of this segment
+    const float* rec = nullptr;
+    if (base + lane < n_pairs) {
+      const int b = b0 + base + lane;
+      const long long lo = max(cta_lo(T_all, b, n_ctas), static_cast<long long>(start));
+      const long long hi = min(cta_lo(T_all, b + 1, n_ctas), static_cast<long long>(end));
+      if (hi > lo) rec = record_base(p.partials, b + sg, tile, D);
     }
-    Lsum += warp_sum(lj * wj);
+    // the maxima, the sums and the outputs of the first U records are requested together
+    const float mj = rec ? rec[rr] : -INFINITY, lj = rec ? rec[kTileRows + rr] : 0.f;
+    constexpr int U = 8;
     const int n = min(32, n_pairs - base);
-    constexpr int U = 4;                            // records whose loads are in flight together
-    for (int i0 = 0; i0 < n; i0 += U) {
-      float w[U], v[U][C];
+    float v[U][C];
+    auto request = [&](int i0) {
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int i = i0 + u;
-        w[u] = (i < n) ? __shfl_sync(0xffffffffu, wj, i & 31) : 0.f;
         const unsigned long long addr = __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(rec), i & 31);
-        const float* src = reinterpret_cast<const float*>(addr) + 2 * kTileRows + rr * D + lane * C;
 #pragma unroll
         for (int c = 0; c < C; ++c) v[u][c] = 0.f;
-        if (w[u] != 0.f) ldv<C>(src, v[u]);
+        if (i < n && addr) ldv<C>(reinterpret_cast<const float*>(addr) + 2 * kTileRows + rr * D + lane * C, v[u]);
       }
+    };
+    request(0);
+    const float M_new = fmaxf(M, warp_max(mj));
+    const float keep = (M == -INFINITY) ? 0.f : (LOG2 ? exp2f(M - M_new) : expf(M - M_new));
+    const float wj = (mj == -INFINITY) ? 0.f : (LOG2 ? exp2f(mj - M_new) : expf(mj - M_new));
+    M = M_new;
+    Lsum = Lsum * keep + warp_sum(lj * wj);
 #pragma unroll
-      for (int u = 0; u < U; ++u)
+    for (int c = 0; c < C; ++c) acc[c] *= keep;
+    for (int i0 = 0; i0 < n; i0 += U) {
+      if (i0 > 0) request(i0);
 #pragma unroll
-        for (int c = 0; c < C; ++c) acc[c] = fmaf(v[u][c], w[u], acc[c]);
+      for (int u = 0; u < U; ++u) {
+        const float w = (i0 + u < n) ? __shfl_sync(0xffffffffu, wj, (i0 + u) & 31) : 0.f;
+        if (w != 0.f) {
+#pragma unroll
+          for (int c = 0; c < C; ++c) acc[c] = fmaf(v[u][c], w, acc[c]);
+        }
+      }
     }
   }
 }
@@ -199,7 +205,7 @@ __global__ void __launch_bounds__(256) attn_combine_kernel(AttnParams p) {
   }
   __syncthreads();
   constexpr int C = D / 32;
-  const int n_ctas = LOG2 ? p.n_ctas : f32_ctas(pre[p.n_seg], p.n_ctas, p.page);   // CTAs of the main kernel that share the list
+  const int n_ctas = LOG2 ? tc5_ctas(pre[p.n_seg], p.n_ctas, p.page) : f32_ctas(pre[p.n_seg], p.n_ctas, p.page);   // CTAs of the main kernel that share the list
   for (int r = blockIdx.y * 8 + warp; r < rows; r += gridDim.y * 8) {   // few CTAs per segment: most row blocks are empty on most steps
     const int row = rg * kRowsPerGroup + r, a = row / p.G, gi = row % p.G;
     const int tok = p.active_idx[s * p.B + a];
@@ -231,24 +237,24 @@ struct FinishParams {
   void* out;
   float* lse_out;
   int32_t* step;
-  const int32_t* slot_map;   // [N*B] slot of a block token in the active list, -1 = stable (null: look it up)
+  const int32_t* slot_map;   // [N*B] slot of a block token in the active list, -1 = stable
   size_t n_rows;
 };
 
 constexpr int kFinishThreads = 128;
 
 template <typename T, int D>
-__global__ void __launch_bounds__(kFinishThreads) attn_finish_kernel(AttnParams p, FinishParams f) {
+__global__ void __launch_bounds__(kFinishThreads, 5) attn_finish_kernel(AttnParams p, FinishParams f) {
   grid_dep_trigger();
   grid_dep_wait();
   constexpr int C = D / 32;
   const int lane = threadIdx.x & 31;
-  const size_t row = static_cast<size_t>(blockIdx.x) * (kFinishThreads / 32) + (threadIdx.x >> 5);
+  const uint32_t row_i = blockIdx.x * (kFinishThreads / 32) + (threadIdx.x >> 5);
+  const size_t row = row_i;
   if (blockIdx.x == 0)
     for (int s = threadIdx.x; s < p.N; s += kFinishThreads) f.step[s] += 1;
   if (row >= f.n_rows) return;
-  const int hq = static_cast<int>(row % p.Hq), tok = static_cast<int>((row / p.Hq) % p.B);
-  const int s = static_cast<int>(row / (static_cast<size_t>(p.Hq) * p.B));
+  const int hq = static_cast<int>(row_i % p.Hq), st = static_cast<int>(row_i / p.Hq), tok = st % p.B, s = st / p.B;   // (32-bit divisions)
   const int kh = hq / p.G, gi = hq % p.G;
   // operands that do not depend on the row being active: requested first (one vector access each)
   const T* q = static_cast<const T*>(f.q);
@@ -261,26 +267,21 @@ __global__ void __launch_bounds__(kFinishThreads) attn_finish_kernel(AttnParams 
   float a[C], Lp;
   ld_state<C>(p.o_p, p.o_p_bf16, row * D + lane * C, a);
   Lp = p.lse_p[row];
-  // the row's slot in the active list, if any (the list has at most B <= 64 entries)
-  int slot = -1;
-  if (f.slot_map) {
-    slot = f.slot_map[s * p.B + tok];
-    if (slot >= p.B) slot = -1;
-  } else {
-    const int na = clamp_active(p.n_active[s], p.B);
-    for (int base = 0; base < na && slot < 0; base += 32) {
-      const int i = base + lane;
-      const unsigned hit = __ballot_sync(0xffffffffu, i < na && p.active_idx[s * p.B + i] == tok);
-      if (hit) slot = base + __ffs(hit) - 1;
-    }
-  }
-  if (slot >= 0) {
+  // where an active row's records are, for the first row group: requested before the slot is known
+  int sg = s * p.Hkv + kh;
+  int v0 = p.seg_prefix[sg], v1 = p.seg_prefix[sg + 1];             // of the charged list: the segment's pages follow its pad
+  const int v_all = p.seg_prefix[p.n_seg], na = clamp_active(p.n_active[s], p.B);
+  const int slot = f.slot_map[s * p.B + tok];                       // in the active list (at most B entries), -1 = stable
+  if (slot >= 0 && slot < p.B) {
     const int rowk = slot * p.G + gi, rg = rowk / kRowsPerGroup, r = rowk % kRowsPerGroup;
-    const int sg = rg * (p.n_seg / p.n_rg) + s * p.Hkv + kh;
+    if (rg > 0) {
+      sg += rg * (p.n_seg / p.n_rg);
+      v0 = p.seg_prefix[sg];
+      v1 = p.seg_prefix[sg + 1];
+    }
     float acc[C], M, Lsum;
-    const int v0 = p.seg_prefix[sg], v1 = p.seg_prefix[sg + 1];      // of the charged list: the segment's pages follow its pad
-    const int pad = v1 > v0 ? segment_pad(rows_in_group(clamp_active(p.n_active[s], p.B), p.G, rg)) : 0;
-    merge_records<D, true>(p, p.n_ctas, sg, r, v0 + pad, v1, p.seg_prefix[p.n_seg], lane, acc, M, Lsum);
+    const int pad = v1 > v0 ? segment_pad(rows_in_group(na, p.G, rg)) : 0;
+    merge_records<D, true>(p, tc5_ctas(v_all, p.n_ctas, p.page), sg, r, v0 + pad, v1, v_all, lane, acc, M, Lsum);
     const bool empty = !(Lsum > 0.f);
     const float inv = empty ? 0.f : 1.f / Lsum;
     Lp = empty ? -INFINITY : (M + log2f(Lsum)) * kLn2;
@@ -528,6 +529,7 @@ int32_t launch_attn_finish(losa_ctx* c, const void* q, const int32_t* active_idx
   ap.Hq = sh.n_q_heads;
   ap.Hkv = sh.n_kv_heads;
   ap.G = sh.n_q_heads / sh.n_kv_heads;
+  ap.page = sh.page_size;
   ap.n_rg = c->lay.n_row_groups;
   ap.n_seg = c->lay.n_segments;
   ap.n_ctas = c->lay.n_ctas;

@@ -239,6 +239,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     for (int i = tid; i <= p.n_seg; i += NT) p.seg_prefix[i] = vpre[i];
   // this CTA's share of the charged list, mapped back to pages: the first page at or after a charged position
   const long long V_all = vpre[p.n_seg];
+  int sg0 = 0;                                       // (of the call below that is made last: the segment of the share's first page, or an empty one before it)
   auto page_at = [&](long long v) {
     if (v >= V_all) return pre[p.n_seg];
     int a = 0, b = p.n_seg;                          // vpre[a] <= v < vpre[b]
@@ -246,17 +247,18 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       const int mid = (a + b) >> 1;
       if (vpre[mid] <= v) a = mid; else b = mid;
     }
+    sg0 = a;
     const int len = pre[a + 1] - pre[a], pad = vpre[a + 1] - vpre[a] - len;
     const int off = static_cast<int>(v - vpre[a]) - pad;
     return pre[a] + (off < 0 ? 0 : off);
   };
-  const int lo = page_at(cta_lo(V_all, blockIdx.x, p.n_ctas));
-  const int hi = page_at(cta_lo(V_all, blockIdx.x + 1, p.n_ctas));
+  const int n_share = tc5_ctas(V_all, p.n_ctas, GP);
+  const int hi = page_at(cta_lo(V_all, blockIdx.x + 1, n_share));
+  const int lo = page_at(cta_lo(V_all, blockIdx.x, n_share));
   if (lo >= hi) {                                  // nothing to do: give the tensor memory back
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(TMEM_COLS) : "memory");
     return;
   }
-  int sg0 = 0;
   while (pre[sg0 + 1] <= lo) ++sg0;
   auto n_active_of = [&](int s) { return staged ? na_s[s] : clamp_active(p.n_active[s], p.B); };
   auto kv_len_of = [&](int s) { return staged ? len_s[s] : p.kv_len[s]; };
@@ -372,9 +374,9 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       }
       return true;
     };
-    Item a = stage_a(lo + lane);
-    Ready b = stage_b(lo + lane, a);
-    a = stage_a(lo + lane + 32);
+    const Item a0 = stage_a(lo + lane);
+    Item a = stage_a(lo + lane + 32);                 // requested beside the first batch: the first copies wait for two loads, not three
+    Ready b = stage_b(lo + lane, a0);
     if constexpr (FP8) {                              // one stage deeper: the scales of a batch are requested a batch ahead
       stage_c(lo + lane, b);
       Ready b1 = stage_b(lo + lane + 32, a);

@@ -356,6 +356,20 @@ def test_many_rows_per_kv_head_fp32():
     run_blocks(cfg, modes=("losa",))
 
 
+@pytest.mark.parametrize("kw", [
+    # one KV head: more than 32 partial records for every row, whole-group shares that leave CTAs without pages
+    dict(n_q_heads=4, n_kv_heads=1, kv_lens=(40000,), block_size=8, steps=2, m_active=2, topk=16),
+    # more (sequence, head) lists than resident selection CTAs: one CTA takes all active slots of its list
+    dict(n_q_heads=28, n_kv_heads=4, kv_lens=(97,) * 36 + (0, 1, 33, 500), block_size=5, steps=3, m_active=3, topk=2),
+    # in-block row tiles of the selection's grid: one partial tile, and a second tile of one row
+    dict(n_q_heads=2, n_kv_heads=2, kv_lens=(70, 300), block_size=1, steps=2, m_active=1, topk=2),
+    dict(n_q_heads=5, n_kv_heads=1, kv_lens=(70, 300), block_size=13, steps=2, m_active=3, topk=2, head_dim=64),
+    dict(n_q_heads=1, n_kv_heads=1, kv_lens=(70, 300), block_size=64, steps=2, m_active=3, topk=2),
+])
+def test_whole_step_call_grids_and_merges_at_their_edges(kw):
+    run_blocks(wl.config("c2", **kw), fused=True)
+
+
 @pytest.mark.parametrize("g,d,m,G", [(16, 64, 1, 1), (32, 128, 4, 4), (64, 64, 5, 4), (16, 128, 8, 4), (32, 64, 11, 3), (64, 128, 16, 4), (32, 128, 13, 5), (16, 64, 16, 8)])
 def test_fp32_attention_by_rows_per_kv_head(g, d, m, G):
     """The fp32 stage-4 kernel at 1, 16, 20, 32, 33, 64, 65 and 128 query rows, odd page counts, empty and one-token prefixes."""
