@@ -37,7 +37,7 @@ int32_t make_layout(const losa_shape_t* sh, int n_ctas, WorkspaceLayout* L) {
   size_t off = 0;
   L->status = off;   off = align_up(off + 16, 256);
   L->counters = off; off = align_up(off + sizeof(uint32_t) * sh->batch, 256);
-  L->seg_prefix = off; off = align_up(off + sizeof(int32_t) * (kMaxSegments + 1), 256);
+  L->seg_records = off; off = align_up(off + 2 * sizeof(int32_t) * kMaxSegments, 256);
   L->slot_map = off; off = align_up(off + sizeof(int32_t) * sh->batch * sh->block_size, 256);
   L->union_bits = off;
   off = align_up(off + sizeof(uint32_t) * static_cast<size_t>(sh->batch) * sh->n_kv_heads * ((sh->max_pages_per_seq + 31) / 32), 256);

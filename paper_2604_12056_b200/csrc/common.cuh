@@ -20,7 +20,7 @@ constexpr float kLn2 = 0.6931471805599453f;
 struct WorkspaceLayout {
   size_t status;     // int32[4]  : device status word (+ padding)
   size_t counters;   // uint32[N] : arrival counters of select_active (self-resetting)
-  size_t seg_prefix; // int32[kMaxSegments + 1] : item prefix of the segments, left by the stage-4 main kernel for its combine kernel
+  size_t seg_records; // int2[kMaxSegments] : first CTA and number of the partial records of every segment, left by the stage-4 main kernel for the kernels that merge them
   size_t slot_map;   // int32[N*B] : slot of every block token in the active list of the whole-step path, -1 = stable
   size_t union_bits;    // uint32[N*H_kv*ceil(P_max/32)] : page bitmaps of the selection that also writes the union (all zero between launches)
   size_t union_tickets; // uint32[N*H_kv] : its arrival counters (self-resetting)
@@ -238,20 +238,38 @@ __device__ __forceinline__ int rows_in_group(int n_active, int G, int rg) {
   const int r = n_active * G - rg * kRowsPerGroup;
   return r < 0 ? 0 : (r > kRowsPerGroup ? kRowsPerGroup : r);
 }
-// floor(T * b / n); in 32 bits where the product fits (a 64-bit division is some 100 dependent instructions)
+// floor(T * b / n) for 0 <= b <= n <= 2^15, in 32 bits: a 64-bit division is some 100 dependent instructions
+__device__ __forceinline__ int cta_lo(int T, int b, int n) {
+  const uint32_t q = static_cast<uint32_t>(T) / static_cast<uint32_t>(n), r = static_cast<uint32_t>(T) - q * n;
+  return static_cast<int>(q * b + r * static_cast<uint32_t>(b) / static_cast<uint32_t>(n));
+}
 __device__ __forceinline__ long long cta_lo(long long T, int b, int n) {
-  if (T < (1 << 22) && b <= 512) return static_cast<uint32_t>(T) * static_cast<uint32_t>(b) / static_cast<uint32_t>(n);
-  return (T * b) / n;
+  return T <= 0x7fffffffll ? static_cast<long long>(cta_lo(static_cast<int>(T), b, n)) : T * b / n;
+}
+// The records of a segment whose items are positions start .. end - 1 of a list of T items cut over n
+// CTAs: x = the first CTA, y = how many CTAs (consecutive; each leaves one record).  The main kernels
+// write this per segment for the kernels that merge the records, which are chains of dependent reads
+// and would otherwise repeat the divisions in theirs.
+__device__ __forceinline__ int2 segment_records(int T, int n, int start, int end) {
+  if (end <= start) return make_int2(0, 0);
+  auto cta_of = [&](int v) {
+    int b = min(n - 1, static_cast<int>(static_cast<float>(v) * n / T));
+    while (b + 1 < n && cta_lo(T, b + 1, n) <= v) ++b;
+    while (b > 0 && cta_lo(T, b, n) > v) --b;
+    return b;
+  };
+  const int b0 = cta_of(start);
+  return make_int2(b0, cta_of(end - 1) - b0 + 1);
 }
 
 // CTAs of the tensor-core kernel that share a charged list of length V (page: tokens per page).  It takes
 // pages in groups of 128 tokens, and a group costs the same whatever it holds: short shares are
 // rounded up to whole groups, which costs the main kernel nothing and leaves the merge fewer records.
-__device__ __forceinline__ int tc5_ctas(long long V, int n_ctas, int page) {
-  const int pg = 128 / page, per = static_cast<int>((V + n_ctas - 1) / n_ctas);
+__device__ __forceinline__ int tc5_ctas(int V, int n_ctas, int page) {
+  const int pg = 128 / page, per = V / n_ctas + (V % n_ctas ? 1 : 0);
   if (per >= 8 * pg || per < 1) return n_ctas;
   const int whole = (per + pg - 1) / pg * pg;
-  return static_cast<int>((V + whole - 1) / whole);
+  return (V + whole - 1) / whole;
 }
 
 // The tensor-core kernel cuts a list in which every non-empty segment is charged segment_pad(rows)

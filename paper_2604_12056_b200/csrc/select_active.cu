@@ -96,6 +96,7 @@ select_active_kernel(const T* __restrict__ x_cur, const T* __restrict__ x_prev, 
     if (t < B) {
       const double dt = s_delta[t];
       int r = 0;
+#pragma unroll 8
       for (int j = 0; j < B; ++j) {
         const double dj = s_delta[j];
         r += (dj > dt || (dj == dt && j < t)) ? 1 : 0;

@@ -39,14 +39,14 @@ struct AttnParams {
   const int32_t* union_pages;
   const int32_t* union_count;
   float* partials;
-  int32_t* seg_prefix;  // workspace copy of the segment prefix (written by the bf16 main kernel, read by its combine kernel)
+  int2* seg_records;    // per segment: first CTA and number of its partial records (written by the main kernels)
   void* o_p;                // cached prefix output, fp32 or bf16 (o_p_bf16)
   int o_p_bf16;
   float* lse_p;
   int32_t* status;
   const float* k_scale;   // FP8 pages: [n_phys, H_kv] power-of-two scales (else null)
   const float* v_scale;
-  int N, B, Hq, Hkv, G, Pmax, page, n_phys, n_rg, n_seg, n_ctas;
+  int N, B, Hq, Hkv, G, Pmax, n_phys, n_rg, n_sk, n_seg, n_ctas;   // n_sk = N * Hkv, n_seg = n_rg * n_sk
   float sm_scale;
   long long wait_cycles;  // bound of every mbarrier wait of the bf16 main kernel, in SM clock cycles
 };
@@ -117,57 +117,39 @@ template <int C> __device__ __forceinline__ void st_state(void* base, int bf16, 
 #include "sparse_prefix_attn_f32.cuh"
 
 // ===================================================================== combine kernel
-// grid (n_seg, 8): warp = one query row of the segment's row group at a time.  The CTAs whose item range
-// meets the segment are consecutive; each of them left one record for the row's 16-row tile.  The
-// merge is a chain of dependent reads (latency bounds it), so lanes take one record's maximum and sum
-// each while the outputs of the first eight records are already on their way, and eight more are
-// requested at a time.  LOG2: partial maxima in base-2 units (tensor-core kernel) or natural units
-// (fp32 kernel).
-// Merge of the partial records of row r of segment sg by one warp: returns the un-normalised
-// output columns lane * C + c in acc, the reference maximum M and the sum of weights Lsum.
+// grid (n_seg, kCombineTiles): warp = one query row of the segment's row group at a time.  The CTAs whose
+// item range meets the segment are consecutive; each of them left one record for the row's 16-row tile.
+// The merge is a chain of dependent reads: latency bounds it.  LOG2: partial maxima in base-2 units
+// (tensor-core kernel) or natural units (fp32 kernel).
+// Merge of the partial records of row r of segment sg by one warp: returns the un-normalised output
+// columns lane * C + c in acc, the reference maximum M and the sum of weights Lsum.  The outputs of up
+// to kMergeBatch records are copied to `buf` (that many rows of D floats of this warp) while their
+// maxima are read; with up to 32 KB per CTA and few registers, more CTAs are resident than with
+// outputs in registers, and the rolled loops keep the code short.  A lane reads back only what it
+// copied itself.
+constexpr int kMergeBatch = 16;
 template <int D, bool LOG2>
-__device__ __forceinline__ void merge_records(const AttnParams& p, int n_ctas, int sg, int r, int start, int end, long long T_all,
-                                              int lane, float (&acc)[D / 32], float& M, float& Lsum) {
+__device__ __forceinline__ void merge_records(const AttnParams& p, float* buf, int sg, int r, int2 records, int lane,
+                                              float (&acc)[D / 32], float& M, float& Lsum) {
   constexpr int C = D / 32;
-  const int tile = r / kTileRows, rr = r % kTileRows;
+  constexpr size_t kSlot = static_cast<size_t>(8) * kTileRows * (D + 2);     // consecutive CTAs, consecutive slots
+  const int rr = r % kTileRows;
 #pragma unroll
   for (int c = 0; c < C; ++c) acc[c] = 0.f;
   M = -INFINITY;
   Lsum = 0.f;
-  if (end <= start) return;
-  // the first and the last CTA whose range can meet start .. end - 1
-  auto cta_of = [&](int v) {
-    int b = T_all < (1 << 22) && n_ctas <= 512 ? static_cast<int>(static_cast<uint32_t>(v) * static_cast<uint32_t>(n_ctas) / static_cast<uint32_t>(T_all))
-                                              : static_cast<int>((static_cast<long long>(v) * n_ctas) / T_all);
-    while (b + 1 < n_ctas && cta_lo(T_all, b + 1, n_ctas) <= v) ++b;
-    return b;
-  };
-  const int b0 = cta_of(start), n_pairs = cta_of(end - 1) - b0 + 1;
-  for (int base = 0; base < n_pairs; base += 32) {
-    // record of piece base + lane, or null when that CTA has no page of this segment
-    const float* rec = nullptr;
-    if (base + lane < n_pairs) {
-      const int b = b0 + base + lane;
-      const long long lo = max(cta_lo(T_all, b, n_ctas), static_cast<long long>(start));
-      const long long hi = min(cta_lo(T_all, b + 1, n_ctas), static_cast<long long>(end));
-      if (hi > lo) rec = record_base(p.partials, b + sg, tile, D);
+  const uint32_t dst = smem_u32(buf + lane * C);
+  for (int base = 0; base < records.y; base += kMergeBatch) {
+    const int n = min(kMergeBatch, records.y - base);
+    const float* rec = record_base(p.partials, records.x + base + sg, r / kTileRows, D);
+    const float mj = lane < n ? rec[lane * kSlot + rr] : -INFINITY, lj = lane < n ? rec[lane * kSlot + kTileRows + rr] : 0.f;
+    const float* src = rec + 2 * kTileRows + rr * D + lane * C;
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {
+      if constexpr (C == 4) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i * D * 4), "l"(src + i * kSlot) : "memory");
+      else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst + i * D * 4), "l"(src + i * kSlot) : "memory");
     }
-    // the maxima, the sums and the outputs of the first U records are requested together
-    const float mj = rec ? rec[rr] : -INFINITY, lj = rec ? rec[kTileRows + rr] : 0.f;
-    constexpr int U = 8;
-    const int n = min(32, n_pairs - base);
-    float v[U][C];
-    auto request = [&](int i0) {
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int i = i0 + u;
-        const unsigned long long addr = __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(rec), i & 31);
-#pragma unroll
-        for (int c = 0; c < C; ++c) v[u][c] = 0.f;
-        if (i < n && addr) ldv<C>(reinterpret_cast<const float*>(addr) + 2 * kTileRows + rr * D + lane * C, v[u]);
-      }
-    };
-    request(0);
+    asm volatile("cp.async.commit_group;" ::: "memory");
     const float M_new = fmaxf(M, warp_max(mj));
     const float keep = (M == -INFINITY) ? 0.f : (LOG2 ? exp2f(M - M_new) : expf(M - M_new));
     const float wj = (mj == -INFINITY) ? 0.f : (LOG2 ? exp2f(mj - M_new) : expf(mj - M_new));
@@ -175,46 +157,39 @@ __device__ __forceinline__ void merge_records(const AttnParams& p, int n_ctas, i
     Lsum = Lsum * keep + warp_sum(lj * wj);
 #pragma unroll
     for (int c = 0; c < C; ++c) acc[c] *= keep;
-    for (int i0 = 0; i0 < n; i0 += U) {
-      if (i0 > 0) request(i0);
+    cp_async_wait<0>();
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {
+      const float w = __shfl_sync(0xffffffffu, wj, i);
+      float v[C];
+      ldv<C>(buf + i * D + lane * C, v);
+      if (w != 0.f) {
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const float w = (i0 + u < n) ? __shfl_sync(0xffffffffu, wj, (i0 + u) & 31) : 0.f;
-        if (w != 0.f) {
-#pragma unroll
-          for (int c = 0; c < C; ++c) acc[c] = fmaf(v[u][c], w, acc[c]);
-        }
+        for (int c = 0; c < C; ++c) acc[c] = fmaf(v[c], w, acc[c]);
       }
     }
   }
 }
 
-template <int D, bool LOG2, bool PRE>
-__global__ void __launch_bounds__(256) attn_combine_kernel(AttnParams p) {
+constexpr int kCombineThreads = 128, kCombineTiles = 16;
+
+template <int D, bool LOG2>
+__global__ void __launch_bounds__(kCombineThreads) attn_combine_kernel(AttnParams p) {
   grid_dep_wait();
-  __shared__ int pre[kMaxSegments + 1];
+  __shared__ __align__(16) float buf[kCombineThreads / 32][kMergeBatch * D];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int sg = blockIdx.x;
-  const int n_sk = p.n_seg / p.n_rg, rg = sg / n_sk, sk = sg % n_sk, s = sk / p.Hkv, kh = sk % p.Hkv;
+  const int rg = sg / p.n_sk, sk = sg % p.n_sk, s = sk / p.Hkv, kh = sk % p.Hkv;
+  const int2 records = p.seg_records[sg];
   const int rows = rows_in_group(clamp_active(p.n_active[s], p.B), p.G, rg);
-  if (blockIdx.y * 8 >= rows) return;                 // whole CTA idle: skip the prefix as well
-  if (PRE) {                                          // the main kernel left the prefix in the workspace
-    if (tid == 0) { pre[sg] = p.seg_prefix[sg]; pre[sg + 1] = p.seg_prefix[sg + 1]; pre[p.n_seg] = p.seg_prefix[p.n_seg]; }
-  } else if (warp == 0) {
-    segment_prefix(pre, p.n_seg, p.n_rg, p.Hkv, p.G, p.n_active, p.union_count, p.B, lane);
-  }
-  __syncthreads();
   constexpr int C = D / 32;
-  const int n_ctas = LOG2 ? tc5_ctas(pre[p.n_seg], p.n_ctas, p.page) : f32_ctas(pre[p.n_seg], p.n_ctas, p.page);   // CTAs of the main kernel that share the list
-  for (int r = blockIdx.y * 8 + warp; r < rows; r += gridDim.y * 8) {   // few CTAs per segment: most row blocks are empty on most steps
+  for (int r = blockIdx.y * (kCombineThreads / 32) + warp; r < rows; r += gridDim.y * (kCombineThreads / 32)) {   // few CTAs per segment: most row blocks are empty on most steps
     const int row = rg * kRowsPerGroup + r, a = row / p.G, gi = row % p.G;
     const int tok = p.active_idx[s * p.B + a];
     if (tok < 0 || tok >= p.B) { set_status(p.status, LOSA_ERR_BOUNDS); continue; }
     const size_t orow = (static_cast<size_t>(s) * p.B + tok) * p.Hq + kh * p.G + gi;
     float acc[C], M, Lsum;
-    // (PRE: the prefix left by the tensor-core kernel is that of the charged list; a segment's pages follow its pad)
-    const int pad = (PRE && pre[sg + 1] > pre[sg]) ? segment_pad(rows) : 0;
-    merge_records<D, LOG2>(p, n_ctas, sg, r, pre[sg] + pad, pre[sg + 1], pre[p.n_seg], lane, acc, M, Lsum);
+    merge_records<D, LOG2>(p, buf[warp], sg, r, records, lane, acc, M, Lsum);
     const bool empty = !(Lsum > 0.f);
     const float inv = empty ? 0.f : 1.f / Lsum;
 #pragma unroll
@@ -244,7 +219,8 @@ struct FinishParams {
 constexpr int kFinishThreads = 128;
 
 template <typename T, int D>
-__global__ void __launch_bounds__(kFinishThreads, 5) attn_finish_kernel(AttnParams p, FinishParams f) {
+__global__ void __launch_bounds__(kFinishThreads) attn_finish_kernel(AttnParams p, FinishParams f) {
+  __shared__ __align__(16) float buf[kFinishThreads / 32][kMergeBatch * D];
   grid_dep_trigger();
   grid_dep_wait();
   constexpr int C = D / 32;
@@ -267,21 +243,20 @@ __global__ void __launch_bounds__(kFinishThreads, 5) attn_finish_kernel(AttnPara
   float a[C], Lp;
   ld_state<C>(p.o_p, p.o_p_bf16, row * D + lane * C, a);
   Lp = p.lse_p[row];
-  // where an active row's records are, for the first row group: requested before the slot is known
+  // an active row's records, for the first row group: requested before the slot is known (volatile: a
+  // plain load would sink into the branch and add a round trip)
   int sg = s * p.Hkv + kh;
-  int v0 = p.seg_prefix[sg], v1 = p.seg_prefix[sg + 1];             // of the charged list: the segment's pages follow its pad
-  const int v_all = p.seg_prefix[p.n_seg], na = clamp_active(p.n_active[s], p.B);
+  int2 records;
+  asm volatile("ld.global.v2.s32 {%0, %1}, [%2];" : "=r"(records.x), "=r"(records.y) : "l"(p.seg_records + sg));
   const int slot = f.slot_map[s * p.B + tok];                       // in the active list (at most B entries), -1 = stable
   if (slot >= 0 && slot < p.B) {
     const int rowk = slot * p.G + gi, rg = rowk / kRowsPerGroup, r = rowk % kRowsPerGroup;
     if (rg > 0) {
-      sg += rg * (p.n_seg / p.n_rg);
-      v0 = p.seg_prefix[sg];
-      v1 = p.seg_prefix[sg + 1];
+      sg += rg * p.n_sk;
+      records = p.seg_records[sg];
     }
     float acc[C], M, Lsum;
-    const int pad = v1 > v0 ? segment_pad(rows_in_group(na, p.G, rg)) : 0;
-    merge_records<D, true>(p, tc5_ctas(v_all, p.n_ctas, p.page), sg, r, v0 + pad, v1, v_all, lane, acc, M, Lsum);
+    merge_records<D, true>(p, buf[threadIdx.x >> 5], sg, r, records, lane, acc, M, Lsum);
     const bool empty = !(Lsum > 0.f);
     const float inv = empty ? 0.f : 1.f / Lsum;
     Lp = empty ? -INFINITY : (M + log2f(Lsum)) * kLn2;
@@ -420,7 +395,7 @@ int32_t launch_tc5(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool with
   if (c->profile) LOSA_CUDA_TRY(c, cudaEventRecord(c->ev_end, st));
   int32_t rc = after_launch(c);
   if (rc != LOSA_OK || !with_combine) return rc;
-  launch_k(attn_combine_kernel<D, true, true>, dim3(ap.n_seg, 8), 256, 0, st, ap);
+  launch_k(attn_combine_kernel<D, true>, dim3(ap.n_seg, kCombineTiles), kCombineThreads, 0, st, ap);
   return after_launch(c);
 }
 
@@ -437,7 +412,7 @@ int32_t launch_f32(losa_ctx* c, const AttnParams& ap, cudaStream_t st) {
   if (c->profile) LOSA_CUDA_TRY(c, cudaEventRecord(c->ev_end, st));
   int32_t rc = after_launch(c);
   if (rc != LOSA_OK) return rc;
-  launch_k(attn_combine_kernel<D, false, false>, dim3(ap.n_seg, 8), 256, 0, st, ap);
+  launch_k(attn_combine_kernel<D, false>, dim3(ap.n_seg, kCombineTiles), kCombineThreads, 0, st, ap);
   return after_launch(c);
 }
 
@@ -484,7 +459,7 @@ int32_t launch_sparse_prefix_attn(losa_ctx* c, const void* q, const losa_kv_t* k
   ap.union_pages = union_pages;
   ap.union_count = union_count;
   ap.partials = reinterpret_cast<float*>(c->ws + c->lay.partials);
-  ap.seg_prefix = reinterpret_cast<int32_t*>(c->ws + c->lay.seg_prefix);
+  ap.seg_records = reinterpret_cast<int2*>(c->ws + c->lay.seg_records);
   ap.o_p = state->o_p;
   ap.o_p_bf16 = state->o_p_format == LOSA_STATE_BF16 ? 1 : 0;
   ap.lse_p = state->lse_p;
@@ -498,10 +473,10 @@ int32_t launch_sparse_prefix_attn(losa_ctx* c, const void* q, const losa_kv_t* k
   ap.Hkv = sh.n_kv_heads;
   ap.G = sh.n_q_heads / sh.n_kv_heads;
   ap.Pmax = sh.max_pages_per_seq;
-  ap.page = sh.page_size;
   ap.n_phys = kv->n_phys_pages;
   ap.n_rg = c->lay.n_row_groups;
   ap.n_seg = c->lay.n_segments;
+  ap.n_sk = sh.batch * sh.n_kv_heads;
   ap.n_ctas = c->lay.n_ctas;
   ap.sm_scale = sh.sm_scale;
   ap.wait_cycles = c->wait_cycles > 0 ? c->wait_cycles : kWaitCycles;
@@ -519,7 +494,7 @@ int32_t launch_attn_finish(losa_ctx* c, const void* q, const int32_t* active_idx
   ap.active_idx = active_idx;
   ap.n_active = n_active;
   ap.partials = reinterpret_cast<float*>(c->ws + c->lay.partials);
-  ap.seg_prefix = reinterpret_cast<int32_t*>(c->ws + c->lay.seg_prefix);
+  ap.seg_records = reinterpret_cast<int2*>(c->ws + c->lay.seg_records);
   ap.o_p = state->o_p;
   ap.o_p_bf16 = state->o_p_format == LOSA_STATE_BF16 ? 1 : 0;
   ap.lse_p = state->lse_p;
@@ -529,9 +504,9 @@ int32_t launch_attn_finish(losa_ctx* c, const void* q, const int32_t* active_idx
   ap.Hq = sh.n_q_heads;
   ap.Hkv = sh.n_kv_heads;
   ap.G = sh.n_q_heads / sh.n_kv_heads;
-  ap.page = sh.page_size;
   ap.n_rg = c->lay.n_row_groups;
   ap.n_seg = c->lay.n_segments;
+  ap.n_sk = sh.batch * sh.n_kv_heads;
   ap.n_ctas = c->lay.n_ctas;
   FinishParams fp;
   fp.q = q;

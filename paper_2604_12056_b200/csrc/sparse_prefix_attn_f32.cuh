@@ -27,9 +27,9 @@ constexpr int kF32Chunk = 256;      // pages whose numbers are resolved at once
 // CTAs that share the list of T pages: at least 64 tokens each (a CTA's start-up costs more than their
 // arithmetic, and every further CTA is another record for the combine kernel to merge one after the
 // other: 64 pages of 16 tokens as 64 records took that kernel 25 us, as 16 records 5.8 us).
-__device__ __forceinline__ int f32_ctas(long long T, int n_ctas, int page) {
-  const long long n = (T * page + 63) / 64;
-  return n < 1 ? 1 : (n < n_ctas ? static_cast<int>(n) : n_ctas);
+__device__ __forceinline__ int f32_ctas(int T, int n_ctas, int page) {
+  if (T >= 64 * n_ctas) return n_ctas;
+  return min(n_ctas, max(1, (T * page + 63) / 64));
 }
 
 template <int D> struct F32Smem {
@@ -64,7 +64,7 @@ __device__ __forceinline__ void f32_piece(const AttnParams& p, F32Smem<D>& sm, i
   constexpr int RG = 4 * NB, TG = 4 / NB, TPT = kF32Tok / TG;   // second product: row groups of 8, token groups, tokens per thread
   constexpr int CV = D / 64;                        // 16-byte column runs per thread
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n_sk = p.n_seg / p.n_rg, rg = sg / n_sk, sk = sg % n_sk, s = sk / p.Hkv, kh = sk % p.Hkv;
+  const int rg = sg / p.n_sk, sk = sg % p.n_sk, s = sk / p.Hkv, kh = sk % p.Hkv;
   const int rows = rows_in_group(clamp_active(p.n_active[s], p.B), p.G, rg);
   const int len = p.kv_len[s];
   const float* kp = static_cast<const float*>(p.k_pages) + static_cast<size_t>(kh) * p.stride_head;
@@ -281,16 +281,17 @@ __global__ void __launch_bounds__(kF32Threads, 1) attn_f32_kernel(AttnParams p) 
   static_assert(sizeof(float) * 2 * kF32Stages * kF32Tok * D >= sizeof(float) * kRowsPerGroup * D, "the partial outputs fit the tiles");
   if (threadIdx.x < 32) segment_prefix(sm.pre, p.n_seg, p.n_rg, p.Hkv, p.G, p.n_active, p.union_count, p.B, threadIdx.x);
   __syncthreads();
-  const long long T_all = sm.pre[p.n_seg];
+  const int T_all = sm.pre[p.n_seg];
   const int n = f32_ctas(T_all, p.n_ctas, GP);
+  for (int seg = blockIdx.x * kF32Threads + threadIdx.x; seg < p.n_seg; seg += gridDim.x * kF32Threads)
+    p.seg_records[seg] = segment_records(T_all, n, sm.pre[seg], sm.pre[seg + 1]);
   if (static_cast<int>(blockIdx.x) >= n) return;
-  const int lo = static_cast<int>(cta_lo(T_all, blockIdx.x, n)), hi = static_cast<int>(cta_lo(T_all, blockIdx.x + 1, n));
+  const int lo = cta_lo(T_all, blockIdx.x, n), hi = cta_lo(T_all, blockIdx.x + 1, n);
   int sg = 0, item = lo;
   while (item < hi) {
     while (sm.pre[sg + 1] <= item) ++sg;
     const int seg_end = min(hi, sm.pre[sg + 1]), u0 = item - sm.pre[sg], u1 = seg_end - sm.pre[sg];
-    const int n_sk = p.n_seg / p.n_rg;
-    const int rows = rows_in_group(clamp_active(p.n_active[(sg % n_sk) / p.Hkv], p.B), p.G, sg / n_sk);
+    const int rows = rows_in_group(clamp_active(p.n_active[(sg % p.n_sk) / p.Hkv], p.B), p.G, sg / p.n_sk);
     if (rows <= 16) f32_piece<D, GP, 1, 4>(p, sm, sg, u0, u1);
     else if (rows <= 32) f32_piece<D, GP, 1, 8>(p, sm, sg, u0, u1);
     else if (rows <= 64) f32_piece<D, GP, 2, 8>(p, sm, sg, u0, u1);

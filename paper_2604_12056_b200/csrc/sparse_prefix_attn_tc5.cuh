@@ -235,26 +235,29 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   __syncthreads();
   tc5_fence_after();
   const uint32_t tmem = *tmem_slot;
-  if (blockIdx.x == 0)                             // the combine kernel reads the prefix instead of recomputing it
-    for (int i = tid; i <= p.n_seg; i += NT) p.seg_prefix[i] = vpre[i];
   // this CTA's share of the charged list, mapped back to pages: the first page at or after a charged position
-  const long long V_all = vpre[p.n_seg];
-  int sg0 = 0;                                       // (of the call below that is made last: the segment of the share's first page, or an empty one before it)
-  auto page_at = [&](long long v) {
-    if (v >= V_all) return pre[p.n_seg];
-    int a = 0, b = p.n_seg;                          // vpre[a] <= v < vpre[b]
-    while (b - a > 1) {
-      const int mid = (a + b) >> 1;
-      if (vpre[mid] <= v) a = mid; else b = mid;
+  const int V_all = vpre[p.n_seg], n_share = tc5_ctas(V_all, p.n_ctas, GP);
+  if (warp == kTc5PvWarp)                          // (this warp is needed last) for the merging kernels
+    for (int seg = blockIdx.x * 32 + lane; seg < p.n_seg; seg += gridDim.x * 32) {
+      const int n_pages = pre[seg + 1] - pre[seg], end = vpre[seg + 1];
+      p.seg_records[seg] = segment_records(V_all, n_share, end - n_pages, end);
     }
-    sg0 = a;
-    const int len = pre[a + 1] - pre[a], pad = vpre[a + 1] - vpre[a] - len;
-    const int off = static_cast<int>(v - vpre[a]) - pad;
-    return pre[a] + (off < 0 ? 0 : off);
-  };
-  const int n_share = tc5_ctas(V_all, p.n_ctas, GP);
-  const int hi = page_at(cta_lo(V_all, blockIdx.x + 1, n_share));
-  const int lo = page_at(cta_lo(V_all, blockIdx.x, n_share));
+  int lo = pre[p.n_seg], hi = lo, sg0 = 0;         // sg0: the segment of the share's first page, or one before it
+  if (static_cast<int>(blockIdx.x) < n_share) {
+    const int v_lo = cta_lo(V_all, blockIdx.x, n_share), v_hi = cta_lo(V_all, blockIdx.x + 1, n_share);
+    int a = 0, b = p.n_seg, c = 0, d = p.n_seg;    // vpre[a] <= v_lo < vpre[b], vpre[c] <= v_hi (< vpre[d]): two searches side by side
+    while (b - a > 1 || d - c > 1) {
+      const int m0 = (a + b) >> 1, m1 = (c + d) >> 1;
+      const int x0 = vpre[m0], x1 = vpre[m1];
+      if (b - a > 1) { if (x0 <= v_lo) a = m0; else b = m0; }
+      if (d - c > 1) { if (x1 <= v_hi) c = m1; else d = m1; }
+    }
+    auto page_at = [&](int a, int v) {             // the pages of a segment lie at the end of its charged run
+      return pre[a] + max(0, v - vpre[a + 1] + (pre[a + 1] - pre[a]));
+    };
+    if (v_lo < V_all) { sg0 = a; lo = page_at(a, v_lo); }
+    if (v_hi < V_all) hi = page_at(c, v_hi);
+  }
   if (lo >= hi) {                                  // nothing to do: give the tensor memory back
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(TMEM_COLS) : "memory");
     return;
@@ -291,7 +294,8 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
           pstart = pre[cursor];
         }
         const int q = i - pstart, seg_end = min(hi, pre[cursor + 1]);
-        it.sk = cursor % (p.n_seg / p.n_rg);
+        it.sk = cursor;
+        while (it.sk >= p.n_sk) it.sk -= p.n_sk;
         it.grp = gbase + q / PG;
         it.j = q % PG;
         it.ng = min(PG, seg_end - (i - it.j));
@@ -552,7 +556,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     bool ok = true;
     while (item < hi && ok) {
       const int seg_end = min(hi, pre[sg + 1]);
-      const int n_sk = p.n_seg / p.n_rg, rg = sg / n_sk, sk = sg % n_sk, s = sk / p.Hkv, kh = sk % p.Hkv;
+      const int rg = sg / p.n_sk, sk = sg % p.n_sk, s = sk / p.Hkv, kh = sk % p.Hkv;
       const int rows = rows_in_group(n_active_of(s), p.G, rg);
       const bool warp_has_rows = quarter * 32 < rows;          // the same for both warps of a pair
       // ---- the piece's Q tile: this thread's half row, two bf16 per tensor-memory column
