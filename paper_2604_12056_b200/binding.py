@@ -80,22 +80,51 @@ def lib() -> C.CDLL:
     return _lib
 
 
+# Argument types of the entry points a denoising step calls (p: pointer, i: int32, d: double).  With
+# them ctypes converts plain integers itself; without, every argument is wrapped in an object first,
+# and a step of six calls spends more time in that than in its launches.
+_SIGNATURES = {
+    "losa_select_active": "pppipppppp", "losa_select_active_tau": "pppidpppppp",
+    "losa_select_active_static": "pppipppppp", "losa_page_scores_topk": "ppppppippp",
+    "losa_page_scores_topk_pooled": "ppppppippp", "losa_page_scores_topk_mma": "ppppppippp",
+    "losa_page_union": "ppppippppp", "losa_sparse_prefix_attn": "ppppppppp", "losa_block_attn_merge": "pppppppp",
+    "losa_update_prefix_cache": "ppppppip", "losa_quantize_kv_pages": "pppp", "losa_build_page_summaries": "ppp",
+    "losa_denoise_step": "ppppppppppip", "losa_denoise_step_host": "pppppppppip",
+}
+_typed = None
+
+
+def _typed_lib() -> C.CDLL:
+    """The library's functions with argument types (a handle of its own: `lib()` stays untyped)."""
+    global _typed
+    if _typed is None:
+        lib()                                               # raises when it has not been built
+        t = C.CDLL(LIB_PATH)
+        kinds = {"p": C.c_void_p, "i": C.c_int32, "d": C.c_double}
+        for name, sig in _SIGNATURES.items():
+            f = getattr(t, name)
+            f.restype, f.argtypes = C.c_int32, [kinds[k] for k in sig]
+        _typed = t
+    return _typed
+
+
 def _ptr(t):
     if t is None:
         return None
     if isinstance(t, torch.Tensor):
         assert t.is_cuda and t.is_contiguous(), "device tensors must be contiguous CUDA tensors"
-        return C.c_void_p(t.data_ptr())
-    return C.c_void_p(int(t))
+        return t.data_ptr()
+    return int(t)
 
 
 def _hptr(t):
     assert isinstance(t, torch.Tensor) and not t.is_cuda and t.is_contiguous()
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """The raw handle of torch's current stream (without building a Stream object for every call)."""
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def torch_dtype(dtype: int):
@@ -191,19 +220,19 @@ class Context:
         return float(ms.value)
 
     def poll_status(self) -> int:
-        return int(lib().losa_poll_status(self._h, _stream()))
+        return int(lib().losa_poll_status(self._h, C.c_void_p(_stream())))
 
 
 def losa_select_active(ctx, x_cur, x_prev, row_width, m_per_seq, step, active_idx, n_active, delta_opt=None):
-    ctx._check("losa_select_active", lib().losa_select_active(
-        ctx._h, _ptr(x_cur), _ptr(x_prev), C.c_int32(row_width), _ptr(m_per_seq), _ptr(step),
+    ctx._check("losa_select_active", _typed_lib().losa_select_active(
+        ctx._h, _ptr(x_cur), _ptr(x_prev), row_width, _ptr(m_per_seq), _ptr(step),
         _ptr(active_idx), _ptr(n_active), _ptr(delta_opt), _stream()))
 
 
 def losa_select_active_tau(ctx, x_cur, x_prev, row_width, tau, m_cap_opt, step, active_idx, n_active, delta_opt=None):
     """Stage 1, threshold variant: tokens are kept until their Delta reach tau of the block's total."""
-    ctx._check("losa_select_active_tau", lib().losa_select_active_tau(
-        ctx._h, _ptr(x_cur), _ptr(x_prev), C.c_int32(row_width), C.c_double(tau), _ptr(m_cap_opt), _ptr(step),
+    ctx._check("losa_select_active_tau", _typed_lib().losa_select_active_tau(
+        ctx._h, _ptr(x_cur), _ptr(x_prev), row_width, tau, _ptr(m_cap_opt), _ptr(step),
         _ptr(active_idx), _ptr(n_active), _ptr(delta_opt), _stream()))
 
 
@@ -212,7 +241,7 @@ def losa_select_active_static(shape: ShapeT, x_cur, x_prev, row_width, m_per_seq
     """Stage 1 for callers that must not allocate device memory: no context, no workspace; the
     scratch lives in a fixed array inside the library (batch <= 64).  Calls on one device share
     that array, so they must not overlap on the GPU."""
-    rc = lib().losa_select_active_static(C.byref(shape), _ptr(x_cur), _ptr(x_prev), C.c_int32(row_width),
+    rc = _typed_lib().losa_select_active_static(C.byref(shape), _ptr(x_cur), _ptr(x_prev), row_width,
                                          _ptr(m_per_seq), _ptr(step), _ptr(active_idx), _ptr(n_active),
                                          _ptr(delta_opt), _stream())
     if rc != LOSA_OK:
@@ -220,63 +249,63 @@ def losa_select_active_static(shape: ShapeT, x_cur, x_prev, row_width, m_per_seq
 
 
 def losa_page_scores_topk(ctx, q, kv, active_idx, n_active, step, k, topk_pages, topk_scores_opt=None):
-    ctx._check("losa_page_scores_topk", lib().losa_page_scores_topk(
-        ctx._h, _ptr(q), C.byref(kv), _ptr(active_idx), _ptr(n_active), _ptr(step), C.c_int32(k),
+    ctx._check("losa_page_scores_topk", _typed_lib().losa_page_scores_topk(
+        ctx._h, _ptr(q), C.byref(kv), _ptr(active_idx), _ptr(n_active), _ptr(step), k,
         _ptr(topk_pages), _ptr(topk_scores_opt), _stream()))
 
 
 def losa_page_scores_topk_pooled(ctx, q, kv, active_idx, n_active, step, k, topk_pages, topk_scores_opt=None):
-    ctx._check("losa_page_scores_topk_pooled", lib().losa_page_scores_topk_pooled(
-        ctx._h, _ptr(q), C.byref(kv), _ptr(active_idx), _ptr(n_active), _ptr(step), C.c_int32(k),
+    ctx._check("losa_page_scores_topk_pooled", _typed_lib().losa_page_scores_topk_pooled(
+        ctx._h, _ptr(q), C.byref(kv), _ptr(active_idx), _ptr(n_active), _ptr(step), k,
         _ptr(topk_pages), _ptr(topk_scores_opt), _stream()))
 
 
 def losa_page_scores_topk_mma(ctx, q, kv, active_idx, n_active, step, k, topk_pages, topk_scores_opt=None):
     """Stage 2 with tensor-core scores (bf16): lists valid under the relaxed rule, not entry by entry."""
-    ctx._check("losa_page_scores_topk_mma", lib().losa_page_scores_topk_mma(
-        ctx._h, _ptr(q), C.byref(kv), _ptr(active_idx), _ptr(n_active), _ptr(step), C.c_int32(k),
+    ctx._check("losa_page_scores_topk_mma", _typed_lib().losa_page_scores_topk_mma(
+        ctx._h, _ptr(q), C.byref(kv), _ptr(active_idx), _ptr(n_active), _ptr(step), k,
         _ptr(topk_pages), _ptr(topk_scores_opt), _stream()))
 
 
 def losa_page_union(ctx, topk_pages, active_idx, n_active, k, kv_len, step, union_pages, union_count):
-    ctx._check("losa_page_union", lib().losa_page_union(
-        ctx._h, _ptr(topk_pages), _ptr(active_idx), _ptr(n_active), C.c_int32(k), _ptr(kv_len), _ptr(step),
+    ctx._check("losa_page_union", _typed_lib().losa_page_union(
+        ctx._h, _ptr(topk_pages), _ptr(active_idx), _ptr(n_active), k, _ptr(kv_len), _ptr(step),
         _ptr(union_pages), _ptr(union_count), _stream()))
 
 
 def losa_sparse_prefix_attn(ctx, q, kv, active_idx, n_active, union_pages, union_count, state):
-    ctx._check("losa_sparse_prefix_attn", lib().losa_sparse_prefix_attn(
+    ctx._check("losa_sparse_prefix_attn", _typed_lib().losa_sparse_prefix_attn(
         ctx._h, _ptr(q), C.byref(kv), _ptr(active_idx), _ptr(n_active), _ptr(union_pages),
         _ptr(union_count), C.byref(state), _stream()))
 
 
 def losa_block_attn_merge(ctx, q, k_blk, v_blk, state, out, lse_out_opt=None):
-    ctx._check("losa_block_attn_merge", lib().losa_block_attn_merge(
+    ctx._check("losa_block_attn_merge", _typed_lib().losa_block_attn_merge(
         ctx._h, _ptr(q), _ptr(k_blk), _ptr(v_blk), C.byref(state), _ptr(out), _ptr(lse_out_opt), _stream()))
 
 
 def losa_update_prefix_cache(ctx, kv, state, q, k_blk, v_blk, finalize_block):
-    ctx._check("losa_update_prefix_cache", lib().losa_update_prefix_cache(
+    ctx._check("losa_update_prefix_cache", _typed_lib().losa_update_prefix_cache(
         ctx._h, C.byref(kv), C.byref(state), _ptr(q), _ptr(k_blk), _ptr(v_blk),
-        C.c_int32(1 if finalize_block else 0), _stream()))
+        1 if finalize_block else 0, _stream()))
 
 
 def losa_quantize_kv_pages(ctx, src_kv, dst_kv):
     """bf16 cache -> FP8 cache (codes, per-page scales, summaries of the dequantised keys)."""
-    ctx._check("losa_quantize_kv_pages", lib().losa_quantize_kv_pages(ctx._h, C.byref(src_kv), C.byref(dst_kv), _stream()))
+    ctx._check("losa_quantize_kv_pages", _typed_lib().losa_quantize_kv_pages(ctx._h, C.byref(src_kv), C.byref(dst_kv), _stream()))
 
 
 def losa_build_page_summaries(ctx, kv):
-    ctx._check("losa_build_page_summaries", lib().losa_build_page_summaries(ctx._h, C.byref(kv), _stream()))
+    ctx._check("losa_build_page_summaries", _typed_lib().losa_build_page_summaries(ctx._h, C.byref(kv), _stream()))
 
 
 def losa_denoise_step(ctx, q, k_blk, v_blk, out, lse_out_opt, kv, state, buf, m_per_seq, k):
-    ctx._check("losa_denoise_step", lib().losa_denoise_step(
+    ctx._check("losa_denoise_step", _typed_lib().losa_denoise_step(
         ctx._h, _ptr(q), _ptr(k_blk), _ptr(v_blk), _ptr(out), _ptr(lse_out_opt), C.byref(kv), C.byref(state),
-        C.byref(buf), _ptr(m_per_seq), C.c_int32(k), _stream()))
+        C.byref(buf), _ptr(m_per_seq), k, _stream()))
 
 
 def losa_denoise_step_host(ctx, h_q, h_k_blk, h_v_blk, h_out, kv, state, buf, m_per_seq, k):
-    ctx._check("losa_denoise_step_host", lib().losa_denoise_step_host(
+    ctx._check("losa_denoise_step_host", _typed_lib().losa_denoise_step_host(
         ctx._h, _hptr(h_q), _hptr(h_k_blk), _hptr(h_v_blk), _hptr(h_out), C.byref(kv), C.byref(state),
-        C.byref(buf), _ptr(m_per_seq), C.c_int32(k), _stream()))
+        C.byref(buf), _ptr(m_per_seq), k, _stream()))
