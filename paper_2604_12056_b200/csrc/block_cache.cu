@@ -403,7 +403,7 @@ int32_t launch_summaries_t(losa_ctx* c, losa_kv_t* kv, cudaStream_t st) {
   const losa_shape_t& sh = c->shape;
   if (sh.max_pages_per_seq == 0) return LOSA_OK;
   const dim3 grid((sh.max_pages_per_seq * sh.n_kv_heads + kSumWarps - 1) / kSumWarps, 1, sh.batch);
-  launch_k(build_summaries_kernel<T, D>, grid, kSumWarps * 32, 0, st, 
+  launch_streaming(build_summaries_kernel<T, D>, grid, kSumWarps * 32, 0, st, 
       static_cast<const T*>(kv->k_pages), static_cast<T*>(kv->kmin), static_cast<T*>(kv->kmax),
       kv->page_table, kv->kv_len, kv->stride_page, kv->stride_head, kv->stride_tok, sh.n_kv_heads,
       sh.page_size, sh.max_pages_per_seq, kv->n_phys_pages, status_ptr(c));

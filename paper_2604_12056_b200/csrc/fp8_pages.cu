@@ -211,10 +211,14 @@ __global__ void __launch_bounds__(kFp8Warps * 32) fp8_pages_kernel(Fp8Params p) 
 template <int MODE, int D>
 void launch_fp8_d(const losa_shape_t& sh, const Fp8Params& p, int pages, cudaStream_t st) {
   const dim3 grid((pages * sh.n_kv_heads + kFp8Warps - 1) / kFp8Warps, MODE == 1 ? 1 : 2, sh.batch);
+  auto launch = [&](void (*kernel)(Fp8Params)) {      // (mode 2 is a small kernel between the steps of two blocks)
+    if (MODE == 2) launch_k(kernel, grid, kFp8Warps * 32, 0, st, p);
+    else launch_streaming(kernel, grid, kFp8Warps * 32, 0, st, p);
+  };
   switch (sh.page_size) {
-    case 16: launch_k(fp8_pages_kernel<MODE, D, 16>, grid, kFp8Warps * 32, 0, st, p); break;
-    case 32: launch_k(fp8_pages_kernel<MODE, D, 32>, grid, kFp8Warps * 32, 0, st, p); break;
-    default: launch_k(fp8_pages_kernel<MODE, D, 64>, grid, kFp8Warps * 32, 0, st, p); break;
+    case 16: launch(fp8_pages_kernel<MODE, D, 16>); break;
+    case 32: launch(fp8_pages_kernel<MODE, D, 32>); break;
+    default: launch(fp8_pages_kernel<MODE, D, 64>); break;
   }
 }
 // `pages`: logical pages per sequence that the grid covers
