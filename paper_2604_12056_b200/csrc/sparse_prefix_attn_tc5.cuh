@@ -26,28 +26,39 @@ constexpr int kTc5QkWarp = 8, kTc5PvWarp = 9, kTc5KWarp = 10, kTc5VWarp = 11;
 constexpr int kTc5CvtWarp = 12;                  // FP8 pages: four converting warps, two for K and two for V
 template <bool FP8> constexpr int tc5_threads() { return FP8 ? 512 : 384; }
 constexpr int kTc5Tok = 128;                     // tokens per group = N of Q K^T = columns of one S buffer
-constexpr int kTc5PgMax = 8;                     // pages per group at the smallest page size (16)
-constexpr int kTc5MetaRing = 16;                 // groups whose per-page token counts are kept (producer lead < 16)
 constexpr float kTc5Tau = 8.0f;                  // reference maximum moves only when it would grow by more than this (log2 units)
 constexpr int kTc5XchgBytes = (2 * 2 + 1) * kRowsPerGroup * 4;   // row maxima [group parity][set][row], row sums [row]
 constexpr int kTc5StgMax = 20;                   // FP8 pages: staging slots per tensor, one page each, at most
-constexpr int kTc5StgTail = kTc5StgMax * 2 * (8 + 8) + 2 * kTc5MetaRing * kTc5PgMax * 4;   // ... their barriers (landed, emptied), K and V; the page scales of the groups in flight
-constexpr int kTc5TailBytes = kTailBytes + 512 + kTc5XchgBytes + kTc5StgTail + (kMaxSegments + 2) * 4;  // 1024 bytes of barriers + page meta, the segment prefix and index cache, the exchange arrays, the scales
+// Groups whose per-page data (token counts; FP8: scales) is kept.  The K producer writes a page's entry
+// when it issues the page's copy, so the ring must be longer than its lead over the softmax warps.  A
+// group never spans two segments, so in a run of one-page segments every page in flight is a group of
+// its own.  The first page of group g is issued once its slot is free:
+//   bf16  Q K^T of group g - NR has run, hence P V of group g - NR - 2: group g - NR - 1 may still be
+//         read, a lead of NR + 1;
+//   FP8   page, and so at worst group, g - NSP has been converted (NSP staging slots), hence Q K^T of
+//         group g - NSP - NR has run: a lead of NSP + NR + 1.
+// Small pages have up to 20 staging slots, a lead of 23; the others at most 10.
+template <int D, int GP, bool FP8> constexpr int tc5_meta_ring() { return FP8 && GP * D <= 2048 ? 32 : 16; }
+// Barriers, the segment prefix and index cache, the exchange arrays, the charged prefix, the staging
+// barriers (landed, emptied; K and V), two words per page of the meta ring
+template <int D, int GP, bool FP8> constexpr int tc5_tail_bytes() {
+  return kTailBytes + kTc5XchgBytes + (kMaxSegments + 2) * 4 + kTc5StgMax * 2 * (8 + 8) + tc5_meta_ring<D, GP, FP8>() * (kTc5Tok / GP) * 8;
+}
 
 template <int D> constexpr int tc5_slot_bytes() { return kTc5Tok * D * 2; }
-template <int D, bool FP8> constexpr int tc5_ring_slots() {     // per ring (K and V have one each)
+template <int D, int GP, bool FP8> constexpr int tc5_ring_slots() {     // per ring (K and V have one each)
   if (FP8) return 2;                                            // the staging slots take the rest
-  const int n = (kSmemBudget - 1024 - kTc5TailBytes) / tc5_slot_bytes<D>() / 2;
+  const int n = (kSmemBudget - 1024 - tc5_tail_bytes<D, GP, FP8>()) / tc5_slot_bytes<D>() / 2;
   return n > 6 ? 6 : n;
 }
 // FP8: pages per staging ring (one for K, one for V): what the ring slots leave, up to five groups
 template <int D, int GP> constexpr int tc5_stg_slots() {
-  const int fit = (kSmemBudget - 1024 - kTc5TailBytes - 4 * tc5_slot_bytes<D>()) / 2 / (GP * D), five = 5 * (kTc5Tok / GP);
+  const int fit = (kSmemBudget - 1024 - tc5_tail_bytes<D, GP, true>() - 4 * tc5_slot_bytes<D>()) / 2 / (GP * D), five = 5 * (kTc5Tok / GP);
   const int n = fit < five ? fit : five;
   return n < kTc5StgMax ? n : kTc5StgMax;
 }
 template <int D, int GP, bool FP8> constexpr int tc5_smem_bytes() {
-  return 1024 + 2 * tc5_ring_slots<D, FP8>() * tc5_slot_bytes<D>() + (FP8 ? 2 * tc5_stg_slots<D, GP>() * GP * D : 0) + kTc5TailBytes;
+  return 1024 + 2 * tc5_ring_slots<D, GP, FP8>() * tc5_slot_bytes<D>() + (FP8 ? 2 * tc5_stg_slots<D, GP>() * GP * D : 0) + tc5_tail_bytes<D, GP, FP8>();
 }
 
 // Shared-memory matrix descriptor: 128-byte swizzle, 8-row groups 1024 bytes apart; lbo = distance
@@ -141,12 +152,13 @@ __device__ __forceinline__ uint32_t tc5_sw(int t, int c) { return static_cast<ui
 template <int D, int GP, bool FP8>
 __global__ void __launch_bounds__(tc5_threads<FP8>(), 1)
 attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, AttnParams p) {
-  constexpr int NR = tc5_ring_slots<D, FP8>();  // slots per ring
+  constexpr int NR = tc5_ring_slots<D, GP, FP8>();  // slots per ring
   constexpr int NSP = FP8 ? tc5_stg_slots<D, GP>() : 1, STG = GP * D;   // FP8: staging slots per tensor, bytes of a slot (one page of codes)
   constexpr int NT = tc5_threads<FP8>();
   constexpr uint32_t FMT = FP8 ? 0u : 1u;       // operand format of the MMAs: fp16 / bf16
   constexpr int SLOT = tc5_slot_bytes<D>();
   constexpr int PG = kTc5Tok / GP;              // pages per group
+  constexpr int MR = tc5_meta_ring<D, GP, FP8>();   // groups of the meta ring
   constexpr int HALVES = D / 64;                // 64-column (128-byte) blocks of a K or V row
   constexpr int HS = kTc5Tok * 128;             // bytes of one such block of a whole group
   constexpr int PAGE_BYTES = GP * D * 2;        // of K, and of V
@@ -154,9 +166,10 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   constexpr int TMEM_COLS = 512;
   static_assert(D == 64 || D == 128, "head dimensions of the tensor-core path");
   static_assert(GP == 16 || GP == 32 || GP == 64, "page sizes of the tensor-core path");
-  static_assert(NR >= 2 && PG <= kTc5PgMax, "ring too shallow / group too long");
+  static_assert(NR >= 2, "ring too shallow");
   static_assert(!FP8 || (NSP >= PG && NSP <= kTc5StgMax), "staging ring");
-  static_assert(8 * (4 * 6 + 14) + 4 * kTc5MetaRing * kTc5PgMax + 16 <= 1024, "tail layout");
+  static_assert((FP8 ? NSP : 0) + NR + 1 < MR, "the producer's lead fits the meta ring");
+  static_assert(8 * (4 * 6 + 14) + 16 <= 512, "tail layout");
 
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -170,21 +183,21 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   const uint32_t kfull = tail_s, kfree = kfull + 8 * NR, vfull = kfree + 8 * NR, vfree = vfull + 8 * NR;
   const uint32_t s_full = vfree + 8 * NR, s_free = s_full + 16, p_full = s_free + 16, q_full = p_full + 16, q_free = q_full + 8, xbar = q_free + 8;
   const uint32_t drain_bar = xbar + 32;            // two barriers: the issuing threads' last commit when the CTA gives up
-  volatile int* meta = reinterpret_cast<volatile int*>(tail + 8 * (4 * 6 + 14));   // [kTc5MetaRing][kTc5PgMax] valid tokens per page
-  volatile int* abort_flag = meta + kTc5MetaRing * kTc5PgMax;
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 8 * (4 * 6 + 14));
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(const_cast<int*>(abort_flag) + 1);
-  int* pre = reinterpret_cast<int*>(tail + 1024);
+  int* pre = reinterpret_cast<int*>(tail + 512);
   int* tok_s = pre + kMaxSegments + 2;
   int* na_s = tok_s + kStageIdx;
   int* len_s = na_s + kStageSeq;
   float* xmax = reinterpret_cast<float*>(len_s + kStageSeq);   // [2][2][128]
   float* xsum = xmax + 4 * kRowsPerGroup;                        // [128]
   int* vpre = reinterpret_cast<int*>(xsum + kRowsPerGroup);      // prefix of the charged segment lengths (pages + pad)
-  // FP8: per tensor, a staging slot's page has landed / has been converted; the scales of the groups' pages
+  // FP8: per tensor, a staging slot's page has landed / has been converted
   const uint32_t stg_bars = smem_u32(vpre + kMaxSegments + 1) + 4;   // (kMaxSegments + 1 is odd)
   const uint32_t kstg_full = stg_bars, vstg_full = kstg_full + 8 * kTc5StgMax, kstg_free = vstg_full + 8 * kTc5StgMax, vstg_free = kstg_free + 8 * kTc5StgMax;
-  volatile float* kscale_meta = reinterpret_cast<volatile float*>(vpre + kMaxSegments + 2 + 8 * kTc5StgMax);   // [kTc5MetaRing][kTc5PgMax]
-  volatile float* vscale_meta = kscale_meta + kTc5MetaRing * kTc5PgMax;
+  // per page of the groups in flight, [MR][PG]: valid tokens (FP8: and the value scale's exponent field << 8), FP8: key scale
+  volatile int* meta = vpre + kMaxSegments + 2 + 8 * kTc5StgMax;
+  volatile float* kscale_meta = reinterpret_cast<volatile float*>(const_cast<int*>(meta) + MR * PG);
   const bool staged = p.N * p.B <= kStageIdx && p.N <= kStageSeq;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -338,10 +351,9 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             if (round > 0) ok = mbar_wait(emptied + 8 * slot, (round - 1) & 1, abort_flag, p.status, p.wait_cycles);
             if (ok) {
               if (!is_v) {
-                const int at = (b.grp % kTc5MetaRing) * kTc5PgMax + b.j;
-                meta[at] = b.valid;
+                const int at = (b.grp % MR) * PG + b.j;
+                meta[at] = b.valid | ((__float_as_int(b.vs) >> 23) & 0xff) << 8;
                 kscale_meta[at] = b.ks;
-                vscale_meta[at] = b.vs;
               }
               mbar_expect_tx(landed + 8 * slot, STG);
               tma_load_4d(stg + slot * STG, map, landed + 8 * slot, 0, 0, b.kh, b.phys, policy);
@@ -364,7 +376,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
           if (__shfl_sync(0xffffffffu, ok, 0) == 0) return false;
         }
         const bool mine = lane >= pos && lane < pos + cnt;
-        if (!is_v && mine) meta[(grp % kTc5MetaRing) * kTc5PgMax + b.j] = b.valid;
+        if (!is_v && mine) meta[(grp % MR) * PG + b.j] = b.valid;
         __syncwarp();
         if (j0 == 0 && lane == 0) mbar_expect_tx(full0 + 8 * slot, ng * PAGE_BYTES);
         __syncwarp();
@@ -596,17 +608,18 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       for (int first = item; first < seg_end && ok; first += PG, ++g) {
         const int ng = min(PG, seg_end - first), ncol = ng * GP, b = g & 1, use = g >> 1;
         const uint32_t s_addr = lane_addr + COL_S + b * kTc5Tok;
-        volatile int* gmeta = meta + (g % kTc5MetaRing) * kTc5PgMax;
+        volatile int* gmeta = meta + (g % MR) * PG;
+        auto valid_of = [&](int j) { return FP8 ? gmeta[j] & 0xff : gmeta[j]; };     // tokens of the group's page j
         ok = warp_wait(s_full + 8 * b, use & 1);
         if (!ok) break;
         tc5_fence_after();
         // pages with fewer than GP tokens (the last page of a prefix), or a group that ends inside a
         // 32-column chunk, need per-column masks; everything else takes the plain path
         bool ragged = (ncol & 31) != 0;
-        for (int j = 0; j < ng; ++j) ragged |= gmeta[j] < GP;
+        for (int j = 0; j < ng; ++j) ragged |= valid_of(j) < GP;
         auto masked = [&](int col) {
           const int j = col / GP, t = col % GP;
-          return j >= ng || t >= gmeta[j];
+          return j >= ng || t >= valid_of(j);
         };
         const int col0 = 64 * h;                                // this thread's columns: col0 .. col0+63, below ncol
         if (warp_has_rows) {
@@ -634,9 +647,9 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
           if constexpr (FP8) {
 #pragma unroll
             for (int x = 0; x < 2 * NP; ++x) {
-              const int j = (col0 + x * PW) / GP, at = (g % kTc5MetaRing) * kTc5PgMax + j;
-              kmul[x] = j < ng ? scale2 * kscale_meta[at] : 1.f;
-              vexp[x] = j < ng ? static_cast<float>((__float_as_int(vscale_meta[at]) >> 23) - 127) : 0.f;
+              const int j = (col0 + x * PW) / GP;
+              kmul[x] = j < ng ? scale2 * kscale_meta[(g % MR) * PG + j] : 1.f;
+              vexp[x] = j < ng ? static_cast<float>((gmeta[j] >> 8) - 127) : 0.f;
             }
           }
           float mx_own = -INFINITY;
@@ -717,14 +730,14 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
           // rows of V past the end of the prefix may hold anything (even NaN): clear them once the
           // tile has landed (all softmax warps, whether or not they own rows)
           bool any_short = false;
-          for (int j = 0; j < ng; ++j) any_short |= gmeta[j] < GP;
+          for (int j = 0; j < ng; ++j) any_short |= valid_of(j) < GP;
           if (any_short) {
             const int slot = g % NR;
             ok = warp_wait(vfull + 8 * slot, (g / NR) & 1);
             if (!ok) break;
             uint8_t* vg = gen + (NR + slot) * SLOT;
             for (int j = 0; j < ng; ++j) {
-              const int valid = gmeta[j];
+              const int valid = valid_of(j);
               for (int idx = tid; idx < (GP - valid) * (D / 8); idx += kTc5SoftmaxWarps * 32) {
                 const int t = j * GP + valid + idx / (D / 8), ch = idx % (D / 8);
                 *reinterpret_cast<uint4*>(vg + (ch >> 3) * HS + tc5_sw(t, ch & 7)) = make_uint4(0u, 0u, 0u, 0u);

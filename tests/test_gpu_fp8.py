@@ -128,6 +128,63 @@ def test_fp8_pages_of_very_different_scales(g, d):
         assert (np.abs(snap["lse_p"] - ref["lse_p"]) <= 1e-3).all()
 
 
+def dequantised_prefix(layer, cfg, s, h):
+    """Keys and values [L, d] of sequence s and KV head h as stage 4 must see them: code times scale, in float64."""
+    import torch
+    L = int(layer.kv_len[s])
+    phys = layer.page_table[s, :-(-L // cfg.page_size)].long()
+    return [(codes[phys, h].view(torch.float8_e4m3fn).double() * scale[phys, h].double()[:, None, None]).reshape(-1, cfg.head_dim)[:L]
+            for codes, scale in ((layer.k_codes, layer.k_scale), (layer.v_codes, layer.v_scale))]
+
+
+def assert_dense_rows_exact_to_p(layer, cfg, q, s, what):
+    """o_p and lse_p of a dense step against float64, column by column.  P is rounded to fp16 relative to the row's
+    largest weight: half a unit of its 11 bits, below 2^-14 half a unit of 2^-24, so that a column is off by at most
+    2^-11 sum p |v| + 2^-25 p_max sum |v|; as much again for the sums in fp32 and 2^x."""
+    import torch
+    G = cfg.n_q_heads // cfg.n_kv_heads
+    for h in range(cfg.n_kv_heads):
+        k, v = dequantised_prefix(layer, cfg, s, h)
+        for i in range(h * G, (h + 1) * G):
+            sc = q[s, :, i].double() @ k.T * cfg.sm_scale
+            p = torch.softmax(sc, -1)
+            bound = 2.0 ** -10 * (p @ v.abs()) + 2.0 ** -24 * p.amax(-1, keepdim=True) * v.abs().sum(0)
+            err = (layer.o_p[s, :, i].double() - p @ v).abs()
+            assert (err <= bound).all(), f"{what}: sequence {s} head {i}, worst {(err / bound).max():.3g} of the bound"
+            assert (layer.lse_p[s, :, i].double() - torch.logsumexp(sc, -1)).abs().max() <= 1e-3, what
+
+
+@pytest.mark.parametrize("g,d", [(16, 64), (16, 128), (32, 64), (32, 128), (64, 64), (64, 128)])
+def test_fp8_runs_of_one_page_prompts_in_one_share(g, d):
+    """One long prompt beside 40 of a single page, lengths 1 .. g and scales of every size: a CTA's share of the list
+    then holds some twenty groups of one page, as many as the staging rings have slots."""
+    import torch
+    from paper_2604_12056_b200.layer import LosaLayer
+    # a one-page segment is charged 11 items: 148 shares of at least 26 of them
+    N, Hkv, Bk = 41, 8, 4
+    P = 26 * 11 * 148 // Hkv
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(g + d)
+    lens = [P * g] + [1 + int(x) for x in torch.randint(0, g, (N - 1,), generator=gen, device="cuda")]
+    cfg = wl.config("c2", n_q_heads=Hkv, n_kv_heads=Hkv, head_dim=d, page_size=g, kv_lens=tuple(lens), block_size=Bk, steps=1,
+                    topk=1, m_active=1)
+    n_phys = P + N - 1
+    f = torch.exp2(torch.randint(-2, 9, (2, n_phys, Hkv, 1, 1), generator=gen, device="cuda"))
+    kp = (torch.randn(n_phys, Hkv, g, d, generator=gen, device="cuda") * f[0].clamp_max(4.0)).bfloat16()
+    vp = (torch.randn(n_phys, Hkv, g, d, generator=gen, device="cuda") * f[1].clamp_max(64.0)).bfloat16()
+    order = torch.randperm(n_phys, generator=gen, device="cuda").to(torch.int32)
+    table = torch.zeros(N, cfg.max_pages_per_seq, dtype=torch.int32, device="cuda")
+    table[0, :P] = order[:P]
+    table[1:, 0] = order[P:]
+    q = torch.randn(N, Bk, Hkv, d, generator=gen, device="cuda").bfloat16()
+    kb, vb = (torch.randn(N, Bk, Hkv, d, generator=gen, device="cuda").bfloat16() for _ in range(2))
+    layer = LosaLayer(cfg, kp, vp, table, torch.tensor(lens, dtype=torch.int32, device="cuda"), fp8_kv=True)
+    layer.run_step(q, kb, vb, torch.ones(N, dtype=torch.int32, device="cuda"))
+    assert layer.ctx.poll_status() == 0
+    for s in range(1, N):
+        assert_dense_rows_exact_to_p(layer, cfg, q, s, f"page {g} d {d}, {lens[s]} tokens")
+
+
 def test_fp8_cache_dense_mode_and_two_row_groups():
     cfg = wl.config("c4", kv_lens=(64 * 40 + 17,), steps=2, topk=8, m_active=40, heavy_frac=0.0)
     run_fp8_blocks(cfg)
