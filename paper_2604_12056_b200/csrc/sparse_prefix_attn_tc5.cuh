@@ -28,7 +28,12 @@ template <bool FP8> constexpr int tc5_threads() { return FP8 ? 512 : 384; }
 constexpr int kTc5Tok = 128;                     // tokens per group = N of Q K^T = columns of one S buffer
 constexpr float kTc5Tau = 8.0f;                  // reference maximum moves only when it would grow by more than this (log2 units)
 constexpr int kTc5XchgBytes = (2 * 2 + 1) * kRowsPerGroup * 4;   // row maxima [group parity][set][row], row sums [row]
+// FP8 pages: binary places by which P is held above the reference maximum.  P stays below 2^(8 + 7) < 65504.
+constexpr float kTc5Fp8Lift = 7.0f;
 constexpr int kTc5StgMax = 20;                   // FP8 pages: staging slots per tensor, one page each, at most
+// FP8: value pages whose multiplier is kept.  Page x + 32 is issued once page x + 32 - 20 or a later one has
+// been converted, and with it the whole group of page x (at most 8 pages).
+constexpr int kTc5VmulRing = 32;
 // Groups whose per-page data (token counts; FP8: scales) is kept.  The K producer writes a page's entry
 // when it issues the page's copy, so the ring must be longer than its lead over the softmax warps.  A
 // group never spans two segments, so in a run of one-page segments every page in flight is a group of
@@ -40,9 +45,9 @@ constexpr int kTc5StgMax = 20;                   // FP8 pages: staging slots per
 // Small pages have up to 20 staging slots, a lead of 23; the others at most 10.
 template <int D, int GP, bool FP8> constexpr int tc5_meta_ring() { return FP8 && GP * D <= 2048 ? 32 : 16; }
 // Barriers, the segment prefix and index cache, the exchange arrays, the charged prefix, the staging
-// barriers (landed, emptied; K and V), two words per page of the meta ring
+// barriers (landed, emptied; K and V) and the value pages' multipliers, two words per page of the meta ring
 template <int D, int GP, bool FP8> constexpr int tc5_tail_bytes() {
-  return kTailBytes + kTc5XchgBytes + (kMaxSegments + 2) * 4 + kTc5StgMax * 2 * (8 + 8) + tc5_meta_ring<D, GP, FP8>() * (kTc5Tok / GP) * 8;
+  return kTailBytes + kTc5XchgBytes + (kMaxSegments + 2) * 4 + kTc5StgMax * 2 * (8 + 8) + kTc5VmulRing * 4 + tc5_meta_ring<D, GP, FP8>() * (kTc5Tok / GP) * 8;
 }
 
 template <int D> constexpr int tc5_slot_bytes() { return kTc5Tok * D * 2; }
@@ -140,8 +145,12 @@ __device__ __forceinline__ uint32_t tc5_sw(int t, int c) { return static_cast<ui
 // converted to fp16 instead of bf16).  The scales stay out of the conversion, which is bound by its
 // instruction count: the key scale joins the softmax scale of the page's columns, and the value
 // scale 2^e is added to their exponent, so that P' = p 2^e multiplies the codes of V and the row sum
-// takes its columns back by 2^-e.  The reference maximum is that of the shifted exponents: every P'
-// has the same headroom, and with equal scales the bits are those of scaled operands.  A group is 2 x 16 KiB of codes:
+// takes its columns back by 2^-e.  P' is rounded to fp16 relative to the largest p 2^e, so a page whose
+// scale lies below another's would lose that many places of fp16's range.  Two things keep every
+// weight at least as precise as an unscaled one: only the scales' part from 2^-6 to 2^0 goes into the
+// exponent (pages of values up to 448; once a share has met a larger one, the converters go over each
+// group of V a second time and multiply by the rest, exactly), and the reference lies 2^7 below the maximum.  A weight is then subnormal only 2^-15 or more
+// below its row's largest, 2^-14 without scales.  A group is 2 x 16 KiB of codes:
 // one warp needs about 3.8 us for 16 KiB, and while the two producing warps did this work it set the
 // pace (eight 32K prompts: dense step 372 us, sparse step at three active tokens 120 us).  Now 224 and
 // 81 us (scaling in the converters: 245 and 87; bit moves instead of the conversion instruction: 306
@@ -195,8 +204,11 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   // FP8: per tensor, a staging slot's page has landed / has been converted
   const uint32_t stg_bars = smem_u32(vpre + kMaxSegments + 1) + 4;   // (kMaxSegments + 1 is odd)
   const uint32_t kstg_full = stg_bars, vstg_full = kstg_full + 8 * kTc5StgMax, kstg_free = vstg_full + 8 * kTc5StgMax, vstg_free = kstg_free + 8 * kTc5StgMax;
-  // per page of the groups in flight, [MR][PG]: valid tokens (FP8: and the value scale's exponent field << 8), FP8: key scale
-  volatile int* meta = vpre + kMaxSegments + 2 + 8 * kTc5StgMax;
+  // FP8: multipliers of the newest value pages' codes, as two fp16; whether any was other than one
+  volatile uint32_t* vmul = reinterpret_cast<volatile uint32_t*>(vpre + kMaxSegments + 2 + 8 * kTc5StgMax);
+  volatile int* vmul_used = abort_flag + 2;
+  // per page of the groups in flight, [MR][PG]: valid tokens (FP8: and the exponent field of the value scale's part in P << 8), FP8: key scale
+  volatile int* meta = vpre + kMaxSegments + 2 + 8 * kTc5StgMax + kTc5VmulRing;
   volatile float* kscale_meta = reinterpret_cast<volatile float*>(const_cast<int*>(meta) + MR * PG);
   const bool staged = p.N * p.B <= kStageIdx && p.N <= kStageSeq;
 
@@ -226,6 +238,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         mbar_init(vstg_free + 8 * i, 2);
       }
     *abort_flag = 0;
+    *vmul_used = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -327,15 +340,15 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       }
       return r;
     };
-    auto stage_c = [&](int i, Ready& r) {             // bounds; FP8, K warp: the page's scales (their address needs the physical page)
+    auto stage_c = [&](int i, Ready& r) {             // bounds; FP8: the page's scales (their address needs the physical page)
       if (i < hi) {
         if (r.phys < 0 || r.phys >= p.n_phys || r.valid <= 0) {
           set_status(p.status, LOSA_ERR_BOUNDS);
           r.phys = 0;
           r.valid = 0;
         }
-        if (FP8 && !is_v) {
-          r.ks = __ldg(p.k_scale + static_cast<size_t>(r.phys) * p.Hkv + r.kh);
+        if (FP8) {
+          if (!is_v) r.ks = __ldg(p.k_scale + static_cast<size_t>(r.phys) * p.Hkv + r.kh);
           r.vs = __ldg(p.v_scale + static_cast<size_t>(r.phys) * p.Hkv + r.kh);
         }
       }
@@ -344,15 +357,22 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     auto issue = [&](int b0, const Ready& b) {
       const int nb = min(32, hi - b0);
       if constexpr (FP8) {                            // page by page: every lane handles its own staging slot
+        // the value scale: 2^-6 .. 2^0 of it go into P (as an exponent field), the rest onto the codes
+        const int e = (__float_as_int(b.vs) >> 23) & 0xff, in_p = min(max(e, 127 - 6), 127);
+        const __half2 in_v = __float2half2_rn(__int_as_float((e - in_p + 127) << 23));
         for (int pos = 0; pos < nb; ++pos) {
           int ok = 1;
           if (lane == pos) {
             const int x = b0 + pos - lo, slot = x % NSP, round = x / NSP;
             if (round > 0) ok = mbar_wait(emptied + 8 * slot, (round - 1) & 1, abort_flag, p.status, p.wait_cycles);
             if (ok) {
-              if (!is_v) {
+              if (is_v) {
+                const uint32_t m2 = *reinterpret_cast<const uint32_t*>(&in_v);
+                vmul[x % kTc5VmulRing] = m2;
+                if (m2 != 0x3c003c00u) *vmul_used = 1;
+              } else {
                 const int at = (b.grp % MR) * PG + b.j;
-                meta[at] = b.valid | ((__float_as_int(b.vs) >> 23) & 0xff) << 8;
+                meta[at] = b.valid | in_p << 8;
                 kscale_meta[at] = b.ks;
               }
               mbar_expect_tx(landed + 8 * slot, STG);
@@ -472,6 +492,22 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
           if (lane == 0) mbar_arrive(emptied + 8 * ss, 1);
         }
         if (!ok) break;
+        if (is_v && *vmul_used) {                     // this lane's chunks once more, times what of the scales is not in P
+#pragma unroll 1
+          for (int i = 0; i < ng * NU; ++i) {
+            const int pg = i / NU, u = i % NU;
+            const uint32_t mul = vmul[(first + pg - lo) % kTc5VmulRing];
+            const __half2 m2 = *reinterpret_cast<const __half2*>(&mul);
+            uint4* at = reinterpret_cast<uint4*>(ring_gen + sr * SLOT + (c >> 3) * HS + tc5_sw(pg * GP + tl + u * TPI, c & 7));
+            uint4 x = *at;
+            auto scale = [&](uint32_t& y) {
+              const __half2 v = __hmul2(*reinterpret_cast<const __half2*>(&y), m2);
+              y = *reinterpret_cast<const uint32_t*>(&v);
+            };
+            scale(x.x); scale(x.y); scale(x.z); scale(x.w);
+            *at = x;
+          }
+        }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs read the slot through the async proxy
         __syncwarp();
         if (lane == 0) mbar_arrive(full0 + 8 * sr, 1);
@@ -672,9 +708,10 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
           ok = pair_sync();
           const float m_new = fmaxf(mx_own, xmax[(b * 2 + (h ^ 1)) * kRowsPerGroup + r]) * (FP8 ? 1.f : scale2);
           float corr = 1.f;
-          if (m_new > m_ref + kTc5Tau || (m_ref == -INFINITY && m_new > -INFINITY)) {
-            corr = (m_ref == -INFINITY) ? 0.f : ex2(m_ref - m_new);
-            m_ref = m_new;
+          constexpr float LIFT = FP8 ? kTc5Fp8Lift : 0.f;
+          if (m_new > m_ref + (kTc5Tau + LIFT) || (m_ref == -INFINITY && m_new > -INFINITY)) {
+            corr = (m_ref == -INFINITY) ? 0.f : ex2(m_ref - (m_new - LIFT));
+            m_ref = m_new - LIFT;
             l *= corr;
           }
           // ---- rescale O (rare): the previous group's P V must have run; all lanes of the warp take

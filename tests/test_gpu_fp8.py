@@ -128,30 +128,90 @@ def test_fp8_pages_of_very_different_scales(g, d):
         assert (np.abs(snap["lse_p"] - ref["lse_p"]) <= 1e-3).all()
 
 
-def dequantised_prefix(layer, cfg, s, h):
-    """Keys and values [L, d] of sequence s and KV head h as stage 4 must see them: code times scale, in float64."""
+def listed_prefix(layer, cfg, s, h):
+    """Keys and values [n, d] of the pages listed for sequence s and KV head h as stage 4 must see them: code times
+    scale, in float64."""
     import torch
-    L = int(layer.kv_len[s])
-    phys = layer.page_table[s, :-(-L // cfg.page_size)].long()
-    return [(codes[phys, h].view(torch.float8_e4m3fn).double() * scale[phys, h].double()[:, None, None]).reshape(-1, cfg.head_dim)[:L]
+    pages = layer.union_pages[s, h, :int(layer.union_count[s, h])].long()
+    valid = (pages[:, None] * cfg.page_size + torch.arange(cfg.page_size, device="cuda")) < layer.kv_len[s]
+    phys = layer.page_table[s, pages].long()
+    return [(codes[phys, h].view(torch.float8_e4m3fn).double() * scale[phys, h].double()[:, None, None])[valid]
             for codes, scale in ((layer.k_codes, layer.k_scale), (layer.v_codes, layer.v_scale))]
 
 
-def assert_dense_rows_exact_to_p(layer, cfg, q, s, what):
-    """o_p and lse_p of a dense step against float64, column by column.  P is rounded to fp16 relative to the row's
-    largest weight: half a unit of its 11 bits, below 2^-14 half a unit of 2^-24, so that a column is off by at most
-    2^-11 sum p |v| + 2^-25 p_max sum |v|; as much again for the sums in fp32 and 2^x."""
+def assert_rows_exact_to_p(layer, cfg, q, s, what, p_bits=11):
+    """o_p and lse_p of the last step's active rows against float64 over the listed pages, column by column.  P is
+    rounded to fp16 relative to the row's largest weight: half a unit of its 11 bits, below 2^-14 half a unit of
+    2^-24, so that a column is off by at most 2^-11 sum p |v| + 2^-25 p_max sum |v|; as much again for the sums in
+    fp32 and 2^x."""
     import torch
     G = cfg.n_q_heads // cfg.n_kv_heads
+    act = layer.active_idx[s, :int(layer.n_active[s])].long()
     for h in range(cfg.n_kv_heads):
-        k, v = dequantised_prefix(layer, cfg, s, h)
+        k, v = listed_prefix(layer, cfg, s, h)
         for i in range(h * G, (h + 1) * G):
-            sc = q[s, :, i].double() @ k.T * cfg.sm_scale
+            sc = q[s, act, i].double() @ k.T * cfg.sm_scale
             p = torch.softmax(sc, -1)
-            bound = 2.0 ** -10 * (p @ v.abs()) + 2.0 ** -24 * p.amax(-1, keepdim=True) * v.abs().sum(0)
-            err = (layer.o_p[s, :, i].double() - p @ v).abs()
+            bound = 2.0 ** (1 - p_bits) * (p @ v.abs()) + 2.0 ** -24 * p.amax(-1, keepdim=True) * v.abs().sum(0)
+            err = (layer.o_p[s, act, i].double() - p @ v).abs()
             assert (err <= bound).all(), f"{what}: sequence {s} head {i}, worst {(err / bound).max():.3g} of the bound"
-            assert (layer.lse_p[s, :, i].double() - torch.logsumexp(sc, -1)).abs().max() <= 1e-3, what
+            assert (layer.lse_p[s, act, i].double() - torch.logsumexp(sc, -1)).abs().max() <= 1e-3, what
+
+
+def hot_token_layer(g, d, at, channel, above, n_tokens, N=1, Hkv=2, G=2):
+    """Prompts whose values are those of ordinary low-scale pages (N(0.5, 1)), except for one page of zeros with one
+    token of a single large channel; that token's score lies `above` (log2 units) over all others, which are about
+    equal.  Returns the layer after its dense step, the config, the queries and sequence 0's expected output."""
+    import torch
+    from paper_2604_12056_b200.layer import LosaLayer
+    Bk = 4
+    cfg = wl.config("c2", n_q_heads=Hkv * G, n_kv_heads=Hkv, head_dim=d, page_size=g, kv_lens=(n_tokens,) * N, block_size=Bk, steps=1,
+                    topk=1, m_active=1)
+    P = N * cfg.max_pages_per_seq
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(7 * g + d + at)
+    rnd = lambda *shape: torch.randn(*shape, generator=gen, device="cuda")
+    u = rnd(d)
+    u /= u.norm()
+    kp = 0.05 * rnd(P, Hkv, g, d)
+    kp -= (kp @ u)[..., None] * u                           # orthogonal to the queries' direction
+    vp = 0.5 + rnd(P, Hkv, g, d)
+    page, tok = torch.arange(N, device="cuda") * cfg.max_pages_per_seq + at // g, at % g
+    vp[page] = 0.0
+    vp[page, :, tok, 0] = channel
+    kp[page, :, tok] = u * (above * float(np.log(2.0)) / (4.0 * cfg.sm_scale))
+    q = (4.0 * u + 0.02 * rnd(N, Bk, Hkv * G, d)).bfloat16()
+    kb, vb = (rnd(N, Bk, Hkv, d).bfloat16() for _ in range(2))
+    table = torch.arange(P, dtype=torch.int32, device="cuda").view(N, -1).contiguous()
+    layer = LosaLayer(cfg, kp.bfloat16(), vp.bfloat16(), table, torch.full((N,), n_tokens, dtype=torch.int32, device="cuda"), fp8_kv=True)
+    layer.run_step(q, kb, vb, torch.ones(N, dtype=torch.int32, device="cuda"))
+    assert layer.ctx.poll_status() == 0
+    out = torch.empty(q.shape[1:], dtype=torch.float64, device="cuda")
+    for i in range(Hkv * G):
+        k, v = listed_prefix(layer, cfg, 0, i // G)
+        k, v = (torch.cat([a, b[0, :, i // G].double()]) for a, b in ((k, kb), (v, vb)))
+        out[:, i] = torch.softmax(q[0, :, i].double() @ k.T * cfg.sm_scale, -1) @ v
+    return layer, cfg, q, out
+
+
+@pytest.mark.parametrize("g,d", [(16, 64), (32, 64), (64, 64), (16, 128), (32, 128), (64, 128)])
+@pytest.mark.parametrize("above,channel,at", [(13.0, 30000.0, 3), (14.0, 16000.0, 100), (13.0, 57000.0, 700), (6.0, 400.0, 3), (10.0, 600.0, 3)])
+def test_fp8_weights_beside_a_page_of_large_scale(g, d, above, channel, at):
+    """The value scale of a page must not cost the weights of pages with smaller scales their bits: the columns that
+    only low-scale pages fill are as good as with weights that carry no scale."""
+    layer, cfg, q, out = hot_token_layer(g, d, at, channel, above, 1000)
+    assert float(layer.v_scale.max()) >= 64 * float(layer.v_scale.min())
+    assert_rows_exact_to_p(layer, cfg, q, 0, f"page {g} d {d}")
+    assert ((layer.out[0].double() - out).abs() <= 2e-2 + 1e-2 * out.abs()).all()
+
+
+def test_fp8_output_beside_a_page_of_large_scale_in_a_batch():
+    """Eight prompts of 32,000 tokens: a share holds some 440 pages, and the hot token's page is in the first of each
+    prompt's.  The low-scale tokens of that share are a sixth of the output's other columns."""
+    layer, cfg, q, out = hot_token_layer(16, 128, 3, 30000.0, 13.0, 32000, N=8, Hkv=8, G=1)
+    err = (layer.out[0].double() - out).abs()
+    assert (err <= 2e-2 + 1e-2 * out.abs()).all(), f"worst {err[..., 1:].max():.3g}"
+    assert_rows_exact_to_p(layer, cfg, q, 0, "batch")
 
 
 @pytest.mark.parametrize("g,d", [(16, 64), (16, 128), (32, 64), (32, 128), (64, 64), (64, 128)])
@@ -182,7 +242,7 @@ def test_fp8_runs_of_one_page_prompts_in_one_share(g, d):
     layer.run_step(q, kb, vb, torch.ones(N, dtype=torch.int32, device="cuda"))
     assert layer.ctx.poll_status() == 0
     for s in range(1, N):
-        assert_dense_rows_exact_to_p(layer, cfg, q, s, f"page {g} d {d}, {lens[s]} tokens")
+        assert_rows_exact_to_p(layer, cfg, q, s, f"page {g} d {d}, {lens[s]} tokens")
 
 
 def test_fp8_cache_dense_mode_and_two_row_groups():
