@@ -357,9 +357,10 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     auto issue = [&](int b0, const Ready& b) {
       const int nb = min(32, hi - b0);
       if constexpr (FP8) {                            // page by page: every lane handles its own staging slot
-        // the value scale: 2^-6 .. 2^0 of it go into P (as an exponent field), the rest onto the codes
+        // the value scale: 2^-6 .. 2^0 of it go into P (as an exponent field), the rest onto the codes (also
+        // what a caller's own scale has beside its power of two)
         const int e = (__float_as_int(b.vs) >> 23) & 0xff, in_p = min(max(e, 127 - 6), 127);
-        const __half2 in_v = __float2half2_rn(__int_as_float((e - in_p + 127) << 23));
+        const __half2 in_v = __float2half2_rn(b.vs * __int_as_float((254 - in_p) << 23));
         for (int pos = 0; pos < nb; ++pos) {
           int ok = 1;
           if (lane == pos) {

@@ -141,9 +141,9 @@ def listed_prefix(layer, cfg, s, h):
 
 def assert_rows_exact_to_p(layer, cfg, q, s, what, p_bits=11):
     """o_p and lse_p of the last step's active rows against float64 over the listed pages, column by column.  P is
-    rounded to fp16 relative to the row's largest weight: half a unit of its 11 bits, below 2^-14 half a unit of
-    2^-24, so that a column is off by at most 2^-11 sum p |v| + 2^-25 p_max sum |v|; as much again for the sums in
-    fp32 and 2^x."""
+    rounded to fp16 relative to the row's largest weight: half a unit of its p_bits = 11 bits, below 2^-14 half a unit
+    of 2^-24, so that a column is off by at most 2^-11 sum p |v| + 2^-25 p_max sum |v|; as much again for the sums
+    in fp32 and 2^x."""
     import torch
     G = cfg.n_q_heads // cfg.n_kv_heads
     act = layer.active_idx[s, :int(layer.n_active[s])].long()
@@ -212,6 +212,20 @@ def test_fp8_output_beside_a_page_of_large_scale_in_a_batch():
     err = (layer.out[0].double() - out).abs()
     assert (err <= 2e-2 + 1e-2 * out.abs()).all(), f"worst {err[..., 1:].max():.3g}"
     assert_rows_exact_to_p(layer, cfg, q, 0, "batch")
+
+
+@pytest.mark.parametrize("g,d", [(16, 64), (32, 128), (64, 128)])
+def test_fp8_scales_of_any_value(g, d):
+    """A caller's own scales, not powers of two and below 2^-6 too: every page's code times its scale.  The multiplier, its
+    product with a code and P are each rounded to 11 bits: three times 2^-11, so 2^-9 takes their place in the bound."""
+    import torch
+    from paper_2604_12056_b200 import binding as B
+    layer, cfg, q, _ = hot_token_layer(g, d, 3, 400.0, 1.0, 1000)
+    for scale, factors in ((layer.k_scale, (1.0, 0.81, 1.3)), (layer.v_scale, (1.0, 1.37, 0.0137, 91.0))):
+        scale *= torch.tensor(factors, device="cuda")[torch.arange(len(scale), device="cuda") % len(factors)][:, None]
+    B.losa_sparse_prefix_attn(layer.ctx, q, layer.kv, layer.active_idx, layer.n_active, layer.union_pages, layer.union_count, layer.state)
+    assert layer.ctx.poll_status() == 0
+    assert_rows_exact_to_p(layer, cfg, q, 0, f"page {g} d {d}", p_bits=9)
 
 
 @pytest.mark.parametrize("g,d", [(16, 64), (16, 128), (32, 64), (32, 128), (64, 64), (64, 128)])
