@@ -272,16 +272,6 @@ __device__ __forceinline__ int2 segment_records(int T, int n, int start, int end
   return make_int2(b0, cta_of(end - 1) - b0 + 1);
 }
 
-// CTAs of the tensor-core kernel that share a charged list of length V (page: tokens per page).  It takes
-// pages in groups of 128 tokens, and a group costs the same whatever it holds: short shares are
-// rounded up to whole groups, which costs the main kernel nothing and leaves the merge fewer records.
-__device__ __forceinline__ int tc5_ctas(int V, int n_ctas, int page) {
-  const int pg = 128 / page, per = V / n_ctas + (V % n_ctas ? 1 : 0);
-  if (per >= 8 * pg || per < 1) return n_ctas;
-  const int whole = (per + pg - 1) / pg * pg;
-  return (V + whole - 1) / whole;
-}
-
 // The tensor-core kernel cuts a list in which every non-empty segment is charged segment_pad(rows)
 // items on top of its pages (placed before them): entering a segment costs a CTA about as much as
 // that many pages (drain of the pipeline, the record, the new Q tile, refill), so equal shares of

@@ -357,7 +357,7 @@ def test_many_rows_per_kv_head_fp32():
 
 
 @pytest.mark.parametrize("kw", [
-    # one KV head: more than 32 partial records for every row, whole-group shares that leave CTAs without pages
+    # one KV head: more than 32 partial records for every row
     dict(n_q_heads=4, n_kv_heads=1, kv_lens=(40000,), block_size=8, steps=2, m_active=2, topk=16),
     # more (sequence, head) lists than resident selection CTAs: one CTA takes all active slots of its list
     dict(n_q_heads=28, n_kv_heads=4, kv_lens=(97,) * 36 + (0, 1, 33, 500), block_size=5, steps=3, m_active=3, topk=2),
@@ -368,6 +368,36 @@ def test_many_rows_per_kv_head_fp32():
 ])
 def test_whole_step_call_grids_and_merges_at_their_edges(kw):
     run_blocks(wl.config("c2", **kw), fused=True)
+
+
+@pytest.mark.parametrize("g,d", [(16, 64), (32, 128), (64, 128)])
+def test_short_lists_are_cut_into_single_pages(g, d):
+    """bf16, a list shorter than the number of CTAs: a page is a share of its own, so P is rounded relative to the page's
+    largest weight.  With one token far above the others on every page that weight is 1, and the output is as good as
+    fp32: scores of about 10 with a relative error of 2^-20, 2^x and the sums below that."""
+    import torch
+    from paper_2604_12056_b200.layer import LosaLayer
+    P, Hq, Bk = 40, 4, 4
+    cfg = wl.config("c2", n_q_heads=Hq, n_kv_heads=1, head_dim=d, page_size=g, kv_lens=(P * g,), block_size=Bk, steps=1, topk=1,
+                    m_active=1)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(g + d)
+    n = cfg.max_pages_per_seq
+    u = torch.nn.functional.normalize(torch.randn(d, generator=gen, device="cuda"), dim=0)
+    far = torch.full((n, 1, g, 1), -60.0, device="cuda")
+    far[:, :, 3] = 10.0 + torch.rand(n, 1, 1, generator=gen, device="cuda")
+    kp = (far * u / (4.0 * cfg.sm_scale)).bfloat16()
+    vp = torch.randn(n, 1, g, d, generator=gen, device="cuda").bfloat16()
+    q = (4.0 * u + 0.02 * torch.randn(1, Bk, Hq, d, generator=gen, device="cuda")).bfloat16()
+    kb, vb = (torch.randn(1, Bk, 1, d, generator=gen, device="cuda").bfloat16() for _ in range(2))
+    table = torch.arange(n, dtype=torch.int32, device="cuda")[None].contiguous()
+    layer = LosaLayer(cfg, kp, vp, table, torch.tensor([P * g], dtype=torch.int32, device="cuda"))
+    layer.run_step(q, kb, vb, torch.ones(1, dtype=torch.int32, device="cuda"))
+    assert layer.ctx.poll_status() == 0
+    k, v = (t[:P, 0].reshape(-1, d).double() for t in (kp, vp))
+    p = torch.softmax(q[0].double() @ k.T * cfg.sm_scale, -1)
+    err = (layer.o_p[0].double() - p @ v).abs() / (p @ v.abs())
+    assert err.max() < 2e-5, f"{err.max():.3g}"
 
 
 @pytest.mark.parametrize("g,d,m,G", [(16, 64, 1, 1), (32, 128, 4, 4), (64, 64, 5, 4), (16, 128, 8, 4), (32, 64, 11, 3), (64, 128, 16, 4), (32, 128, 13, 5), (16, 64, 16, 8)])
