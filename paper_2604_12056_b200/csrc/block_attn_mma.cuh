@@ -56,14 +56,16 @@ struct BlockAttnParams {
 // MERGE = true (stage 5 of the six-call path): the in-block part is merged with the prefix
 // statistics by log-sum-exp and the attention output is written (Section 2.2 / 4.3); MERGE = false
 // (whole-step path): the normalised in-block part goes to `ob_out` and L_b to `lse_out`.
-// Row tile rt (64 rows) of (sequence s, KV head kh), by the kMmaThreads threads of a CTA.
-template <int D, int BK, bool MERGE>
+// Row tile rt (64 rows) of (sequence s, KV head kh), by the kMmaThreads threads of a CTA.  CW: columns of O
+// per pass.  All D at once is the faster way (K_b V_b and o_p are requested once); 64 take 32 registers
+// less, which the refinement's CTAs do not have.
+template <int D, int BK, bool MERGE, int CW>
 __device__ __forceinline__ void block_attn_mma_cta(const BlockAttnParams& p, BlockAttnSmem<D, BK>& sm, int rt, int kh, int s) {
   const int B = p.B, Hq = p.Hq, Hkv = p.Hkv;
   const float sm_scale = p.sm_scale;
   constexpr int KS = BlockAttnSmem<D, BK>::KS, VS = BlockAttnSmem<D, BK>::VS;
   constexpr int NT = BK / 8;         // key tiles of S
-  constexpr int NO = D / 8;          // column tiles of O
+  constexpr int NO = CW / 8;         // column tiles of O per pass
   __nv_bfloat16* Ks = sm.k;
   __nv_bfloat16* Vt = sm.vt;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -147,20 +149,20 @@ __device__ __forceinline__ void block_attn_mma_cta(const BlockAttnParams& p, Blo
   l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
   l1 += __shfl_xor_sync(0xffffffffu, l1, 1);
   l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
-  // ---- O = P V_b, 64 columns at a time (all at once would take 32 more registers than the refinement's CTAs have)
+  // ---- O = P V_b
   const float Lb0 = m0 + logf(l0), Lb1 = m1 + logf(l1);
 #pragma unroll
-  for (int j0 = 0; j0 < NO; j0 += 8) {
-    float o[8][4];
+  for (int j0 = 0; j0 < D / 8; j0 += NO) {
+    float o[NO][4];
 #pragma unroll
-    for (int jn = 0; jn < 8; ++jn)
+    for (int jn = 0; jn < NO; ++jn)
 #pragma unroll
       for (int e = 0; e < 4; ++e) o[jn][e] = 0.f;
 #pragma unroll
     for (int kk = 0; kk < BK / 16; ++kk) {
       const uint32_t a[4] = {pa[2 * kk][0], pa[2 * kk][1], pa[2 * kk + 1][0], pa[2 * kk + 1][1]};
 #pragma unroll
-      for (int jn = 0; jn < 8; ++jn) {
+      for (int jn = 0; jn < NO; ++jn) {
         const uint32_t* vr = reinterpret_cast<const uint32_t*>(Vt + (8 * (j0 + jn) + g) * VS + 16 * kk);
         mma_bf16_16816(o[jn], a, vr[t4], vr[4 + t4]);
       }
@@ -174,20 +176,27 @@ __device__ __forceinline__ void block_attn_mma_cta(const BlockAttnParams& p, Blo
         const float M2 = fmaxf(Lp, Lb);
         const float L = M2 + logf(expf(Lp - M2) + expf(Lb - M2));
         const float wp = expf(Lp - L), wb = expf(Lb - L) / l;
+        // the cached prefix output as it is stored (fp32 or bf16); all of it is requested before the first store,
+        // which the compiler cannot tell apart from these loads (stage 5 in a graph: 5.7 us, one by one 11.7)
+        float2 pv[NO];
+        if (p.o_p_bf16) {
 #pragma unroll
-        for (int jn = 0; jn < 8; ++jn) {
-          float2 pv;                                 // the cached prefix output as it is stored (fp32 or bf16)
-          if (p.o_p_bf16) pv = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(static_cast<const __nv_bfloat16*>(p.o_p) + at + 8 * jn));
-          else pv = *reinterpret_cast<const float2*>(static_cast<const float*>(p.o_p) + at + 8 * jn);
-          const float x = (wp > 0.f ? wp * pv.x : 0.f) + wb * o[jn][e0];
-          const float y = (wp > 0.f ? wp * pv.y : 0.f) + wb * o[jn][e0 + 1];
+          for (int jn = 0; jn < NO; ++jn) pv[jn] = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(static_cast<const __nv_bfloat16*>(p.o_p) + at + 8 * jn));
+        } else {
+#pragma unroll
+          for (int jn = 0; jn < NO; ++jn) pv[jn] = *reinterpret_cast<const float2*>(static_cast<const float*>(p.o_p) + at + 8 * jn);
+        }
+#pragma unroll
+        for (int jn = 0; jn < NO; ++jn) {
+          const float x = (wp > 0.f ? wp * pv[jn].x : 0.f) + wb * o[jn][e0];
+          const float y = (wp > 0.f ? wp * pv[jn].y : 0.f) + wb * o[jn][e0 + 1];
           *reinterpret_cast<__nv_bfloat162*>(p.out + at + 8 * jn) = __floats2bfloat162_rn(x, y);
         }
         if (j0 == 0 && p.lse_out && t4 == 0) p.lse_out[gr] = L;
       } else {
         const float inv = 1.f / l;
 #pragma unroll
-        for (int jn = 0; jn < 8; ++jn)
+        for (int jn = 0; jn < NO; ++jn)
           *reinterpret_cast<float2*>(p.ob_out + at + 8 * jn) = make_float2(o[jn][e0] * inv, o[jn][e0 + 1] * inv);
         if (j0 == 0 && t4 == 0) p.lse_out[gr] = Lb;
       }

@@ -160,7 +160,7 @@ template <int D, int BK, bool MERGE>
 __global__ void __launch_bounds__(kMmaThreads) block_attn_mma_kernel(BlockAttnParams p) {
   grid_dep_wait();
   __shared__ __align__(16) BlockAttnSmem<D, BK> sm;
-  block_attn_mma_cta<D, BK, MERGE>(p, sm, blockIdx.x, blockIdx.y, blockIdx.z);
+  block_attn_mma_cta<D, BK, MERGE, D>(p, sm, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
 // Whole-step path, last kernel: one warp per (token, head) row merges the prefix statistics with

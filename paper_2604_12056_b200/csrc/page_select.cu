@@ -409,7 +409,7 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
     const int t = qid - n_refine, sk = t / p.blk_tiles;
     if (!(p.step && __ldcg(p.step + sk / p.Hkv) == 0)) grid_dep_trigger();      // (as below)
     grid_dep_wait();
-    block_attn_mma_cta<D, BK, false>(bp, sm.b, t % p.blk_tiles, sk % p.Hkv, sk / p.Hkv);
+    block_attn_mma_cta<D, BK, false, 64>(bp, sm.b, t % p.blk_tiles, sk % p.Hkv, sk / p.Hkv);
     return;
   }
   const int pool = POOLED ? p.Hq / p.Hkv : 1, Hl = p.Hq / pool;
