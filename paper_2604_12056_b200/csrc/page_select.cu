@@ -114,7 +114,7 @@ __device__ __forceinline__ unsigned long long make_key(uint32_t ob, int p) {
 // (P <= kSelThreads * kSelPerThread) their order bits stay in registers for the whole selection.
 constexpr int kSelThreads = 128;
 constexpr int kSelPerThread = 8;
-constexpr int kSelSlots = 8;        // CTAs per (sequence, head): active slots are dealt out round-robin
+constexpr int kSelSlots = 8;        // CTAs per (sequence, head), at most: active slots are dealt out round-robin
 
 template <bool CACHED, typename Row, typename F>
 __device__ __forceinline__ void for_each_key(const uint32_t (&cache)[kSelPerThread], const Row& row,
@@ -841,6 +841,22 @@ int32_t topk_max_sortable(const losa_ctx* c) {
   return n;
 }
 
+// CTAs of the refinement per list, i.e. (sequence, head) or (sequence, KV head): the fewest from three up that
+// fill at least five sixths of the waves they take, else eight; no more than block tokens.  Most slots are idle
+// on most steps, and an idle CTA costs its dispatch; on steps with many active tokens a last wave that is
+// nearly empty doubles the time.  Whole step, us, at 3 / 8 / 32 active tokens (888 resident CTAs):
+//   256 lists (8 x 32K tokens)  3 CTAs 107 / 163 / 364, 4 CTAs (1.15 waves) 108 / 176 / 405, 8 CTAs 111 / 171 / 370
+//   512 lists (16 x 8K)         3 CTAs 130 / 178 / 362, 2 CTAs (1.15 waves) 128 / 190 / 416, 8 CTAs 134 / 182 / 353
+//   128 lists (4 x 24K)         6 CTAs 63 / 87 / 172, 7 CTAs (1.01 waves) 64 / 92 / 184, 3 CTAs 64 / 94 / 198
+int refine_slots(int lists, int resident, int block_size) {
+  int slots = kSelSlots;
+  for (int n = kSelSlots - 1; n >= 3; --n) {
+    const int ctas = n * lists, waves = (ctas + resident - 1) / resident;
+    if (6 * ctas >= 5 * waves * resident) slots = n;
+  }
+  return std::min(slots, block_size);
+}
+
 bool selects_by_refinement(const losa_ctx* c, int32_t k, int selector) {
   return c->shape.dtype == LOSA_BF16 && (selector == kSelectorExact || selector == kSelectorPooled) && k <= kSelCap &&
          c->shape.max_pages_per_seq > 0;
@@ -883,11 +899,8 @@ int32_t launch_page_scores_topk(losa_ctx* c, const void* q, const losa_kv_t* kv,
     rp.union_pages = union_pages;
     rp.union_count = union_count;
     if (with_union) *union_done = true;
-    // CTAs per (sequence, head): up to eight, but no more than are resident together - most slots are
-    // idle on most steps, and an idle CTA costs its dispatch (eight sequences of 32 heads: 2,048 CTAs for
-    // 768 busy ones kept the grid's tail waiting)
-    const int lists = sh.batch * (sh.n_q_heads / pool), resident = c->n_sms * (pool > 1 ? 4 : 6);
-    rp.slots = std::max(1, std::min({kSelSlots, sh.block_size, (resident + lists - 1) / lists}));
+    const int lists = sh.batch * (sh.n_q_heads / pool);
+    rp.slots = refine_slots(lists, c->n_sms * (pool > 1 ? 4 : 6), sh.block_size);
     rp.blk_tiles = block_attn_tiles(sh);
     const bool with_block = blk && blk->q;
     const BlockAttnParams bp = with_block ? block_attn_params(c, blk->q, blk->k_blk, blk->v_blk) : BlockAttnParams{};

@@ -359,7 +359,9 @@ def test_many_rows_per_kv_head_fp32():
 @pytest.mark.parametrize("kw", [
     # one KV head: more than 32 partial records for every row
     dict(n_q_heads=4, n_kv_heads=1, kv_lens=(40000,), block_size=8, steps=2, m_active=2, topk=16),
-    # more (sequence, head) lists than resident selection CTAs: one CTA takes all active slots of its list
+    # 256 (sequence, head) lists: three selection CTAs each, which take the active slots round-robin
+    dict(n_q_heads=32, n_kv_heads=8, kv_lens=(97,) * 6 + (1, 500), block_size=13, steps=3, m_active=11, topk=2),
+    # more lists than resident selection CTAs
     dict(n_q_heads=28, n_kv_heads=4, kv_lens=(97,) * 36 + (0, 1, 33, 500), block_size=5, steps=3, m_active=3, topk=2),
     # in-block row tiles of the selection's grid: one partial tile, and a second tile of one row
     dict(n_q_heads=2, n_kv_heads=2, kv_lens=(70, 300), block_size=1, steps=2, m_active=1, topk=2),
