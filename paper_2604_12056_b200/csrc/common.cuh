@@ -118,7 +118,7 @@ inline void launch_split(int carveout, void (*kernel)(KArgs...), dim3 grid, dim3
   attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
   attr[1].val.sharedMemCarveout = carveout;
   cfg.attrs = attr;
-  cfg.numAttrs = 2;
+  cfg.numAttrs = carveout == cudaSharedmemCarveoutDefault ? 1 : 2;      // default: the driver's choice
   (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);   // the error, if any, is read by after_launch()
 }
 // The kernels of a step: one shared-memory / L1 split for all of them.  An SM changes its split only

@@ -900,15 +900,20 @@ int32_t launch_page_scores_topk(losa_ctx* c, const void* q, const losa_kv_t* kv,
     rp.union_count = union_count;
     if (with_union) *union_done = true;
     const int lists = sh.batch * (sh.n_q_heads / pool);
-    rp.slots = refine_slots(lists, c->n_sms * (pool > 1 ? 4 : 6), sh.block_size);
+    // As a call of its own (six-call path) the kernel has nothing beside or behind it: eight CTAs per list, and the
+    // driver's shared-memory / L1 split, under which the summaries that a list's queries share are found in
+    // L1 (eight 32K prompts, 32 active tokens: 188 us with bounds, 200 with a step's CTAs and split; three: 28.4 and 29.2).
+    const bool in_step = blk != nullptr;
+    rp.slots = in_step ? refine_slots(lists, c->n_sms * (pool > 1 ? 4 : 6), sh.block_size) : std::min(kSelSlots, sh.block_size);
     rp.blk_tiles = block_attn_tiles(sh);
     const bool with_block = blk && blk->q;
     const BlockAttnParams bp = with_block ? block_attn_params(c, blk->q, blk->k_blk, blk->v_blk) : BlockAttnParams{};
     const int grid = lists * rp.slots + (with_block ? rp.blk_tiles * sh.n_kv_heads * sh.batch : 0);
     with_block_attn_shape(sh, [&](auto d, auto bk) {
       constexpr int D = decltype(d)::value, BK = decltype(bk)::value;
-      if (pool > 1) launch_k(topk_refine_kernel<D, true, BK>, grid, kSelThreads, 0, st, rp, bp);
-      else launch_k(topk_refine_kernel<D, false, BK>, grid, kSelThreads, 0, st, rp, bp);
+      const int split = in_step ? cudaSharedmemCarveoutMaxShared : cudaSharedmemCarveoutDefault;
+      if (pool > 1) launch_split(split, topk_refine_kernel<D, true, BK>, grid, kSelThreads, 0, st, rp, bp);
+      else launch_split(split, topk_refine_kernel<D, false, BK>, grid, kSelThreads, 0, st, rp, bp);
     });
     return after_launch(c);
   }
