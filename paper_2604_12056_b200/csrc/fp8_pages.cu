@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kFp8Warps * 32) fp8_pages_kernel(Fp8Params p) 
       if (p.blk_aligned) {
         raw[i] = *reinterpret_cast<const uint4*>(src);
       } else {
-        __nv_bfloat16 e[8];
+        alignas(16) __nv_bfloat16 e[8];
 #pragma unroll
         for (int x = 0; x < 8; ++x) e[x] = src[x];
         raw[i] = *reinterpret_cast<const uint4*>(e);
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kFp8Warps * 32) fp8_pages_kernel(Fp8Params p) 
       if (t0 + i * RPI < n_old) {
         float v[8];
         fp8_decode8(old[i], v);
-        __nv_bfloat162 h[4];
+        alignas(16) __nv_bfloat162 h[4];
 #pragma unroll
         for (int x = 0; x < 4; ++x) h[x] = __floats2bfloat162_rn(v[2 * x] * old_scale, v[2 * x + 1] * old_scale);
         raw[i] = *reinterpret_cast<const uint4*>(h);
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(kFp8Warps * 32) fp8_pages_kernel(Fp8Params p) 
       for (int x = 0; x < 8; ++x)
         if (lo[x] <= hi[x]) { lo[x] = a[x] * new_scale; hi[x] = b[x] * new_scale; }
     }
-    __nv_bfloat162 a[4], b[4];                                      // exact: four significant bits
+    alignas(16) __nv_bfloat162 a[4], b[4];                                      // exact: four significant bits
 #pragma unroll
     for (int x = 0; x < 4; ++x) {
       a[x] = __floats2bfloat162_rn(lo[2 * x], lo[2 * x + 1]);
