@@ -352,7 +352,7 @@ int32_t losa_denoise_step(losa_ctx* ctx, const void* q, const void* k_blk, const
   const cudaError_t joined = fork ? cudaStreamWaitEvent(st, ctx->ev_join, 0) : cudaSuccess;
   if (rc != LOSA_OK) return rc;
   LOSA_CUDA_TRY(ctx, joined);
-  if (finish_fuses_combine(ctx)) return launch_attn_finish(ctx, q, buf->active_idx, buf->n_active, slot_map, state, out, lse_out_opt, st);
+  if (finish_fuses_combine(ctx)) return launch_attn_finish(ctx, q, slot_map, state, out, lse_out_opt, st);
   return launch_merge_commit(ctx, q, state, out, lse_out_opt, st);
 }
 

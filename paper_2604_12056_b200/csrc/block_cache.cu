@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(kMmaThreads) block_attn_mma_kernel(BlockAttnPa
   block_attn_mma_cta<D, BK, MERGE, D>(p, sm, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
-// Whole-step path, last kernel: one warp per (token, head) row merges the prefix statistics with
+// Whole-step path, last kernel in fp32 (bf16: attn_finish_kernel): one warp per (token, head) row merges the prefix statistics with
 // the in-block part (Section 2.2 / 4.3), writes the output, and keeps the row's query for the next
 // step's Eq. 1; block 0 also bumps the step counters.
 template <typename T, int D>
@@ -452,9 +452,6 @@ int32_t launch_block_attn(losa_ctx* c, const void* q, const void* k_blk, const v
 
 int32_t launch_merge_commit(losa_ctx* c, const void* q, losa_state_t* state, void* out, float* lse_out_opt,
                             cudaStream_t st) {
-  const bool bf = c->shape.dtype == LOSA_BF16;
-  if (bf && c->shape.head_dim == 128) return launch_merge_commit_t<__nv_bfloat16, 128>(c, q, state, out, lse_out_opt, st);
-  if (bf) return launch_merge_commit_t<__nv_bfloat16, 64>(c, q, state, out, lse_out_opt, st);
   if (c->shape.head_dim == 128) return launch_merge_commit_t<float, 128>(c, q, state, out, lse_out_opt, st);
   return launch_merge_commit_t<float, 64>(c, q, state, out, lse_out_opt, st);
 }

@@ -55,14 +55,14 @@ int32_t launch_sparse_prefix_attn(losa_ctx* c, const void* q, const losa_kv_t* k
 // launch_attn_finish merges them, merges with the in-block part, writes the output, keeps the
 // queries and bumps the step (one kernel instead of combine + merge_commit).
 bool finish_fuses_combine(const losa_ctx* c);
-int32_t launch_attn_finish(losa_ctx* c, const void* q, const int32_t* active_idx, const int32_t* n_active, const int32_t* slot_map,
-                           losa_state_t* state, void* out, float* lse_out_opt, cudaStream_t st);
+int32_t launch_attn_finish(losa_ctx* c, const void* q, const int32_t* slot_map, losa_state_t* state, void* out,
+                           float* lse_out_opt, cudaStream_t st);
 
 int32_t launch_block_attn_merge(losa_ctx* c, const void* q, const void* k_blk, const void* v_blk,
                                 const losa_state_t* state, void* out, float* lse_out_opt,
                                 cudaStream_t st);
 
-// Whole-step path: in-block attention alone (o_b, L_b into the workspace), then merge with the
+// Whole-step path: in-block attention alone (o_b, L_b into the workspace); fp32: then merge with the
 // prefix statistics, write the output, keep the queries and bump the step counters.
 int32_t launch_block_attn(losa_ctx* c, const void* q, const void* k_blk, const void* v_blk, cudaStream_t st);
 int32_t launch_merge_commit(losa_ctx* c, const void* q, losa_state_t* state, void* out, float* lse_out_opt,

@@ -487,28 +487,21 @@ int32_t launch_sparse_prefix_attn(losa_ctx* c, const void* q, const losa_kv_t* k
 
 bool finish_fuses_combine(const losa_ctx* c) { return c->shape.dtype == LOSA_BF16; }
 
-int32_t launch_attn_finish(losa_ctx* c, const void* q, const int32_t* active_idx, const int32_t* n_active,
-                           const int32_t* slot_map,
-                           losa_state_t* state, void* out, float* lse_out_opt, cudaStream_t st) {
+int32_t launch_attn_finish(losa_ctx* c, const void* q, const int32_t* slot_map, losa_state_t* state, void* out,
+                           float* lse_out_opt, cudaStream_t st) {
   const losa_shape_t& sh = c->shape;
-  AttnParams ap = {};
-  ap.active_idx = active_idx;
-  ap.n_active = n_active;
+  AttnParams ap = {};                       // (what the merge reads of it)
   ap.partials = reinterpret_cast<float*>(c->ws + c->lay.partials);
   ap.seg_records = reinterpret_cast<int2*>(c->ws + c->lay.seg_records);
   ap.o_p = state->o_p;
   ap.o_p_bf16 = state->o_p_format == LOSA_STATE_BF16 ? 1 : 0;
   ap.lse_p = state->lse_p;
-  ap.status = status_ptr(c);
   ap.N = sh.batch;
   ap.B = sh.block_size;
   ap.Hq = sh.n_q_heads;
   ap.Hkv = sh.n_kv_heads;
   ap.G = sh.n_q_heads / sh.n_kv_heads;
-  ap.n_rg = c->lay.n_row_groups;
-  ap.n_seg = c->lay.n_segments;
   ap.n_sk = sh.batch * sh.n_kv_heads;
-  ap.n_ctas = c->lay.n_ctas;
   FinishParams fp;
   fp.q = q;
   fp.slot_map = slot_map;
