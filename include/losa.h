@@ -360,12 +360,13 @@ typedef struct {
  * finalize_block = 0) in one call, with the same results as the six calls in order: the index
  * buffers of `buf` receive what stages 1-3 produce, state->o_p / lse_p what stage 4 produces,
  * out / lse_out_opt what stage 5 produces; q_prev and step are updated as by stage 6.
- * Being one call, it may schedule freely inside: the in-block attention of stage 5 (which needs
- * nothing from stages 1-4) runs on a second stream owned by the context and is joined before a
- * final merge kernel that also keeps the queries; where stage 2 runs the candidate refinement
- * (bf16, k <= 512) that kernel also writes stage 3's union.  All work is ordered after prior work on
- * `stream` and complete when `stream` reaches the end of the call's work; the call can be captured
- * in a CUDA graph after one un-captured call on the context (which creates the second stream). */
+ * Being one call, it may schedule freely inside.  The in-block attention of stage 5 needs nothing from
+ * stages 1-4: where stage 2 runs the candidate refinement (bf16, exact or pooled lists, k <= 512) that
+ * kernel's grid carries it and also writes stage 3's union; elsewhere it runs on a second stream
+ * owned by the context, which the first such call creates, and is joined before the final merge
+ * kernel, which also keeps the queries.  All work is ordered after prior work on `stream` and
+ * complete when `stream` reaches the end of the call's work; the call can be captured in a CUDA graph
+ * after one un-captured call on the context. */
 int32_t losa_denoise_step(losa_ctx* ctx, const void* q, const void* k_blk, const void* v_blk, void* out,
                           float* lse_out_opt, losa_kv_t* kv, losa_state_t* state,
                           const losa_step_buffers_t* buf, const int32_t* m_per_seq, int32_t k,

@@ -575,7 +575,7 @@ __global__ void __launch_bounds__(kPsThreads, 1) page_scores_stream_kernel(PsPar
 constexpr float kMmaErrCoef = 1.0f / 8192.0f;
 constexpr int kMmaWP = 16;                          // pages per warp and tile
 constexpr int kMmaTP = kPsWarps * kMmaWP;           // pages per tile
-constexpr int kMmaStages = 2;                       // tiles in shared memory: two leave room for the CTAs of the in-block attention, which runs beside
+constexpr int kMmaStages = 2;                       // tiles in shared memory (one ahead of the one in use)
 
 __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                                uint32_t b0, uint32_t b1) {
