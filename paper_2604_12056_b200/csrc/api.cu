@@ -325,6 +325,9 @@ int32_t losa_denoise_step(losa_ctx* ctx, const void* q, const void* k_blk, const
   // refinement, that kernel's grid carries it; elsewhere (fp32, long lists) it runs on a second stream.
   const BlockInputs blk = {q, k_blk, v_blk};
   const bool fork = !selects_by_refinement(ctx, k, ctx->pooled_selection);
+  const bool from_bits = union_from_bits(ctx, k);   // stage 4 takes the union from the selection's page bitmaps
+  rc = prepare_sparse_prefix_attn(ctx, kv);
+  if (rc != LOSA_OK) return rc;
   if (fork) {
     if (!ctx->side_stream) {
       // lowest priority: when CTAs of both streams are pending, those of stages 1-4 go first
@@ -341,19 +344,19 @@ int32_t losa_denoise_step(losa_ctx* ctx, const void* q, const void* k_blk, const
     LOSA_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_join, ctx->side_stream));
   }
   rc = launch_select_active(ctx, q, state->q_prev, sh.n_q_heads * sh.head_dim, m_per_seq, state->step,
-                            buf->active_idx, buf->n_active, nullptr, st, 0.0, slot_map);
+                            buf->active_idx, buf->n_active, nullptr, st, 0.0, slot_map,
+                            reinterpret_cast<uint32_t*>(ctx->ws + ctx->lay.union_bits), from_bits ? sh.n_kv_heads * union_words(ctx) : 0);
   bool union_done = false;                              // stage 3 written by the selection kernel itself
   if (rc == LOSA_OK) rc = launch_page_scores_topk(ctx, q, kv, buf->active_idx, buf->n_active, state->step, k, buf->topk_pages, nullptr, st, ctx->pooled_selection, true, buf->union_pages, buf->union_count, &union_done, fork ? nullptr : &blk);
   if (rc == LOSA_OK && !union_done) rc = launch_page_union(ctx, buf->topk_pages, buf->active_idx, buf->n_active, k, kv->kv_len, state->step, buf->union_pages, buf->union_count, st);
-  if (rc == LOSA_OK) rc = launch_sparse_prefix_attn(ctx, q, kv, buf->active_idx, buf->n_active, buf->union_pages, buf->union_count, state, st, true);
+  if (rc == LOSA_OK) rc = launch_sparse_prefix_attn(ctx, q, kv, buf->active_idx, buf->n_active, buf->union_pages, buf->union_count, state, st, true, from_bits);
   // (join, also when a launch above failed: the forked kernel must not be left reading the caller's
   // buffers, nor a capture be left with an unjoined branch;) then one pass over the rows: (merge of
   // the partial records,) merge with the block part, commit
   const cudaError_t joined = fork ? cudaStreamWaitEvent(st, ctx->ev_join, 0) : cudaSuccess;
   if (rc != LOSA_OK) return rc;
   LOSA_CUDA_TRY(ctx, joined);
-  if (finish_fuses_combine(ctx)) return launch_attn_finish(ctx, q, slot_map, state, out, lse_out_opt, st);
-  return launch_merge_commit(ctx, q, state, out, lse_out_opt, st);
+  return launch_attn_finish(ctx, q, slot_map, state, out, lse_out_opt, st);
 }
 
 int32_t losa_denoise_step_host(losa_ctx* ctx, const void* h_q, const void* h_k_blk, const void* h_v_blk,

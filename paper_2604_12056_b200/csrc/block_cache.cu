@@ -163,42 +163,6 @@ __global__ void __launch_bounds__(kMmaThreads) block_attn_mma_kernel(BlockAttnPa
   block_attn_mma_cta<D, BK, MERGE, D>(p, sm, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
-// Whole-step path, last kernel in fp32 (bf16: attn_finish_kernel): one warp per (token, head) row merges the prefix statistics with
-// the in-block part (Section 2.2 / 4.3), writes the output, and keeps the row's query for the next
-// step's Eq. 1; block 0 also bumps the step counters.
-template <typename T, int D>
-__global__ void __launch_bounds__(kThreads)
-merge_commit_kernel(const T* __restrict__ q, T* __restrict__ q_prev, const float* __restrict__ o_p,
-                    const float* __restrict__ lse_p, const float* __restrict__ o_b,
-                    const float* __restrict__ lse_b, T* __restrict__ out, float* __restrict__ lse_out,
-                    int32_t* __restrict__ step, int N, size_t n_rows) {
-  grid_dep_wait();
-  const int lane = threadIdx.x & 31;
-  const size_t row = static_cast<size_t>(blockIdx.x) * (kThreads / 32) + (threadIdx.x >> 5);
-  if (blockIdx.x == 0)
-    for (int s = threadIdx.x; s < N; s += kThreads) step[s] += 1;
-  if (row >= n_rows) return;
-  constexpr int C = D / 32;
-  float a[C], b[C];
-  T qv[C];
-#pragma unroll
-  for (int c = 0; c < C; ++c) {
-    a[c] = o_p[row * D + lane + 32 * c];
-    b[c] = o_b[row * D + lane + 32 * c];
-    qv[c] = q[row * D + lane + 32 * c];
-  }
-  const float Lp = lse_p[row], Lb = lse_b[row];
-  const float M = fmaxf(Lp, Lb);
-  const float L = M + logf(expf(Lp - M) + expf(Lb - M));
-  const float wp = expf(Lp - L), wb = expf(Lb - L);
-#pragma unroll
-  for (int c = 0; c < C; ++c) {
-    out[row * D + lane + 32 * c] = from_f32<T>((wp > 0.f ? wp * a[c] : 0.f) + wb * b[c]);
-    q_prev[row * D + lane + 32 * c] = qv[c];
-  }
-  if (lse_out && lane == 0) lse_out[row] = L;
-}
-
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
 commit_step_kernel(const uint4* __restrict__ q, uint4* __restrict__ q_prev, size_t n_vec,
@@ -353,19 +317,6 @@ int32_t launch_merge_t(losa_ctx* c, const void* q, const void* k_blk, const void
   return after_launch(c);
 }
 
-template <typename T, int D>
-int32_t launch_merge_commit_t(losa_ctx* c, const void* q, losa_state_t* state, void* out, float* lse_out,
-                              cudaStream_t st) {
-  const losa_shape_t& sh = c->shape;
-  const size_t n_rows = static_cast<size_t>(sh.batch) * sh.block_size * sh.n_q_heads;
-  const int blocks = static_cast<int>((n_rows + kThreads / 32 - 1) / (kThreads / 32));
-  launch_k(merge_commit_kernel<T, D>, blocks, kThreads, 0, st, 
-      static_cast<const T*>(q), static_cast<T*>(state->q_prev), static_cast<const float*>(state->o_p), state->lse_p,
-      reinterpret_cast<const float*>(c->ws + c->lay.block_o), reinterpret_cast<const float*>(c->ws + c->lay.block_lse),
-      static_cast<T*>(out), lse_out, state->step, sh.batch, n_rows);
-  return after_launch(c);
-}
-
 template <typename T>
 int32_t launch_update_t(losa_ctx* c, losa_kv_t* kv, losa_state_t* state, const void* q,
                         const void* k_blk, const void* v_blk, int32_t finalize_block, cudaStream_t st) {
@@ -448,12 +399,6 @@ int32_t launch_block_attn(losa_ctx* c, const void* q, const void* k_blk, const v
   }
   if (c->shape.head_dim == 128) return launch_merge_t<float, 128, false>(c, q, k_blk, v_blk, nullptr, nullptr, lb, ob, st);
   return launch_merge_t<float, 64, false>(c, q, k_blk, v_blk, nullptr, nullptr, lb, ob, st);
-}
-
-int32_t launch_merge_commit(losa_ctx* c, const void* q, losa_state_t* state, void* out, float* lse_out_opt,
-                            cudaStream_t st) {
-  if (c->shape.head_dim == 128) return launch_merge_commit_t<float, 128>(c, q, state, out, lse_out_opt, st);
-  return launch_merge_commit_t<float, 64>(c, q, state, out, lse_out_opt, st);
 }
 
 int32_t launch_update_prefix_cache(losa_ctx* c, losa_kv_t* kv, losa_state_t* state, const void* q,

@@ -281,9 +281,11 @@ constexpr int kSegPadBase = 10, kSegPadRowsPer = 8;
 __device__ __forceinline__ int segment_pad(int rows) { return rows > 0 ? kSegPadBase + rows / kSegPadRowsPer : 0; }
 
 // Exclusive prefix of segment item counts into pre[0..n_seg] (shared memory), by one warp; with
-// vpre, also the prefix of the charged counts (pages + pad of every non-empty segment).
+// vpre, also the prefix of the charged counts (pages + pad of every non-empty segment).  count(sk): length of
+// the list of (sequence, KV head) sk.
+template <typename Count>
 __device__ __forceinline__ void segment_prefix(int* pre, int n_seg, int n_rg, int H_kv, int G,
-                                               const int32_t* n_active, const int32_t* union_count,
+                                               const int32_t* n_active, Count&& count,
                                                int B, int lane, int* vpre = nullptr) {
   int run = 0, vrun = 0;
   for (int base = 0; base < n_seg; base += 32) {
@@ -294,7 +296,7 @@ __device__ __forceinline__ void segment_prefix(int* pre, int n_seg, int n_rg, in
       int na = n_active[s];
       na = na < 0 ? 0 : (na > B ? B : na);
       const int rows = rows_in_group(na, G, rg);
-      c = rows > 0 ? max(union_count[sk], 0) : 0;
+      c = rows > 0 ? max(count(sk), 0) : 0;
       vc = c > 0 ? c + segment_pad(rows) : 0;
     }
     int inc = c, vinc = vc;

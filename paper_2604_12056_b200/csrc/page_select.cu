@@ -102,7 +102,7 @@ topk_kernel(const float* __restrict__ scores, const int32_t* __restrict__ kv_len
 // every key above that bin, and either finishes by sorting "taken + threshold bin" (a few dozen
 // keys) or narrows the range to the threshold bin and repeats.  A range of one value means the
 // remaining candidates tie on the score: the lowest page ids win, taken in page order.
-constexpr int kSelCap = 512;     // candidate keys a warp can sort; also the largest k of this path
+constexpr int kSelCap = kListCap;   // candidate keys a CTA can sort; also the largest k of this path
 constexpr int kSelBins = 256;
 
 __device__ __forceinline__ unsigned long long make_key(uint32_t ob, int p) {
@@ -130,10 +130,11 @@ __device__ __forceinline__ void for_each_key(const uint32_t (&cache)[kSelPerThre
   }
 }
 
+// bits: page bitmap that the chosen pages are ORed into, or null.
 template <bool CACHED, typename Row>
 __device__ __forceinline__ void topk_select_body(const Row& row, int P, int kk, int k,
-                                                 int32_t* out_pages, float* out_scores, int n_out) {
-  __shared__ unsigned long long cand[kSelCap];
+                                                 int32_t* out_pages, float* out_scores, int n_out, uint32_t* bits) {
+  __shared__ __align__(16) unsigned long long cand[kSelCap];
   __shared__ int hist[kSelBins];
   __shared__ uint32_t s_red[2][kSelThreads / 32];
   __shared__ int s_ncand, s_bstar, s_above, s_thr;
@@ -227,34 +228,43 @@ __device__ __forceinline__ void topk_select_body(const Row& row, int P, int kk, 
     __syncthreads();
   }
   __syncthreads();
-  // sort the candidates (descending) and emit the first kk
+  // order the candidates (descending) and emit the first kk
   const int ncand = s_ncand;
-  int n2 = 2;
-  while (n2 < ncand) n2 <<= 1;
-  for (int i = ncand + tid; i < n2; i += kSelThreads) cand[i] = 0ull;
-  __syncthreads();
-  for (int k2 = 2; k2 <= n2; k2 <<= 1) {
-    for (int j = k2 >> 1; j > 0; j >>= 1) {
-      for (int t = tid; t < (n2 >> 1); t += kSelThreads) {
-        const int i = ((t & ~(j - 1)) << 1) | (t & (j - 1));
-        const int x = i | j;
-        const unsigned long long ka = cand[i], kb = cand[x];
-        if ((ka < kb) == ((i & k2) == 0)) { cand[i] = kb; cand[x] = ka; }
-      }
-      __syncthreads();
+  auto emit = [&](int rank, unsigned long long key) {
+    const int pg = static_cast<int32_t>(0xffffffffu - static_cast<uint32_t>(key));
+    for (int gi = 0; gi < n_out; ++gi) {               // pooled: the list goes to every head of the group
+      out_pages[gi * k + rank] = pg;
+      if (out_scores) out_scores[gi * k + rank] = unorder_bits(static_cast<uint32_t>(key >> 32));
     }
-  }
-  for (int gi = 0; gi < n_out; ++gi) {               // pooled: the list goes to every head of the group
-    for (int j = tid; j < k; j += kSelThreads) {
-      if (j < kk) {
-        const unsigned long long key = cand[j];
-        out_pages[gi * k + j] = static_cast<int32_t>(0xffffffffu - static_cast<uint32_t>(key));
-        if (out_scores) out_scores[gi * k + j] = unorder_bits(static_cast<uint32_t>(key >> 32));
-      } else {
-        out_pages[gi * k + j] = -1;
+    if (bits) atomicOr(&bits[pg >> 5], 1u << (pg & 31));
+  };
+  if (ncand <= kSelThreads) {                          // few: a candidate's position is the number of larger keys (all differ)
+    if ((tid & ~31) < ncand) {
+      const unsigned long long mine = tid < ncand ? cand[tid] : ~0ull;
+      int rank = 0;
+      for (int i = 0; i < ncand; ++i) rank += cand[i] > mine ? 1 : 0;
+      if (tid < ncand && rank < kk) emit(rank, mine);
+    }
+  } else {
+    int n2 = 2;
+    while (n2 < ncand) n2 <<= 1;
+    for (int i = ncand + tid; i < n2; i += kSelThreads) cand[i] = 0ull;
+    __syncthreads();
+    for (int k2 = 2; k2 <= n2; k2 <<= 1) {
+      for (int j = k2 >> 1; j > 0; j >>= 1) {
+        for (int t = tid; t < (n2 >> 1); t += kSelThreads) {
+          const int i = ((t & ~(j - 1)) << 1) | (t & (j - 1));
+          const int x = i | j;
+          const unsigned long long ka = cand[i], kb = cand[x];
+          if ((ka < kb) == ((i & k2) == 0)) { cand[i] = kb; cand[x] = ka; }
+        }
+        __syncthreads();
       }
     }
+    for (int j = tid; j < kk; j += kSelThreads) emit(j, cand[j]);
   }
+  for (int gi = 0; gi < n_out; ++gi)
+    for (int j = kk + tid; j < k; j += kSelThreads) out_pages[gi * k + j] = -1;
 }
 
 
@@ -619,10 +629,8 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
       }
       __syncthreads();
       const RowView<false> rv{row, 1, p.score_stride};
-      topk_select_body<false>(rv, P, kk, p.k, out_pages, out_scores, pool);
+      topk_select_body<false>(rv, P, kk, p.k, out_pages, out_scores, pool, bits);
       __syncthreads();
-      if (bits)
-        for (int j = tid; j < kk; j += kSelThreads) mark(out_pages[j]);     // this CTA's own stores
       continue;
     }
     // a group of four lanes per candidate, 32 candidates per round; the physical page ids of four
@@ -726,7 +734,7 @@ topk_select_kernel(float* __restrict__ scores, const int32_t* __restrict__ kv_le
                    const int32_t* __restrict__ active_idx, const int32_t* __restrict__ n_active,
                    const int32_t* __restrict__ step, int32_t* __restrict__ topk_pages,
                    float* __restrict__ topk_scores, int N, int B, int Hq, int g, int k, int Pmax, int score_stride, int pool,
-                   int32_t* __restrict__ status) {
+                   uint32_t* __restrict__ union_bits, int G, int W, int32_t* __restrict__ status) {
   grid_dep_trigger();
   grid_dep_wait();
   // A CTA serves the active slots a = j, j + kSelSlots, ... of one (sequence, head): launching a CTA
@@ -734,7 +742,16 @@ topk_select_kernel(float* __restrict__ scores, const int32_t* __restrict__ kv_le
   // pool > 1 (pooled selector): one list per KV head from the maximum of its `pool` heads' rows
   const int qid = blockIdx.x, Hl = Hq / pool;
   const int h = (qid % Hl) * pool, s = (qid / Hl) % N, j = qid / (Hl * N);
-  if (step && step[s] == 0) return;
+  // fp32 whole step: the chosen pages go into the bitmap of the KV head's list, from which stage 4 takes the union (all
+  // zero at the start; on the first step of a block the whole prefix)
+  uint32_t* bits = union_bits ? union_bits + (static_cast<size_t>(s) * (Hq / G) + h / G) * W : nullptr;
+  if (step && step[s] == 0) {
+    if (bits && j == 0 && h % G == 0) {
+      const int P0 = min(pages_of(kv_len[s], g), Pmax);
+      for (int w = threadIdx.x; w < W; w += kSelThreads) bits[w] = prefix_word(w, P0);
+    }
+    return;
+  }
   int na = n_active[s];
   na = na > B ? B : na;
   int P = pages_of(kv_len[s], g);
@@ -746,7 +763,7 @@ topk_select_kernel(float* __restrict__ scores, const int32_t* __restrict__ kv_le
     RowView<POOLED> row{scores + ((static_cast<size_t>(s) * B + a) * Hq + h) * score_stride, pool, score_stride};
     const size_t o = ((static_cast<size_t>(s) * B + tok) * Hq + h) * k;
     if (P <= kSelThreads * kSelPerThread) {
-      topk_select_body<true>(row, P, kk, k, topk_pages + o, topk_scores ? topk_scores + o : nullptr, pool);
+      topk_select_body<true>(row, P, kk, k, topk_pages + o, topk_scores ? topk_scores + o : nullptr, pool, bits);
     } else {
       if (POOLED && pool > 1) {
         // the selection reads the row several times: pool once, into the group's first row (the
@@ -764,7 +781,7 @@ topk_select_kernel(float* __restrict__ scores, const int32_t* __restrict__ kv_le
         __syncthreads();
         row.g = 1;
       }
-      topk_select_body<false>(row, P, kk, k, topk_pages + o, topk_scores ? topk_scores + o : nullptr, pool);
+      topk_select_body<false>(row, P, kk, k, topk_pages + o, topk_scores ? topk_scores + o : nullptr, pool, bits);
     }
     __syncthreads();                                 // the shared state is reused by the next slot
   }
@@ -918,20 +935,23 @@ int32_t launch_page_scores_topk(losa_ctx* c, const void* q, const losa_kv_t* kv,
     return after_launch(c);
   }
   int32_t rc = selector == kSelectorMma ? launch_page_bounds(c, q, kv, active_idx, n_active, step, st, true, after_stage1)
-                                        : launch_page_scores(c, q, kv, active_idx, n_active, step, st);
+                                        : launch_page_scores(c, q, kv, active_idx, n_active, step, st, after_stage1);
   if (rc != LOSA_OK) return rc;
 
   float* sc = reinterpret_cast<float*>(c->ws + c->lay.scores);
   if (k <= kSelCap) {
+    uint32_t* bits = union_pages && union_done && union_from_bits(c, k) ? reinterpret_cast<uint32_t*>(c->ws + c->lay.union_bits) : nullptr;
+    const int G = sh.n_q_heads / sh.n_kv_heads;
+    if (bits) *union_done = true;
     const int queries = sh.batch * std::min<int>(sh.block_size, kSelSlots) * (sh.n_q_heads / pool);
     if (pool > 1)
       launch_k(topk_select_kernel<true>, queries, kSelThreads, 0, st,
           sc, kv->kv_len, active_idx, n_active, step, topk_pages, topk_scores_opt, sh.batch, sh.block_size,
-          sh.n_q_heads, sh.page_size, k, sh.max_pages_per_seq, c->lay.score_stride, pool, status_ptr(c));
+          sh.n_q_heads, sh.page_size, k, sh.max_pages_per_seq, c->lay.score_stride, pool, bits, G, union_words(c), status_ptr(c));
     else
       launch_k(topk_select_kernel<false>, queries, kSelThreads, 0, st,
           sc, kv->kv_len, active_idx, n_active, step, topk_pages, topk_scores_opt, sh.batch, sh.block_size,
-          sh.n_q_heads, sh.page_size, k, sh.max_pages_per_seq, c->lay.score_stride, 1, status_ptr(c));
+          sh.n_q_heads, sh.page_size, k, sh.max_pages_per_seq, c->lay.score_stride, 1, bits, G, union_words(c), status_ptr(c));
     return after_launch(c);
   }
   // budgets beyond what one warp can sort: whole-list bitonic sort, one CTA per query

@@ -20,7 +20,8 @@ select_active_kernel(const T* __restrict__ x_cur, const T* __restrict__ x_prev, 
                      const int32_t* __restrict__ m_per_seq, const int32_t* __restrict__ step,
                      int32_t* __restrict__ active_idx, int32_t* __restrict__ n_active,
                      float* __restrict__ delta_opt, double* __restrict__ delta_ws,
-                     unsigned int* __restrict__ counters, double tau, int32_t* __restrict__ slot_map) {
+                     unsigned int* __restrict__ counters, double tau, int32_t* __restrict__ slot_map,
+                     uint32_t* __restrict__ clear, int clear_words) {
   // Wait first, release afterwards: a kernel released by this one may read, before its own wait, what
   // earlier kernels of the stream wrote (the cache's lengths, summaries and step counters), so those
   // must have completed by then.
@@ -31,6 +32,8 @@ select_active_kernel(const T* __restrict__ x_cur, const T* __restrict__ x_prev, 
   const int m_given = m_per_seq ? m_per_seq[s] : -1;
   const int step_now = step ? step[s] : 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // the page bitmaps of the step that begins: read last by the step before, marked next by the selection
+  for (int w = i * kThreads + tid; w < clear_words; w += B * kThreads) clear[static_cast<size_t>(s) * clear_words + w] = 0u;
   const size_t row = (static_cast<size_t>(s) * B + i) * row_width;
   constexpr int kVec = 8;
   double acc = 0.0;
@@ -145,7 +148,8 @@ select_active_kernel(const T* __restrict__ x_cur, const T* __restrict__ x_prev, 
 
 int32_t launch_select_active(losa_ctx* c, const void* x_cur, const void* x_prev, int32_t row_width,
                              const int32_t* m_per_seq, const int32_t* step, int32_t* active_idx,
-                             int32_t* n_active, float* delta_opt, cudaStream_t st, double tau, int32_t* slot_map_opt) {
+                             int32_t* n_active, float* delta_opt, cudaStream_t st, double tau, int32_t* slot_map_opt,
+                             uint32_t* clear, int32_t clear_words) {
   const losa_shape_t& sh = c->shape;
   dim3 grid(sh.block_size, sh.batch);
   double* dws = reinterpret_cast<double*>(c->ws + c->lay.delta);
@@ -153,11 +157,11 @@ int32_t launch_select_active(losa_ctx* c, const void* x_cur, const void* x_prev,
   if (sh.dtype == LOSA_BF16) {
     launch_k(select_active_kernel<__nv_bfloat16>, grid, kThreads, 0, st, 
         static_cast<const __nv_bfloat16*>(x_cur), static_cast<const __nv_bfloat16*>(x_prev), row_width,
-        sh.block_size, m_per_seq, step, active_idx, n_active, delta_opt, dws, ctr, tau, slot_map_opt);
+        sh.block_size, m_per_seq, step, active_idx, n_active, delta_opt, dws, ctr, tau, slot_map_opt, clear, clear_words);
   } else {
     launch_k(select_active_kernel<float>, grid, kThreads, 0, st, 
         static_cast<const float*>(x_cur), static_cast<const float*>(x_prev), row_width, sh.block_size,
-        m_per_seq, step, active_idx, n_active, delta_opt, dws, ctr, tau, slot_map_opt);
+        m_per_seq, step, active_idx, n_active, delta_opt, dws, ctr, tau, slot_map_opt, clear, clear_words);
   }
   return after_launch(c);
 }
@@ -223,11 +227,11 @@ extern "C" int32_t losa_select_active_static(const losa_shape_t* shape, const vo
   if (shape->dtype == LOSA_BF16) {
     losa::launch_k(losa::select_active_kernel<__nv_bfloat16>, grid, losa::kThreads, 0, st, 
         static_cast<const __nv_bfloat16*>(x_cur), static_cast<const __nv_bfloat16*>(x_prev), row_width,
-        shape->block_size, m_per_seq, step, active_idx, n_active, delta_opt, scratch->delta, scratch->counters, 0.0, nullptr);
+        shape->block_size, m_per_seq, step, active_idx, n_active, delta_opt, scratch->delta, scratch->counters, 0.0, nullptr, nullptr, 0);
   } else {
     losa::launch_k(losa::select_active_kernel<float>, grid, losa::kThreads, 0, st, 
         static_cast<const float*>(x_cur), static_cast<const float*>(x_prev), row_width, shape->block_size,
-        m_per_seq, step, active_idx, n_active, delta_opt, scratch->delta, scratch->counters, 0.0, nullptr);
+        m_per_seq, step, active_idx, n_active, delta_opt, scratch->delta, scratch->counters, 0.0, nullptr, nullptr, 0);
   }
   return cudaGetLastError() == cudaSuccess ? LOSA_OK : LOSA_ERR_CUDA;
 }

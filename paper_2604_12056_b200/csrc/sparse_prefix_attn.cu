@@ -39,6 +39,10 @@ struct AttnParams {
   const int32_t* n_active;
   const int32_t* union_pages;
   const int32_t* union_count;
+  const uint32_t* union_bits;   // whole step: the lists as page bitmaps [n_sk][W], to be written to ...
+  int32_t* union_pages_out;     // ... these (fp32 kernel); null: the lists are in union_pages / union_count
+  int32_t* union_count_out;
+  int W;
   float* partials;
   int2* seg_records;    // per segment: first CTA and number of its partial records (written by the main kernels)
   void* o_p;                // cached prefix output, fp32 or bf16 (o_p_bf16)
@@ -61,6 +65,73 @@ __device__ __forceinline__ float* record_base(float* partials, int slot, int w, 
 }
 
 __device__ __forceinline__ int clamp_active(int na, int B) { return na < 0 ? 0 : (na > B ? B : na); }
+
+// Whole step: the lists as page bitmaps [n_sk][W] (written by the selection) in shared memory, with the number of
+// set bits of the list before every word, so that a page is found by its position in the list.
+struct UnionBits {
+  uint32_t* bits;
+  uint16_t* before;
+  int W;
+  // all lists, by the warps of the CTA (the caller synchronises)
+  __device__ __forceinline__ void load(const uint32_t* __restrict__ src, int n_sk, int warp, int n_warps, int lane) const {
+    for (int sk = warp; sk < n_sk; sk += n_warps) {
+      int run = 0;
+      for (int w0 = 0; w0 < W; w0 += 32) {
+        const int w = w0 + lane;
+        const uint32_t v = w < W ? src[sk * W + w] : 0u;
+        const int c = __popc(v);
+        int inc = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(0xffffffffu, inc, o);
+          if (lane >= o) inc += t;
+        }
+        if (w < W) {
+          bits[sk * W + w] = v;
+          before[sk * W + w] = static_cast<uint16_t>(run + inc - c);
+        }
+        run += __shfl_sync(0xffffffffu, inc, 31);
+      }
+    }
+  }
+  __device__ __forceinline__ int count(int sk) const {
+    const int e = (sk + 1) * W - 1;
+    return before[e] + __popc(bits[e]);
+  }
+  __device__ __forceinline__ int page(int sk, int u) const {     // entry u of list sk: its word, then the bit in the word
+    const uint16_t* first = before + sk * W;
+    int a = 0, b = W;                               // first[a] <= u (< first[b])
+    while (b - a > 1) {
+      const int m = (a + b) >> 1;
+      if (first[m] <= u) a = m; else b = m;
+    }
+    uint32_t v = bits[sk * W + a];
+    int n = u - first[a], at = 0;                   // the bit with n set bits below it
+#pragma unroll
+    for (int half = 16; half > 0; half >>= 1) {
+      const int c = __popc(v & ((1u << half) - 1u));
+      if (n >= c) { n -= c; at += half; v >>= half; }
+    }
+    return a * 32 + at;
+  }
+  // stage 3's output for the lists of this CTA, by one warp
+  __device__ __forceinline__ void write(const AttnParams& p, int lane) const {
+    for (int sk = blockIdx.x; sk < p.n_sk; sk += gridDim.x) {
+      int32_t* out = p.union_pages_out + static_cast<size_t>(sk) * p.Pmax;
+      for (int w = lane; w < W; w += 32) {
+        uint32_t v = bits[sk * W + w];
+        int pos = before[sk * W + w];
+        while (v) {
+          out[pos++] = w * 32 + __ffs(v) - 1;
+          v &= v - 1;
+        }
+      }
+      const int n = count(sk);
+      for (int t = n + lane; t < p.Pmax; t += 32) out[t] = -1;
+      if (lane == 0) p.union_count_out[sk] = n;
+    }
+  }
+};
 
 // C (2 or 4) consecutive elements as one vector access; a lane of the row-wise kernels below owns
 // columns lane * C .. lane * C + C - 1 of a row of D = 32 C elements.
@@ -200,7 +271,7 @@ __global__ void __launch_bounds__(kCombineThreads) attn_combine_kernel(AttnParam
   }
 }
 
-// Whole-step path, last kernel (bf16 main kernel): one warp per (sequence, block token, head) row.
+// Whole-step path, last kernel: one warp per (sequence, block token, head) row.
 // An active row merges its partial records (as the combine kernel does) and stores the new prefix
 // statistics; a stable row reads its cached ones (reuse rule, Section 4.2).  Either way the row is
 // then merged with the in-block part by log-sum-exp (Section 2.2 / 4.3), the output is written and
@@ -221,6 +292,7 @@ constexpr int kFinishThreads = 128;
 
 template <typename T, int D>
 __global__ void __launch_bounds__(kFinishThreads) attn_finish_kernel(AttnParams p, FinishParams f) {
+  constexpr bool LOG2 = !std::is_same_v<T, float>;     // partial maxima in base-2 units (tensor-core kernel)
   __shared__ __align__(16) float buf[kFinishThreads / 32][kMergeBatch * D];
   grid_dep_trigger();
   grid_dep_wait();
@@ -237,7 +309,10 @@ __global__ void __launch_bounds__(kFinishThreads) attn_finish_kernel(AttnParams 
   const T* q = static_cast<const T*>(f.q);
   float b[C];
   ldv<C>(f.o_b + row * D + lane * C, b);
-  const RawRow<C> qv = ld_raw<C>(q + row * D + lane * C);
+  RawRow<C> qv;                                         // (fp32: qf)
+  float qf[C];
+  if constexpr (LOG2) qv = ld_raw<C>(q + row * D + lane * C);
+  else ldv<C>(q + row * D + lane * C, qf);
   const float Lb = f.lse_b[row];
   // the cached prefix statistics as well: nine rows in ten are stable, and asking now saves them
   // a second round trip (an active row overwrites these below)
@@ -257,10 +332,10 @@ __global__ void __launch_bounds__(kFinishThreads) attn_finish_kernel(AttnParams 
       records = p.seg_records[sg];
     }
     float acc[C], M, Lsum;
-    merge_records<D, true>(p, buf[threadIdx.x >> 5], sg, r, records, lane, acc, M, Lsum);
+    merge_records<D, LOG2>(p, buf[threadIdx.x >> 5], sg, r, records, lane, acc, M, Lsum);
     const bool empty = !(Lsum > 0.f);
     const float inv = empty ? 0.f : 1.f / Lsum;
-    Lp = empty ? -INFINITY : (M + log2f(Lsum)) * kLn2;
+    Lp = empty ? -INFINITY : (LOG2 ? (M + log2f(Lsum)) * kLn2 : M + logf(Lsum));
 #pragma unroll
     for (int c = 0; c < C; ++c) a[c] = acc[c] * inv;
     st_state<C>(p.o_p, p.o_p_bf16, row * D + lane * C, a);
@@ -274,8 +349,13 @@ __global__ void __launch_bounds__(kFinishThreads) attn_finish_kernel(AttnParams 
   float o[C];
 #pragma unroll
   for (int c = 0; c < C; ++c) o[c] = (wp > 0.f ? wp * a[c] : 0.f) + wb * b[c];
-  st_bf16<C>(out + row * D + lane * C, o);
-  st_raw<C>(q_prev + row * D + lane * C, qv);
+  if constexpr (LOG2) {
+    st_bf16<C>(out + row * D + lane * C, o);
+    st_raw<C>(q_prev + row * D + lane * C, qv);
+  } else {
+    stv<C>(out + row * D + lane * C, o);
+    stv<C>(q_prev + row * D + lane * C, qf);
+  }
   if (f.lse_out && lane == 0) f.lse_out[row] = L;
 }
 
@@ -328,7 +408,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
                                   CUtensorMapFloatOOBfill);
 
-int32_t encode_pool_map(losa_ctx* c, unsigned char* blob, const void* pool, const losa_kv_t* kv) {
+int32_t encode_pool_map(losa_ctx* c, unsigned char* blob, const void* pool, const losa_kv_t* kv, bool is_v) {
   const losa_shape_t& sh = c->shape;
   if (!c->encode_fn) {
     void* fn = nullptr;
@@ -340,7 +420,7 @@ int32_t encode_pool_map(losa_ctx* c, unsigned char* blob, const void* pool, cons
   const cuuint64_t dims[4] = {static_cast<cuuint64_t>(sh.head_dim), static_cast<cuuint64_t>(sh.page_size),
                               static_cast<cuuint64_t>(sh.n_kv_heads), static_cast<cuuint64_t>(kv->n_phys_pages)};
   // bf16 pages: 64-element (128-byte) boxes with the 128-byte swizzle, as the MMA descriptors expect them;
-  // FP8 pages: whole rows of d bytes, unswizzled, into the staging slots (the kernel converts them)
+  // FP8 pages: whole rows of d bytes; K swizzled over the row (an MMA operand), V as it lies (the kernel converts it)
   const bool fp8 = kv->kv_format == LOSA_KV_FP8_E4M3;
   const cuuint64_t es = fp8 ? 1 : 2;
   const cuuint64_t strides[3] = {static_cast<cuuint64_t>(kv->stride_tok) * es, static_cast<cuuint64_t>(kv->stride_head) * es,
@@ -365,9 +445,9 @@ int32_t ensure_tensor_maps(losa_ctx* c, const losa_kv_t* kv) {
                     c->tmap_strides[2] == kv->stride_tok && c->tmap_n_phys == kv->n_phys_pages &&
                     c->tmap_format == kv->kv_format;
   if (same) return LOSA_OK;
-  int32_t rc = encode_pool_map(c, c->tmap_k, kv->k_pages, kv);
+  int32_t rc = encode_pool_map(c, c->tmap_k, kv->k_pages, kv, false);
   if (rc != LOSA_OK) return rc;
-  rc = encode_pool_map(c, c->tmap_v, kv->v_pages, kv);
+  rc = encode_pool_map(c, c->tmap_v, kv->v_pages, kv, true);
   if (rc != LOSA_OK) return rc;
   c->tmap_key_k = kv->k_pages;
   c->tmap_key_v = kv->v_pages;
@@ -401,7 +481,7 @@ int32_t launch_tc5(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool with
 }
 
 template <int D, int GP>
-int32_t launch_f32(losa_ctx* c, const AttnParams& ap, cudaStream_t st) {
+int32_t launch_f32(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool with_combine) {
   constexpr int smem = sizeof(F32Smem<D>);
   static_assert(smem <= kSmemBudget, "shared memory of the fp32 stage-4 kernel");
   if (!(c->attn_attr_set & 1)) {
@@ -412,7 +492,7 @@ int32_t launch_f32(losa_ctx* c, const AttnParams& ap, cudaStream_t st) {
   launch_k(attn_f32_kernel<D, GP>, ap.n_ctas, kF32Threads, smem, st, ap);
   if (c->profile) LOSA_CUDA_TRY(c, cudaEventRecord(c->ev_end, st));
   int32_t rc = after_launch(c);
-  if (rc != LOSA_OK) return rc;
+  if (rc != LOSA_OK || !with_combine) return rc;
   launch_k(attn_combine_kernel<D, false>, dim3(ap.n_seg, kCombineTiles), kCombineThreads, 0, st, ap);
   return after_launch(c);
 }
@@ -428,24 +508,26 @@ int32_t dispatch_page(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool w
     }
   }
   switch (c->shape.page_size) {
-    case 16: return bf ? launch_tc5<D, 16, false>(c, ap, st, with_combine) : launch_f32<D, 16>(c, ap, st);
-    case 32: return bf ? launch_tc5<D, 32, false>(c, ap, st, with_combine) : launch_f32<D, 32>(c, ap, st);
-    default: return bf ? launch_tc5<D, 64, false>(c, ap, st, with_combine) : launch_f32<D, 64>(c, ap, st);
+    case 16: return bf ? launch_tc5<D, 16, false>(c, ap, st, with_combine) : launch_f32<D, 16>(c, ap, st, with_combine);
+    case 32: return bf ? launch_tc5<D, 32, false>(c, ap, st, with_combine) : launch_f32<D, 32>(c, ap, st, with_combine);
+    default: return bf ? launch_tc5<D, 64, false>(c, ap, st, with_combine) : launch_f32<D, 64>(c, ap, st, with_combine);
   }
 }
 
 }  // namespace
 
 
+int32_t prepare_sparse_prefix_attn(losa_ctx* c, const losa_kv_t* kv) {
+  return c->shape.dtype == LOSA_BF16 ? ensure_tensor_maps(c, kv) : LOSA_OK;
+}
+
 int32_t launch_sparse_prefix_attn(losa_ctx* c, const void* q, const losa_kv_t* kv,
                                   const int32_t* active_idx, const int32_t* n_active,
                                   const int32_t* union_pages, const int32_t* union_count,
-                                  losa_state_t* state, cudaStream_t st, bool defer_combine) {
+                                  losa_state_t* state, cudaStream_t st, bool defer_combine, bool from_bits) {
   const losa_shape_t& sh = c->shape;
-  if (sh.dtype == LOSA_BF16) {
-    int32_t rc = ensure_tensor_maps(c, kv);
-    if (rc != LOSA_OK) return rc;
-  }
+  const int32_t rc = prepare_sparse_prefix_attn(c, kv);
+  if (rc != LOSA_OK) return rc;
   AttnParams ap;
   ap.q = q;
   ap.k_pages = kv->k_pages;
@@ -459,6 +541,10 @@ int32_t launch_sparse_prefix_attn(losa_ctx* c, const void* q, const losa_kv_t* k
   ap.n_active = n_active;
   ap.union_pages = union_pages;
   ap.union_count = union_count;
+  ap.union_bits = from_bits ? reinterpret_cast<const uint32_t*>(c->ws + c->lay.union_bits) : nullptr;
+  ap.union_pages_out = from_bits ? const_cast<int32_t*>(union_pages) : nullptr;
+  ap.union_count_out = from_bits ? const_cast<int32_t*>(union_count) : nullptr;
+  ap.W = union_words(c);
   ap.partials = reinterpret_cast<float*>(c->ws + c->lay.partials);
   ap.seg_records = reinterpret_cast<int2*>(c->ws + c->lay.seg_records);
   ap.o_p = state->o_p;
@@ -481,11 +567,8 @@ int32_t launch_sparse_prefix_attn(losa_ctx* c, const void* q, const losa_kv_t* k
   ap.n_ctas = c->lay.n_ctas;
   ap.sm_scale = sh.sm_scale;
   ap.wait_cycles = c->wait_cycles > 0 ? c->wait_cycles : kWaitCycles;
-  const bool with_combine = !(defer_combine && finish_fuses_combine(c));
-  return sh.head_dim == 128 ? dispatch_page<128>(c, ap, st, with_combine) : dispatch_page<64>(c, ap, st, with_combine);
+  return sh.head_dim == 128 ? dispatch_page<128>(c, ap, st, !defer_combine) : dispatch_page<64>(c, ap, st, !defer_combine);
 }
-
-bool finish_fuses_combine(const losa_ctx* c) { return c->shape.dtype == LOSA_BF16; }
 
 int32_t launch_attn_finish(losa_ctx* c, const void* q, const int32_t* slot_map, losa_state_t* state, void* out,
                            float* lse_out_opt, cudaStream_t st) {
@@ -513,8 +596,13 @@ int32_t launch_attn_finish(losa_ctx* c, const void* q, const int32_t* slot_map, 
   fp.step = state->step;
   fp.n_rows = static_cast<size_t>(sh.batch) * sh.block_size * sh.n_q_heads;
   const int blocks = static_cast<int>((fp.n_rows + kFinishThreads / 32 - 1) / (kFinishThreads / 32));
-  if (sh.head_dim == 128) launch_k(attn_finish_kernel<__nv_bfloat16, 128>, blocks, kFinishThreads, 0, st, ap, fp);
-  else launch_k(attn_finish_kernel<__nv_bfloat16, 64>, blocks, kFinishThreads, 0, st, ap, fp);
+  if (sh.dtype == LOSA_BF16) {
+    if (sh.head_dim == 128) launch_k(attn_finish_kernel<__nv_bfloat16, 128>, blocks, kFinishThreads, 0, st, ap, fp);
+    else launch_k(attn_finish_kernel<__nv_bfloat16, 64>, blocks, kFinishThreads, 0, st, ap, fp);
+  } else {
+    if (sh.head_dim == 128) launch_k(attn_finish_kernel<float, 128>, blocks, kFinishThreads, 0, st, ap, fp);
+    else launch_k(attn_finish_kernel<float, 64>, blocks, kFinishThreads, 0, st, ap, fp);
+  }
   return after_launch(c);
 }
 

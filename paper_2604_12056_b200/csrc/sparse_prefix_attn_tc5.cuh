@@ -249,7 +249,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   grid_dep_trigger();
   grid_dep_wait();                                 // nothing above touches global memory
   if (warp == 0) {
-    segment_prefix(pre, p.n_seg, p.n_rg, p.Hkv, p.G, p.n_active, p.union_count, p.B, lane, vpre);
+    segment_prefix(pre, p.n_seg, p.n_rg, p.Hkv, p.G, p.n_active, [&](int sk) { return p.union_count[sk]; }, p.B, lane, vpre);
   } else if (staged) {
     for (int i = tid - 32; i < p.N * p.B; i += NT - 32) tok_s[i] = p.active_idx[i];
     for (int i = tid - 32; i < p.N; i += NT - 32) {

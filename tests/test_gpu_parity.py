@@ -410,6 +410,16 @@ def test_fp32_attention_by_rows_per_kv_head(g, d, m, G):
     run_blocks(cfg)
 
 
+@pytest.mark.parametrize("kw", [
+    # 72 lists of 32 words: the most page bitmaps that the fp32 stage-4 kernel keeps; 33 words: stage 3 in a kernel of its own
+    dict(kv_lens=(16 * 1020,) + (40,) * 8, n_q_heads=16, n_kv_heads=8), dict(kv_lens=(16 * 1030,) + (40,) * 8, n_q_heads=16, n_kv_heads=8),
+    # a list that ends inside a word, one word, an empty and a one-token prefix; more than 16 rows per KV head
+    dict(kv_lens=(16 * 31, 16 * 33 + 1, 0, 1, 16 * 130), n_q_heads=8, n_kv_heads=2, m_active=5),
+])
+def test_fp32_whole_step_takes_the_union_from_page_bitmaps(kw):
+    run_blocks(wl.config("c1", **{**dict(head_dim=64, page_size=16, block_size=6, steps=3, topk=7, m_active=2, hidden_width=0), **kw}), fused=True)
+
+
 def test_fp32_attention_over_more_pages_than_a_cta_resolves_at_once():
     """48,000 pages: more than 256 for every CTA; compared with softmax in float64."""
     import torch
