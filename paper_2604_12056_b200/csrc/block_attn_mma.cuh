@@ -70,21 +70,8 @@ __device__ __forceinline__ void block_attn_mma_cta(const BlockAttnParams& p, Blo
   __nv_bfloat16* Vt = sm.vt;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int G = Hq / Hkv, nrow = B * G;
-  // ---- stage K_b (row-major) and V_b (transposed); keys >= B are zero
-  for (int idx = tid; idx < BK * (D / 8); idx += kMmaThreads) {
-    const int t = idx % BK, ch = idx / BK;             // key fastest: the transposed stores of a warp fall into one row
-    uint4 kv = make_uint4(0u, 0u, 0u, 0u), vv = kv;
-    if (t < B) {
-      const size_t src = ((static_cast<size_t>(s) * B + t) * Hkv + kh) * D + ch * 8;
-      kv = *reinterpret_cast<const uint4*>(p.k_blk + src);
-      vv = *reinterpret_cast<const uint4*>(p.v_blk + src);
-    }
-    *reinterpret_cast<uint4*>(Ks + t * KS + ch * 8) = kv;
-    const __nv_bfloat16* ve = reinterpret_cast<const __nv_bfloat16*>(&vv);
-#pragma unroll
-    for (int e = 0; e < 8; ++e) Vt[(ch * 8 + e) * VS + t] = ve[e];
-  }
-  // ---- this warp's 16 rows: rows g and g + 8 of the tile for this lane
+  // ---- this warp's 16 rows: rows g and g + 8 of the tile for this lane; the queries are
+  //      requested before the staging's stores, which the compiler cannot tell apart from these loads
   const int g = lane >> 2, t4 = lane & 3;
   const int lr0 = rt * kMmaRows + warp * 16 + g, lr1 = lr0 + 8;
   auto global_row = [&](int lr) {
@@ -101,6 +88,20 @@ __device__ __forceinline__ void block_attn_mma_cta(const BlockAttnParams& p, Blo
     qa[ks][1] = q1[ks * 8 + t4];
     qa[ks][2] = q0[ks * 8 + 4 + t4];
     qa[ks][3] = q1[ks * 8 + 4 + t4];
+  }
+  // ---- stage K_b (row-major) and V_b (transposed); keys >= B are zero
+  for (int idx = tid; idx < BK * (D / 8); idx += kMmaThreads) {
+    const int t = idx % BK, ch = idx / BK;             // key fastest: the transposed stores of a warp fall into one row
+    uint4 kv = make_uint4(0u, 0u, 0u, 0u), vv = kv;
+    if (t < B) {
+      const size_t src = ((static_cast<size_t>(s) * B + t) * Hkv + kh) * D + ch * 8;
+      kv = *reinterpret_cast<const uint4*>(p.k_blk + src);
+      vv = *reinterpret_cast<const uint4*>(p.v_blk + src);
+    }
+    *reinterpret_cast<uint4*>(Ks + t * KS + ch * 8) = kv;
+    const __nv_bfloat16* ve = reinterpret_cast<const __nv_bfloat16*>(&vv);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) Vt[(ch * 8 + e) * VS + t] = ve[e];
   }
   __syncthreads();
   if (rt * kMmaRows + warp * 16 >= nrow) return;       // no row of this warp exists

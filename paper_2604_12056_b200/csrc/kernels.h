@@ -49,7 +49,12 @@ int32_t launch_page_scores(losa_ctx* c, const void* q, const losa_kv_t* kv, cons
 // With approx_only the tensor-core value itself is written as an fp32 score row (relaxed selector).
 int32_t launch_page_bounds(losa_ctx* c, const void* q, const losa_kv_t* kv, const int32_t* active_idx,
                            const int32_t* n_active, const int32_t* step, cudaStream_t st, bool approx_only = false,
-                           bool after_stage1 = false);
+                           bool after_stage1 = false, bool pooled = false);
+// pooled: the largest bounds of a KV head's heads go into the first one's row (bounds_can_pool).
+inline bool bounds_can_pool(const losa_ctx* c) {
+  const int G = c->shape.n_q_heads / c->shape.n_kv_heads;
+  return G == 2 || G == 4 || G == 8;                 // an aligned run of rows of the MMA tile
+}
 // after_stage1: the previous kernel on `st` is stage 1 of the same step, which releases its dependents only
 // after everything before it has completed: the kernel then takes its work list and first copies (kv_len,
 // step, page table, summaries - nothing stage 1 writes) before stage 1 ends.

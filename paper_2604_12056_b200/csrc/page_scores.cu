@@ -73,6 +73,7 @@ struct PsParams {
   int32_t* status;
   int N, B, Hq, Hkv, G, g, Pmax, n_phys, score_stride, n_ctas, n_stages;
   int early;   // the kernel before this one in the stream is stage 1 of the same step: the list and the first copies may be taken before it ends
+  int pool;         // tensor-core bounds kernel: 1, or the heads of a KV head (2, 4 or 8) whose largest bounds are written, into the first one's row
   int tile_pages;   // tensor-core bounds kernel: pages per tile of this launch (16 .. 128, chosen on the host)
 };
 
@@ -784,10 +785,28 @@ __global__ void __launch_bounds__(kPsThreads, 1) page_bounds_mma_kernel(PsParams
           mma_bf16_16816(m1, a_lo.z, a_hi.z, a_lo.w, a_hi.w, b_1.z, b_1.w);
         }
         // c[0], c[1]: row g, pages 2 t4, 2 t4 + 1 of the 8-page tile; c[2], c[3]: row g + 8
+        if (!APPROX) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {               // bounds: A - delta in c, A + delta in m
+            const float d0 = kMmaErrCoef * m0[e], d1 = kMmaErrCoef * m1[e];
+            m0[e] = c0[e] + d0; c0[e] -= d0;
+            m1[e] = c1[e] + d1; c1[e] -= d1;
+          }
+          // pooled lists: the largest bounds of the heads, which are consecutive rows (an aligned run of 2, 4 or 8)
+          for (int off = 1; off < p.pool; off <<= 1) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              c0[e] = fmaxf(c0[e], __shfl_xor_sync(0xffffffffu, c0[e], 4 * off));
+              c1[e] = fmaxf(c1[e], __shfl_xor_sync(0xffffffffu, c1[e], 4 * off));
+              m0[e] = fmaxf(m0[e], __shfl_xor_sync(0xffffffffu, m0[e], 4 * off));
+              m1[e] = fmaxf(m1[e], __shfl_xor_sync(0xffffffffu, m1[e], 4 * off));
+            }
+          }
+        }
 #pragma unroll
         for (int hr = 0; hr < 2; ++hr) {
           const int r = 16 * mt + g + 8 * hr;
-          if (r < nr) {
+          if (r < nr && (g & (p.pool - 1)) == 0) {
             const int row = r0 + r, a = row / p.G, gi = row % p.G;
             const size_t at = ((static_cast<size_t>(w.s) * p.B + a) * p.Hq + w.kh * p.G + gi) * p.score_stride + w.p0 + warp * WP + 2 * t4;
 #pragma unroll
@@ -797,9 +816,8 @@ __global__ void __launch_bounds__(kPsThreads, 1) page_bounds_mma_kernel(PsParams
                 if (col < w.np) p.scores[at + e] = c0[2 * hr + e];
                 if (col + 8 < w.np) p.scores[at + e + 8] = c1[2 * hr + e];
               } else {
-                const float d0 = kMmaErrCoef * m0[2 * hr + e], d1 = kMmaErrCoef * m1[2 * hr + e];
-                if (col < w.np) bounds[at + e] = make_float2(c0[2 * hr + e] - d0, c0[2 * hr + e] + d0);
-                if (col + 8 < w.np) bounds[at + e + 8] = make_float2(c1[2 * hr + e] - d1, c1[2 * hr + e] + d1);
+                if (col < w.np) bounds[at + e] = make_float2(c0[2 * hr + e], m0[2 * hr + e]);
+                if (col + 8 < w.np) bounds[at + e + 8] = make_float2(c1[2 * hr + e], m1[2 * hr + e]);
               }
             }
           }
@@ -879,6 +897,7 @@ PsParams make_params(losa_ctx* c, const void* q, const losa_kv_t* kv, const int3
   p.n_stages = 0;
   p.early = 0;
   p.tile_pages = 0;
+  p.pool = 1;
   return p;
 }
 
@@ -886,8 +905,9 @@ PsParams make_params(losa_ctx* c, const void* q, const losa_kv_t* kv, const int3
 
 // bf16 only: (lower, upper) bound pairs of the page scores into the workspace's score rows (as float2)
 int32_t launch_page_bounds(losa_ctx* c, const void* q, const losa_kv_t* kv, const int32_t* active_idx,
-                           const int32_t* n_active, const int32_t* step, cudaStream_t st, bool approx_only, bool after_stage1) {
+                           const int32_t* n_active, const int32_t* step, cudaStream_t st, bool approx_only, bool after_stage1, bool pooled) {
   PsParams p = make_params(c, q, kv, active_idx, n_active, step);
+  p.pool = pooled ? p.G : 1;
   p.early = after_stage1 ? 1 : 0;
   // Pages per tile: a tile costs a fixed part plus a part per page (about 0.8 us + 2 us per 128 pages),
   // and the kernel lasts as many tiles as its busiest CTA gets; of the sizes 16, 32 .. 128 the one that

@@ -273,22 +273,26 @@ __device__ __forceinline__ void topk_select_body(const Row& row, int P, int kk, 
 // fp32 in shared memory): lane u runs the chains of runs u, u + 4(, u + 8, u + 12) - 16 fused
 // multiply-adds per run of 8 dimensions - and the butterfly c[i] += c[i ^ off], off = D/16 .. 1, is
 // taken inside the lane while off >= 4 and with two shuffles below that.  All four lanes return it.
+template <int D> struct SummaryRuns { uint4 lo[D / 32], hi[D / 32]; };      // a lane's runs of one page's kmin and kmax
 template <int D>
-__device__ __forceinline__ float exact_score4(const float* __restrict__ qs, const __nv_bfloat16* __restrict__ lo_p,
-                                              const __nv_bfloat16* __restrict__ hi_p, int u) {
-  constexpr int RPL = D / 32;      // runs per lane
-  uint4 lo_raw[RPL], hi_raw[RPL];  // requested together, converted run by run
+__device__ __forceinline__ SummaryRuns<D> load_summary(const __nv_bfloat16* __restrict__ lo_p, const __nv_bfloat16* __restrict__ hi_p, int u) {
+  SummaryRuns<D> r;                // requested together, converted run by run
 #pragma unroll
-  for (int w = 0; w < RPL; ++w) {
-    lo_raw[w] = __ldg(reinterpret_cast<const uint4*>(lo_p + 8 * (u + 4 * w)));
-    hi_raw[w] = __ldg(reinterpret_cast<const uint4*>(hi_p + 8 * (u + 4 * w)));
+  for (int w = 0; w < D / 32; ++w) {
+    r.lo[w] = __ldg(reinterpret_cast<const uint4*>(lo_p + 8 * (u + 4 * w)));
+    r.hi[w] = __ldg(reinterpret_cast<const uint4*>(hi_p + 8 * (u + 4 * w)));
   }
+  return r;
+}
+template <int D>
+__device__ __forceinline__ float exact_score4(const float* __restrict__ qs, const SummaryRuns<D>& r, int u) {
+  constexpr int RPL = D / 32;      // runs per lane
   float c[RPL];
 #pragma unroll
   for (int w = 0; w < RPL; ++w) {
     const int t = u + 4 * w;
-    const uint32_t lw[4] = {lo_raw[w].x, lo_raw[w].y, lo_raw[w].z, lo_raw[w].w};
-    const uint32_t hw[4] = {hi_raw[w].x, hi_raw[w].y, hi_raw[w].z, hi_raw[w].w};
+    const uint32_t lw[4] = {r.lo[w].x, r.lo[w].y, r.lo[w].z, r.lo[w].w};
+    const uint32_t hw[4] = {r.hi[w].x, r.hi[w].y, r.hi[w].z, r.hi[w].w};
     float acc = 0.f;
 #pragma unroll
     for (int j4 = 0; j4 < 2; ++j4) {
@@ -335,6 +339,7 @@ struct RefineParams {
   int32_t* union_pages;
   int32_t* union_count;
   int W;                          // words per bitmap, ceil(Pmax / 32) <= kSelBins
+  int bound_rows;                 // pooled: rows of bounds per list: the heads' own, or 1 where the bounds kernel has pooled them
   int slots;                      // CTAs per (sequence, head or KV head): active slots are dealt out round-robin
   int blk_tiles;                  // row tiles of the in-block attention per (sequence, KV head)
 };
@@ -398,7 +403,7 @@ template <int D, bool POOLED>
 struct RefineSmem {
   float qs[(POOLED ? kMaxPool : 1) * 2 * D];
   unsigned long long ckey[kSelCap];
-  int cpage[kSelCap];
+  int cpage[kSelCap], cphys[kSelCap];
   int hist[kSelBins];
   uint32_t red[2][kSelThreads / 32];
   int ncand, bstar;
@@ -480,7 +485,7 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
     // most kSelThreads * kSelPerThread pages
     const bool cached = P <= kSelThreads * kSelPerThread;
     if constexpr (POOLED) {
-      if (!cached) {
+      if (!cached && p.bound_rows > 1) {
         // the passes below read the row several times: pool once, into the group's first row (the
         // rows are scratch, this CTA is their only reader, and a thread reads back only what it wrote)
         constexpr int U = 4;                                   // pages per thread whose loads are in flight together
@@ -488,7 +493,7 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
           float2 v[U];
 #pragma unroll
           for (int e = 0; e < U; ++e) v[e] = p0 + e * kSelThreads < P ? row2[p0 + e * kSelThreads] : make_float2(0.f, 0.f);
-          for (int gi = 1; gi < pool; ++gi) {
+          for (int gi = 1; gi < p.bound_rows; ++gi) {
             float2 w[U];
 #pragma unroll
             for (int e = 0; e < U; ++e)
@@ -512,7 +517,7 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
         bv[i] = pg < P ? row2[pg] : make_float2(0.f, 0.f);
       }
       if constexpr (POOLED) {
-        for (int gi = 1; gi < pool; ++gi) {
+        for (int gi = 1; gi < p.bound_rows; ++gi) {
           float2 bg[kSelPerThread];
 #pragma unroll
           for (int i = 0; i < kSelPerThread; ++i) {
@@ -615,9 +620,12 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
     };
     auto exact_at = [&](int ph) {                 // called by the four lanes of a group with the same page
       const size_t so = static_cast<size_t>(ph) * p.Hkv * D;
-      float e = exact_score4<D>(qs, lo_base + so, hi_base + so, u);
-      if constexpr (POOLED)
-        for (int gi = 1; gi < pool; ++gi) e = fmaxf(e, exact_score4<D>(qs + gi * 2 * D, lo_base + so, hi_base + so, u));
+      const SummaryRuns<D> sr = load_summary<D>(lo_base + so, hi_base + so, u);
+      float e = exact_score4<D>(qs, sr, u);
+      if constexpr (POOLED) {                      // the summary serves all heads of the group
+#pragma unroll 1
+        for (int gi = 1; gi < pool; ++gi) e = fmaxf(e, exact_score4<D>(qs + gi * 2 * D, sr, u));
+      }
       return e;
     };
     if (ncand > kSelCap) {
@@ -633,24 +641,18 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
       __syncthreads();
       continue;
     }
-    // a group of four lanes per candidate, 32 candidates per round; the physical page ids of four
-    // rounds are requested together (one round trip instead of four)
-    constexpr int kPer = kSelThreads / 4, kAhead = 4;
-    for (int i0 = 0; i0 < ncand; i0 += kPer * kAhead) {
-      int pgs[kAhead], phs[kAhead];
-#pragma unroll
-      for (int r = 0; r < kAhead; ++r) {
-        pgs[r] = cpage[min(i0 + r * kPer + tid / 4, ncand - 1)];
-        phs[r] = phys_of(pgs[r]);
-      }
-#pragma unroll
-      for (int r = 0; r < kAhead; ++r) {
-        if (i0 + r * kPer < ncand) {                     // uniform over the CTA
-          const float e = exact_at(phs[r]);
-          const int i = i0 + r * kPer + tid / 4;
-          if (u == 0 && i < ncand) ckey[i] = make_key(order_bits(e), pgs[r]);
-        }
-      }
+    // a group of four lanes per candidate, 32 candidates per round, all physical page ids in one round trip
+    // (through shared memory: with four rounds' ids in registers the loop was unrolled, spilled, and a whole step
+    // took 1 us longer with one 8K sequence, 2 us with eight of 32K)
+    int* cphys = sm.r.cphys;
+    for (int i = tid; i < ncand; i += kSelThreads) cphys[i] = phys_of(cpage[i]);
+    __syncthreads();
+    constexpr int kPer = kSelThreads / 4;
+#pragma unroll 1
+    for (int i0 = 0; i0 < ncand; i0 += kPer) {           // uniform over the CTA
+      const int i = i0 + tid / 4, ic = min(i, ncand - 1);
+      const float e = exact_at(cphys[ic]);
+      if (u == 0 && i < ncand) ckey[i] = make_key(order_bits(e), cpage[i]);
     }
     // ---- order the candidates (descending) and emit the first kk
     __syncthreads();
@@ -892,7 +894,8 @@ int32_t launch_page_scores_topk(losa_ctx* c, const void* q, const losa_kv_t* kv,
   if (selects_by_refinement(c, k, selector)) {
     // bf16, exact lists (per query head, or per KV head from the group's maximum): bounds from the
     // tensor cores, exact scores for the candidates only
-    int32_t rc = launch_page_bounds(c, q, kv, active_idx, n_active, step, st, false, after_stage1);
+    const bool pool_bounds = pooled && bounds_can_pool(c);
+    int32_t rc = launch_page_bounds(c, q, kv, active_idx, n_active, step, st, false, after_stage1, pool_bounds);
     if (rc != LOSA_OK) return rc;
     RefineParams rp;
     rp.bounds = reinterpret_cast<float2*>(c->ws + c->lay.scores);
@@ -912,6 +915,7 @@ int32_t launch_page_scores_topk(losa_ctx* c, const void* q, const losa_kv_t* kv,
     rp.W = (sh.max_pages_per_seq + 31) / 32;
     const bool with_union = union_pages && union_count && union_done && rp.W <= kSelBins;
     rp.union_bits = with_union ? reinterpret_cast<uint32_t*>(c->ws + c->lay.union_bits) : nullptr;
+    rp.bound_rows = pool_bounds ? 1 : pool;
     rp.union_tickets = reinterpret_cast<unsigned int*>(c->ws + c->lay.union_tickets);
     rp.union_pages = union_pages;
     rp.union_count = union_count;

@@ -198,8 +198,8 @@ template <int C> __device__ __forceinline__ void st_state(void* base, int bf16, 
 // to kMergeBatch records are copied to `buf` (that many rows of D floats of this warp) while their
 // maxima are read; with up to 32 KB per CTA and few registers, more CTAs are resident than with
 // outputs in registers, and the rolled loops keep the code short.  A lane reads back only what it
-// copied itself.
-constexpr int kMergeBatch = 16;
+// copied itself.  20: what one sequence's eight KV heads have over 148 CTAs, in one round trip (16: two; 1.5 us per step).
+constexpr int kMergeBatch = 20;
 template <int D, bool LOG2>
 __device__ __forceinline__ void merge_records(const AttnParams& p, float* buf, int sg, int r, int2 records, int lane,
                                               float (&acc)[D / 32], float& M, float& Lsum) {

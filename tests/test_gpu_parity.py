@@ -175,6 +175,17 @@ def test_whole_step_call_beyond_the_bitmap_of_the_selection_kernel():
     run_blocks(cfg, modes=("losa",), fused=True, want_scores=False)
 
 
+@pytest.mark.parametrize("pooled", [False, True])
+@pytest.mark.parametrize("kw", [
+    # bounds in registers up to 1,024 pages, from L2 beyond; heads pooled by the bounds kernel (2, 4, 8) or by the selection (3, 16)
+    dict(n_q_heads=4, n_kv_heads=2, kv_lens=(16 * 1024, 16 * 1025)), dict(n_q_heads=12, n_kv_heads=3, kv_lens=(16 * 1100 + 1, 700)),
+    dict(n_q_heads=16, n_kv_heads=2, kv_lens=(16 * 129, 33)), dict(n_q_heads=6, n_kv_heads=2, kv_lens=(16 * 1100, 16 * 90)),
+    dict(n_q_heads=16, n_kv_heads=1, kv_lens=(16 * 1100, 16 * 90), m_active=3),
+])
+def test_whole_step_selection_by_prefix_length_and_group(kw, pooled):
+    run_blocks(wl.config("c2", **{**dict(head_dim=64, page_size=16, block_size=5, steps=3, topk=7, m_active=5), **kw}), fused=True, pooled=pooled)
+
+
 @pytest.mark.parametrize("kw", [
     dict(kv_lens=(2048, 1500), steps=4),
     dict(n_q_heads=4, n_kv_heads=2, head_dim=64, page_size=16, kv_lens=(16 * 1100 + 5, 700), block_size=8, steps=3, topk=8,
