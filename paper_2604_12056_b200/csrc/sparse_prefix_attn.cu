@@ -430,7 +430,7 @@ int32_t encode_pool_map(losa_ctx* c, unsigned char* blob, const void* pool, cons
   const CUresult r = reinterpret_cast<EncodeTiledFn>(c->encode_fn)(
       reinterpret_cast<CUtensorMap*>(blob), fp8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4,
       const_cast<void*>(pool), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-      fp8 ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B,
+      fp8 && is_v ? CU_TENSOR_MAP_SWIZZLE_NONE : (fp8 && sh.head_dim == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B),
       CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     c->last_cuda_error = static_cast<int32_t>(r);
@@ -466,6 +466,10 @@ int32_t launch_tc5(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool with
   constexpr int bit = FP8 ? 2 : 1;  // a context has one shape on one device: one instantiation per cache format
   if (!(c->attn_attr_set & bit)) {
     LOSA_CUDA_TRY(c, cudaFuncSetAttribute(attn_tc5_kernel<D, GP, FP8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    // the kernel moves registers between its warps: a build that is launched with fewer than it deals out would wait for ever
+    cudaFuncAttributes fa;
+    LOSA_CUDA_TRY(c, cudaFuncGetAttributes(&fa, attn_tc5_kernel<D, GP, FP8>));
+    if (fa.numRegs < (FP8 ? kTc5LaunchRegs8 : kTc5LaunchRegs)) return LOSA_ERR_UNSUPPORTED;
     c->attn_attr_set |= bit;
   }
   CUtensorMap mk, mv;

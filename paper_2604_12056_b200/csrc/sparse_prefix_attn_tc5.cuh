@@ -3,67 +3,76 @@
 //
 // A CTA owns up to 128 GQA-grouped query rows of one (sequence, KV head) at a time: the M = 128 rows
 // of every MMA, one row per tensor-memory lane.  Pages are taken in groups of 128 tokens (PG pages):
-//   S[128 x 128]  = Q . K^T      A = Q from tensor memory (bf16, written there once per piece),
+//   S[128 x 128]  = Q . K^T      A = Q from shared memory (written there once per piece),
 //                                B = the group's K tiles, K-major in shared memory (128-byte swizzle,
 //                                as TMA wrote them); D / 16 instructions
-//   softmax       eight warps, thread = (query row, half of the columns): the row's scores are read
-//                 from tensor memory once, the maximum is exchanged with the partner thread, then
-//                 P = 2^(s - m); the reference maximum m only moves when it would grow by more than
-//                 2^8 (then O is rescaled in place); P is rounded to bf16 and written over the
-//                 scores it came from
+//   softmax       three sets of four warps, thread = query row; the sets take every third group: the row's
+//                 maximum in one pass, P = 2^(s - m) in a second, rounded to bf16 and written over the scores;
+//                 the reference maximum m passes from group to group and only moves when it would grow by
+//                 more than 2^8 (then O is rescaled in place)
 //   O[128 x D]   += P . V        A = P from tensor memory, B = the group's V tiles as they lie in
 //                                memory (tokens x d: MN-major); 8 instructions
-// Issuing one tcgen05.mma costs the issuing thread ~120 cycles whatever its shape (measured), so the
-// shapes are as large as the layout allows and the two products have an issuing thread each.
-// K and V have a ring of group-sized slots each, filled by one producer warp each (lane = page:
-// 32 pages' copies are issued by one instruction); a K slot is free again as soon as its Q K^T has
-// run, a V slot after its P V.  S is double-buffered.  Completion is tracked with tcgen05.commit on
-// mbarriers; every wait is bounded; tensor memory is returned on every path.
+// An instruction of either product takes the pipe 64 cycles (128 x 128 x 16); each product has an issuing
+// thread of its own.  K and V have a ring of group-sized slots each, filled by one producer warp each
+// (lane = page: 32 pages' copies are issued by one instruction); a K slot is free again as soon as its
+// Q K^T has run, a V slot after its P V.  There is an S buffer per set (tensor memory: O 128 + 3 x 128
+// columns; Q therefore lies in shared memory).  Completion is tracked with tcgen05.commit on mbarriers; every wait is
+// bounded; tensor memory is returned on every path.
 #pragma once
 
-constexpr int kTc5SoftmaxWarps = 8;              // two sets of four: set h takes columns 64h .. 64h+63 of every group
-constexpr int kTc5QkWarp = 8, kTc5PvWarp = 9, kTc5KWarp = 10, kTc5VWarp = 11;
-constexpr int kTc5CvtWarp = 12;                  // FP8 pages: four converting warps, two for K and two for V
-template <bool FP8> constexpr int tc5_threads() { return FP8 ? 512 : 384; }
+constexpr int kTc5Sets = 3, kTc5SetWarps = 4;    // sets of softmax warps: set h takes every third group, thread = one query row
+constexpr int kTc5SoftmaxWarps = kTc5Sets * kTc5SetWarps;
+constexpr int kTc5QkWarp = 12, kTc5PvWarp = 13, kTc5KWarp = 14, kTc5VWarp = 15;
+constexpr int kTc5CvtWarp = 16, kTc5CvtWarps = 4; // FP8 pages: four warps that convert V
+template <bool FP8> constexpr int tc5_threads() { return FP8 ? 640 : 512; }
+// Registers per thread at the launch, and as they are dealt out to the softmax warps and the others:
+// 12 x 32 x 136 + 4 x 32 x 104 = 512 x 128; FP8 12 x 32 x 112 + 8 x 32 x 72 = 640 x 96.
+constexpr int kTc5LaunchRegs = 128, kTc5SoftmaxRegs = 136, kTc5OtherRegs = 104;
+constexpr int kTc5LaunchRegs8 = 96, kTc5SoftmaxRegs8 = 112, kTc5OtherRegs8 = 72;
+static_assert(kTc5SoftmaxWarps * kTc5SoftmaxRegs + 4 * kTc5OtherRegs <= 16 * kTc5LaunchRegs, "registers");
+static_assert(kTc5SoftmaxWarps * kTc5SoftmaxRegs8 + 8 * kTc5OtherRegs8 <= 20 * kTc5LaunchRegs8, "registers, FP8");
 constexpr int kTc5Tok = 128;                     // tokens per group = N of Q K^T = columns of one S buffer
 constexpr float kTc5Tau = 8.0f;                  // reference maximum moves only when it would grow by more than this (log2 units)
-constexpr int kTc5XchgBytes = (2 * 2 + 1) * kRowsPerGroup * 4;   // row maxima [group parity][set][row], row sums [row]
+constexpr int kTc5XchgBytes = 3 * kTc5Sets * kRowsPerGroup * 4;   // reference maxima, row sums and the references of these, each [set][row]
 // FP8 pages: binary places by which P is held above the reference maximum.  P stays below 2^(8 + 7) < 65504.
 constexpr float kTc5Fp8Lift = 7.0f;
-constexpr int kTc5StgMax = 20;                   // FP8 pages: staging slots per tensor, one page each, at most
+constexpr int kTc5StgMax = 20;                   // FP8 pages: staging slots of V, one page each, at most
 // FP8: value pages whose multiplier is kept.  Page x + 32 is issued once page x + 32 - 20 or a later one has
 // been converted, and with it the whole group of page x (at most 8 pages).
 constexpr int kTc5VmulRing = 32;
 // Groups whose per-page data (token counts; FP8: scales) is kept.  The K producer writes a page's entry
 // when it issues the page's copy, so the ring must be longer than its lead over the softmax warps.  A
 // group never spans two segments, so in a run of one-page segments every page in flight is a group of
-// its own.  The first page of group g is issued once its slot is free:
-//   bf16  Q K^T of group g - NR has run, hence P V of group g - NR - 2: group g - NR - 1 may still be
-//         read, a lead of NR + 1;
-//   FP8   page, and so at worst group, g - NSP has been converted (NSP staging slots), hence Q K^T of
-//         group g - NSP - NR has run: a lead of NSP + NR + 1.
-// Small pages have up to 20 staging slots, a lead of 23; the others at most 10.
-template <int D, int GP, bool FP8> constexpr int tc5_meta_ring() { return FP8 && GP * D <= 2048 ? 32 : 16; }
+// its own.  The first page of group g is issued once its K slot is free: Q K^T of group g - NRK has run,
+// hence P V of group g - NRK - 3 has released its S buffer: group g - NRK - 2 may still be read.
+constexpr int kTc5MetaRing = 16;
 // Barriers, the segment prefix and index cache, the exchange arrays, the charged prefix, the staging
-// barriers (landed, emptied; K and V) and the value pages' multipliers, two words per page of the meta ring
-template <int D, int GP, bool FP8> constexpr int tc5_tail_bytes() {
-  return kTailBytes + kTc5XchgBytes + (kMaxSegments + 2) * 4 + kTc5StgMax * 2 * (8 + 8) + kTc5VmulRing * 4 + tc5_meta_ring<D, GP, FP8>() * (kTc5Tok / GP) * 8;
+// barriers (landed, emptied) and the value pages' multipliers, two words per page of the meta ring
+template <int GP> constexpr int tc5_tail_bytes() {
+  return kTailBytes + kTc5XchgBytes + (kMaxSegments + 2) * 4 + kTc5StgMax * (8 + 8) + kTc5VmulRing * 4 + kTc5MetaRing * (kTc5Tok / GP) * 8;
 }
 
-template <int D> constexpr int tc5_slot_bytes() { return kTc5Tok * D * 2; }
-template <int D, int GP, bool FP8> constexpr int tc5_ring_slots() {     // per ring (K and V have one each)
-  if (FP8) return 2;                                            // the staging slots take the rest
-  const int n = (kSmemBudget - 1024 - tc5_tail_bytes<D, GP, FP8>()) / tc5_slot_bytes<D>() / 2;
-  return n > 6 ? 6 : n;
+// Shared memory: the Q tile (FP8: two tiles of codes), a ring of group-sized slots for K and one for V, FP8: a
+// ring of page-sized slots where the codes of V land.
+template <int D> constexpr int tc5_slot_bytes() { return kTc5Tok * D * 2; }                              // V, and bf16 K
+template <int D, bool FP8> constexpr int tc5_kslot_bytes() { return kTc5Tok * D * (FP8 ? 1 : 2); }
+template <int D> constexpr int tc5_q_bytes() { return kRowsPerGroup * D * 2; }
+template <int D, int GP, bool FP8> constexpr int tc5_ring_slots(bool v) {
+  if (FP8) return v ? 2 : (D == 128 ? 4 : 6);                   // the staging slots take the rest
+  const int n = (kSmemBudget - 1024 - tc5_tail_bytes<GP>() - tc5_q_bytes<D>()) / tc5_slot_bytes<D>();
+  const int own = v ? n / 2 : (n + 1) / 2;                      // K is ahead of V by the S buffers
+  return own > 6 ? 6 : own;
 }
-// FP8: pages per staging ring (one for K, one for V): what the ring slots leave, up to five groups
+// FP8: pages of the staging ring of V: what the ring slots leave, up to five groups
 template <int D, int GP> constexpr int tc5_stg_slots() {
-  const int fit = (kSmemBudget - 1024 - tc5_tail_bytes<D, GP, true>() - 4 * tc5_slot_bytes<D>()) / 2 / (GP * D), five = 5 * (kTc5Tok / GP);
+  const int fit = (kSmemBudget - 1024 - tc5_tail_bytes<GP>() - tc5_q_bytes<D>() - tc5_ring_slots<D, GP, true>(false) * tc5_kslot_bytes<D, true>() -
+                   tc5_ring_slots<D, GP, true>(true) * tc5_slot_bytes<D>()) / (GP * D), five = 5 * (kTc5Tok / GP);
   const int n = fit < five ? fit : five;
   return n < kTc5StgMax ? n : kTc5StgMax;
 }
 template <int D, int GP, bool FP8> constexpr int tc5_smem_bytes() {
-  return 1024 + 2 * tc5_ring_slots<D, GP, FP8>() * tc5_slot_bytes<D>() + (FP8 ? 2 * tc5_stg_slots<D, GP>() * GP * D : 0) + tc5_tail_bytes<D, GP, FP8>();
+  return 1024 + tc5_q_bytes<D>() + tc5_ring_slots<D, GP, FP8>(false) * tc5_kslot_bytes<D, FP8>() + tc5_ring_slots<D, GP, FP8>(true) * tc5_slot_bytes<D>() +
+         (FP8 ? tc5_stg_slots<D, GP>() * GP * D : 0) + tc5_tail_bytes<GP>();
 }
 
 // Shared-memory matrix descriptor: 128-byte swizzle, 8-row groups 1024 bytes apart; lbo = distance
@@ -72,8 +81,18 @@ __device__ __forceinline__ uint64_t tc5_desc(uint32_t saddr, uint32_t lbo) {
   return static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4) | (static_cast<uint64_t>((lbo >> 4) & 0x3FFFu) << 16) |
          (static_cast<uint64_t>(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
 }
-// Instruction descriptor, kind::f16: fp32 accumulate, A and B both bf16 (fmt 1) or both fp16 (fmt 0),
-// M x N tile, B optionally MN-major.
+// K-major tile of E4M3 codes, rows of D bytes: the 128-byte swizzle for D = 128, the 64-byte one (8-row groups 512
+// bytes apart) for D = 64.
+template <int D> __device__ __forceinline__ uint64_t tc5_desc8(uint32_t saddr) {
+  return static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4) | (1ull << 16) | (static_cast<uint64_t>((8 * D) >> 4) << 32) | (1ull << 46) |
+         (static_cast<uint64_t>(D == 128 ? 2 : 4) << 61);
+}
+// byte offset of 16-byte chunk c of row t of such a tile
+template <int D> __device__ __forceinline__ uint32_t tc5_sw8(int t, int c) {
+  return static_cast<uint32_t>(t * D + ((D == 128 ? c ^ (t & 7) : c ^ ((t >> 1) & 3)) << 4));
+}
+// Instruction descriptor: fp32 accumulate, M x N tile, B optionally MN-major; kind::f16: A and B both bf16
+// (fmt 1) or both fp16 (fmt 0); kind::f8f6f4: both E4M3 (fmt 0).
 __device__ __forceinline__ uint32_t tc5_idesc(int M, int N, int b_mn_major, uint32_t fmt = 1u) {
   return (1u << 4) | (fmt << 7) | (fmt << 10) | (static_cast<uint32_t>(b_mn_major) << 16) |
          (static_cast<uint32_t>(N >> 3) << 17) | (static_cast<uint32_t>(M >> 4) << 24);
@@ -84,6 +103,19 @@ __device__ __forceinline__ void tc5_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uin
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
       ::"r"(d_tmem), "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+}
+// D[tmem] (+)= A[smem descriptor] . B[smem descriptor], bf16 operands, or E4M3
+__device__ __forceinline__ void tc5_mma_ss(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void tc5_mma_ss8(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
 }
 __device__ __forceinline__ void tc5_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -113,6 +145,14 @@ __device__ __forceinline__ void tc5_ld32_nowait(uint32_t taddr, uint32_t* r) {
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr) : "memory");
 }
+__device__ __forceinline__ void tc5_ld16(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+        "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr) : "memory");
+}
 __device__ __forceinline__ void tc5_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tc5_pin32(uint32_t* r) {
 #pragma unroll
@@ -138,104 +178,104 @@ __device__ __forceinline__ void tc5_wait_st() { asm volatile("tcgen05.wait::st.s
 // byte offset of 16-byte chunk c (0..7) of row t in a [rows][128 B] tile with the 128-byte swizzle
 __device__ __forceinline__ uint32_t tc5_sw(int t, int c) { return static_cast<uint32_t>(t * 128 + ((c ^ (t & 7)) << 4)); }
 
-// FP8: the K / V pools hold E4M3 bytes with one power-of-two scale per (page, KV head).  The page
-// copies land in staging rings as they lie in memory (half the bytes); four converting warps, one
-// per scheduler, turn a landed page's codes into fp16 (exact) in the group's ring slot, in the layout
-// the tensor maps of the bf16 path produce, and every MMA runs on fp16 operands (Q and P are
-// converted to fp16 instead of bf16).  The scales stay out of the conversion, which is bound by its
-// instruction count: the key scale joins the softmax scale of the page's columns, and the value
-// scale 2^e is added to their exponent, so that P' = p 2^e multiplies the codes of V and the row sum
-// takes its columns back by 2^-e.  P' is rounded to fp16 relative to the largest p 2^e, so a page whose
-// scale lies below another's would lose that many places of fp16's range.  Two things keep every
-// weight at least as precise as an unscaled one: only the scales' part from 2^-6 to 2^0 goes into the
-// exponent (pages of values up to 448; once a share has met a larger one, the converters go over each
-// group of V a second time and multiply by the rest, exactly), and the reference lies 2^7 below the maximum.  A weight is then subnormal only 2^-15 or more
-// below its row's largest, 2^-14 without scales.  A group is 2 x 16 KiB of codes:
-// one warp needs about 3.8 us for 16 KiB, and while the two producing warps did this work it set the
-// pace (eight 32K prompts: dense step 372 us, sparse step at three active tokens 120 us).  Now 224 and
-// 81 us (scaling in the converters: 245 and 87; bit moves instead of the conversion instruction: 306
-// and 105; no conversion at all: 207 and 77).  Staging slots are single pages, so that one is refilled
-// while its neighbours are converted.  The
-// CTA's 512 threads start with 128 registers each; the softmax warps take 168 and the other eight
-// give theirs up to 88 (2 x 128 x 168 + 2 x 128 x 88 = 512 x 128).
+// FP8: the K / V pools hold E4M3 bytes with one power-of-two scale per (page, KV head).  K is an operand as
+// it lies: Q goes to shared memory as two E4M3 tiles whose sum is the bf16 query (four significant bits each),
+// and both are multiplied with the codes by kind::f8f6f4, at twice the 16-bit rate and with fp32 sums of the
+// same accuracy (against float64 on random codes: 1.0e-7, bf16 1.6e-7).  V cannot: P needs more than two terms.
+// Its codes land in a staging ring as they lie in memory; four converting warps, one per scheduler, turn a
+// landed page into fp16 (exact) in the group's ring slot, in the layout the tensor maps of the bf16 path
+// produce, and P is fp16.  The scales stay out of the conversion, which is bound by its instruction count: the
+// key scale joins the softmax scale of the page's columns, and the value scale 2^e is added to their
+// exponent, so that P' = p 2^e multiplies the codes of V and the row sum takes its columns back by 2^-e.  P'
+// is rounded to fp16 relative to the largest p 2^e, so a page whose scale lies below another's would lose that
+// many places of fp16's range.  Two things keep every weight at least as precise as an unscaled one: only the
+// scales' part from 2^-6 to 2^0 goes into the exponent (pages of values up to 448; once a share has met a
+// larger one, the converters go over each group of V a second time and multiply by the rest, exactly), and
+// the reference lies 2^7 below the maximum.  A weight is then subnormal only 2^-15 or more below its row's
+// largest, 2^-14 without scales.  Staging slots are single pages, so that one is refilled while its
+// neighbours are converted.
 template <int D, int GP, bool FP8>
 __global__ void __launch_bounds__(tc5_threads<FP8>(), 1)
 attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, AttnParams p) {
-  constexpr int NR = tc5_ring_slots<D, GP, FP8>();  // slots per ring
-  constexpr int NSP = FP8 ? tc5_stg_slots<D, GP>() : 1, STG = GP * D;   // FP8: staging slots per tensor, bytes of a slot (one page of codes)
+  constexpr int NRK = tc5_ring_slots<D, GP, FP8>(false), NRV = tc5_ring_slots<D, GP, FP8>(true);   // slots per ring
+  constexpr int NSP = FP8 ? tc5_stg_slots<D, GP>() : 1, STG = GP * D;   // FP8: staging slots of V, bytes of a slot (one page of codes)
   constexpr int NT = tc5_threads<FP8>();
-  constexpr uint32_t FMT = FP8 ? 0u : 1u;       // operand format of the MMAs: fp16 / bf16
-  constexpr int SLOT = tc5_slot_bytes<D>();
+  constexpr int KSLOT = tc5_kslot_bytes<D, FP8>(), SLOT = tc5_slot_bytes<D>(), QB = tc5_q_bytes<D>();
   constexpr int PG = kTc5Tok / GP;              // pages per group
-  constexpr int MR = tc5_meta_ring<D, GP, FP8>();   // groups of the meta ring
-  constexpr int HALVES = D / 64;                // 64-column (128-byte) blocks of a K or V row
+  constexpr int MR = kTc5MetaRing;              // groups of the meta ring
+  constexpr int HALVES = D / 64;                // 64-column (128-byte) blocks of a 16-bit K or V row
   constexpr int HS = kTc5Tok * 128;             // bytes of one such block of a whole group
-  constexpr int PAGE_BYTES = GP * D * 2;        // of K, and of V
-  constexpr uint32_t COL_O = 0, COL_S = 128, COL_Q = 384;   // tensor-memory columns: O[D], S0[128], S1[128], Q[D/2]
+  constexpr int PAGE_BYTES = GP * D * 2;        // of a 16-bit page of K, and of V
+  constexpr int SB = kTc5Sets;                  // S buffers, one per set
+  constexpr uint32_t COL_O = 0, COL_S = 128;    // tensor-memory columns: O[D], S0[128], S1[128], S2[128]
   constexpr int TMEM_COLS = 512;
   static_assert(D == 64 || D == 128, "head dimensions of the tensor-core path");
   static_assert(GP == 16 || GP == 32 || GP == 64, "page sizes of the tensor-core path");
-  static_assert(NR >= 2, "ring too shallow");
+  static_assert(NRK >= 2 && NRV >= 2 && NRK <= 6 && NRV <= 6, "ring depth");
   static_assert(!FP8 || (NSP >= PG && NSP <= kTc5StgMax), "staging ring");
-  static_assert((FP8 ? NSP : 0) + NR + 1 < MR, "the producer's lead fits the meta ring");
-  static_assert(8 * (4 * 6 + 14) + 16 <= 512, "tail layout");
+  static_assert(NRK + 2 < MR, "the producer's lead fits the meta ring");
+  constexpr int kBars = 4 * 6 + 3 * SB + 3 + 4 + 4 * SB + 2;
+  static_assert(8 * kBars + 16 <= 512, "tail layout");
 
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* gen = smem_raw + (base - raw);
-  const uint32_t kring = base, vring = base + NR * SLOT;
-  constexpr int STG_ALL = FP8 ? 2 * NSP * STG : 0;
-  const uint32_t kstg = base + 2 * NR * SLOT, vstg = kstg + NSP * STG;          // FP8 only
-  uint8_t* tail = gen + 2 * NR * SLOT + STG_ALL;
-  const uint32_t tail_s = base + 2 * NR * SLOT + STG_ALL;
-  const uint32_t kfull = tail_s, kfree = kfull + 8 * NR, vfull = kfree + 8 * NR, vfree = vfull + 8 * NR;
-  const uint32_t s_full = vfree + 8 * NR, s_free = s_full + 16, p_full = s_free + 16, q_full = p_full + 16, q_free = q_full + 8, xbar = q_free + 8;
-  const uint32_t drain_bar = xbar + 32;            // two barriers: the issuing threads' last commit when the CTA gives up
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 8 * (4 * 6 + 14));
+  const uint32_t qtile = base, kring = base + QB, vring = kring + NRK * KSLOT, vstg = vring + NRV * SLOT;   // vstg: FP8 only
+  constexpr int TAIL = QB + NRK * KSLOT + NRV * SLOT + (FP8 ? NSP * STG : 0);
+  uint8_t* tail = gen + TAIL;
+  const uint32_t tail_s = base + TAIL;
+  const uint32_t kfull = tail_s, kfree = kfull + 8 * NRK, vfull = kfree + 8 * NRK, vfree = vfull + 8 * NRV;
+  const uint32_t s_full = vfree + 8 * NRV, s_free = s_full + 8 * SB, p_full = s_free + 8 * SB, q_full = p_full + 8 * SB, q_free = q_full + 8, o_free = q_free + 8;
+  const uint32_t xbar = o_free + 8, mbar = xbar + 32;     // per lane quarter: the sets meet; [set][quarter]: a group's reference is published
+  const uint32_t drain_bar = mbar + 32 * SB;            // two barriers: the issuing threads' last commit when the CTA gives up
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 8 * kBars);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(const_cast<int*>(abort_flag) + 1);
   int* pre = reinterpret_cast<int*>(tail + 512);
   int* tok_s = pre + kMaxSegments + 2;
   int* na_s = tok_s + kStageIdx;
   int* len_s = na_s + kStageSeq;
-  float* xmax = reinterpret_cast<float*>(len_s + kStageSeq);   // [2][2][128]
-  float* xsum = xmax + 4 * kRowsPerGroup;                        // [128]
-  int* vpre = reinterpret_cast<int*>(xsum + kRowsPerGroup);      // prefix of the charged segment lengths (pages + pad)
-  // FP8: per tensor, a staging slot's page has landed / has been converted
-  const uint32_t stg_bars = smem_u32(vpre + kMaxSegments + 1) + 4;   // (kMaxSegments + 1 is odd)
-  const uint32_t kstg_full = stg_bars, vstg_full = kstg_full + 8 * kTc5StgMax, kstg_free = vstg_full + 8 * kTc5StgMax, vstg_free = kstg_free + 8 * kTc5StgMax;
+  float* mref = reinterpret_cast<float*>(len_s + kStageSeq);   // [set][128]
+  float* xsum = mref + SB * kRowsPerGroup;                       // [set][128]: row sums of a piece ...
+  float* xref = xsum + SB * kRowsPerGroup;                       // ... and the references they are relative to
+  int* vpre = reinterpret_cast<int*>(xref + SB * kRowsPerGroup);  // prefix of the charged segment lengths (pages + pad)
+  // FP8: a staging slot's page has landed / has been converted
+  const uint32_t vstg_full = smem_u32(vpre + kMaxSegments + 1) + 4;   // (kMaxSegments + 1 is odd)
+  const uint32_t vstg_free = vstg_full + 8 * kTc5StgMax;
   // FP8: multipliers of the newest value pages' codes, as two fp16; whether any was other than one
-  volatile uint32_t* vmul = reinterpret_cast<volatile uint32_t*>(vpre + kMaxSegments + 2 + 8 * kTc5StgMax);
+  volatile uint32_t* vmul = reinterpret_cast<volatile uint32_t*>(vpre + kMaxSegments + 2 + 4 * kTc5StgMax);
   volatile int* vmul_used = abort_flag + 2;
   // per page of the groups in flight, [MR][PG]: valid tokens (FP8: and the exponent field of the value scale's part in P << 8), FP8: key scale
-  volatile int* meta = vpre + kMaxSegments + 2 + 8 * kTc5StgMax + kTc5VmulRing;
+  volatile int* meta = vpre + kMaxSegments + 2 + 4 * kTc5StgMax + kTc5VmulRing;
   volatile float* kscale_meta = reinterpret_cast<volatile float*>(const_cast<int*>(meta) + MR * PG);
   const bool staged = p.N * p.B <= kStageIdx && p.N <= kStageSeq;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) {
-    for (int i = 0; i < NR; ++i) {
-      mbar_init(kfull + 8 * i, FP8 ? 2 : 1);         // the copies' bytes / the two converting warps
+    for (int i = 0; i < NRK; ++i) {
+      mbar_init(kfull + 8 * i, 1);
       mbar_init(kfree + 8 * i, 1);
-      mbar_init(vfull + 8 * i, FP8 ? 2 : 1);
+    }
+    for (int i = 0; i < NRV; ++i) {
+      mbar_init(vfull + 8 * i, FP8 ? kTc5CvtWarps : 1);   // the converting warps / the copies' bytes
       mbar_init(vfree + 8 * i, 1);
     }
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < SB; ++b) {
       mbar_init(s_full + 8 * b, 1);                  // tcgen05.commit after Q K^T
       mbar_init(s_free + 8 * b, 1);                  // tcgen05.commit after P V: the S buffer is free and O holds the group
-      mbar_init(p_full + 8 * b, kTc5SoftmaxWarps);
+      mbar_init(p_full + 8 * b, kTc5SetWarps);
     }
     mbar_init(q_full, kTc5SoftmaxWarps);
     mbar_init(q_free, 1);
-    for (int i = 0; i < 4; ++i) mbar_init(xbar + 8 * i, 2);      // the two softmax warps of a scheduler meet here
+    mbar_init(o_free, kTc5SoftmaxWarps);
+    for (int i = 0; i < 4; ++i) mbar_init(xbar + 8 * i, kTc5Sets);
+    for (int i = 0; i < 4 * SB; ++i) mbar_init(mbar + 8 * i, 1);
     mbar_init(drain_bar, 1);
     mbar_init(drain_bar + 8, 1);
     if (FP8)
       for (int i = 0; i < NSP; ++i) {
-        mbar_init(kstg_full + 8 * i, 1);
         mbar_init(vstg_full + 8 * i, 1);
-        mbar_init(kstg_free + 8 * i, 2);
-        mbar_init(vstg_free + 8 * i, 2);
+        mbar_init(vstg_free + 8 * i, kTc5CvtWarps);
       }
     *abort_flag = 0;
     *vmul_used = 0;
@@ -298,7 +338,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
 
   int issued = -1;                                   // producer warps: newest group (FP8: page) whose copies have been issued
   if (warp >= kTc5SoftmaxWarps) {
-  if constexpr (FP8) asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");    // whole warpgroups
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(FP8 ? kTc5OtherRegs8 : kTc5OtherRegs));   // whole warpgroups
   if (warp == kTc5KWarp || warp == kTc5VWarp) {
     // ------------------------------------------------------------------ producer warps: one for K, one for V
     // Lane j of a batch of 32 consecutive items resolves item -> logical page -> physical page (a
@@ -310,7 +350,8 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     const unsigned long long policy = l2_evict_first_policy();
     const CUtensorMap* map = is_v ? &tmV : &tmK;
     const uint32_t ring = is_v ? vring : kring, full0 = is_v ? vfull : kfull, free0 = is_v ? vfree : kfree;
-    const uint32_t stg = is_v ? vstg : kstg, landed = is_v ? vstg_full : kstg_full, emptied = is_v ? vstg_free : kstg_free;
+    auto slot_of = [&](int grp) { return is_v ? grp % NRV : grp % NRK; };
+    auto round_of = [&](int grp) { return is_v ? grp / NRV : grp / NRK; };
     int cursor = sg0, gbase = 0, pstart = lo;       // segment of the lane's newest item, groups before its piece, the piece's first item
     struct Item { int page, sk, grp, j, ng; };
     struct Ready { int phys, kh, valid, grp, j, ng; float ks, vs; };
@@ -356,31 +397,25 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         }
       }
     };
+    auto scale_in_p = [](float vs) { return min(max((__float_as_int(vs) >> 23) & 0xff, 127 - 6), 127); };
     // copies of the batch of items b0 .. b0 + 31 (one per lane); false when a wait has run out
     auto issue = [&](int b0, const Ready& b) {
       const int nb = min(32, hi - b0);
-      if constexpr (FP8) {                            // page by page: every lane handles its own staging slot
+      if (FP8 && is_v) {                              // page by page: every lane handles its own staging slot
         // the value scale: 2^-6 .. 2^0 of it go into P (as an exponent field), the rest onto the codes (also
         // what a caller's own scale has beside its power of two)
-        const int e = (__float_as_int(b.vs) >> 23) & 0xff, in_p = min(max(e, 127 - 6), 127);
-        const __half2 in_v = __float2half2_rn(b.vs * __int_as_float((254 - in_p) << 23));
+        const __half2 in_v = __float2half2_rn(b.vs * __int_as_float((254 - scale_in_p(b.vs)) << 23));
         for (int pos = 0; pos < nb; ++pos) {
           int ok = 1;
           if (lane == pos) {
             const int x = b0 + pos - lo, slot = x % NSP, round = x / NSP;
-            if (round > 0) ok = mbar_wait(emptied + 8 * slot, (round - 1) & 1, abort_flag, p.status, p.wait_cycles);
+            if (round > 0) ok = mbar_wait(vstg_free + 8 * slot, (round - 1) & 1, abort_flag, p.status, p.wait_cycles);
             if (ok) {
-              if (is_v) {
-                const uint32_t m2 = *reinterpret_cast<const uint32_t*>(&in_v);
-                vmul[x % kTc5VmulRing] = m2;
-                if (m2 != 0x3c003c00u) *vmul_used = 1;
-              } else {
-                const int at = (b.grp % MR) * PG + b.j;
-                meta[at] = b.valid | in_p << 8;
-                kscale_meta[at] = b.ks;
-              }
-              mbar_expect_tx(landed + 8 * slot, STG);
-              tma_load_4d(stg + slot * STG, map, landed + 8 * slot, 0, 0, b.kh, b.phys, policy);
+              const uint32_t m2 = *reinterpret_cast<const uint32_t*>(&in_v);
+              vmul[x % kTc5VmulRing] = m2;
+              if (m2 != 0x3c003c00u) *vmul_used = 1;
+              mbar_expect_tx(vstg_full + 8 * slot, STG);
+              tma_load_4d(vstg + slot * STG, map, vstg_full + 8 * slot, 0, 0, b.kh, b.phys, policy);
             }
           }
           if (__shfl_sync(0xffffffffu, ok, pos) == 0) return false;
@@ -393,21 +428,29 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         const int grp = __shfl_sync(0xffffffffu, b.grp, pos), j0 = __shfl_sync(0xffffffffu, b.j, pos);
         const int ng = __shfl_sync(0xffffffffu, b.ng, pos);
         const int cnt = min(ng - j0, nb - pos);
-        const int slot = grp % NR, round = grp / NR;
+        const int slot = slot_of(grp), round = round_of(grp);
         if (j0 == 0) {
           int ok = 1;
           if (lane == 0 && round > 0) ok = mbar_wait(free0 + 8 * slot, (round - 1) & 1, abort_flag, p.status, p.wait_cycles);
           if (__shfl_sync(0xffffffffu, ok, 0) == 0) return false;
         }
         const bool mine = lane >= pos && lane < pos + cnt;
-        if (!is_v && mine) meta[(grp % MR) * PG + b.j] = b.valid;
+        if (!is_v && mine) {
+          const int at = (grp % MR) * PG + b.j;
+          meta[at] = FP8 ? b.valid | scale_in_p(b.vs) << 8 : b.valid;
+          if (FP8) kscale_meta[at] = b.ks;
+        }
         __syncwarp();
-        if (j0 == 0 && lane == 0) mbar_expect_tx(full0 + 8 * slot, ng * PAGE_BYTES);
+        if (j0 == 0 && lane == 0) mbar_expect_tx(full0 + 8 * slot, ng * (FP8 ? STG : PAGE_BYTES));
         __syncwarp();
         if (mine) {
-          const uint32_t dst = ring + slot * SLOT + b.j * (GP * 128);
+          if constexpr (FP8) {                        // K: a page of codes, swizzled by the copy, is an operand as it is
+            tma_load_4d(ring + slot * KSLOT + b.j * STG, map, full0 + 8 * slot, 0, 0, b.kh, b.phys, policy);
+          } else {
+            const uint32_t dst = ring + slot * SLOT + b.j * (GP * 128);
 #pragma unroll
-          for (int hf = 0; hf < HALVES; ++hf) tma_load_4d(dst + hf * HS, map, full0 + 8 * slot, hf * 64, 0, b.kh, b.phys, policy);
+            for (int hf = 0; hf < HALVES; ++hf) tma_load_4d(dst + hf * HS, map, full0 + 8 * slot, hf * 64, 0, b.kh, b.phys, policy);
+          }
         }
         issued = grp;
         pos += cnt;
@@ -443,19 +486,16 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       }
     }
   } else if (FP8 && warp >= kTc5CvtWarp) {
-    // ------------------------------------------------------------------ converting warps (FP8 pages)
-    // Two warps per tensor, each half of every page's tokens.  A lane takes eight codes at a time (one
-    // 16-byte chunk of fp16): 8-byte reads of consecutive codes and 16-byte stores of consecutive
-    // swizzled chunks, both without bank conflicts; up to eight are requested before any is converted.
-    const bool is_v = warp >= kTc5CvtWarp + 2;
-    const int half = warp & 1;
-    const uint8_t* stg_gen = gen + ((is_v ? vstg : kstg) - base);
-    uint8_t* ring_gen = gen + ((is_v ? vring : kring) - base);
-    const uint32_t landed = is_v ? vstg_full : kstg_full, emptied = is_v ? vstg_free : kstg_free;
-    const uint32_t full0 = is_v ? vfull : kfull, free0 = is_v ? vfree : kfree;
+    // ------------------------------------------------------------------ converting warps (FP8 pages): V
+    // Each a quarter of every page's tokens.  A lane takes eight codes at a time (one 16-byte chunk of
+    // fp16): 8-byte reads of consecutive codes and 16-byte stores of consecutive swizzled chunks, both
+    // without bank conflicts; all of a page's are requested before any is converted.
+    const uint8_t* stg_gen = gen + (vstg - base);
+    uint8_t* ring_gen = gen + (vring - base);
     constexpr int CPR = D / 8, TPI = 32 / CPR;        // chunks of a row, tokens per warp access
-    constexpr int NU = GP / 2 / TPI, U = NU < 8 ? NU : 8;   // accesses per page and warp, in flight
-    const int tl = half * (GP / 2) + lane / CPR, c = lane % CPR;
+    constexpr int NU = GP / kTc5CvtWarps / TPI, U = NU;   // accesses per page and warp
+    static_assert(NU >= 1 && NU * TPI * kTc5CvtWarps == GP, "a page's tokens over the converting warps");
+    const int tl = (warp - kTc5CvtWarp) * (GP / kTc5CvtWarps) + lane / CPR, c = lane % CPR;
     auto wait = [&](uint32_t bar, uint32_t parity) {
       int ok = 1;
       if (lane == 0) ok = mbar_wait(bar, parity, abort_flag, p.status, p.wait_cycles);
@@ -467,11 +507,11 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     while (item < hi && ok) {
       const int seg_end = min(hi, pre[sg + 1]);
       for (int first = item; first < seg_end && ok; first += PG, ++g) {
-        const int ng = min(PG, seg_end - first), sr = g % NR;
-        if (g >= NR) ok = wait(free0 + 8 * sr, (g / NR - 1) & 1);
+        const int ng = min(PG, seg_end - first), sr = g % NRV;
+        if (g >= NRV) ok = wait(vfree + 8 * sr, (g / NRV - 1) & 1);
         for (int pg = 0; pg < ng; ++pg) {
           const int x = first + pg - lo, ss = x % NSP;
-          ok = ok && wait(landed + 8 * ss, (x / NSP) & 1);
+          ok = ok && wait(vstg_full + 8 * ss, (x / NSP) & 1);
           if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
           const uint8_t* src = stg_gen + ss * STG + tl * D + c * 8;
           uint8_t* dst = ring_gen + sr * SLOT + (c >> 3) * HS;
@@ -493,10 +533,10 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             }
           }
           __syncwarp();
-          if (lane == 0) mbar_arrive(emptied + 8 * ss, 1);
+          if (lane == 0) mbar_arrive(vstg_free + 8 * ss, 1);
         }
         if (!ok) break;
-        if (is_v && *vmul_used) {                     // this lane's chunks once more, times what of the scales is not in P
+        if (*vmul_used) {                     // this lane's chunks once more, times what of the scales is not in P
 #pragma unroll 1
           for (int i = 0; i < ng * NU; ++i) {
             const int pg = i / NU, u = i % NU;
@@ -514,7 +554,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs read the slot through the async proxy
         __syncwarp();
-        if (lane == 0) mbar_arrive(full0 + 8 * sr, 1);
+        if (lane == 0) mbar_arrive(vfull + 8 * sr, 1);
       }
       item = seg_end;
       ++sg;
@@ -529,16 +569,27 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         const int seg_end = min(hi, pre[sg + 1]);
         ok = mbar_wait(q_full, piece & 1, abort_flag, p.status, p.wait_cycles);
         for (int first = item; first < seg_end && ok; first += PG, ++g) {
-          const int ng = min(PG, seg_end - first), b = g & 1, use = g >> 1, slot = g % NR;
-          ok = mbar_wait(kfull + 8 * slot, (g / NR) & 1, abort_flag, p.status, p.wait_cycles);
+          const int ng = min(PG, seg_end - first), b = g % SB, use = g / SB, slot = g % NRK;
+          ok = mbar_wait(kfull + 8 * slot, (g / NRK) & 1, abort_flag, p.status, p.wait_cycles);
           ok = ok && (use == 0 || mbar_wait(s_free + 8 * b, (use - 1) & 1, abort_flag, p.status, p.wait_cycles));
           if (!ok) break;
           tc5_fence_after();
-          const uint32_t idesc = tc5_idesc(kRowsPerGroup, ng * GP, 0, FMT), kt = kring + slot * SLOT;
+          const uint32_t kt = kring + slot * KSLOT, s_col = tmem + COL_S + b * kTc5Tok;
+          if constexpr (FP8) {                       // both terms of Q against the same codes
+            const uint32_t idesc = tc5_idesc(kRowsPerGroup, ng * GP, 0, 0u);
 #pragma unroll
-          for (int ks = 0; ks < D / 16; ++ks)
-            tc5_mma_ts(tmem + COL_S + b * kTc5Tok, tmem + COL_Q + ks * 8, tc5_desc(kt + (ks >> 2) * HS + (ks & 3) * 32, 16),
-                       idesc, ks > 0 ? 1u : 0u);
+            for (int ks = 0; ks < D / 32; ++ks)
+#pragma unroll
+              for (int t = 0; t < 2; ++t)
+                tc5_mma_ss8(s_col, tc5_desc8<D>(qtile + t * (QB / 2) + ks * 32), tc5_desc8<D>(kt + ks * 32), idesc, ks + t > 0 ? 1u : 0u);
+          } else {
+            const uint32_t idesc = tc5_idesc(kRowsPerGroup, ng * GP, 0);
+#pragma unroll
+            for (int ks = 0; ks < D / 16; ++ks) {
+              const uint32_t at = (ks >> 2) * HS + (ks & 3) * 32;
+              tc5_mma_ss(s_col, tc5_desc(qtile + at, 16), tc5_desc(kt + at, 16), idesc, ks > 0 ? 1u : 0u);
+            }
+          }
           tc5_commit(s_full + 8 * b);
           tc5_commit(kfree + 8 * slot);
           if (first + PG >= seg_end) tc5_commit(q_free);        // Q may be replaced once the piece's last product has run
@@ -552,14 +603,15 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   } else if (warp == kTc5PvWarp) {
     // ------------------------------------------------------------------ P V issuer (one thread)
     if (lane == 0) {
-      const uint32_t idesc = tc5_idesc(kRowsPerGroup, D, 1, FMT);
-      int sg = sg0, item = lo, g = 0;
+      const uint32_t idesc = tc5_idesc(kRowsPerGroup, D, 1, FP8 ? 0u : 1u);
+      int sg = sg0, item = lo, piece = 0, g = 0;
       bool ok = true;
       while (item < hi && ok) {
         const int seg_end = min(hi, pre[sg + 1]);
         for (int first = item; first < seg_end && ok; first += PG, ++g) {
-          const int ng = min(PG, seg_end - first), b = g & 1, use = g >> 1, slot = g % NR;
-          ok = mbar_wait(vfull + 8 * slot, (g / NR) & 1, abort_flag, p.status, p.wait_cycles);
+          const int ng = min(PG, seg_end - first), b = g % SB, use = g / SB, slot = g % NRV;
+          ok = mbar_wait(vfull + 8 * slot, (g / NRV) & 1, abort_flag, p.status, p.wait_cycles);
+          if (first == item && piece > 0) ok = ok && mbar_wait(o_free, (piece - 1) & 1, abort_flag, p.status, p.wait_cycles);   // O has been read
           ok = ok && mbar_wait(p_full + 8 * b, use & 1, abort_flag, p.status, p.wait_cycles);
           if (!ok) break;
           tc5_fence_after();
@@ -572,251 +624,307 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         }
         item = seg_end;
         ++sg;
+        ++piece;
         while (item < hi && pre[sg + 1] <= item) ++sg;
       }
     }
   }
   } else {
     // ------------------------------------------------------------------ softmax / epilogue warps
-    if constexpr (FP8) asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
-    // Thread = query row (tensor-memory lane 32 * (warp % 4) + lane) and one half of the columns:
-    // set h = warp / 4 takes columns 64h .. 64h+63 of every group (and half of Q, of O when it is
-    // rescaled or read out).  The exponentials are the bottleneck of this path (one special-function
-    // unit per scheduler); two warps per scheduler keep that unit busy while the partner loads,
-    // packs and stores.  The pair meets once per group (named barrier) to exchange the row maxima.
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(FP8 ? kTc5SoftmaxRegs8 : kTc5SoftmaxRegs));
+    // Thread = query row (tensor-memory lane 32 * (warp % 4) + lane); set h = warp / 4 takes the groups
+    // h, h + 3, ..., all columns, in S buffer h.  The three warps of a scheduler work on different groups, a
+    // third of a period apart, so that one's exponentials (one special-function unit per scheduler) run while
+    // the others load, take maxima, pack and store.  All sets add to the same O, under the same reference
+    // maximum: a group's handler takes the reference over from the group before it, whose set publishes it
+    // as soon as it has decided (before its exponentials).
     const __nv_bfloat16* q = static_cast<const __nv_bfloat16*>(p.q);
-    const int quarter = warp & 3, h = warp >> 2;
+    const int quarter = warp & 3, h = warp >> 2, h_prev = h == 0 ? kTc5Sets - 1 : h - 1;
     const int r = quarter * 32 + lane;                         // row of the tile = tensor-memory lane
     const uint32_t lane_addr = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
-    const float scale2 = p.sm_scale * kLog2e;
-    constexpr int QW = D / 4;                                  // 32-bit words of Q per thread (half a row)
-    constexpr int OC = D / 2;                                  // columns of O per thread
+    const uint32_t s_addr = lane_addr + COL_S + h * kTc5Tok;
     // every wait of these warps ends with one answer for the whole warp: the tensor-memory
     // instructions that follow need all 32 lanes
     auto warp_wait = [&](uint32_t bar, uint32_t parity) {
       return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, p.status, p.wait_cycles)) != 0;
     };
-    int n_meet = 0;
-    auto pair_sync = [&]() {                                    // bounded like every other wait
-      __syncwarp();
-      if (lane == 0) mbar_arrive(xbar + 8 * quarter, 1);
-      const bool met = warp_wait(xbar + 8 * quarter, n_meet & 1);
-      ++n_meet;
-      return met;
-    };
-    int sg = sg0, item = lo, piece = 0, g = 0;
+    int sg = sg0, item = lo, piece = 0, g = 0, n_meet = 0;
+    int n_pub = 0;                                              // references the previous set's warp of this quarter has published, or will have
     bool ok = true;
     while (item < hi && ok) {
       const int seg_end = min(hi, pre[sg + 1]);
       const int rg = sg / p.n_sk, sk = sg % p.n_sk, s = sk / p.Hkv, kh = sk % p.Hkv;
       const int rows = rows_in_group(n_active_of(s), p.G, rg);
-      const bool warp_has_rows = quarter * 32 < rows;          // the same for both warps of a pair
-      // ---- the piece's Q tile: this thread's half row, two bf16 per tensor-memory column
+      const bool warp_has_rows = quarter * 32 < rows;          // the same for the warps of a quarter
+      float scale2 = p.sm_scale * kLog2e;
+      // ---- the piece's Q tile: sets 0 and 1 write half a row per thread
       {
-        uint32_t qw[QW];
         const uint4* src = nullptr;
         if (r < rows) {
           const int row = rg * kRowsPerGroup + r, a = row / p.G, gi = row % p.G;
           int tok = token_of(s, a);
           if (tok < 0 || tok >= p.B) { set_status(p.status, LOSA_ERR_BOUNDS); tok = 0; }
-          src = reinterpret_cast<const uint4*>(q + ((static_cast<size_t>(s) * p.B + tok) * p.Hq + kh * p.G + gi) * D) + h * (QW / 4);
+          src = reinterpret_cast<const uint4*>(q + ((static_cast<size_t>(s) * p.B + tok) * p.Hq + kh * p.G + gi) * D);
         }
+        constexpr int NC = D / 16;                              // 16-byte chunks of half a row
+        uint4 qv[NC];
 #pragma unroll
-        for (int c = 0; c < QW / 4; ++c) {
-          const uint4 v = src ? __ldg(src + c) : make_uint4(0u, 0u, 0u, 0u);
-          qw[4 * c] = v.x; qw[4 * c + 1] = v.y; qw[4 * c + 2] = v.z; qw[4 * c + 3] = v.w;
-        }
-        if constexpr (FP8) {                        // the MMAs of this variant take fp16 operands
+        for (int c = 0; c < NC; ++c) qv[c] = src && h < 2 ? __ldg(src + h * NC + c) : make_uint4(0u, 0u, 0u, 0u);
+        if constexpr (FP8) {
+          // Q in two E4M3 terms.  The row is scaled by the power of two that brings its largest element to
+          // 2^7 .. 2^8; the first term takes four significant bits of an element and the second the other
+          // four, exactly down to 2^-9 of the largest element; below that the error is at most 2^-18 of it.
+          uint32_t top = 0;                                     // of the whole row
+          if (src) {
+#pragma unroll 4
+            for (int c = 0; c < 2 * NC; ++c) {
+              const uint4 v = __ldg(src + c);
+              const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-          for (int c = 0; c < QW; ++c) {
-            const __half2 hq = __floats2half2_rn(__uint_as_float(qw[c] << 16), __uint_as_float(qw[c] & 0xffff0000u));
-            qw[c] = *reinterpret_cast<const uint32_t*>(&hq);
+              for (int e = 0; e < 4; ++e) top = max(top, max((w[e] << 16) & 0x7fffffffu, w[e] & 0x7fff0000u));
+            }
+          }
+          // (exponent field e of the largest element: times 2^(134 - e) in two steps, each a normal number)
+          const int e_top = max(static_cast<int>(top >> 23), 16), up = 134 - e_top, u0 = up / 2, u1 = up - u0;
+          const float f0 = __int_as_float((127 + u0) << 23), f1 = __int_as_float((127 + u1) << 23);
+          scale2 *= __int_as_float((127 - u0) << 23) * __int_as_float((127 - u1) << 23);
+          if ((top >> 23) == 255) scale2 = __int_as_float(top);           // an infinity or NaN among them: in all the row's scores
+          if (piece > 0) ok = warp_wait(q_free, (piece - 1) & 1);
+          if (!ok) break;
+          if (warp_has_rows && h < 2) {
+#pragma unroll
+            for (int c = 0; c < NC; c += 2) {                   // two chunks of bf16 make one of codes
+              uint32_t hi4[4], lo4[4];
+#pragma unroll
+              for (int x = 0; x < 2; ++x) {
+                const uint32_t w[4] = {qv[c + x].x, qv[c + x].y, qv[c + x].z, qv[c + x].w};
+                uint16_t a[4], b[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                  const float v0 = __uint_as_float(w[e] << 16) * f0 * f1, v1 = __uint_as_float(w[e] & 0xffff0000u) * f0 * f1;
+                  a[e] = __nv_cvt_float2_to_fp8x2(make_float2(v0, v1), __NV_SATFINITE, __NV_E4M3);
+                  const __half2_raw back = __nv_cvt_fp8x2_to_halfraw2(a[e], __NV_E4M3);
+                  const float2 bf = __half22float2(__half2(back));
+                  b[e] = __nv_cvt_float2_to_fp8x2(make_float2(v0 - bf.x, v1 - bf.y), __NV_SATFINITE, __NV_E4M3);
+                }
+                hi4[2 * x] = a[0] | static_cast<uint32_t>(a[1]) << 16;
+                hi4[2 * x + 1] = a[2] | static_cast<uint32_t>(a[3]) << 16;
+                lo4[2 * x] = b[0] | static_cast<uint32_t>(b[1]) << 16;
+                lo4[2 * x + 1] = b[2] | static_cast<uint32_t>(b[3]) << 16;
+              }
+              uint8_t* dst = gen + tc5_sw8<D>(r, h * (NC / 2) + c / 2);
+              *reinterpret_cast<uint4*>(dst) = make_uint4(hi4[0], hi4[1], hi4[2], hi4[3]);
+              *reinterpret_cast<uint4*>(dst + QB / 2) = make_uint4(lo4[0], lo4[1], lo4[2], lo4[3]);
+            }
+          }
+        } else {
+          if (piece > 0) ok = warp_wait(q_free, (piece - 1) & 1);
+          if (!ok) break;
+          if (warp_has_rows && h < 2) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {                      // 64-column blocks of 128-byte rows, 128-byte swizzle
+              const int ch = h * NC + c;
+              *reinterpret_cast<uint4*>(gen + (ch >> 3) * HS + tc5_sw(r, ch & 7)) = qv[c];
+            }
           }
         }
-        if (piece > 0) ok = warp_wait(q_free, (piece - 1) & 1);
-        if (!ok) break;
-        tc5_fence_after();
-        if constexpr (QW == 32) tc5_st32(lane_addr + COL_Q + h * QW, qw);
-        else tc5_st16(lane_addr + COL_Q + h * QW, qw);
-        tc5_wait_st();
-        tc5_fence_before();
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs read the tile through the async proxy
         __syncwarp();
         if (lane == 0) mbar_arrive(q_full, 1);
       }
-      float m_ref = -INFINITY, l = 0.f;                         // l: this thread's columns only
-      bool o_valid = false;                                     // O holds at least one group of this piece
+      float m_ref = -INFINITY, l = 0.f;                         // l: the groups of this set, relative to m_ref
       for (int first = item; first < seg_end && ok; first += PG, ++g) {
-        const int ng = min(PG, seg_end - first), ncol = ng * GP, b = g & 1, use = g >> 1;
-        const uint32_t s_addr = lane_addr + COL_S + b * kTc5Tok;
+        const int turn = g % kTc5Sets;
+        if (turn != h) {                                        // another set's
+          if (warp_has_rows && turn == h_prev) ++n_pub;
+          continue;
+        }
+        const int ng = min(PG, seg_end - first), ncol = ng * GP;
         volatile int* gmeta = meta + (g % MR) * PG;
         auto valid_of = [&](int j) { return FP8 ? gmeta[j] & 0xff : gmeta[j]; };     // tokens of the group's page j
-        ok = warp_wait(s_full + 8 * b, use & 1);
+        ok = warp_wait(s_full + 8 * h, (g / kTc5Sets) & 1);
         if (!ok) break;
         tc5_fence_after();
         // pages with fewer than GP tokens (the last page of a prefix), or a group that ends inside a
         // 32-column chunk, need per-column masks; everything else takes the plain path
-        bool ragged = (ncol & 31) != 0;
-        for (int j = 0; j < ng; ++j) ragged |= valid_of(j) < GP;
-        auto masked = [&](int col) {
-          const int j = col / GP, t = col % GP;
-          return j >= ng || t >= valid_of(j);
-        };
-        const int col0 = 64 * h;                                // this thread's columns: col0 .. col0+63, below ncol
+        const bool any_short = __any_sync(0xffffffffu, lane < ng && valid_of(min(lane, PG - 1)) < GP) != 0;
+        const bool ragged = any_short || (ncol & 31) != 0;
         if (warp_has_rows) {
-          // ---- the row's scores: one read of tensor memory into registers, both loads in flight together
-          uint32_t sraw[64];
+          // FP8: the scores of a page carry its key scale, its weights the value scale's part 2^vexp: runs of
+          // PW columns, each of one page
+          constexpr int PW = GP < 32 ? GP : 32;
+          auto run_page = [&](int col) { return min(col / GP, ng - 1); };
+          auto run_mul = [&](int col) { return FP8 ? scale2 * kscale_meta[(g % MR) * PG + run_page(col)] : scale2; };
+          auto run_exp = [&](int col) { return static_cast<float>((gmeta[run_page(col)] >> 8) - 127); };
+          // of columns col .. col + 31 of the scores, those that hold no token become -inf
+          auto mask_chunk = [&](uint32_t* v, int col) {
+            uint32_t keep = 0;
 #pragma unroll
-          for (int c = 0; c < 2; ++c)
-            if (col0 + c * 32 < ncol) tc5_ld32_nowait(s_addr + col0 + 32 * c, sraw + 32 * c);
-          tc5_wait_ld();
-#pragma unroll
-          for (int c = 0; c < 2; ++c)
-            if (col0 + c * 32 < ncol) tc5_pin32(sraw + 32 * c);
-          if (ragged) {
-#pragma unroll
-            for (int c = 0; c < 2; ++c)
-              if (col0 + c * 32 < ncol) {
-#pragma unroll
-                for (int e = 0; e < 32; ++e) if (masked(col0 + 32 * c + e)) sraw[32 * c + e] = 0xff800000u;   // -inf
-              }
-          }
-          // ---- pass 1: the row's maximum over the group (own columns, then the partner's)
-          // (FP8: of the shifted exponents; NP page runs of PW columns per 32, each with its scales)
-          constexpr int PW = (FP8 && GP == 16) ? 16 : 32, NP = 32 / PW;
-          float kmul[2 * NP], vexp[2 * NP];
-          if constexpr (FP8) {
-#pragma unroll
-            for (int x = 0; x < 2 * NP; ++x) {
-              const int j = (col0 + x * PW) / GP;
-              kmul[x] = j < ng ? scale2 * kscale_meta[(g % MR) * PG + j] : 1.f;
-              vexp[x] = j < ng ? static_cast<float>((gmeta[j] >> 8) - 127) : 0.f;
+            for (int x = 0; x < 32 / PW; ++x) {
+              const int c = col + x * PW, j = c / GP, n = j < ng ? min(max(valid_of(j) - c % GP, 0), PW) : 0;
+              keep |= (n >= 32 ? 0xffffffffu : (1u << n) - 1u) << (x * PW % 32);
             }
-          }
+#pragma unroll
+            for (int e = 0; e < 32; ++e) if (!((keep >> e) & 1u)) v[e] = 0xff800000u;
+          };
+          // The scores are read from tensor memory twice, 32 columns at a time in rolled loops.  With the row in registers
+          // and straight code for its 128 columns (two sets of warps), the first group's exponentials of a sparse step
+          // took 2,700 to 7,900 cycles for 15 KB of instructions, fetched behind the page copies that have just filled
+          // the memory queues (2,100 now); 64 columns at a time: eight 32K prompts, dense step 246 against 230 us.
+          // ---- pass 1: the row's maximum over the group (FP8: of the shifted exponents)
           float mx_own = -INFINITY;
-          float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll 1
+          for (int c0 = 0; c0 < ncol; c0 += 32) {
+            uint32_t v[32];
+            tc5_ld32_nowait(s_addr + c0, v);
+            tc5_wait_ld();
+            tc5_pin32(v);
+            if (ragged) mask_chunk(v, c0);
+            float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-          for (int c = 0; c < 2; ++c)
-            if (col0 + c * 32 < ncol) {
-#pragma unroll
-              for (int e = 0; e < 32; ++e) {
-                mx[e & 3] = fmaxf(mx[e & 3], __uint_as_float(sraw[32 * c + e]));
-                if (FP8 && (e + 1) % PW == 0) {
-                  const int x = c * NP + e / PW;
-                  mx_own = fmaxf(mx_own, fmaf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])), kmul[x], vexp[x]));
-                  mx[0] = mx[1] = mx[2] = mx[3] = -INFINITY;
-                }
+            for (int e = 0; e < 32; ++e) {
+              mx[e & 3] = fmaxf(mx[e & 3], __uint_as_float(v[e]));
+              if (FP8 && (e + 1) % PW == 0) {
+                mx_own = fmaxf(mx_own, fmaf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])), run_mul(c0 + e), run_exp(c0 + e)));
+                mx[0] = mx[1] = mx[2] = mx[3] = -INFINITY;
               }
             }
-          if (!FP8) mx_own = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
-          xmax[(b * 2 + h) * kRowsPerGroup + r] = mx_own;
-          ok = pair_sync();
-          const float m_new = fmaxf(mx_own, xmax[(b * 2 + (h ^ 1)) * kRowsPerGroup + r]) * (FP8 ? 1.f : scale2);
-          float corr = 1.f;
-          constexpr float LIFT = FP8 ? kTc5Fp8Lift : 0.f;
-          if (m_new > m_ref + (kTc5Tau + LIFT) || (m_ref == -INFINITY && m_new > -INFINITY)) {
-            corr = (m_ref == -INFINITY) ? 0.f : ex2(m_ref - (m_new - LIFT));
-            m_ref = m_new - LIFT;
-            l *= corr;
+            if (!FP8) mx_own = fmaxf(mx_own, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])));
           }
-          // ---- rescale O (rare): the previous group's P V must have run; all lanes of the warp take
-          //      part, each set on its half of the columns
-          if (__any_sync(0xffffffffu, o_valid && corr != 1.f)) {
-            ok = ok && warp_wait(s_free + 8 * ((g - 1) & 1), ((g - 1) >> 1) & 1);
+          // ---- the reference maximum: the one of the group before, moved when it would grow by more than 2^8
+          float m_prev = -INFINITY;
+          if (first != item) {
+            ok = warp_wait(mbar + 8 * (4 * h_prev + quarter), (n_pub - 1) & 1);
+            m_prev = mref[h_prev * kRowsPerGroup + r];
+          }
+          constexpr float LIFT = FP8 ? kTc5Fp8Lift : 0.f;
+          const float m_own = FP8 ? mx_own : mx_own * scale2;
+          float m_new = m_prev;
+          if (m_own > m_prev + (kTc5Tau + LIFT) || (m_prev == -INFINITY && m_own > -INFINITY)) m_new = m_own - LIFT;
+          mref[h * kRowsPerGroup + r] = m_new;
+          __syncwarp();
+          if (lane == 0) mbar_arrive(mbar + 8 * (4 * h + quarter), 1);
+          if (m_ref != m_new) {
+            l *= m_ref == -INFINITY ? 0.f : ex2(m_ref - m_new);
+            m_ref = m_new;
+          }
+          // ---- rescale O (rare): the previous group's P V must have run, this one's waits for P
+          if (first != item && __any_sync(0xffffffffu, m_prev != m_new)) {
+            const float corr = m_prev == m_new ? 1.f : (m_prev == -INFINITY ? 0.f : ex2(m_prev - m_new));
+            ok = ok && warp_wait(s_free + 8 * h_prev, ((g - 1) / kTc5Sets) & 1);
             if (ok) {
               tc5_fence_after();
+#pragma unroll 1
+              for (int c0 = 0; c0 < D; c0 += 16) {
+                uint32_t w[16];
+                tc5_ld16(lane_addr + COL_O + c0, w);
 #pragma unroll
-              for (int c0 = 0; c0 < OC; c0 += 32) {
-                float t[32];
-                uint32_t w[32];
-                tc5_ld32(lane_addr + COL_O + h * OC + c0, t);
-#pragma unroll
-                for (int e = 0; e < 32; ++e) w[e] = __float_as_uint(t[e] * corr);
-                tc5_st32(lane_addr + COL_O + h * OC + c0, w);
+                for (int e = 0; e < 16; ++e) w[e] = __float_as_uint(__uint_as_float(w[e]) * corr);
+                tc5_st16(lane_addr + COL_O + c0, w);
               }
               tc5_wait_st();
             }
           }
-          // ---- pass 2: P = 2^(s - m) as bf16, written over the scores (column c of P takes the
-          //      place of columns 2c, 2c+1 of S; every score of the group is in registers by now,
-          //      the partner's too: it has passed the pair barrier)
+          // ---- pass 2: P = 2^(s - m) as 16-bit values, written over the scores (columns 2c, 2c+1 of P take the
+          //      place of column c of S, which has been read by then)
           if (ok) {
             const float ms = (m_ref == -INFINITY) ? 0.f : m_ref;
-            float sum[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+            for (int c0 = 0; c0 < ncol; c0 += 32) {
+              uint32_t v[32];
+              tc5_ld32_nowait(s_addr + c0, v);
+                tc5_wait_ld();
+              tc5_pin32(v);
+              if (ragged) mask_chunk(v, c0);
+              float sum[4] = {0.f, 0.f, 0.f, 0.f};
+              float mul = scale2, add = -ms, vexp = 0.f;
+              uint32_t w[16];
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-              if (col0 + c * 32 < ncol) {
-                uint32_t w[16];
-#pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                  const int x = c * NP + 2 * e / PW;
-                  const float mul = FP8 ? kmul[x] : scale2, add = FP8 ? vexp[x] - ms : -ms;
-                  const float p0 = ex2(fmaf(__uint_as_float(sraw[32 * c + 2 * e]), mul, add));
-                  const float p1 = ex2(fmaf(__uint_as_float(sraw[32 * c + 2 * e + 1]), mul, add));
-                  sum[e & 3] += p0 + p1;
-                  w[e] = FP8 ? pack_f16(p0, p1) : pack_bf16(p0, p1);
-                  if (FP8 && (2 * e + 2) % PW == 0) {     // the page run's sum, without the value scale
-                    l = fmaf((sum[0] + sum[1]) + (sum[2] + sum[3]), __int_as_float((127 - static_cast<int>(vexp[x])) << 23), l);
-                    sum[0] = sum[1] = sum[2] = sum[3] = 0.f;
-                  }
+              for (int e = 0; e < 16; ++e) {
+                if (FP8 && (2 * e) % PW == 0) {
+                  mul = run_mul(c0 + 2 * e);
+                  vexp = run_exp(c0 + 2 * e);
+                  add = vexp - ms;
                 }
-                tc5_st16(s_addr + col0 / 2 + 16 * c, w);
+                const float p0 = ex2(fmaf(__uint_as_float(v[2 * e]), mul, add));
+                const float p1 = ex2(fmaf(__uint_as_float(v[2 * e + 1]), mul, add));
+                sum[e & 3] += p0 + p1;
+                w[e] = FP8 ? pack_f16(p0, p1) : pack_bf16(p0, p1);
+                if (FP8 && (2 * e + 2) % PW == 0) {     // the page run's sum, without the value scale
+                  l = fmaf((sum[0] + sum[1]) + (sum[2] + sum[3]), __int_as_float((127 - static_cast<int>(vexp)) << 23), l);
+                  sum[0] = sum[1] = sum[2] = sum[3] = 0.f;
+                }
               }
+              tc5_st16(s_addr + c0 / 2, w);
+              if (!FP8) l += (sum[0] + sum[1]) + (sum[2] + sum[3]);
             }
             tc5_wait_st();
-            if (!FP8) l += (sum[0] + sum[1]) + (sum[2] + sum[3]);
           }
         }
         if (!ok) break;
-        if (ragged) {
-          // rows of V past the end of the prefix may hold anything (even NaN): clear them once the
-          // tile has landed (all softmax warps, whether or not they own rows)
-          bool any_short = false;
-          for (int j = 0; j < ng; ++j) any_short |= valid_of(j) < GP;
-          if (any_short) {
-            const int slot = g % NR;
-            ok = warp_wait(vfull + 8 * slot, (g / NR) & 1);
-            if (!ok) break;
-            uint8_t* vg = gen + (NR + slot) * SLOT;
-            for (int j = 0; j < ng; ++j) {
-              const int valid = valid_of(j);
-              for (int idx = tid; idx < (GP - valid) * (D / 8); idx += kTc5SoftmaxWarps * 32) {
-                const int t = j * GP + valid + idx / (D / 8), ch = idx % (D / 8);
-                *reinterpret_cast<uint4*>(vg + (ch >> 3) * HS + tc5_sw(t, ch & 7)) = make_uint4(0u, 0u, 0u, 0u);
-              }
+        if (any_short) {
+          // rows of V past the end of the prefix may hold anything (even NaN): clear them once the tile has
+          // landed (all warps of the set, whether or not they own rows).  The slot's previous tile must have been
+          // used first: until then its barrier may be a phase behind, with the parity that is waited for.
+          const int slot = g % NRV;
+          if (g >= NRV) ok = warp_wait(vfree + 8 * slot, (g / NRV - 1) & 1);
+          ok = ok && warp_wait(vfull + 8 * slot, (g / NRV) & 1);
+          if (!ok) break;
+          uint8_t* vg = gen + (vring - base) + slot * SLOT;
+          for (int j = 0; j < ng; ++j) {
+            const int valid = valid_of(j);
+            for (int idx = r; idx < (GP - valid) * (D / 8); idx += kTc5SetWarps * 32) {
+              const int t = j * GP + valid + idx / (D / 8), ch = idx % (D / 8);
+              *reinterpret_cast<uint4*>(vg + (ch >> 3) * HS + tc5_sw(t, ch & 7)) = make_uint4(0u, 0u, 0u, 0u);
             }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         }
         tc5_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(p_full + 8 * b, 1);
-        o_valid = true;
+        if (lane == 0) mbar_arrive(p_full + 8 * h, 1);
       }
       if (!ok) break;
       // ---- the piece's record: one 16-row tile record per 16 rows, reference maximum in base-2
-      //      units; each set writes its half of the columns, set 0 the row's maximum and sum
-      ok = warp_wait(s_free + 8 * ((g - 1) & 1), ((g - 1) >> 1) & 1);
+      //      units; the sets share the columns, set 0 writes the row's maximum and sum
+      ok = warp_wait(s_free + 8 * ((g - 1) % kTc5Sets), ((g - 1) / kTc5Sets) & 1);
       if (!ok) break;
       tc5_fence_after();
       if (warp_has_rows) {
-        if (h == 1) xsum[r] = l;
-        ok = pair_sync();
+        xsum[h * kRowsPerGroup + r] = l;
+        xref[h * kRowsPerGroup + r] = m_ref;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(xbar + 8 * quarter, 1);      // the quarter's warps meet
+        ok = warp_wait(xbar + 8 * quarter, n_meet & 1);
+        ++n_meet;
         if (!ok) break;
         float* rec = record_base(p.partials, blockIdx.x + sg, r / kTileRows, D);
         const int rr = r % kTileRows;
-#pragma unroll
-        for (int c0 = 0; c0 < OC; c0 += 32) {
+#pragma unroll 1
+        for (int c0 = 32 * h; c0 < D; c0 += 32 * kTc5Sets) {
           float t[32];
-          tc5_ld32(lane_addr + COL_O + h * OC + c0, t);
+          tc5_ld32(lane_addr + COL_O + c0, t);
           if (r < rows) {
 #pragma unroll
             for (int e = 0; e < 32; e += 4)
-              *reinterpret_cast<float4*>(rec + 2 * kTileRows + rr * D + h * OC + c0 + e) = make_float4(t[e], t[e + 1], t[e + 2], t[e + 3]);
+              *reinterpret_cast<float4*>(rec + 2 * kTileRows + rr * D + c0 + e) = make_float4(t[e], t[e + 1], t[e + 2], t[e + 3]);
           }
         }
-        if (h == 0 && r < rows) { rec[rr] = m_ref; rec[kTileRows + rr] = l + xsum[r]; }
+        if (h == 0 && r < rows) {
+          const float m_last = mref[((g - 1) % kTc5Sets) * kRowsPerGroup + r];
+          float total = 0.f;
+#pragma unroll
+          for (int x = 0; x < kTc5Sets; ++x) {
+            const float m_x = xref[x * kRowsPerGroup + r];
+            if (m_x != -INFINITY) total = fmaf(xsum[x * kRowsPerGroup + r], ex2(m_x - m_last), total);
+          }
+          rec[rr] = m_last;
+          rec[kTileRows + rr] = total;
+        }
       }
       tc5_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(o_free, 1);
       item = seg_end;
       ++sg;
       ++piece;
@@ -832,9 +940,9 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     // round of copies of every ring slot (a group that was begun has had all its copies issued: the
     // producer loop only stops between groups), the issuing threads for the products they issued.
     if ((warp == kTc5KWarp || warp == kTc5VWarp) && lane == 0) {
-      // (FP8 pages: the copies land in the staging slots)
-      const uint32_t full0 = FP8 ? (warp == kTc5VWarp ? vstg_full : kstg_full) : (warp == kTc5VWarp ? vfull : kfull);
-      constexpr int NSL = FP8 ? NSP : NR;
+        const bool is_v = warp == kTc5VWarp;
+      const uint32_t full0 = is_v ? (FP8 ? vstg_full : vfull) : kfull;
+      const int NSL = is_v ? (FP8 ? NSP : NRV) : NRK;
       for (int sl = 0; sl < NSL; ++sl) {
         if (issued < sl) continue;
         const int gl = issued - (issued - sl) % NSL;

@@ -321,3 +321,108 @@ def test_fp8_cache_full_size_c5_layer():
     ref = o.run_step(h1)
     s1["delta"] = ref["delta"]
     compare(s1, ref, cfg, "fp8 c5 layer, LoSA step")
+
+
+@pytest.mark.parametrize("fp8", [False, True])
+@pytest.mark.parametrize("g,d", [(16, 64), (32, 128), (64, 128)])
+def test_reference_maximum_that_passes_between_groups_and_segments(g, d, fp8):
+    """Shares of several groups of 128 tokens that cross segments at odd group counts; the largest score of a group
+    rises, falls or jumps from group to group, by less and by more than the 2^8 that moves the reference maximum,
+    differently for every query row; 36 and 128 query rows (warps without rows)."""
+    import torch
+    from paper_2604_12056_b200.layer import LosaLayer
+    N, Hkv, G, groups = 24, 4, 4, 13
+    for Bk in (9, 32):
+        n_tok = groups * 128 - 37
+        cfg = wl.config("c2", n_q_heads=Hkv * G, n_kv_heads=Hkv, head_dim=d, page_size=g, kv_lens=(n_tok,) * N, block_size=Bk, steps=1,
+                        topk=1, m_active=1)
+        P, mp = N * cfg.max_pages_per_seq, cfg.max_pages_per_seq
+        gen = torch.Generator(device="cuda")
+        gen.manual_seed(11 * g + d + Bk)
+        rnd = lambda *shape: torch.randn(*shape, generator=gen, device="cuda")
+        u = torch.nn.functional.normalize(rnd(2, d), dim=-1)
+        kp, vp = 0.1 * rnd(P, Hkv, g, d), rnd(P, Hkv, g, d)
+        grp = (torch.arange(mp, device="cuda") * g // 128).float().repeat(N)            # group of a sequence's page
+        level = torch.stack([5.0 * grp, 5.0 * (groups - grp), 40.0 * torch.rand(P, generator=gen, device="cuda"), 12.0 * (grp % 2)])   # log2 units
+        level = level[torch.arange(P, device="cuda") // mp % 4, torch.arange(P, device="cuda")]           # one kind per sequence
+        kp[:, :, 5] += (level * float(np.log(2.0)) / (3.0 * cfg.sm_scale))[:, None, None] * u[0]
+        q = 3.0 * u[0] * torch.rand(N, Bk, Hkv * G, 1, generator=gen, device="cuda") + 0.5 * rnd(N, Bk, Hkv * G, d)
+        kb, vb = (rnd(N, Bk, Hkv, d).bfloat16() for _ in range(2))
+        q = q.bfloat16()
+        table = torch.arange(P, dtype=torch.int32, device="cuda").view(N, -1).contiguous()
+        layer = LosaLayer(cfg, kp.bfloat16(), vp.bfloat16(), table, torch.full((N,), n_tok, dtype=torch.int32, device="cuda"), fp8_kv=fp8)
+        layer.run_step(q, kb, vb, torch.ones(N, dtype=torch.int32, device="cuda"))
+        assert layer.ctx.poll_status() == 0
+        for s in range(N):
+            if fp8:
+                assert_rows_exact_to_p(layer, cfg, q, s, f"{Bk} tokens")
+                continue
+            for h in range(Hkv):
+                k, v = (t[table[s].long(), h].reshape(-1, d)[:n_tok].double() for t in (layer.k_pages, layer.v_pages))
+                heads = slice(h * G, (h + 1) * G)
+                sc = q[s, :, heads].double() @ k.T * cfg.sm_scale
+                p = torch.softmax(sc, -1)
+                # P is rounded to 8 significant bits: half a unit of 2^-8 of every weight, as much again for the rest
+                assert ((layer.o_p[s, :, heads].double() - p @ v).abs() <= 2.0 ** -8 * (p @ v.abs())).all(), (s, h, Bk)
+                assert (layer.lse_p[s, :, heads].double() - torch.logsumexp(sc, -1)).abs().max() <= 1e-4
+
+
+@pytest.mark.parametrize("g,d", [(16, 64), (32, 64), (16, 128), (64, 128)])
+@pytest.mark.parametrize("power", [-100, -20, 0, 10])
+def test_fp8_queries_of_any_magnitude(g, d, power):
+    """The queries enter the first product as two E4M3 terms under a scale of the row: rows of every magnitude, elements
+    2^-20 .. 1 of a row's largest, a row of zeros, a row of one element; against float64 on the dequantised keys."""
+    import torch
+    from paper_2604_12056_b200.layer import LosaLayer
+    Hkv, G, Bk, n_tok = 2, 4, 8, 3 * 128 + 5
+    cfg = wl.config("c2", n_q_heads=Hkv * G, n_kv_heads=Hkv, head_dim=d, page_size=g, kv_lens=(n_tok,), block_size=Bk, steps=1, topk=1,
+                    m_active=1)
+    P = cfg.max_pages_per_seq
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(g + d + power)
+    rnd = lambda *shape: torch.randn(*shape, generator=gen, device="cuda")
+    kp, vp = rnd(P, Hkv, g, d) * 2.0 ** max(-6, min(8, -power)), rnd(P, Hkv, g, d)      # (scores of ordinary size where keys can leave them)
+    q = rnd(1, Bk, Hkv * G, d) * torch.exp2(torch.randint(-20, 1, (1, Bk, Hkv * G, d), generator=gen, device="cuda").float())
+    q[0, 1] = 0.0
+    q[0, 2] *= torch.arange(d, device="cuda") == 7
+    q[0, 3] = rnd(Hkv * G, d)
+    q = (q * 2.0 ** power).bfloat16()
+    kb, vb = (rnd(1, Bk, Hkv, d).bfloat16() for _ in range(2))
+    table = torch.arange(P, dtype=torch.int32, device="cuda")[None].contiguous()
+    layer = LosaLayer(cfg, kp.bfloat16(), vp.bfloat16(), table, torch.tensor([n_tok], dtype=torch.int32, device="cuda"), fp8_kv=True)
+    layer.run_step(q, kb, vb, torch.ones(1, dtype=torch.int32, device="cuda"))
+    assert layer.ctx.poll_status() == 0
+    for h in range(Hkv):
+        k, v = listed_prefix(layer, cfg, 0, h)
+        for i in range(h * G, (h + 1) * G):
+            qd = q[0, :, i].double()
+            sc = qd @ k.T * cfg.sm_scale
+            # an element is exact down to 2^-9 of its row's largest, else off by at most 2^-18 of that (2^-17 here);
+            # fp32 sums: 2^-21 of the sum of magnitudes
+            off = cfg.sm_scale * (2.0 ** -17 * (qd.abs().amax(-1, keepdim=True) * (qd.abs() < 2.0 ** -9 * qd.abs().amax(-1, keepdim=True))) @ k.abs().T
+                                  + 2.0 ** -21 * (qd.abs() @ k.abs().T)).amax(-1)
+            lse = torch.logsumexp(sc, -1)
+            assert ((layer.lse_p[0, :, i].double() - lse).abs() <= off + 1e-5 + 2.0 ** -22 * lse.abs()).all(), (h, i)
+            p = torch.softmax(sc, -1)
+            bound = (2.0 ** -10 + 2 * off[:, None]) * (p @ v.abs()) + 2.0 ** -24 * p.amax(-1, keepdim=True) * v.abs().sum(0)
+            assert ((layer.o_p[0, :, i].double() - p @ v).abs() <= bound).all(), (h, i)
+
+
+def test_fp8_query_with_an_infinity_or_nan_spoils_its_row_only():
+    import torch
+    from paper_2604_12056_b200.layer import LosaLayer
+    cfg = wl.config("c2", n_q_heads=4, n_kv_heads=1, kv_lens=(200,), block_size=4, steps=1, topk=1, m_active=1)
+    w = wl.DeviceWorkload(cfg)
+    x = w.start_block()
+    layer = LosaLayer(cfg, w.k_pages, w.v_pages, w.page_table, w.kv_len, fp8_kv=True)
+    q = x.q.clone()
+    q[0, 1, 0, 5] = float("inf")
+    q[0, 2, 3, 9] = float("nan")
+    layer.run_step(q, x.k_blk, x.v_blk, x.m_per_seq)
+    assert layer.ctx.poll_status() == 0
+    bad = torch.zeros(4, 4, dtype=torch.bool, device="cuda")
+    bad[1, 0] = bad[2, 3] = True
+    assert torch.isnan(layer.o_p[0, 1, 0]).all() and torch.isfinite(layer.o_p[0][~bad]).all()
+    clean = LosaLayer(cfg, w.k_pages, w.v_pages, w.page_table, w.kv_len, fp8_kv=True)
+    clean.run_step(x.q, x.k_blk, x.v_blk, x.m_per_seq)
+    assert (layer.o_p[0][~bad] == clean.o_p[0][~bad]).all()
