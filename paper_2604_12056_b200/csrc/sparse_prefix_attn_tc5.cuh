@@ -37,9 +37,10 @@ constexpr int kTc5XchgBytes = 3 * kTc5Sets * kRowsPerGroup * 4;   // reference m
 // FP8 pages: binary places by which P is held above the reference maximum.  P stays below 2^(8 + 7) < 65504.
 constexpr float kTc5Fp8Lift = 7.0f;
 constexpr int kTc5StgMax = 20;                   // FP8 pages: staging slots of V, one page each, at most
-// FP8: value pages whose multiplier is kept.  Page x + 32 is issued once page x + 32 - 20 or a later one has
-// been converted, and with it the whole group of page x (at most 8 pages).
-constexpr int kTc5VmulRing = 32;
+// FP8: value pages whose multiplier is kept.  Page x + 64 is issued once page x + 64 - 20 or a later one has been
+// converted.  That is at least five groups (of at most 8 pages) after page x's, and a converting warp is less than
+// two groups ahead of the others: it refills a V slot after the slot's P V, which waits for all of them.
+constexpr int kTc5VmulRing = 64;
 // Groups whose per-page data (token counts; FP8: scales) is kept.  The K producer writes a page's entry
 // when it issues the page's copy, so the ring must be longer than its lead over the softmax warps.  A
 // group never spans two segments, so in a run of one-page segments every page in flight is a group of
@@ -206,6 +207,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   constexpr int HALVES = D / 64;                // 64-column (128-byte) blocks of a 16-bit K or V row
   constexpr int HS = kTc5Tok * 128;             // bytes of one such block of a whole group
   constexpr int PAGE_BYTES = GP * D * 2;        // of a 16-bit page of K, and of V
+  constexpr int UT = GP < 32 ? GP : 32, UPP = GP / UT;   // FP8: tokens that a converting warp takes at a time, such runs per page
   constexpr int SB = kTc5Sets;                  // S buffers, one per set
   constexpr uint32_t COL_O = 0, COL_S = 128;    // tensor-memory columns: O[D], S0[128], S1[128], S2[128]
   constexpr int TMEM_COLS = 512;
@@ -275,7 +277,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     if (FP8)
       for (int i = 0; i < NSP; ++i) {
         mbar_init(vstg_full + 8 * i, 1);
-        mbar_init(vstg_free + 8 * i, kTc5CvtWarps);
+        mbar_init(vstg_free + 8 * i, UPP);
       }
     *abort_flag = 0;
     *vmul_used = 0;
@@ -487,15 +489,16 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     }
   } else if (FP8 && warp >= kTc5CvtWarp) {
     // ------------------------------------------------------------------ converting warps (FP8 pages): V
-    // Each a quarter of every page's tokens.  A lane takes eight codes at a time (one 16-byte chunk of
-    // fp16): 8-byte reads of consecutive codes and 16-byte stores of consecutive swizzled chunks, both
-    // without bank conflicts; all of a page's are requested before any is converted.
+    // A warp takes every fourth run of UT tokens (a page, or half a page of 64) of a group: one wait and one arrival for
+    // up to 64 conversions (a quarter of every page per warp had four of each; a block of eight 32K prompts 1,032 us, 968 so).
+    // A lane takes eight codes at a time (one 16-byte chunk of fp16): 8-byte reads of consecutive codes and 16-byte
+    // stores of consecutive swizzled chunks, both without bank conflicts; up to eight are requested before any is converted.
     const uint8_t* stg_gen = gen + (vstg - base);
     uint8_t* ring_gen = gen + (vring - base);
     constexpr int CPR = D / 8, TPI = 32 / CPR;        // chunks of a row, tokens per warp access
-    constexpr int NU = GP / kTc5CvtWarps / TPI, U = NU;   // accesses per page and warp
-    static_assert(NU >= 1 && NU * TPI * kTc5CvtWarps == GP, "a page's tokens over the converting warps");
-    const int tl = (warp - kTc5CvtWarp) * (GP / kTc5CvtWarps) + lane / CPR, c = lane % CPR;
+    constexpr int NU = UT / TPI, U = NU < 8 ? NU : 8; // accesses per run, in flight
+    static_assert(NU % U == 0 && NU * TPI == UT, "a run's tokens");
+    const int tl = lane / CPR, c = lane % CPR;
     auto wait = [&](uint32_t bar, uint32_t parity) {
       int ok = 1;
       if (lane == 0) ok = mbar_wait(bar, parity, abort_flag, p.status, p.wait_cycles);
@@ -509,47 +512,49 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       for (int first = item; first < seg_end && ok; first += PG, ++g) {
         const int ng = min(PG, seg_end - first), sr = g % NRV;
         if (g >= NRV) ok = wait(vfree + 8 * sr, (g / NRV - 1) & 1);
-        for (int pg = 0; pg < ng; ++pg) {
-          const int x = first + pg - lo, ss = x % NSP;
+        uint8_t* dst = ring_gen + sr * SLOT + (c >> 3) * HS;
+        for (int u = warp - kTc5CvtWarp; u < ng * UPP; u += kTc5CvtWarps) {
+          const int pg = u / UPP, x = first + pg - lo, ss = x % NSP, t0 = u % UPP * UT + tl;
           ok = ok && wait(vstg_full + 8 * ss, (x / NSP) & 1);
           if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-          const uint8_t* src = stg_gen + ss * STG + tl * D + c * 8;
-          uint8_t* dst = ring_gen + sr * SLOT + (c >> 3) * HS;
-#pragma unroll
+          const uint8_t* src = stg_gen + ss * STG + t0 * D + c * 8;
+#pragma unroll 1
           for (int u0 = 0; u0 < NU; u0 += U) {
             uint2 w[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) w[u] = *reinterpret_cast<const uint2*>(src + (u0 + u) * TPI * D);
+            for (int e = 0; e < U; ++e) w[e] = *reinterpret_cast<const uint2*>(src + (u0 + e) * TPI * D);
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-              const uint32_t x4[4] = {w[u].x & 0xffffu, w[u].x >> 16, w[u].y & 0xffffu, w[u].y >> 16};
+            for (int e = 0; e < U; ++e) {
+              const uint32_t x4[4] = {w[e].x & 0xffffu, w[e].x >> 16, w[e].y & 0xffffu, w[e].y >> 16};
               uint32_t h[4];
 #pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const __half2_raw v = __nv_cvt_fp8x2_to_halfraw2(static_cast<__nv_fp8x2_storage_t>(x4[e]), __NV_E4M3);
-                h[e] = *reinterpret_cast<const uint32_t*>(&v);
+              for (int k = 0; k < 4; ++k) {
+                const __half2_raw v = __nv_cvt_fp8x2_to_halfraw2(static_cast<__nv_fp8x2_storage_t>(x4[k]), __NV_E4M3);
+                h[k] = *reinterpret_cast<const uint32_t*>(&v);
               }
-              *reinterpret_cast<uint4*>(dst + tc5_sw(pg * GP + tl + (u0 + u) * TPI, c & 7)) = make_uint4(h[0], h[1], h[2], h[3]);
+              *reinterpret_cast<uint4*>(dst + tc5_sw(pg * GP + t0 + (u0 + e) * TPI, c & 7)) = make_uint4(h[0], h[1], h[2], h[3]);
             }
           }
           __syncwarp();
           if (lane == 0) mbar_arrive(vstg_free + 8 * ss, 1);
         }
         if (!ok) break;
-        if (*vmul_used) {                     // this lane's chunks once more, times what of the scales is not in P
-#pragma unroll 1
-          for (int i = 0; i < ng * NU; ++i) {
-            const int pg = i / NU, u = i % NU;
+        if (*vmul_used) {                             // this lane's chunks once more, times what of the scales is not in P
+          for (int u = warp - kTc5CvtWarp; u < ng * UPP; u += kTc5CvtWarps) {
+            const int pg = u / UPP;
             const uint32_t mul = vmul[(first + pg - lo) % kTc5VmulRing];
             const __half2 m2 = *reinterpret_cast<const __half2*>(&mul);
-            uint4* at = reinterpret_cast<uint4*>(ring_gen + sr * SLOT + (c >> 3) * HS + tc5_sw(pg * GP + tl + u * TPI, c & 7));
-            uint4 x = *at;
-            auto scale = [&](uint32_t& y) {
-              const __half2 v = __hmul2(*reinterpret_cast<const __half2*>(&y), m2);
-              y = *reinterpret_cast<const uint32_t*>(&v);
-            };
-            scale(x.x); scale(x.y); scale(x.z); scale(x.w);
-            *at = x;
+#pragma unroll 1
+            for (int i = 0; i < NU; ++i) {
+              uint4* at = reinterpret_cast<uint4*>(dst + tc5_sw(pg * GP + u % UPP * UT + tl + i * TPI, c & 7));
+              uint4 x = *at;
+              auto scale = [&](uint32_t& y) {
+                const __half2 v = __hmul2(*reinterpret_cast<const __half2*>(&y), m2);
+                y = *reinterpret_cast<const uint32_t*>(&v);
+              };
+              scale(x.x); scale(x.y); scale(x.z); scale(x.w);
+              *at = x;
+            }
           }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs read the slot through the async proxy
