@@ -292,11 +292,12 @@ __device__ __forceinline__ void segment_prefix(int* pre, int n_seg, int n_rg, in
     const int seg = base + lane;
     int c = 0, vc = 0;
     if (seg < n_seg) {
-      const int n_sk = n_seg / n_rg, rg = seg / n_sk, sk = seg % n_sk, s = sk / H_kv;
+      const int n_sk = n_rg == 1 ? n_seg : n_seg / n_rg, rg = n_rg == 1 ? 0 : seg / n_sk, sk = seg - rg * n_sk, s = sk / H_kv;
       int na = n_active[s];
+      const int listed = count(sk);                  // (both requested before either is used)
       na = na < 0 ? 0 : (na > B ? B : na);
       const int rows = rows_in_group(na, G, rg);
-      c = rows > 0 ? max(count(sk), 0) : 0;
+      c = rows > 0 ? max(listed, 0) : 0;
       vc = c > 0 ? c + segment_pad(rows) : 0;
     }
     int inc = c, vinc = vc;

@@ -53,6 +53,7 @@ struct AttnParams {
   const float* v_scale;
   int N, B, Hq, Hkv, G, Pmax, n_phys, n_rg, n_sk, n_seg, n_ctas;   // n_sk = N * Hkv, n_seg = n_rg * n_sk
   float sm_scale;
+  int early;              // the kernels before this one are stages 1 to 3 of the same step: what is older may be read before they end
   long long wait_cycles;  // bound of every mbarrier wait of the bf16 main kernel, in SM clock cycles
 };
 
@@ -295,36 +296,40 @@ __global__ void __launch_bounds__(kFinishThreads) attn_finish_kernel(AttnParams 
   constexpr bool LOG2 = !std::is_same_v<T, float>;     // partial maxima in base-2 units (tensor-core kernel)
   __shared__ __align__(16) float buf[kFinishThreads / 32][kMergeBatch * D];
   grid_dep_trigger();
-  grid_dep_wait();
+  if constexpr (!LOG2) grid_dep_wait();                 // (fp32: launched behind an event, nothing runs beside it)
   constexpr int C = D / 32;
   const int lane = threadIdx.x & 31;
   const uint32_t row_i = blockIdx.x * (kFinishThreads / 32) + (threadIdx.x >> 5);
   const size_t row = row_i;
-  if (blockIdx.x == 0)
-    for (int s = threadIdx.x; s < p.N; s += kFinishThreads) f.step[s] += 1;
-  if (row >= f.n_rows) return;
+  const bool mine = row < f.n_rows;
+  // Stage 4 of this step runs before: the slots (stage 1), the queries and the cached prefix statistics (the step before)
+  // are final, and requested beside its last CTAs.  Nine rows in ten are stable; an active row overwrites the
+  // statistics below.  (volatile: a plain load would sink below the wait)
   const int hq = static_cast<int>(row_i % p.Hq), st = static_cast<int>(row_i / p.Hq), tok = st % p.B, s = st / p.B;   // (32-bit divisions)
   const int kh = hq / p.G, gi = hq % p.G;
-  // operands that do not depend on the row being active: requested first (one vector access each)
   const T* q = static_cast<const T*>(f.q);
-  float b[C];
-  ldv<C>(f.o_b + row * D + lane * C, b);
   RawRow<C> qv;                                         // (fp32: qf)
   float qf[C];
-  if constexpr (LOG2) qv = ld_raw<C>(q + row * D + lane * C);
-  else ldv<C>(q + row * D + lane * C, qf);
+  float a[C], Lp = 0.f;
+  int slot = -1;
+  if (mine) {
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(slot) : "l"(f.slot_map + s * p.B + tok));      // in the active list (at most B entries), -1 = stable
+    if constexpr (LOG2) qv = ld_raw<C>(q + row * D + lane * C);
+    else ldv<C>(q + row * D + lane * C, qf);
+    ld_state<C>(p.o_p, p.o_p_bf16, row * D + lane * C, a);
+    Lp = p.lse_p[row];
+  }
+  if constexpr (LOG2) grid_dep_wait();
+  if (blockIdx.x == 0)
+    for (int s = threadIdx.x; s < p.N; s += kFinishThreads) f.step[s] += 1;
+  if (!mine) return;
+  float b[C];
+  ldv<C>(f.o_b + row * D + lane * C, b);
   const float Lb = f.lse_b[row];
-  // the cached prefix statistics as well: nine rows in ten are stable, and asking now saves them
-  // a second round trip (an active row overwrites these below)
-  float a[C], Lp;
-  ld_state<C>(p.o_p, p.o_p_bf16, row * D + lane * C, a);
-  Lp = p.lse_p[row];
-  // an active row's records, for the first row group: requested before the slot is known (volatile: a
-  // plain load would sink into the branch and add a round trip)
+  // an active row's records, for the first row group: requested before the slot is looked at (volatile: as above)
   int sg = s * p.Hkv + kh;
   int2 records;
   asm volatile("ld.global.v2.s32 {%0, %1}, [%2];" : "=r"(records.x), "=r"(records.y) : "l"(p.seg_records + sg));
-  const int slot = f.slot_map[s * p.B + tok];                       // in the active list (at most B entries), -1 = stable
   if (slot >= 0 && slot < p.B) {
     const int rowk = slot * p.G + gi, rg = rowk / kRowsPerGroup, r = rowk % kRowsPerGroup;
     if (rg > 0) {
@@ -570,6 +575,7 @@ int32_t launch_sparse_prefix_attn(losa_ctx* c, const void* q, const losa_kv_t* k
   ap.n_sk = sh.batch * sh.n_kv_heads;
   ap.n_ctas = c->lay.n_ctas;
   ap.sm_scale = sh.sm_scale;
+  ap.early = defer_combine ? 1 : 0;
   ap.wait_cycles = c->wait_cycles > 0 ? c->wait_cycles : kWaitCycles;
   return sh.head_dim == 128 ? dispatch_page<128>(c, ap, st, !defer_combine) : dispatch_page<64>(c, ap, st, !defer_combine);
 }

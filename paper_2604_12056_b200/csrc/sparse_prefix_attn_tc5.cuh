@@ -288,15 +288,18 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "n"(TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  // behind the selection of the same step the lengths are final (stage 1 has waited for everything before the step)
+  if (p.early && staged)
+    for (int i = tid; i < p.N; i += NT) len_s[i] = p.kv_len[i];
   grid_dep_trigger();
-  grid_dep_wait();                                 // nothing above touches global memory
+  grid_dep_wait();                                 // nothing above reads what the kernels of this step write
   if (warp == 0) {
     segment_prefix(pre, p.n_seg, p.n_rg, p.Hkv, p.G, p.n_active, [&](int sk) { return p.union_count[sk]; }, p.B, lane, vpre);
   } else if (staged) {
     for (int i = tid - 32; i < p.N * p.B; i += NT - 32) tok_s[i] = p.active_idx[i];
     for (int i = tid - 32; i < p.N; i += NT - 32) {
       na_s[i] = clamp_active(p.n_active[i], p.B);
-      len_s[i] = p.kv_len[i];
+      if (!p.early) len_s[i] = p.kv_len[i];
     }
   }
   tc5_fence_before();
@@ -459,33 +462,30 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       }
       return true;
     };
-    const Item a0 = stage_a(lo + lane);
-    Item a = stage_a(lo + lane + 32);                 // requested beside the first batch: the first copies wait for two loads, not three
-    Ready b = stage_b(lo + lane, a0);
-    if constexpr (FP8) {                              // one stage deeper: the scales of a batch are requested a batch ahead
-      stage_c(lo + lane, b);
-      Ready b1 = stage_b(lo + lane + 32, a);
-      a = stage_a(lo + lane + 64);
-      bool go = true;
-      for (int b0 = lo; b0 < hi && go; b0 += 32) {
-        const Item a_next = stage_a(b0 + lane + 96);
-        const Ready b2 = stage_b(b0 + lane + 64, a);
-        stage_c(b0 + lane + 32, b1);
-        go = issue(b0, b);
-        a = a_next;
+    // One batch of items per trip, every stage of another one: a list entry is requested two (FP8: three) trips before
+    // its page is copied.  The pipeline fills and drains inside the loop, so that its code is there, and fetched, once.
+    constexpr int DEEP = FP8 ? 32 : 0;                // FP8: the scales of a batch are requested a batch ahead
+    Item a{};
+    Ready b{}, b1{};
+    bool go = true;
+#pragma unroll 1
+    for (int b0 = lo - 64 - DEEP; b0 < hi && go; b0 += 32) {
+      const Item a_next = stage_a(b0 + lane + 64 + DEEP);
+      Ready b_next{};
+      if (b0 >= lo - 32 - DEEP) b_next = stage_b(b0 + lane + 32 + DEEP, a);
+      if constexpr (FP8) {
+        if (b0 >= lo - 32) stage_c(b0 + lane + 32, b1);
+        if (b0 >= lo) go = issue(b0, b);
         b = b1;
-        b1 = b2;
-      }
-    } else {
-      bool go = true;
-      for (int b0 = lo; b0 < hi && go; b0 += 32) {
-        const Item a_next = stage_a(b0 + lane + 64);
-        const Ready b_next = stage_b(b0 + lane + 32, a);
-        stage_c(b0 + lane, b);
-        go = issue(b0, b);
-        a = a_next;
+        b1 = b_next;
+      } else {
+        if (b0 >= lo) {
+          stage_c(b0 + lane, b);
+          go = issue(b0, b);
+        }
         b = b_next;
       }
+      a = a_next;
     }
   } else if (FP8 && warp >= kTc5CvtWarp) {
     // ------------------------------------------------------------------ converting warps (FP8 pages): V
