@@ -605,12 +605,33 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
       __syncthreads();
     }
     // ---- candidates: pages whose upper bound reaches tau
-    for_each_page([&](uint32_t, uint32_t ub, int pg) {
-      if (ub >= tau) {
-        const int i = atomicAdd(&s_ncand, 1);
-        if (i < kSelCap) cpage[i] = pg;
+    // (one ticket per warp for all of its pages: a ticket per page is a chain of eight shared-memory round trips, which
+    // five CTAs per SM share; eight 32K prompts 4,200 cycles, 1,200 now)
+    if (cached) {
+      uint32_t hit[kSelPerThread];
+      int total = 0;
+#pragma unroll
+      for (int i = 0; i < kSelPerThread; ++i) {
+        hit[i] = __ballot_sync(0xffffffffu, tid + kSelThreads * i < P && ubc[i] >= tau);
+        total += __popc(hit[i]);
       }
-    });
+      int at = 0;
+      if (lane == 0 && total > 0) at = atomicAdd(&s_ncand, total);
+      at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+      for (int i = 0; i < kSelPerThread; ++i) {
+        const int mine = at + __popc(hit[i] & ((1u << lane) - 1u));
+        if (((hit[i] >> lane) & 1u) && mine < kSelCap) cpage[mine] = tid + kSelThreads * i;
+        at += __popc(hit[i]);
+      }
+    } else {
+      for_each_page([&](uint32_t, uint32_t ub, int pg) {
+        if (ub >= tau) {
+          const int i = atomicAdd(&s_ncand, 1);
+          if (i < kSelCap) cpage[i] = pg;
+        }
+      });
+    }
     __syncthreads();
     const int ncand = s_ncand;
     auto phys_of = [&](int pg) {
