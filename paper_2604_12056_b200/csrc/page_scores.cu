@@ -841,10 +841,11 @@ int32_t launch_stream(losa_ctx* c, const PsParams& pp, cudaStream_t st) {
                                           128 + ns * C::STAGE_BYTES + C::QBUF_BYTES + tail));
     c->scores_attr_set = 1;
   }
-  // no more stages than a CTA can have tiles (short prefixes): a CTA that asks for less room starts beside stage 1's
+  // Behind stage 1 of the same step, no more stages than a CTA can have tiles (short prefixes): a CTA that asks for less
+  // room starts beside stage 1's.  As a call of its own it has the whole ring: there is nothing that it could start beside.
   const losa_shape_t& sh = c->shape;
   const long long pages = (static_cast<long long>(sh.batch) * sh.n_kv_heads * sh.max_pages_per_seq + p.n_ctas - 1) / p.n_ctas;
-  if (pages + C::TP < static_cast<long long>(ns) * C::TP) ns = std::max<int>(2, static_cast<int>(pages / C::TP) + 1);
+  if (p.early && pages + C::TP < static_cast<long long>(ns) * C::TP) ns = std::max<int>(2, static_cast<int>(pages / C::TP) + 1);
   p.n_stages = ns;
   const int smem = 128 + ns * C::STAGE_BYTES + C::QBUF_BYTES + tail;
   launch_k(page_scores_stream_kernel<T, D, PG>, p.n_ctas, kPsThreads, smem, st, p);

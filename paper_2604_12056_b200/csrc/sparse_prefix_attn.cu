@@ -9,7 +9,7 @@
 // (o_p, L_p) of the ACTIVE tokens only, which is what keeps the reuse rule exact for the others.
 //
 // bf16 kernel (sparse_prefix_attn_tc5.cuh): TMA streams the pages of K and V into rings of shared
-//   memory; Q K^T and P V run on the tcgen05 tensor cores with Q, S, P and O in tensor memory; the
+//   memory; Q K^T and P V run on the tcgen05 tensor cores with S, P and O in tensor memory; the
 //   softmax warps own one query row per thread.  Query rows are the GQA-grouped (active token,
 //   head) pairs of the KV head, up to 128 per row group.
 // fp32 kernel: CUDA cores, fp32 FMA (bf16 tensor cores cannot meet the 1e-5 fp32 tolerance).
