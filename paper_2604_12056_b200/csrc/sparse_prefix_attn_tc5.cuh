@@ -33,7 +33,8 @@ static_assert(kTc5SoftmaxWarps * kTc5SoftmaxRegs + 4 * kTc5OtherRegs <= 16 * kTc
 static_assert(kTc5SoftmaxWarps * kTc5SoftmaxRegs8 + 8 * kTc5OtherRegs8 <= 20 * kTc5LaunchRegs8, "registers, FP8");
 constexpr int kTc5Tok = 128;                     // tokens per group = N of Q K^T = columns of one S buffer
 constexpr float kTc5Tau = 8.0f;                  // reference maximum moves only when it would grow by more than this (log2 units)
-constexpr int kTc5XchgBytes = 3 * kTc5Sets * kRowsPerGroup * 4;   // reference maxima, row sums and the references of these, each [set][row]
+// Reference maxima [set][row]; row sums and the references they are relative to [piece parity][set][row]
+constexpr int kTc5XchgBytes = 5 * kTc5Sets * kRowsPerGroup * 4;
 // FP8 pages: binary places by which P is held above the reference maximum.  P stays below 2^(8 + 7) < 65504.
 constexpr float kTc5Fp8Lift = 7.0f;
 constexpr int kTc5StgMax = 20;                   // FP8 pages: staging slots of V, one page each, at most
@@ -238,9 +239,9 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   int* na_s = tok_s + kStageIdx;
   int* len_s = na_s + kStageSeq;
   float* mref = reinterpret_cast<float*>(len_s + kStageSeq);   // [set][128]
-  float* xsum = mref + SB * kRowsPerGroup;                       // [set][128]: row sums of a piece ...
-  float* xref = xsum + SB * kRowsPerGroup;                       // ... and the references they are relative to
-  int* vpre = reinterpret_cast<int*>(xref + SB * kRowsPerGroup);  // prefix of the charged segment lengths (pages + pad)
+  float* xsum = mref + SB * kRowsPerGroup;                       // [piece parity][set][128]: row sums of a piece ...
+  float* xref = xsum + 2 * SB * kRowsPerGroup;                   // ... and the references they are relative to
+  int* vpre = reinterpret_cast<int*>(xref + 2 * SB * kRowsPerGroup);  // prefix of the charged segment lengths (pages + pad)
   // FP8: a staging slot's page has landed / has been converted
   const uint32_t vstg_full = smem_u32(vpre + kMaxSegments + 1) + 4;   // (kMaxSegments + 1 is odd)
   const uint32_t vstg_free = vstg_full + 8 * kTc5StgMax;
@@ -653,7 +654,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     auto warp_wait = [&](uint32_t bar, uint32_t parity) {
       return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, p.status, p.wait_cycles)) != 0;
     };
-    int sg = sg0, item = lo, piece = 0, g = 0, n_meet = 0;
+    int sg = sg0, item = lo, piece = 0, g = 0;
     int n_pub = 0;                                              // references the previous set's warp of this quarter has published, or will have
     bool ok = true;
     while (item < hi && ok) {
@@ -891,18 +892,27 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       }
       if (!ok) break;
       // ---- the piece's record: one 16-row tile record per 16 rows, reference maximum in base-2
-      //      units; the sets share the columns, set 0 writes the row's maximum and sum
-      ok = warp_wait(s_free + 8 * ((g - 1) % kTc5Sets), ((g - 1) / kTc5Sets) & 1);
+      //      units; the sets share the columns, set 0 writes the row's maximum and sum.
+      // O is complete when the P V of the piece's last group has run.  Only the set that handled that group may wait for it on the
+      // group's S buffer: for the others the buffer's barrier can still be a phase behind, with the parity waited for.  The meeting
+      // of a quarter's three warps, rows or not, hands the set's knowledge on, and keeps every warp from running ahead: without
+      // it one could arrive on o_free for two pieces while another still reads O.  The next piece's sums go to the other buffer: they
+      // can be written while set 0 reads these, those of the piece after it only behind its meeting, which waits for o_free.
+      if ((g - 1) % kTc5Sets == h) {
+        ok = warp_wait(s_free + 8 * h, ((g - 1) / kTc5Sets) & 1);
+        if (!ok) break;
+        tc5_fence_after();
+      }
+      const int sums = (piece & 1) * SB * kRowsPerGroup;
+      xsum[sums + h * kRowsPerGroup + r] = l;
+      xref[sums + h * kRowsPerGroup + r] = m_ref;
+      tc5_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(xbar + 8 * quarter, 1);
+      ok = warp_wait(xbar + 8 * quarter, piece & 1);
       if (!ok) break;
       tc5_fence_after();
       if (warp_has_rows) {
-        xsum[h * kRowsPerGroup + r] = l;
-        xref[h * kRowsPerGroup + r] = m_ref;
-        __syncwarp();
-        if (lane == 0) mbar_arrive(xbar + 8 * quarter, 1);      // the quarter's warps meet
-        ok = warp_wait(xbar + 8 * quarter, n_meet & 1);
-        ++n_meet;
-        if (!ok) break;
         float* rec = record_base(p.partials, blockIdx.x + sg, r / kTileRows, D);
         const int rr = r % kTileRows;
 #pragma unroll 1
@@ -920,8 +930,8 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
           float total = 0.f;
 #pragma unroll
           for (int x = 0; x < kTc5Sets; ++x) {
-            const float m_x = xref[x * kRowsPerGroup + r];
-            if (m_x != -INFINITY) total = fmaf(xsum[x * kRowsPerGroup + r], ex2(m_x - m_last), total);
+            const float m_x = xref[sums + x * kRowsPerGroup + r];
+            if (m_x != -INFINITY) total = fmaf(xsum[sums + x * kRowsPerGroup + r], ex2(m_x - m_last), total);
           }
           rec[rr] = m_last;
           rec[kTileRows + rr] = total;

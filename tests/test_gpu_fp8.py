@@ -367,6 +367,60 @@ def test_reference_maximum_that_passes_between_groups_and_segments(g, d, fp8):
                 assert (layer.lse_p[s, :, heads].double() - torch.logsumexp(sc, -1)).abs().max() <= 1e-4
 
 
+@pytest.mark.parametrize("fp8", [False, True])
+@pytest.mark.parametrize("g,d", [(16, 128), (32, 64), (64, 128)])
+def test_shares_of_several_short_pieces_with_and_without_rows(g, d, fp8):
+    """Some four pieces per CTA of 1 to 7 groups of 128 tokens, 8 to 128 query rows each, in an order in which most softmax
+    warps have rows in one piece and none in the next: a piece's output must be read before the next one's first product,
+    by warps that handled the last group and by those that did not.  Against float64, and the same bits every time."""
+    import torch
+    from paper_2604_12056_b200 import binding as B
+    from paper_2604_12056_b200.layer import LosaLayer
+    N, Hkv, G, Bk = 64, 8, 8, 16
+    n_tok = 7 * 128 - 3
+    cfg = wl.config("c2", n_q_heads=Hkv * G, n_kv_heads=Hkv, head_dim=d, page_size=g, kv_lens=(n_tok,) * N, block_size=Bk, steps=1,
+                    topk=1, m_active=1)
+    mp, n_pages = cfg.max_pages_per_seq, 7 * 128 // g
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(3 * g + d)
+    rnd = lambda *shape: torch.randn(*shape, generator=gen, device="cuda").bfloat16()
+    table = torch.arange(N * mp, dtype=torch.int32, device="cuda").view(N, mp)
+    layer = LosaLayer(cfg, rnd(N * mp, Hkv, g, d), rnd(N * mp, Hkv, g, d), table, torch.full((N,), n_tok, dtype=torch.int32, device="cuda"), fp8_kv=fp8)
+    q = rnd(N, Bk, Hkv * G, d)
+    layer.n_active.copy_(torch.tensor([16, 1, 5, 9, 13, 2, 12, 4], dtype=torch.int32).repeat(N // 8))
+    layer.active_idx.fill_(-1)
+    layer.union_pages.fill_(-1)
+    for s in range(N):
+        na = int(layer.n_active[s])
+        layer.active_idx[s, :na] = torch.arange(Bk - na, Bk, dtype=torch.int32)
+        for h in range(Hkv):
+            n = min(n_pages, int(torch.randint(1, 8, (1,), generator=gen, device="cuda")) * (128 // g) - (s + h) % 3 * (g < 64))
+            layer.union_pages[s, h, :n] = torch.randperm(n_pages, generator=gen, device="cuda")[:n].sort().values.int()
+            layer.union_count[s, h] = n
+    first = None
+    for _ in range(10):
+        layer.o_p.zero_()
+        B.losa_sparse_prefix_attn(layer.ctx, q, layer.kv, layer.active_idx, layer.n_active, layer.union_pages, layer.union_count, layer.state)
+        assert layer.ctx.poll_status() == 0
+        first = (layer.o_p.clone(), layer.lse_p.clone()) if first is None else first
+        assert torch.equal(layer.o_p, first[0]) and torch.equal(layer.lse_p, first[1])
+    for s in range(N):
+        if fp8:
+            assert_rows_exact_to_p(layer, cfg, q, s, "fp8")
+            continue
+        act = layer.active_idx[s, :int(layer.n_active[s])].long()
+        for h in range(Hkv):
+            pages = layer.union_pages[s, h, :int(layer.union_count[s, h])].long()
+            valid = (pages[:, None] * g + torch.arange(g, device="cuda")) < n_tok
+            k, v = (t[table[s, pages].long(), h][valid].double() for t in (layer.k_pages, layer.v_pages))
+            for i in range(h * G, (h + 1) * G):
+                sc = q[s, act, i].double() @ k.T * cfg.sm_scale
+                p = torch.softmax(sc, -1)
+                # P is rounded to 8 significant bits: half a unit of 2^-8 of every weight, as much again for the rest
+                assert ((layer.o_p[s, act, i].double() - p @ v).abs() <= 2.0 ** -8 * (p @ v.abs())).all(), (s, i)
+                assert (layer.lse_p[s, act, i].double() - torch.logsumexp(sc, -1)).abs().max() <= 1e-4
+
+
 @pytest.mark.parametrize("g,d", [(16, 64), (32, 64), (16, 128), (64, 128)])
 @pytest.mark.parametrize("power", [-100, -20, 0, 10])
 def test_fp8_queries_of_any_magnitude(g, d, power):
