@@ -330,13 +330,15 @@ int32_t losa_update_prefix_cache(losa_ctx* ctx, losa_kv_t* kv, losa_state_t* sta
  * tensor:  amax = largest |x| over the page's valid tokens;  scale = 2^e with e the smallest integer
  * such that amax <= 448 * 2^e, clamped to [-6, 7];  code = round-to-nearest-even of x / scale,
  * saturated at +-448;  the value every stage works with is scale * value(code) (exact in bf16 and
- * fp16).  Slots of a page past the prefix's end hold code 0.  Stage 4 streams half the bytes and takes
- * fp16 operands with fp32 accumulation: the keys' codes, with the key scale on the scores, and the values'
- * codes, with the value scale partly on the codes (exact) and partly on the softmax weights before
- * they are rounded to fp16.  A weight keeps 11 significant bits down to 2^-14 of its row's largest whatever
- * the scales of the row's other pages, and an absolute 2^-25 of it below that; results are held to
- * the bf16 tolerances against the definition evaluated on the dequantised cache.  Stages 2, 3, 5 are unchanged (the summaries are those of the dequantised
- * keys); block finalisation re-quantises every touched page from its dequantised old rows and the
+ * fp16).  Slots of a page past the prefix's end hold code 0.  Stage 4 streams half the bytes; both its products
+ * accumulate in fp32.  The scores come from the keys' codes as they are and the query as a sum of three E5M2
+ * terms under a power of two of its row, with the key scale on the score: an element of the query counts with all
+ * its bits down to 2^-24 of its row's largest, a smaller one to within 2^-32 of that largest.  The second product takes
+ * fp16 operands: the values' codes, with the value scale partly on the codes (exact) and partly on the softmax
+ * weights before they are rounded to fp16.  A weight keeps 11 significant bits down to 2^-14 of its row's
+ * largest whatever the scales of the row's other pages, and an absolute 2^-25 of it below that; results are held to
+ * the bf16 tolerances against the definition evaluated on the dequantised cache.  Stages 2, 3, 5 are unchanged
+ * (the summaries are those of the dequantised keys); block finalisation re-quantises every touched page from its dequantised old rows and the
  * new rows together.  Inputs must satisfy |x| <= 448 * 2^7 (larger magnitudes saturate).
  *
  * losa_quantize_kv_pages: src is a native bf16 cache, dst an FP8 cache with the same page_table,

@@ -54,26 +54,27 @@ template <int GP> constexpr int tc5_tail_bytes() {
   return kTailBytes + kTc5XchgBytes + (kMaxSegments + 2) * 4 + kTc5StgMax * (8 + 8) + kTc5VmulRing * 4 + kTc5MetaRing * (kTc5Tok / GP) * 8;
 }
 
-// Shared memory: the Q tile (FP8: two tiles of codes), a ring of group-sized slots for K and one for V, FP8: a
+// Shared memory: the Q tile (FP8: one tile of codes per term), a ring of group-sized slots for K and one for V, FP8: a
 // ring of page-sized slots where the codes of V land.
 template <int D> constexpr int tc5_slot_bytes() { return kTc5Tok * D * 2; }                              // V, and bf16 K
 template <int D, bool FP8> constexpr int tc5_kslot_bytes() { return kTc5Tok * D * (FP8 ? 1 : 2); }
-template <int D> constexpr int tc5_q_bytes() { return kRowsPerGroup * D * 2; }
+constexpr int kTc5QTerms = 3;                    // FP8: E5M2 terms of a query
+template <int D, bool FP8> constexpr int tc5_q_bytes() { return kRowsPerGroup * D * (FP8 ? kTc5QTerms : 2); }
 template <int D, int GP, bool FP8> constexpr int tc5_ring_slots(bool v) {
-  if (FP8) return v ? 2 : (D == 128 ? 4 : 6);                   // the staging slots take the rest
-  const int n = (kSmemBudget - 1024 - tc5_tail_bytes<GP>() - tc5_q_bytes<D>()) / tc5_slot_bytes<D>();
+  if (FP8) return v ? 2 : (D == 128 ? 3 : 6);                   // the staging slots take the rest
+  const int n = (kSmemBudget - 1024 - tc5_tail_bytes<GP>() - tc5_q_bytes<D, false>()) / tc5_slot_bytes<D>();
   const int own = v ? n / 2 : (n + 1) / 2;                      // K is ahead of V by the S buffers
   return own > 6 ? 6 : own;
 }
 // FP8: pages of the staging ring of V: what the ring slots leave, up to five groups
 template <int D, int GP> constexpr int tc5_stg_slots() {
-  const int fit = (kSmemBudget - 1024 - tc5_tail_bytes<GP>() - tc5_q_bytes<D>() - tc5_ring_slots<D, GP, true>(false) * tc5_kslot_bytes<D, true>() -
+  const int fit = (kSmemBudget - 1024 - tc5_tail_bytes<GP>() - tc5_q_bytes<D, true>() - tc5_ring_slots<D, GP, true>(false) * tc5_kslot_bytes<D, true>() -
                    tc5_ring_slots<D, GP, true>(true) * tc5_slot_bytes<D>()) / (GP * D), five = 5 * (kTc5Tok / GP);
   const int n = fit < five ? fit : five;
   return n < kTc5StgMax ? n : kTc5StgMax;
 }
 template <int D, int GP, bool FP8> constexpr int tc5_smem_bytes() {
-  return 1024 + tc5_q_bytes<D>() + tc5_ring_slots<D, GP, FP8>(false) * tc5_kslot_bytes<D, FP8>() + tc5_ring_slots<D, GP, FP8>(true) * tc5_slot_bytes<D>() +
+  return 1024 + tc5_q_bytes<D, FP8>() + tc5_ring_slots<D, GP, FP8>(false) * tc5_kslot_bytes<D, FP8>() + tc5_ring_slots<D, GP, FP8>(true) * tc5_slot_bytes<D>() +
          (FP8 ? tc5_stg_slots<D, GP>() * GP * D : 0) + tc5_tail_bytes<GP>();
 }
 
@@ -83,7 +84,7 @@ __device__ __forceinline__ uint64_t tc5_desc(uint32_t saddr, uint32_t lbo) {
   return static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4) | (static_cast<uint64_t>((lbo >> 4) & 0x3FFFu) << 16) |
          (static_cast<uint64_t>(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
 }
-// K-major tile of E4M3 codes, rows of D bytes: the 128-byte swizzle for D = 128, the 64-byte one (8-row groups 512
+// K-major tile of 8-bit codes, rows of D bytes: the 128-byte swizzle for D = 128, the 64-byte one (8-row groups 512
 // bytes apart) for D = 64.
 template <int D> __device__ __forceinline__ uint64_t tc5_desc8(uint32_t saddr) {
   return static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4) | (1ull << 16) | (static_cast<uint64_t>((8 * D) >> 4) << 32) | (1ull << 46) |
@@ -94,9 +95,9 @@ template <int D> __device__ __forceinline__ uint32_t tc5_sw8(int t, int c) {
   return static_cast<uint32_t>(t * D + ((D == 128 ? c ^ (t & 7) : c ^ ((t >> 1) & 3)) << 4));
 }
 // Instruction descriptor: fp32 accumulate, M x N tile, B optionally MN-major; kind::f16: A and B both bf16
-// (fmt 1) or both fp16 (fmt 0); kind::f8f6f4: both E4M3 (fmt 0).
-__device__ __forceinline__ uint32_t tc5_idesc(int M, int N, int b_mn_major, uint32_t fmt = 1u) {
-  return (1u << 4) | (fmt << 7) | (fmt << 10) | (static_cast<uint32_t>(b_mn_major) << 16) |
+// (format 1) or both fp16 (0); kind::f8f6f4: each E4M3 (0) or E5M2 (1).
+__device__ __forceinline__ uint32_t tc5_idesc(int M, int N, int b_mn_major, uint32_t fmt_a, uint32_t fmt_b) {
+  return (1u << 4) | (fmt_a << 7) | (fmt_b << 10) | (static_cast<uint32_t>(b_mn_major) << 16) |
          (static_cast<uint32_t>(N >> 3) << 17) | (static_cast<uint32_t>(M >> 4) << 24);
 }
 // D[tmem] (+)= A[tmem] . B[smem descriptor]
@@ -106,7 +107,7 @@ __device__ __forceinline__ void tc5_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uin
       "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
       ::"r"(d_tmem), "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
 }
-// D[tmem] (+)= A[smem descriptor] . B[smem descriptor], bf16 operands, or E4M3
+// D[tmem] (+)= A[smem descriptor] . B[smem descriptor], bf16 operands, or 8-bit ones
 __device__ __forceinline__ void tc5_mma_ss(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
@@ -181,9 +182,12 @@ __device__ __forceinline__ void tc5_wait_st() { asm volatile("tcgen05.wait::st.s
 __device__ __forceinline__ uint32_t tc5_sw(int t, int c) { return static_cast<uint32_t>(t * 128 + ((c ^ (t & 7)) << 4)); }
 
 // FP8: the K / V pools hold E4M3 bytes with one power-of-two scale per (page, KV head).  K is an operand as
-// it lies: Q goes to shared memory as two E4M3 tiles whose sum is the bf16 query (four significant bits each),
-// and both are multiplied with the codes by kind::f8f6f4, at twice the 16-bit rate and with fp32 sums of the
-// same accuracy (against float64 on random codes: 1.0e-7, bf16 1.6e-7).  V cannot: P needs more than two terms.
+// it lies: Q goes to shared memory as three E5M2 tiles whose sum is the bf16 query under a power of two of the row, and each is
+// multiplied with the codes by kind::f8f6f4, at twice the 16-bit rate and with fp32 sums.  A term takes three significant bits and
+// leaves at most half a unit of them, so three terms hold the eight of a bf16 value; with the row's largest element at
+// 2^15 .. 2^16 that is exact down to 2^-9, 2^-24 of the largest, and below to within 2^-17, 2^-32 of it - more than the fp16
+// value of an element keeps in a row below 256.  (Two E4M3 terms lose an element's low bits from 2^-9 of the row's largest
+// on: with them the block of eight 32K prompts takes 954 us, 976 with three, of which K's ring gives one slot to the third.)  V cannot: P needs more than three terms.
 // Its codes land in a staging ring as they lie in memory; four converting warps, one per scheduler, turn a
 // landed page into fp16 (exact) in the group's ring slot, in the layout the tensor maps of the bf16 path
 // produce, and P is fp16.  The scales stay out of the conversion, which is bound by its instruction count: the
@@ -202,7 +206,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   constexpr int NRK = tc5_ring_slots<D, GP, FP8>(false), NRV = tc5_ring_slots<D, GP, FP8>(true);   // slots per ring
   constexpr int NSP = FP8 ? tc5_stg_slots<D, GP>() : 1, STG = GP * D;   // FP8: staging slots of V, bytes of a slot (one page of codes)
   constexpr int NT = tc5_threads<FP8>();
-  constexpr int KSLOT = tc5_kslot_bytes<D, FP8>(), SLOT = tc5_slot_bytes<D>(), QB = tc5_q_bytes<D>();
+  constexpr int KSLOT = tc5_kslot_bytes<D, FP8>(), SLOT = tc5_slot_bytes<D>(), QB = tc5_q_bytes<D, FP8>();
   constexpr int PG = kTc5Tok / GP;              // pages per group
   constexpr int MR = kTc5MetaRing;              // groups of the meta ring
   constexpr int HALVES = D / 64;                // 64-column (128-byte) blocks of a 16-bit K or V row
@@ -581,15 +585,15 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
           if (!ok) break;
           tc5_fence_after();
           const uint32_t kt = kring + slot * KSLOT, s_col = tmem + COL_S + b * kTc5Tok;
-          if constexpr (FP8) {                       // both terms of Q against the same codes
-            const uint32_t idesc = tc5_idesc(kRowsPerGroup, ng * GP, 0, 0u);
+          if constexpr (FP8) {                       // the terms of Q (E5M2) against the same codes (E4M3)
+            const uint32_t idesc = tc5_idesc(kRowsPerGroup, ng * GP, 0, 1u, 0u);
 #pragma unroll
             for (int ks = 0; ks < D / 32; ++ks)
 #pragma unroll
-              for (int t = 0; t < 2; ++t)
-                tc5_mma_ss8(s_col, tc5_desc8<D>(qtile + t * (QB / 2) + ks * 32), tc5_desc8<D>(kt + ks * 32), idesc, ks + t > 0 ? 1u : 0u);
+              for (int t = 0; t < kTc5QTerms; ++t)
+                tc5_mma_ss8(s_col, tc5_desc8<D>(qtile + t * (QB / kTc5QTerms) + ks * 32), tc5_desc8<D>(kt + ks * 32), idesc, ks + t > 0 ? 1u : 0u);
           } else {
-            const uint32_t idesc = tc5_idesc(kRowsPerGroup, ng * GP, 0);
+            const uint32_t idesc = tc5_idesc(kRowsPerGroup, ng * GP, 0, 1u, 1u);
 #pragma unroll
             for (int ks = 0; ks < D / 16; ++ks) {
               const uint32_t at = (ks >> 2) * HS + (ks & 3) * 32;
@@ -609,7 +613,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   } else if (warp == kTc5PvWarp) {
     // ------------------------------------------------------------------ P V issuer (one thread)
     if (lane == 0) {
-      const uint32_t idesc = tc5_idesc(kRowsPerGroup, D, 1, FP8 ? 0u : 1u);
+      const uint32_t idesc = tc5_idesc(kRowsPerGroup, D, 1, FP8 ? 0u : 1u, FP8 ? 0u : 1u);
       int sg = sg0, item = lo, piece = 0, g = 0;
       bool ok = true;
       while (item < hi && ok) {
@@ -677,9 +681,8 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
 #pragma unroll
         for (int c = 0; c < NC; ++c) qv[c] = src && h < 2 ? __ldg(src + h * NC + c) : make_uint4(0u, 0u, 0u, 0u);
         if constexpr (FP8) {
-          // Q in two E4M3 terms.  The row is scaled by the power of two that brings its largest element to
-          // 2^7 .. 2^8; the first term takes four significant bits of an element and the second the other
-          // four, exactly down to 2^-9 of the largest element; below that the error is at most 2^-18 of it.
+          // Q in three E5M2 terms, under the power of two that brings the row's largest element to 2^15 .. 2^16 (what of it
+          // lies above 57344, the largest E5M2 value, is left to the second term).
           uint32_t top = 0;                                     // of the whole row
           if (src) {
 #pragma unroll 4
@@ -690,8 +693,8 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
               for (int e = 0; e < 4; ++e) top = max(top, max((w[e] << 16) & 0x7fffffffu, w[e] & 0x7fff0000u));
             }
           }
-          // (exponent field e of the largest element: times 2^(134 - e) in two steps, each a normal number)
-          const int e_top = max(static_cast<int>(top >> 23), 16), up = 134 - e_top, u0 = up / 2, u1 = up - u0;
+          // (exponent field e of the largest element: times 2^(142 - e) in two steps, each a normal number)
+          const int e_top = max(static_cast<int>(top >> 23), 16), up = 142 - e_top, u0 = up / 2, u1 = up - u0;
           const float f0 = __int_as_float((127 + u0) << 23), f1 = __int_as_float((127 + u1) << 23);
           scale2 *= __int_as_float((127 - u0) << 23) * __int_as_float((127 - u1) << 23);
           if ((top >> 23) == 255) scale2 = __int_as_float(top);           // an infinity or NaN among them: in all the row's scores
@@ -700,27 +703,28 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
           if (warp_has_rows && h < 2) {
 #pragma unroll
             for (int c = 0; c < NC; c += 2) {                   // two chunks of bf16 make one of codes
-              uint32_t hi4[4], lo4[4];
+              uint32_t w4[kTc5QTerms][4];
 #pragma unroll
               for (int x = 0; x < 2; ++x) {
                 const uint32_t w[4] = {qv[c + x].x, qv[c + x].y, qv[c + x].z, qv[c + x].w};
-                uint16_t a[4], b[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                  const float v0 = __uint_as_float(w[e] << 16) * f0 * f1, v1 = __uint_as_float(w[e] & 0xffff0000u) * f0 * f1;
-                  a[e] = __nv_cvt_float2_to_fp8x2(make_float2(v0, v1), __NV_SATFINITE, __NV_E4M3);
-                  const __half2_raw back = __nv_cvt_fp8x2_to_halfraw2(a[e], __NV_E4M3);
-                  const float2 bf = __half22float2(__half2(back));
-                  b[e] = __nv_cvt_float2_to_fp8x2(make_float2(v0 - bf.x, v1 - bf.y), __NV_SATFINITE, __NV_E4M3);
+                  float2 v = make_float2(__uint_as_float(w[e] << 16) * f0 * f1, __uint_as_float(w[e] & 0xffff0000u) * f0 * f1);
+#pragma unroll
+                  for (int t = 0; t < kTc5QTerms; ++t) {
+                    const uint32_t code = __nv_cvt_float2_to_fp8x2(v, __NV_SATFINITE, __NV_E5M2);
+                    const float2 part = __half22float2(__half2(__nv_cvt_fp8x2_to_halfraw2(code, __NV_E5M2)));
+                    v.x -= part.x;
+                    v.y -= part.y;
+                    if (e % 2 == 0) w4[t][2 * x + e / 2] = code;
+                    else w4[t][2 * x + e / 2] |= code << 16;
+                  }
                 }
-                hi4[2 * x] = a[0] | static_cast<uint32_t>(a[1]) << 16;
-                hi4[2 * x + 1] = a[2] | static_cast<uint32_t>(a[3]) << 16;
-                lo4[2 * x] = b[0] | static_cast<uint32_t>(b[1]) << 16;
-                lo4[2 * x + 1] = b[2] | static_cast<uint32_t>(b[3]) << 16;
               }
               uint8_t* dst = gen + tc5_sw8<D>(r, h * (NC / 2) + c / 2);
-              *reinterpret_cast<uint4*>(dst) = make_uint4(hi4[0], hi4[1], hi4[2], hi4[3]);
-              *reinterpret_cast<uint4*>(dst + QB / 2) = make_uint4(lo4[0], lo4[1], lo4[2], lo4[3]);
+#pragma unroll
+              for (int t = 0; t < kTc5QTerms; ++t)
+                *reinterpret_cast<uint4*>(dst + t * (QB / kTc5QTerms)) = make_uint4(w4[t][0], w4[t][1], w4[t][2], w4[t][3]);
             }
           }
         } else {

@@ -424,7 +424,7 @@ def test_shares_of_several_short_pieces_with_and_without_rows(g, d, fp8):
 @pytest.mark.parametrize("g,d", [(16, 64), (32, 64), (16, 128), (64, 128)])
 @pytest.mark.parametrize("power", [-100, -20, 0, 10])
 def test_fp8_queries_of_any_magnitude(g, d, power):
-    """The queries enter the first product as two E4M3 terms under a scale of the row: rows of every magnitude, elements
+    """The queries enter the first product as three E5M2 terms under a scale of the row: rows of every magnitude, elements
     2^-20 .. 1 of a row's largest, a row of zeros, a row of one element; against float64 on the dequantised keys."""
     import torch
     from paper_2604_12056_b200.layer import LosaLayer
@@ -451,10 +451,47 @@ def test_fp8_queries_of_any_magnitude(g, d, power):
         for i in range(h * G, (h + 1) * G):
             qd = q[0, :, i].double()
             sc = qd @ k.T * cfg.sm_scale
-            # an element is exact down to 2^-9 of its row's largest, else off by at most 2^-18 of that (2^-17 here);
-            # fp32 sums: 2^-21 of the sum of magnitudes
-            off = cfg.sm_scale * (2.0 ** -17 * (qd.abs().amax(-1, keepdim=True) * (qd.abs() < 2.0 ** -9 * qd.abs().amax(-1, keepdim=True))) @ k.abs().T
-                                  + 2.0 ** -21 * (qd.abs() @ k.abs().T)).amax(-1)
+            # an element is exact down to 2^-24 of its row's largest, which no element here is below: what remains are the
+            # fp32 sums, 2^-21 of the sum of magnitudes
+            off = cfg.sm_scale * 2.0 ** -21 * (qd.abs() @ k.abs().T).amax(-1)
+            lse = torch.logsumexp(sc, -1)
+            assert ((layer.lse_p[0, :, i].double() - lse).abs() <= off + 1e-5 + 2.0 ** -22 * lse.abs()).all(), (h, i)
+            p = torch.softmax(sc, -1)
+            bound = (2.0 ** -10 + 2 * off[:, None]) * (p @ v.abs()) + 2.0 ** -24 * p.amax(-1, keepdim=True) * v.abs().sum(0)
+            assert ((layer.o_p[0, :, i].double() - p @ v).abs() <= bound).all(), (h, i)
+
+
+@pytest.mark.parametrize("g,d", [(16, 128), (64, 64)])
+@pytest.mark.parametrize("top,below", [(2, 8), (2, 14), (8, 10), (8, 16), (8, 22), (15, 12), (15, 22)])
+def test_fp8_query_elements_far_below_a_large_one_keep_their_bits(g, d, top, below):
+    """One element of 2^top per row meets keys of zero, the others are 2^-below of it and make the scores: all eight bits of
+    them count.  Against float64 on the dequantised keys; no error but that of fp32 sums."""
+    import torch
+    from paper_2604_12056_b200.layer import LosaLayer
+    Hkv, G, Bk, n_tok = 2, 4, 8, 3 * 128 + 5
+    cfg = wl.config("c2", n_q_heads=Hkv * G, n_kv_heads=Hkv, head_dim=d, page_size=g, kv_lens=(n_tok,), block_size=Bk, steps=1, topk=1,
+                    m_active=1)
+    P = cfg.max_pages_per_seq
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(g + d + top + below)
+    rnd = lambda *shape: torch.randn(*shape, generator=gen, device="cuda")
+    kp, vp = rnd(P, Hkv, g, d) * 2.0 ** min(13, max(-4, below - top)), rnd(P, Hkv, g, d)       # (keys as large as FP8 pages hold them)
+    kp[..., 3] = 0.0
+    q = rnd(1, Bk, Hkv * G, d)
+    q = q.sign() * (0.5 + q.abs()).clamp_max(3.9) * 2.0 ** (top - below - 1)             # 2^-24 of the largest or more
+    q[..., 3] = 1.5 * 2.0 ** top
+    q = q.bfloat16()
+    kb, vb = (rnd(1, Bk, Hkv, d).bfloat16() for _ in range(2))
+    table = torch.arange(P, dtype=torch.int32, device="cuda")[None].contiguous()
+    layer = LosaLayer(cfg, kp.bfloat16(), vp.bfloat16(), table, torch.tensor([n_tok], dtype=torch.int32, device="cuda"), fp8_kv=True)
+    layer.run_step(q, kb, vb, torch.ones(1, dtype=torch.int32, device="cuda"))
+    assert layer.ctx.poll_status() == 0
+    for h in range(Hkv):
+        k, v = listed_prefix(layer, cfg, 0, h)
+        for i in range(h * G, (h + 1) * G):
+            qd = q[0, :, i].double()
+            sc = qd @ k.T * cfg.sm_scale
+            off = cfg.sm_scale * 2.0 ** -21 * (qd.abs() @ k.abs().T).amax(-1)       # fp32 sums
             lse = torch.logsumexp(sc, -1)
             assert ((layer.lse_p[0, :, i].double() - lse).abs() <= off + 1e-5 + 2.0 ** -22 * lse.abs()).all(), (h, i)
             p = torch.softmax(sc, -1)
