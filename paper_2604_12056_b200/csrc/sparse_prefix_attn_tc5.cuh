@@ -219,7 +219,9 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   static_assert(D == 64 || D == 128, "head dimensions of the tensor-core path");
   static_assert(GP == 16 || GP == 32 || GP == 64, "page sizes of the tensor-core path");
   static_assert(NRK >= 2 && NRV >= 2 && NRK <= 6 && NRV <= 6, "ring depth");
-  static_assert(!FP8 || (NSP >= PG && NSP <= kTc5StgMax), "staging ring");
+  // A converting warp waits on the parity of a staging slot whose page before, NSP pages back, another warp may have taken: that page
+  // has to lie two groups back at least, where all four warps have finished (less than two groups lie between them).
+  static_assert(!FP8 || (NSP >= 2 * PG && NSP <= kTc5StgMax), "staging ring");
   static_assert(NRK + 2 < MR, "the producer's lead fits the meta ring");
   constexpr int kBars = 4 * 6 + 3 * SB + 3 + 4 + 4 * SB + 2;
   static_assert(8 * kBars + 16 <= 512, "tail layout");
