@@ -302,18 +302,17 @@ __global__ void __launch_bounds__(kFinishThreads) attn_finish_kernel(AttnParams 
   const uint32_t row_i = blockIdx.x * (kFinishThreads / 32) + (threadIdx.x >> 5);
   const size_t row = row_i;
   const bool mine = row < f.n_rows;
-  // Stage 4 of this step runs before: the slots (stage 1), the queries and the cached prefix statistics (the step before)
-  // are final, and requested beside its last CTAs.  Nine rows in ten are stable; an active row overwrites the
-  // statistics below.  (volatile: a plain load would sink below the wait)
+  // The queries and the cached prefix statistics are older than the step, whose stage 1 has waited for all that is: they
+  // are requested beside the kernels before this one.  Nine rows in ten are stable; an active row overwrites the
+  // statistics below.  What the step itself writes, also in stage 1 (the slots), is read behind the wait: the kernels in
+  // between release their dependents before they wait themselves.
   const int hq = static_cast<int>(row_i % p.Hq), st = static_cast<int>(row_i / p.Hq), tok = st % p.B, s = st / p.B;   // (32-bit divisions)
   const int kh = hq / p.G, gi = hq % p.G;
   const T* q = static_cast<const T*>(f.q);
   RawRow<C> qv;                                         // (fp32: qf)
   float qf[C];
   float a[C], Lp = 0.f;
-  int slot = -1;
   if (mine) {
-    asm volatile("ld.global.s32 %0, [%1];" : "=r"(slot) : "l"(f.slot_map + s * p.B + tok));      // in the active list (at most B entries), -1 = stable
     if constexpr (LOG2) qv = ld_raw<C>(q + row * D + lane * C);
     else ldv<C>(q + row * D + lane * C, qf);
     ld_state<C>(p.o_p, p.o_p_bf16, row * D + lane * C, a);
@@ -323,10 +322,13 @@ __global__ void __launch_bounds__(kFinishThreads) attn_finish_kernel(AttnParams 
   if (blockIdx.x == 0)
     for (int s = threadIdx.x; s < p.N; s += kFinishThreads) f.step[s] += 1;
   if (!mine) return;
+  // the slot in the active list (at most B entries), -1 = stable, and an active row's records, for the first row group, are
+  // requested together (volatile: the records would sink below the look at the slot)
+  int slot;
+  asm volatile("ld.global.s32 %0, [%1];" : "=r"(slot) : "l"(f.slot_map + s * p.B + tok));
   float b[C];
   ldv<C>(f.o_b + row * D + lane * C, b);
   const float Lb = f.lse_b[row];
-  // an active row's records, for the first row group: requested before the slot is looked at (volatile: as above)
   int sg = s * p.Hkv + kh;
   int2 records;
   asm volatile("ld.global.v2.s32 {%0, %1}, [%2];" : "=r"(records.x), "=r"(records.y) : "l"(p.seg_records + sg));
