@@ -70,7 +70,8 @@ int32_t launch_sparse_prefix_attn(losa_ctx* c, const void* q, const losa_kv_t* k
                                   losa_state_t* state, cudaStream_t st, bool defer_combine = false, bool from_bits = false);
 // from_bits (whole step, fp32): the lists come from the page bitmaps in the workspace and are written to
 // union_pages / union_count by this kernel.
-// Encodes what stage 4 needs on the host; a failure here leaves nothing launched.
+// All that stage 4 needs on the host, and can be refused for: tensor maps, kernel attributes.  The whole-step call does this
+// before its first launch.
 int32_t prepare_sparse_prefix_attn(losa_ctx* c, const losa_kv_t* kv);
 // Whole-step path: with defer_combine the main kernel leaves its partial records unmerged and
 // launch_attn_finish merges them, merges with the in-block part, writes the output, keeps the

@@ -466,24 +466,51 @@ int32_t ensure_tensor_maps(losa_ctx* c, const losa_kv_t* kv) {
   return LOSA_OK;
 }
 
+// f(head dimension, page size) as compile-time numbers
+template <typename F>
+int32_t with_page_shape(const losa_shape_t& sh, F&& f) {
+  auto page = [&](auto d) {
+    switch (sh.page_size) {
+      case 16: return f(d, std::integral_constant<int, 16>{});
+      case 32: return f(d, std::integral_constant<int, 32>{});
+      default: return f(d, std::integral_constant<int, 64>{});
+    }
+  };
+  return sh.head_dim == 128 ? page(std::integral_constant<int, 128>{}) : page(std::integral_constant<int, 64>{});
+}
+
 template <int D, int GP, bool FP8>
-int32_t launch_tc5(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool with_combine) {
+int32_t prepare_tc5(losa_ctx* c) {
   constexpr int smem = tc5_smem_bytes<D, GP, FP8>();
   static_assert(smem <= kSmemBudget, "shared memory of the stage-4 kernel");
   constexpr int bit = FP8 ? 2 : 1;  // a context has one shape on one device: one instantiation per cache format
-  if (!(c->attn_attr_set & bit)) {
-    LOSA_CUDA_TRY(c, cudaFuncSetAttribute(attn_tc5_kernel<D, GP, FP8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    // the kernel moves registers between its warps: a build that is launched with fewer than it deals out would wait for ever
-    cudaFuncAttributes fa;
-    LOSA_CUDA_TRY(c, cudaFuncGetAttributes(&fa, attn_tc5_kernel<D, GP, FP8>));
-    if (fa.numRegs < (FP8 ? kTc5LaunchRegs8 : kTc5LaunchRegs)) return LOSA_ERR_UNSUPPORTED;
-    c->attn_attr_set |= bit;
-  }
+  if (c->attn_attr_set & bit) return LOSA_OK;
+  LOSA_CUDA_TRY(c, cudaFuncSetAttribute(attn_tc5_kernel<D, GP, FP8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  // the kernel moves registers between its warps: a build that is launched with fewer than it deals out would wait for ever
+  cudaFuncAttributes fa;
+  LOSA_CUDA_TRY(c, cudaFuncGetAttributes(&fa, attn_tc5_kernel<D, GP, FP8>));
+  if (fa.numRegs < (FP8 ? kTc5LaunchRegs8 : kTc5LaunchRegs)) return LOSA_ERR_UNSUPPORTED;
+  c->attn_attr_set |= bit;
+  return LOSA_OK;
+}
+
+template <int D, int GP>
+int32_t prepare_f32(losa_ctx* c) {
+  constexpr int smem = sizeof(F32Smem<D>);
+  static_assert(smem <= kSmemBudget, "shared memory of the fp32 stage-4 kernel");
+  if (c->attn_attr_set & 1) return LOSA_OK;
+  LOSA_CUDA_TRY(c, cudaFuncSetAttribute(attn_f32_kernel<D, GP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  c->attn_attr_set |= 1;
+  return LOSA_OK;
+}
+
+template <int D, int GP, bool FP8>
+int32_t launch_tc5(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool with_combine) {
   CUtensorMap mk, mv;
   memcpy(&mk, c->tmap_k, sizeof(mk));
   memcpy(&mv, c->tmap_v, sizeof(mv));
   if (c->profile) LOSA_CUDA_TRY(c, cudaEventRecord(c->ev_begin, st));
-  launch_k(attn_tc5_kernel<D, GP, FP8>, ap.n_ctas, tc5_threads<FP8>(), smem, st, mk, mv, ap);
+  launch_k(attn_tc5_kernel<D, GP, FP8>, ap.n_ctas, tc5_threads<FP8>(), tc5_smem_bytes<D, GP, FP8>(), st, mk, mv, ap);
   if (c->profile) LOSA_CUDA_TRY(c, cudaEventRecord(c->ev_end, st));
   int32_t rc = after_launch(c);
   if (rc != LOSA_OK || !with_combine) return rc;
@@ -493,14 +520,8 @@ int32_t launch_tc5(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool with
 
 template <int D, int GP>
 int32_t launch_f32(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool with_combine) {
-  constexpr int smem = sizeof(F32Smem<D>);
-  static_assert(smem <= kSmemBudget, "shared memory of the fp32 stage-4 kernel");
-  if (!(c->attn_attr_set & 1)) {
-    LOSA_CUDA_TRY(c, cudaFuncSetAttribute(attn_f32_kernel<D, GP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    c->attn_attr_set |= 1;
-  }
   if (c->profile) LOSA_CUDA_TRY(c, cudaEventRecord(c->ev_begin, st));
-  launch_k(attn_f32_kernel<D, GP>, ap.n_ctas, kF32Threads, smem, st, ap);
+  launch_k(attn_f32_kernel<D, GP>, ap.n_ctas, kF32Threads, sizeof(F32Smem<D>), st, ap);
   if (c->profile) LOSA_CUDA_TRY(c, cudaEventRecord(c->ev_end, st));
   int32_t rc = after_launch(c);
   if (rc != LOSA_OK || !with_combine) return rc;
@@ -508,28 +529,17 @@ int32_t launch_f32(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool with
   return after_launch(c);
 }
 
-template <int D>
-int32_t dispatch_page(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool with_combine) {
-  const bool bf = c->shape.dtype == LOSA_BF16;
-  if (ap.k_scale) {                 // FP8 pages (bf16 contexts only, checked by the C-ABI layer)
-    switch (c->shape.page_size) {
-      case 16: return launch_tc5<D, 16, true>(c, ap, st, with_combine);
-      case 32: return launch_tc5<D, 32, true>(c, ap, st, with_combine);
-      default: return launch_tc5<D, 64, true>(c, ap, st, with_combine);
-    }
-  }
-  switch (c->shape.page_size) {
-    case 16: return bf ? launch_tc5<D, 16, false>(c, ap, st, with_combine) : launch_f32<D, 16>(c, ap, st, with_combine);
-    case 32: return bf ? launch_tc5<D, 32, false>(c, ap, st, with_combine) : launch_f32<D, 32>(c, ap, st, with_combine);
-    default: return bf ? launch_tc5<D, 64, false>(c, ap, st, with_combine) : launch_f32<D, 64>(c, ap, st, with_combine);
-  }
-}
-
 }  // namespace
 
 
 int32_t prepare_sparse_prefix_attn(losa_ctx* c, const losa_kv_t* kv) {
-  return c->shape.dtype == LOSA_BF16 ? ensure_tensor_maps(c, kv) : LOSA_OK;
+  const bool bf = c->shape.dtype == LOSA_BF16, fp8 = kv->kv_format == LOSA_KV_FP8_E4M3;     // (FP8 pages: bf16 contexts only)
+  const int32_t rc = bf ? ensure_tensor_maps(c, kv) : LOSA_OK;
+  if (rc != LOSA_OK) return rc;
+  return with_page_shape(c->shape, [&](auto d, auto gp) {
+    constexpr int D = decltype(d)::value, GP = decltype(gp)::value;
+    return fp8 ? prepare_tc5<D, GP, true>(c) : bf ? prepare_tc5<D, GP, false>(c) : prepare_f32<D, GP>(c);
+  });
 }
 
 int32_t launch_sparse_prefix_attn(losa_ctx* c, const void* q, const losa_kv_t* kv,
@@ -579,7 +589,12 @@ int32_t launch_sparse_prefix_attn(losa_ctx* c, const void* q, const losa_kv_t* k
   ap.sm_scale = sh.sm_scale;
   ap.early = defer_combine ? 1 : 0;
   ap.wait_cycles = c->wait_cycles > 0 ? c->wait_cycles : kWaitCycles;
-  return sh.head_dim == 128 ? dispatch_page<128>(c, ap, st, !defer_combine) : dispatch_page<64>(c, ap, st, !defer_combine);
+  const bool bf = sh.dtype == LOSA_BF16, with_combine = !defer_combine;
+  return with_page_shape(sh, [&](auto d, auto gp) {
+    constexpr int D = decltype(d)::value, GP = decltype(gp)::value;
+    return fp8 ? launch_tc5<D, GP, true>(c, ap, st, with_combine)
+               : bf ? launch_tc5<D, GP, false>(c, ap, st, with_combine) : launch_f32<D, GP>(c, ap, st, with_combine);
+  });
 }
 
 int32_t launch_attn_finish(losa_ctx* c, const void* q, const int32_t* slot_map, losa_state_t* state, void* out,
