@@ -307,8 +307,9 @@ int32_t launch_merge_t(losa_ctx* c, const void* q, const void* k_blk, const void
   const losa_shape_t& sh = c->shape;
   const int G = sh.n_q_heads / sh.n_kv_heads;
   const size_t smem = (static_cast<size_t>(sh.block_size) * (2 * D + 4) + static_cast<size_t>(kTokTile) * G * D) * sizeof(float);
-  if (smem > 48 * 1024)
-    LOSA_CUDA_TRY(c, cudaFuncSetAttribute(block_attn_merge_kernel<T, D, MERGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+  constexpr int most = (LOSA_MAX_BLOCK * (2 * D + 4) + kTokTile * 16 * D) * static_cast<int>(sizeof(float));   // (16 heads per KV head)
+  if (smem > 48 * 1024)               // (the most that any context asks for: the attribute is shared by all of them)
+    LOSA_CUDA_TRY(c, cudaFuncSetAttribute(block_attn_merge_kernel<T, D, MERGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
   dim3 grid((sh.block_size + kTokTile - 1) / kTokTile, sh.n_kv_heads, sh.batch);
   launch_k(block_attn_merge_kernel<T, D, MERGE>, grid, kBaThreads, smem, st, 
       static_cast<const T*>(q), static_cast<const T*>(k_blk), static_cast<const T*>(v_blk),

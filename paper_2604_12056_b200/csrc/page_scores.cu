@@ -837,8 +837,8 @@ int32_t launch_stream(losa_ctx* c, const PsParams& pp, cudaStream_t st) {
   ns = ns > kPsMaxStages ? kPsMaxStages : ns;
   if (ns < 2) return LOSA_ERR_UNSUPPORTED;
   if (!c->scores_attr_set) {
-    LOSA_CUDA_TRY(c, cudaFuncSetAttribute(page_scores_stream_kernel<T, D, PG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          128 + ns * C::STAGE_BYTES + C::QBUF_BYTES + tail));
+    // (the whole budget, whatever this context needs: the attribute is the kernel's, and shared by all contexts)
+    LOSA_CUDA_TRY(c, cudaFuncSetAttribute(page_scores_stream_kernel<T, D, PG>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPsSmemBudget));
     c->scores_attr_set = 1;
   }
   // Behind stage 1 of the same step, no more stages than a CTA can have tiles (short prefixes): a CTA that asks for less
@@ -864,7 +864,7 @@ int32_t launch_bounds_t(losa_ctx* c, const PsParams& pp, cudaStream_t st) {
   const int smem = 128 + ns * C::STAGE_BYTES + C::QBUF_BYTES + tail;
   int32_t& attr_set = APPROX ? c->approx_attr_set : c->bounds_attr_set;
   if (!attr_set) {
-    LOSA_CUDA_TRY(c, cudaFuncSetAttribute(page_bounds_mma_kernel<D, APPROX>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    LOSA_CUDA_TRY(c, cudaFuncSetAttribute(page_bounds_mma_kernel<D, APPROX>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPsSmemBudget));
     attr_set = 1;
   }
   launch_k(page_bounds_mma_kernel<D, APPROX>, p.n_ctas, kPsThreads, smem, st, p);

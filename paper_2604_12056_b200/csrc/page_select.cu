@@ -981,8 +981,9 @@ int32_t launch_page_scores_topk(losa_ctx* c, const void* q, const losa_kv_t* kv,
   }
   // budgets beyond what one warp can sort: whole-list bitonic sort, one CTA per query
   const size_t smem = static_cast<size_t>(pow2_at_least(sh.max_pages_per_seq)) * sizeof(unsigned long long);
-  if (smem > 48 * 1024)
-    LOSA_CUDA_TRY(c, cudaFuncSetAttribute(topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+  if (smem > 48 * 1024)               // (the most that any context asks for: the attribute is shared by all of them)
+    LOSA_CUDA_TRY(c, cudaFuncSetAttribute(topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          topk_max_sortable(c) * static_cast<int>(sizeof(unsigned long long))));
   dim3 grid(sh.n_q_heads / pool, sh.block_size, sh.batch);
   launch_k(topk_kernel, grid, kThreads, smem, st, sc, kv->kv_len, active_idx, n_active, step, topk_pages,
                                             topk_scores_opt, sh.block_size, sh.n_q_heads, sh.page_size,

@@ -457,6 +457,26 @@ def test_fp32_attention_over_more_pages_than_a_cta_resolves_at_once():
         assert (layer.lse_p[s] - torch.logsumexp(sc, -1)).abs().max() < 1e-5
 
 
+@pytest.mark.parametrize("dtype,topk", [("f32", 4), ("bf16", 4), ("bf16", 600)])
+def test_contexts_of_different_batches_in_turn(dtype, topk):
+    """Contexts of 8, 1 and 3 sequences in one process, a step of each in turn: what one sets up must not refuse the next
+    call of another (a kernel's limit of shared memory is the kernel's, not the context's)."""
+    from paper_2604_12056_b200.layer import LosaLayer, to_device
+    runs = []
+    for n in (8, 1, 3):
+        cfg = wl.config("c1" if dtype == "f32" else "c2", n_q_heads=8, n_kv_heads=2, head_dim=128, page_size=16, kv_lens=(16 * 610 + 5,) * n,
+                        block_size=4, steps=2, topk=topk, m_active=2, **({"hidden_width": 0} if dtype == "f32" else {}))
+        w = wl.Workload(cfg)
+        runs.append((LosaLayer(cfg, w.k_pages, w.v_pages, w.page_table, w.kv_len), OracleLayer(w), cfg, w.block_steps()))
+    for t in range(2):
+        for g, o, cfg, steps in runs:
+            inp = steps[t]
+            g.run_step(to_device(inp.q), to_device(inp.k_blk), to_device(inp.v_blk), to_device(inp.m_per_seq))
+            snap, ref = g.snapshot(), o.run_step(inp)
+            assert g.ctx.poll_status() == 0
+            compare(snap, ref, cfg, f"{cfg.batch} sequences, step {t}")
+
+
 def test_multi_block_append():
     cfg = wl.config("c5", kv_lens=(200, 90, 64), n_blocks=3, steps=3, topk=4)
     run_blocks(cfg, n_blocks=3)
