@@ -22,7 +22,7 @@ struct WorkspaceLayout {
   size_t counters;   // uint32[N] : arrival counters of select_active (self-resetting)
   size_t seg_records; // int2[kMaxSegments] : first CTA and number of the partial records of every segment, left by the stage-4 main kernel for the kernels that merge them
   size_t slot_map;   // int32[N*B] : slot of every block token in the active list of the whole-step path, -1 = stable
-  size_t union_bits;    // uint32[N*H_kv*ceil(P_max/32)] : page bitmaps of the selection that also writes the union (all zero between launches)
+  size_t union_bits;    // uint32[N*H_kv*ceil(P_max/32)] : page bitmaps of the selection.  bf16: the selection writes the union from them, all zero between launches; fp32: stage 4 does, and stage 1 of the next whole step clears them
   size_t union_tickets; // uint32[N*H_kv] : its arrival counters (self-resetting)
   size_t delta;      // double[N*B]
   size_t scores;     // float[2*N*B*H_q*score_stride]: page scores, or (lower, upper) bound pairs of them

@@ -68,7 +68,8 @@ __device__ __forceinline__ float* record_base(float* partials, int slot, int w, 
 __device__ __forceinline__ int clamp_active(int na, int B) { return na < 0 ? 0 : (na > B ? B : na); }
 
 // Whole step: the lists as page bitmaps [n_sk][W] (written by the selection) in shared memory, with the number of
-// set bits of the list before every word, so that a page is found by its position in the list.
+// set bits of the list before every word, so that a page is found by its position in the list.  (16 bits hold it: a context
+// has at most topk_max_sortable() pages per sequence, 16,384, or is refused.)
 struct UnionBits {
   uint32_t* bits;
   uint16_t* before;

@@ -168,15 +168,6 @@ __device__ __forceinline__ void tc5_st16(uint32_t taddr, const uint32_t* w) {
         "r"(w[9]), "r"(w[10]), "r"(w[11]), "r"(w[12]), "r"(w[13]), "r"(w[14]), "r"(w[15])
       : "memory");
 }
-__device__ __forceinline__ void tc5_st32(uint32_t taddr, const uint32_t* w) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};"
-      ::"r"(taddr), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]), "r"(w[8]),
-        "r"(w[9]), "r"(w[10]), "r"(w[11]), "r"(w[12]), "r"(w[13]), "r"(w[14]), "r"(w[15]), "r"(w[16]), "r"(w[17]),
-        "r"(w[18]), "r"(w[19]), "r"(w[20]), "r"(w[21]), "r"(w[22]), "r"(w[23]), "r"(w[24]), "r"(w[25]), "r"(w[26]),
-        "r"(w[27]), "r"(w[28]), "r"(w[29]), "r"(w[30]), "r"(w[31])
-      : "memory");
-}
 __device__ __forceinline__ void tc5_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // byte offset of 16-byte chunk c (0..7) of row t in a [rows][128 B] tile with the 128-byte swizzle
 __device__ __forceinline__ uint32_t tc5_sw(int t, int c) { return static_cast<uint32_t>(t * 128 + ((c ^ (t & 7)) << 4)); }
@@ -845,7 +836,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             for (int c0 = 0; c0 < ncol; c0 += 32) {
               uint32_t v[32];
               tc5_ld32_nowait(s_addr + c0, v);
-                tc5_wait_ld();
+              tc5_wait_ld();
               tc5_pin32(v);
               if (ragged) mask_chunk(v, c0);
               float sum[4] = {0.f, 0.f, 0.f, 0.f};
@@ -961,7 +952,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     // round of copies of every ring slot (a group that was begun has had all its copies issued: the
     // producer loop only stops between groups), the issuing threads for the products they issued.
     if ((warp == kTc5KWarp || warp == kTc5VWarp) && lane == 0) {
-        const bool is_v = warp == kTc5VWarp;
+      const bool is_v = warp == kTc5VWarp;
       const uint32_t full0 = is_v ? (FP8 ? vstg_full : vfull) : kfull;
       const int NSL = is_v ? (FP8 ? NSP : NRV) : NRK;
       for (int sl = 0; sl < NSL; ++sl) {

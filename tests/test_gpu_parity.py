@@ -431,6 +431,44 @@ def test_fp32_whole_step_takes_the_union_from_page_bitmaps(kw):
     run_blocks(wl.config("c1", **{**dict(head_dim=64, page_size=16, block_size=6, steps=3, topk=7, m_active=2, hidden_width=0), **kw}), fused=True)
 
 
+def test_fp32_whole_step_at_the_most_pages_of_a_sequence():
+    """One list of 16,384 pages, the most that a context admits: the union of the first step is all of them, that of a
+    sparse step the pages listed; one page more is refused."""
+    import torch
+    from paper_2604_12056_b200 import binding as B
+    from paper_2604_12056_b200.layer import LosaLayer
+    g, d, P = 16, 64, 16384
+    cfg = wl.config("c1", n_q_heads=2, n_kv_heads=1, head_dim=d, page_size=g, kv_lens=(P * g - 5,), block_size=3, steps=2, topk=9,
+                    m_active=1, hidden_width=0)
+    assert cfg.max_pages_per_seq == P
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(4)
+    rnd = lambda *shape: torch.randn(*shape, generator=gen, device="cuda")
+    table = torch.randperm(P, generator=gen, device="cuda").to(torch.int32)[None].contiguous()
+    kv_len = torch.tensor([P * g - 5], dtype=torch.int32, device="cuda")
+    layer = LosaLayer(cfg, rnd(P, 1, g, d), rnd(P, 1, g, d), table, kv_len)
+    k, v = (t[table[0].long(), 0] for t in (layer.k_pages, layer.v_pages))
+    q = rnd(1, 3, 2, d)
+    for step in range(2):
+        if step:
+            q = q.clone()
+            q[0, 1] = rnd(2, d)
+        layer.run_step_fused(q, rnd(1, 3, 1, d), rnd(1, 3, 1, d), torch.ones(1, dtype=torch.int32, device="cuda"))
+        assert layer.ctx.poll_status() == 0
+        act = [1] if step else [0, 1, 2]
+        pages = torch.unique(layer.topk_pages[0, 1]) if step else torch.arange(P, dtype=torch.int32, device="cuda")
+        n = len(pages)
+        assert int(layer.union_count[0, 0]) == n and torch.equal(layer.union_pages[0, 0, :n], pages) and (layer.union_pages[0, 0, n:] == -1).all()
+        ok = (pages[:, None].long() * g + torch.arange(g, device="cuda")) < P * g - 5
+        sc = q[0, act].double() @ k[pages.long()][ok].double().T * cfg.sm_scale
+        # (fp32 sums of up to 256K terms that cancel, as in the test below)
+        assert (layer.o_p[0, act] - torch.softmax(sc, -1) @ v[pages.long()][ok].double()).abs().max() < (2e-6 if step else 1e-6)
+        assert (layer.lse_p[0, act] - torch.logsumexp(sc, -1)).abs().max() < 1e-5
+    with pytest.raises(B.LosaError) as e:
+        B.Context(1, 2, 1, d, 3, g, P + 1, B.LOSA_F32, cfg.sm_scale, "cuda")
+    assert e.value.code == B.LOSA_ERR_UNSUPPORTED
+
+
 def test_fp32_attention_over_more_pages_than_a_cta_resolves_at_once():
     """48,000 pages: more than 256 for every CTA; compared with softmax in float64."""
     import torch
