@@ -6,6 +6,7 @@
 // (self-resetting counter) ranks the B scores by (Delta descending, token ascending) and emits the
 // first m tokens in ascending order.
 #include <mutex>
+#include <type_traits>
 
 #include "kernels.h"
 
@@ -14,14 +15,23 @@ namespace {
 
 constexpr int kThreads = 256;
 
-template <typename T>
+// What a whole step asks of this kernel besides: the inverse of the active list, and words per sequence to be cleared.  (The
+// stage as a call of its own is launched without these arguments: with them its host time was 0.5 us of 6 longer.)
+struct StepExtras {
+  int32_t* slot_map;
+  uint32_t* clear;
+  int clear_words;
+};
+struct NoExtras {};
+
+template <typename T, typename Extras>
 __global__ void __launch_bounds__(kThreads)
 select_active_kernel(const T* __restrict__ x_cur, const T* __restrict__ x_prev, int row_width, int B,
                      const int32_t* __restrict__ m_per_seq, const int32_t* __restrict__ step,
                      int32_t* __restrict__ active_idx, int32_t* __restrict__ n_active,
                      float* __restrict__ delta_opt, double* __restrict__ delta_ws,
-                     unsigned int* __restrict__ counters, double tau, int32_t* __restrict__ slot_map,
-                     uint32_t* __restrict__ clear, int clear_words) {
+                     unsigned int* __restrict__ counters, double tau, Extras x) {
+  constexpr bool STEP = std::is_same_v<Extras, StepExtras>;
   // Wait first, release afterwards: a kernel released by this one may read, before its own wait, what
   // earlier kernels of the stream wrote (the cache's lengths, summaries and step counters), so those
   // must have completed by then.
@@ -33,7 +43,8 @@ select_active_kernel(const T* __restrict__ x_cur, const T* __restrict__ x_prev, 
   const int step_now = step ? step[s] : 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // the page bitmaps of the step that begins: read last by the step before, marked next by the selection
-  for (int w = i * kThreads + tid; w < clear_words; w += B * kThreads) clear[static_cast<size_t>(s) * clear_words + w] = 0u;
+  if constexpr (STEP)
+    for (int w = i * kThreads + tid; w < x.clear_words; w += B * kThreads) x.clear[static_cast<size_t>(s) * x.clear_words + w] = 0u;
   const size_t row = (static_cast<size_t>(s) * B + i) * row_width;
   constexpr int kVec = 8;
   double acc = 0.0;
@@ -136,9 +147,9 @@ select_active_kernel(const T* __restrict__ x_cur, const T* __restrict__ x_prev, 
   int32_t* out = active_idx + static_cast<size_t>(s) * B;
   if (act[0]) out[__popc(b0 & below)] = lane;
   if (act[1]) out[n0 + __popc(b1 & below)] = lane + 32;
-  if (slot_map) {                                     // the inverse map, for the kernel that finishes the step
-    if (lane < B) slot_map[s * B + lane] = act[0] ? __popc(b0 & below) : -1;
-    if (lane + 32 < B) slot_map[s * B + lane + 32] = act[1] ? n0 + __popc(b1 & below) : -1;
+  if constexpr (STEP) {                               // the inverse map, for the kernel that finishes the step
+    if (lane < B) x.slot_map[s * B + lane] = act[0] ? __popc(b0 & below) : -1;
+    if (lane + 32 < B) x.slot_map[s * B + lane + 32] = act[1] ? n0 + __popc(b1 & below) : -1;
   }
   for (int t = n0 + n1 + lane; t < B; t += 32) out[t] = -1;
   if (lane == 0) n_active[s] = n0 + n1;
@@ -154,15 +165,17 @@ int32_t launch_select_active(losa_ctx* c, const void* x_cur, const void* x_prev,
   dim3 grid(sh.block_size, sh.batch);
   double* dws = reinterpret_cast<double*>(c->ws + c->lay.delta);
   unsigned int* ctr = reinterpret_cast<unsigned int*>(c->ws + c->lay.counters);
-  if (sh.dtype == LOSA_BF16) {
-    launch_k(select_active_kernel<__nv_bfloat16>, grid, kThreads, 0, st, 
-        static_cast<const __nv_bfloat16*>(x_cur), static_cast<const __nv_bfloat16*>(x_prev), row_width,
-        sh.block_size, m_per_seq, step, active_idx, n_active, delta_opt, dws, ctr, tau, slot_map_opt, clear, clear_words);
-  } else {
-    launch_k(select_active_kernel<float>, grid, kThreads, 0, st, 
-        static_cast<const float*>(x_cur), static_cast<const float*>(x_prev), row_width, sh.block_size,
-        m_per_seq, step, active_idx, n_active, delta_opt, dws, ctr, tau, slot_map_opt, clear, clear_words);
-  }
+  auto launch = [&](auto t, auto x) {
+    using T = decltype(t);
+    launch_k(select_active_kernel<T, decltype(x)>, grid, kThreads, 0, st, static_cast<const T*>(x_cur), static_cast<const T*>(x_prev),
+             row_width, sh.block_size, m_per_seq, step, active_idx, n_active, delta_opt, dws, ctr, tau, x);
+  };
+  auto launch_t = [&](auto t) {
+    if (slot_map_opt) launch(t, StepExtras{slot_map_opt, clear, clear_words});
+    else launch(t, NoExtras{});
+  };
+  if (sh.dtype == LOSA_BF16) launch_t(__nv_bfloat16{});
+  else launch_t(float{});
   return after_launch(c);
 }
 
@@ -225,13 +238,13 @@ extern "C" int32_t losa_select_active_static(const losa_shape_t* shape, const vo
   if (cudaMemsetAsync(scratch->counters, 0, sizeof(unsigned int) * shape->batch, st) != cudaSuccess) return LOSA_ERR_CUDA;
   dim3 grid(shape->block_size, shape->batch);
   if (shape->dtype == LOSA_BF16) {
-    losa::launch_k(losa::select_active_kernel<__nv_bfloat16>, grid, losa::kThreads, 0, st, 
+    losa::launch_k(losa::select_active_kernel<__nv_bfloat16, losa::NoExtras>, grid, losa::kThreads, 0, st,
         static_cast<const __nv_bfloat16*>(x_cur), static_cast<const __nv_bfloat16*>(x_prev), row_width,
-        shape->block_size, m_per_seq, step, active_idx, n_active, delta_opt, scratch->delta, scratch->counters, 0.0, nullptr, nullptr, 0);
+        shape->block_size, m_per_seq, step, active_idx, n_active, delta_opt, scratch->delta, scratch->counters, 0.0, losa::NoExtras{});
   } else {
-    losa::launch_k(losa::select_active_kernel<float>, grid, losa::kThreads, 0, st, 
+    losa::launch_k(losa::select_active_kernel<float, losa::NoExtras>, grid, losa::kThreads, 0, st,
         static_cast<const float*>(x_cur), static_cast<const float*>(x_prev), row_width, shape->block_size,
-        m_per_seq, step, active_idx, n_active, delta_opt, scratch->delta, scratch->counters, 0.0, nullptr, nullptr, 0);
+        m_per_seq, step, active_idx, n_active, delta_opt, scratch->delta, scratch->counters, 0.0, losa::NoExtras{});
   }
   return cudaGetLastError() == cudaSuccess ? LOSA_OK : LOSA_ERR_CUDA;
 }
