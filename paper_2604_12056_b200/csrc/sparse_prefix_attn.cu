@@ -500,7 +500,8 @@ int32_t prepare_f32(losa_ctx* c) {
   constexpr int smem = sizeof(F32Smem<D>);
   static_assert(smem <= kSmemBudget, "shared memory of the fp32 stage-4 kernel");
   if (c->attn_attr_set & 1) return LOSA_OK;
-  LOSA_CUDA_TRY(c, cudaFuncSetAttribute(attn_f32_kernel<D, GP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  LOSA_CUDA_TRY(c, cudaFuncSetAttribute(attn_f32_kernel<D, GP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  LOSA_CUDA_TRY(c, cudaFuncSetAttribute(attn_f32_kernel<D, GP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   c->attn_attr_set |= 1;
   return LOSA_OK;
 }
@@ -522,7 +523,7 @@ int32_t launch_tc5(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool with
 template <int D, int GP>
 int32_t launch_f32(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool with_combine) {
   if (c->profile) LOSA_CUDA_TRY(c, cudaEventRecord(c->ev_begin, st));
-  launch_k(attn_f32_kernel<D, GP>, ap.n_ctas, kF32Threads, sizeof(F32Smem<D>), st, ap);
+  launch_k(ap.union_bits ? attn_f32_kernel<D, GP, true> : attn_f32_kernel<D, GP, false>, ap.n_ctas, kF32Threads, sizeof(F32Smem<D>), st, ap);
   if (c->profile) LOSA_CUDA_TRY(c, cudaEventRecord(c->ev_end, st));
   int32_t rc = after_launch(c);
   if (rc != LOSA_OK || !with_combine) return rc;

@@ -70,11 +70,13 @@ __device__ __forceinline__ void cp_async16_or_zero(uint32_t dst, const void* src
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // Pages c0 .. c0 + n - 1 of list sk (n <= kF32Chunk): physical page and number of valid tokens; the caller synchronises.
-template <int D, int GP>
+// BITS, here and below: the lists are page bitmaps (whole step).  A kernel of its own: with the choice at run time the dense pass
+// over lists (4,096 + 2,875 tokens, 128 rows) took 114 us instead of 111.
+template <int D, int GP, bool BITS>
 __device__ __forceinline__ void f32_resolve(const AttnParams& p, F32Smem<D>& sm, int sk, int c0, int n, int len) {
   const int tid = threadIdx.x, s = sk / p.Hkv;
   if (tid < n) {
-    const int page = p.union_bits ? sm.lists(p.W).page(sk, c0 + tid) : p.union_pages[static_cast<size_t>(sk) * p.Pmax + c0 + tid];
+    const int page = BITS ? sm.lists(p.W).page(sk, c0 + tid) : p.union_pages[static_cast<size_t>(sk) * p.Pmax + c0 + tid];
     bool ok = page >= 0 && page < p.Pmax;
     const int phys = ok ? p.page_table[static_cast<size_t>(s) * p.Pmax + page] : 0;
     ok = ok && phys >= 0 && phys < p.n_phys;
@@ -86,7 +88,7 @@ __device__ __forceinline__ void f32_resolve(const AttnParams& p, F32Smem<D>& sm,
 }
 
 // One piece, more than kF32Few rows: union positions u0 .. u1 - 1 of segment sg.
-template <int D, int GP, int NB>
+template <int D, int GP, int NB, bool BITS>
 __device__ __forceinline__ void f32_piece(const AttnParams& p, F32Smem<D>& sm, int sg, int u0, int u1) {
   constexpr int DI = D / 32, JM = 8;                // 16-byte reads of a key per lane, rows per lane
   constexpr int TS = kF32Warps / NB, TPW = kF32Tok / TS;   // warps per row block, tokens of a tile per warp
@@ -133,7 +135,7 @@ __device__ __forceinline__ void f32_piece(const AttnParams& p, F32Smem<D>& sm, i
   for (int c0 = u0; c0 < u1; c0 += kF32Chunk) {
     const int n = min(kF32Chunk, u1 - c0), n_tiles = (n * GP + kF32Tok - 1) / kF32Tok;
     __syncthreads();                                // the tiles and page numbers of the previous chunk (or piece) are done with
-    f32_resolve<D, GP>(p, sm, sk, c0, n, len);
+    f32_resolve<D, GP, BITS>(p, sm, sk, c0, n, len);
     __syncthreads();
     auto valid_token = [&](int t) {                 // token t of the chunk
       const int it = t / GP;
@@ -280,7 +282,7 @@ __device__ __forceinline__ void f32_piece(const AttnParams& p, F32Smem<D>& sm, i
 }
 
 // One piece of at most kF32Few rows: every warp has tokens of its own.
-template <int D, int GP>
+template <int D, int GP, bool BITS>
 __device__ __forceinline__ void f32_piece_few(const AttnParams& p, F32Smem<D>& sm, int sg, int u0, int u1) {
   constexpr int DI = D / 32, JM = 4, WT = kF32WTok;  // a lane's rows rs + 4 j
   constexpr int NSC = WT / 2;                        // scores per lane and step: lane bit 2 picks the token of a pair
@@ -324,7 +326,7 @@ __device__ __forceinline__ void f32_piece_few(const AttnParams& p, F32Smem<D>& s
   for (int c0 = u0; c0 < u1; c0 += kF32Chunk) {
     const int n = min(kF32Chunk, u1 - c0), n_steps = n * (GP / WT);
     __syncthreads();                                 // the page numbers and rings of the previous chunk (or piece) are done with
-    f32_resolve<D, GP>(p, sm, sk, c0, n, len);
+    f32_resolve<D, GP, BITS>(p, sm, sk, c0, n, len);
     __syncthreads();
     auto load = [&](int step, int slot) {
       if (step < n_steps) {
@@ -464,19 +466,19 @@ __device__ __forceinline__ void f32_piece_few(const AttnParams& p, F32Smem<D>& s
   }
 }
 
-template <int D, int GP>
+template <int D, int GP, bool BITS>
 __global__ void __launch_bounds__(kF32Threads, 1) attn_f32_kernel(AttnParams p) {
   grid_dep_wait();
   extern __shared__ __align__(16) uint8_t f32_smem[];
   F32Smem<D>& sm = *reinterpret_cast<F32Smem<D>*>(f32_smem);
   static_assert(sizeof(float) * 2 * kF32Stages * kF32Tok * D >= sizeof(float) * kRowsPerGroup * D, "the partial outputs fit the tiles");
   const UnionBits lists = sm.lists(p.W);
-  if (p.union_bits) {
+  if constexpr (BITS) {
     lists.load(p.union_bits, p.n_sk, threadIdx.x >> 5, kF32Warps, threadIdx.x & 31);
     __syncthreads();
   }
-  if (threadIdx.x < 32) segment_prefix(sm.pre, p.n_seg, p.n_rg, p.Hkv, p.G, p.n_active, [&](int sk) { return p.union_bits ? lists.count(sk) : p.union_count[sk]; }, p.B, threadIdx.x);
-  else if (p.union_bits && threadIdx.x < 64) lists.write(p, threadIdx.x & 31);
+  if (threadIdx.x < 32) segment_prefix(sm.pre, p.n_seg, p.n_rg, p.Hkv, p.G, p.n_active, [&](int sk) { return BITS ? lists.count(sk) : p.union_count[sk]; }, p.B, threadIdx.x);
+  else if (BITS && threadIdx.x < 64) lists.write(p, threadIdx.x & 31);
   __syncthreads();
   const int T_all = sm.pre[p.n_seg];
   const int n = f32_ctas(T_all, p.n_ctas, GP);
@@ -489,10 +491,10 @@ __global__ void __launch_bounds__(kF32Threads, 1) attn_f32_kernel(AttnParams p) 
     while (sm.pre[sg + 1] <= item) ++sg;
     const int seg_end = min(hi, sm.pre[sg + 1]), u0 = item - sm.pre[sg], u1 = seg_end - sm.pre[sg];
     const int rows = rows_in_group(clamp_active(p.n_active[(sg % p.n_sk) / p.Hkv], p.B), p.G, sg / p.n_sk);
-    if (rows <= kF32Few) f32_piece_few<D, GP>(p, sm, sg, u0, u1);
-    else if (rows <= 32) f32_piece<D, GP, 1>(p, sm, sg, u0, u1);
-    else if (rows <= 64) f32_piece<D, GP, 2>(p, sm, sg, u0, u1);
-    else f32_piece<D, GP, 4>(p, sm, sg, u0, u1);
+    if (rows <= kF32Few) f32_piece_few<D, GP, BITS>(p, sm, sg, u0, u1);
+    else if (rows <= 32) f32_piece<D, GP, 1, BITS>(p, sm, sg, u0, u1);
+    else if (rows <= 64) f32_piece<D, GP, 2, BITS>(p, sm, sg, u0, u1);
+    else f32_piece<D, GP, 4, BITS>(p, sm, sg, u0, u1);
     item = seg_end;
   }
 }
