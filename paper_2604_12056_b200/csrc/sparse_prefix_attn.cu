@@ -198,9 +198,11 @@ template <int C> __device__ __forceinline__ void st_state(void* base, int bf16, 
 // Merge of the partial records of row r of segment sg by one warp: returns the un-normalised output
 // columns lane * C + c in acc, the reference maximum M and the sum of weights Lsum.  The outputs of up
 // to kMergeBatch records are copied to `buf` (that many rows of D floats of this warp) while their
-// maxima are read; with up to 32 KB per CTA and few registers, more CTAs are resident than with
+// maxima are read; with up to 40 KB per CTA and few registers, five CTAs are resident per SM, more than with
 // outputs in registers, and the rolled loops keep the code short.  A lane reads back only what it
-// copied itself.  20: what one sequence's eight KV heads have over 148 CTAs, in one round trip (16: two; 1.5 us per step).
+// copied itself.  20: a list cut over 148 CTAs leaves each of
+// eight segments 19 or 20 records, one round trip instead of two with 16 (eight steps of one 8K sequence 293 us against 298); more segments have
+// fewer records each, and five resident CTAs instead of six cost them nothing (four steps of eight 32K sequences 436 and 435 us).
 constexpr int kMergeBatch = 20;
 template <int D, bool LOG2>
 __device__ __forceinline__ void merge_records(const AttnParams& p, float* buf, int sg, int r, int2 records, int lane,

@@ -178,7 +178,8 @@ __device__ __forceinline__ uint32_t tc5_sw(int t, int c) { return static_cast<ui
 // leaves at most half a unit of them, so three terms hold the eight of a bf16 value; with the row's largest element at
 // 2^15 .. 2^16 that is exact down to 2^-9, 2^-24 of the largest, and below to within 2^-17, 2^-32 of it - more than the fp16
 // value of an element keeps in a row below 256.  (Two E4M3 terms lose an element's low bits from 2^-9 of the row's largest
-// on: with them the block of eight 32K prompts takes 954 us, 976 with three, of which K's ring gives one slot to the third.)  V cannot: P needs more than three terms.
+// on: with them the block of eight 32K prompts takes 954 us, 976 with three.  That is the third product; the slot of K's ring that its
+// tile takes at d = 128 costs nothing: four slots and fewer staging pages are no faster.)  V cannot: P needs more than three terms.
 // Its codes land in a staging ring as they lie in memory; four converting warps, one per scheduler, turn a
 // landed page into fp16 (exact) in the group's ring slot, in the layout the tensor maps of the bf16 path
 // produce, and P is fp16.  The scales stay out of the conversion, which is bound by its instruction count: the
