@@ -13,7 +13,7 @@
 //   O[128 x D]   += P . V        A = P from tensor memory, B = the group's V tiles as they lie in
 //                                memory (tokens x d: MN-major); 8 instructions
 // An instruction of either product takes the pipe 64 cycles (128 x 128 x 16); each product has an issuing
-// thread of its own.  K and V have a ring of group-sized slots each, filled by one producer warp each
+// warp of its own (one elected lane).  K and V have a ring of group-sized slots each, filled by one producer warp each
 // (lane = page: 32 pages' copies are issued by one instruction); a K slot is free again as soon as its
 // Q K^T has run, a V slot after its P V.  There is an S buffer per set (tensor memory: O 128 + 3 x 128
 // columns; Q therefore lies in shared memory).  Completion is tracked with tcgen05.commit on mbarriers; every wait is
@@ -119,6 +119,19 @@ __device__ __forceinline__ void tc5_mma_ss8(uint32_t d_tmem, uint64_t a, uint64_
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
       ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+}
+// A warp's value that is the same in all lanes, in a form the compiler knows to be so, and the lane that issues for its warp.
+// With `lane == 0` around the products and operands from ordinary registers an issuing warp took 75 to 100 cycles per
+// instruction, whatever its shape (eight of them 600 to 820); chosen by elect.sync, 17 (eight 134), and the pipe's 64 count.
+template <typename T> __device__ __forceinline__ T warp_uniform(T v) { return __shfl_sync(0xffffffffu, v, 0); }
+__device__ __forceinline__ bool elect_one() {
+  uint32_t one;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one) :: "memory");
+  return one != 0;
+}
+// one answer for the whole warp
+__device__ __forceinline__ bool warp_mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status, long long limit) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status, limit)) != 0;
 }
 __device__ __forceinline__ void tc5_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -251,7 +264,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   volatile float* kscale_meta = reinterpret_cast<volatile float*>(const_cast<int*>(meta) + MR * PG);
   const bool staged = p.N * p.B <= kStageIdx && p.N <= kStageSeq;
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = warp_uniform(tid >> 5);
   if (tid == 0) {
     for (int i = 0; i < NRK; ++i) {
       mbar_init(kfull + 8 * i, 1);
@@ -565,72 +578,86 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       while (item < hi && pre[sg + 1] <= item) ++sg;
     }
   } else if (warp == kTc5QkWarp) {
-    // ------------------------------------------------------------------ Q K^T issuer (one thread)
-    if (lane == 0) {
-      int sg = sg0, item = lo, piece = 0, g = 0;
-      bool ok = true;
-      while (item < hi && ok) {
-        const int seg_end = min(hi, pre[sg + 1]);
-        ok = mbar_wait(q_full, piece & 1, abort_flag, p.status, p.wait_cycles);
-        for (int first = item; first < seg_end && ok; first += PG, ++g) {
-          const int ng = min(PG, seg_end - first), b = g % SB, use = g / SB, slot = g % NRK;
-          ok = mbar_wait(kfull + 8 * slot, (g / NRK) & 1, abort_flag, p.status, p.wait_cycles);
-          ok = ok && (use == 0 || mbar_wait(s_free + 8 * b, (use - 1) & 1, abort_flag, p.status, p.wait_cycles));
-          if (!ok) break;
-          tc5_fence_after();
-          const uint32_t kt = kring + slot * KSLOT, s_col = tmem + COL_S + b * kTc5Tok;
+    // ------------------------------------------------------------------ Q K^T issuer (a warp, one elected lane issues)
+    const uint32_t qt = warp_uniform(qtile), kr = warp_uniform(kring), s_col0 = warp_uniform(tmem) + COL_S;
+    const int end = warp_uniform(hi);
+    auto wait = [&](uint32_t bar, uint32_t parity) { return warp_mbar_wait(bar, parity, abort_flag, p.status, p.wait_cycles); };
+    int sg = sg0, item = warp_uniform(lo), piece = 0, g = 0;
+    bool ok = true;
+    while (item < end && ok) {
+      const int seg_end = warp_uniform(min(end, pre[sg + 1]));
+      ok = wait(q_full, piece & 1);
+      for (int first = item; first < seg_end && ok; first += PG, ++g) {
+        const int ng = min(PG, seg_end - first), b = g % SB, use = g / SB, slot = g % NRK;
+        ok = wait(kfull + 8 * slot, (g / NRK) & 1);
+        ok = ok && (use == 0 || wait(s_free + 8 * b, (use - 1) & 1));
+        if (!ok) break;
+        tc5_fence_after();
+        if (elect_one()) {
+          const uint32_t kt = kr + slot * KSLOT, s_col = s_col0 + b * kTc5Tok;
           if constexpr (FP8) {                       // the terms of Q (E5M2) against the same codes (E4M3)
             const uint32_t idesc = tc5_idesc(kRowsPerGroup, ng * GP, 0, 1u, 0u);
+            const uint64_t qd = tc5_desc8<D>(qt), kd = tc5_desc8<D>(kt);
 #pragma unroll
             for (int ks = 0; ks < D / 32; ++ks)
 #pragma unroll
               for (int t = 0; t < kTc5QTerms; ++t)
-                tc5_mma_ss8(s_col, tc5_desc8<D>(qtile + t * (QB / kTc5QTerms) + ks * 32), tc5_desc8<D>(kt + ks * 32), idesc, ks + t > 0 ? 1u : 0u);
+                tc5_mma_ss8(s_col, qd + (t * (kRowsPerGroup * D) + ks * 32) / 16, kd + ks * 2, idesc, ks + t > 0 ? 1u : 0u);
           } else {
             const uint32_t idesc = tc5_idesc(kRowsPerGroup, ng * GP, 0, 1u, 1u);
+            const uint64_t qd = tc5_desc(qt, 16), kd = tc5_desc(kt, 16);
 #pragma unroll
             for (int ks = 0; ks < D / 16; ++ks) {
-              const uint32_t at = (ks >> 2) * HS + (ks & 3) * 32;
-              tc5_mma_ss(s_col, tc5_desc(qtile + at, 16), tc5_desc(kt + at, 16), idesc, ks > 0 ? 1u : 0u);
+              const uint32_t at = ((ks >> 2) * HS + (ks & 3) * 32) / 16;
+              tc5_mma_ss(s_col, qd + at, kd + at, idesc, ks > 0 ? 1u : 0u);
             }
           }
           tc5_commit(s_full + 8 * b);
           tc5_commit(kfree + 8 * slot);
           if (first + PG >= seg_end) tc5_commit(q_free);        // Q may be replaced once the piece's last product has run
         }
-        item = seg_end;
-        ++sg;
-        ++piece;
-        while (item < hi && pre[sg + 1] <= item) ++sg;
+        __syncwarp();
       }
+      item = seg_end;
+      ++sg;
+      ++piece;
+      while (item < end && warp_uniform(pre[sg + 1]) <= item) ++sg;
     }
   } else if (warp == kTc5PvWarp) {
-    // ------------------------------------------------------------------ P V issuer (one thread)
-    if (lane == 0) {
-      const uint32_t idesc = tc5_idesc(kRowsPerGroup, D, 1, FP8 ? 0u : 1u, FP8 ? 0u : 1u);
-      int sg = sg0, item = lo, piece = 0, g = 0;
-      bool ok = true;
-      while (item < hi && ok) {
-        const int seg_end = min(hi, pre[sg + 1]);
-        for (int first = item; first < seg_end && ok; first += PG, ++g) {
-          const int ng = min(PG, seg_end - first), b = g % SB, use = g / SB, slot = g % NRV;
-          ok = mbar_wait(vfull + 8 * slot, (g / NRV) & 1, abort_flag, p.status, p.wait_cycles);
-          if (first == item && piece > 0) ok = ok && mbar_wait(o_free, (piece - 1) & 1, abort_flag, p.status, p.wait_cycles);   // O has been read
-          ok = ok && mbar_wait(p_full + 8 * b, use & 1, abort_flag, p.status, p.wait_cycles);
-          if (!ok) break;
-          tc5_fence_after();
-          const uint32_t vt = vring + slot * SLOT;
-          for (int ks = 0; ks < ng * GP / 16; ++ks)
-            tc5_mma_ts(tmem + COL_O, tmem + COL_S + b * kTc5Tok + ks * 8, tc5_desc(vt + ks * 2048, HS), idesc,
-                       (first == item && ks == 0) ? 0u : 1u);
+    // ------------------------------------------------------------------ P V issuer (a warp, one elected lane issues)
+    const uint32_t idesc = tc5_idesc(kRowsPerGroup, D, 1, FP8 ? 0u : 1u, FP8 ? 0u : 1u);
+    const uint32_t vr = warp_uniform(vring), tm = warp_uniform(tmem);
+    const int end = warp_uniform(hi);
+    auto wait = [&](uint32_t bar, uint32_t parity) { return warp_mbar_wait(bar, parity, abort_flag, p.status, p.wait_cycles); };
+    int sg = sg0, item = warp_uniform(lo), piece = 0, g = 0;
+    bool ok = true;
+    while (item < end && ok) {
+      const int seg_end = warp_uniform(min(end, pre[sg + 1]));
+      for (int first = item; first < seg_end && ok; first += PG, ++g) {
+        const int ng = min(PG, seg_end - first), b = g % SB, use = g / SB, slot = g % NRV;
+        ok = wait(vfull + 8 * slot, (g / NRV) & 1);
+        if (first == item && piece > 0) ok = ok && wait(o_free, (piece - 1) & 1);   // O has been read
+        ok = ok && wait(p_full + 8 * b, use & 1);
+        if (!ok) break;
+        tc5_fence_after();
+        if (elect_one()) {
+          const uint64_t vd = tc5_desc(vr + slot * SLOT, HS);
+          const uint32_t p_col = tm + COL_S + b * kTc5Tok, fresh = first == item ? 0u : 1u;
+          if (ng == PG) {
+#pragma unroll
+            for (int ks = 0; ks < kTc5Tok / 16; ++ks) tc5_mma_ts(tm + COL_O, p_col + ks * 8, vd + ks * 128, idesc, ks == 0 ? fresh : 1u);
+          } else {
+            for (int ks = 0; ks < ng * GP / 16; ++ks) tc5_mma_ts(tm + COL_O, p_col + ks * 8, vd + ks * 128, idesc, ks == 0 ? fresh : 1u);
+          }
           tc5_commit(vfree + 8 * slot);
           tc5_commit(s_free + 8 * b);
         }
-        item = seg_end;
-        ++sg;
-        ++piece;
-        while (item < hi && pre[sg + 1] <= item) ++sg;
+        __syncwarp();
       }
+      item = seg_end;
+      ++sg;
+      ++piece;
+      while (item < end && warp_uniform(pre[sg + 1]) <= item) ++sg;
     }
   }
   } else {
@@ -718,7 +745,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
               uint8_t* dst = gen + tc5_sw8<D>(r, h * (NC / 2) + c / 2);
 #pragma unroll
               for (int t = 0; t < kTc5QTerms; ++t)
-                *reinterpret_cast<uint4*>(dst + t * (QB / kTc5QTerms)) = make_uint4(w4[t][0], w4[t][1], w4[t][2], w4[t][3]);
+                *reinterpret_cast<uint4*>(dst + t * (kRowsPerGroup * D)) = make_uint4(w4[t][0], w4[t][1], w4[t][2], w4[t][3]);
             }
           }
         } else {
@@ -962,7 +989,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         mbar_drain(full0 + 8 * sl, (gl / NSL) & 1);
       }
     }
-    if ((warp == kTc5QkWarp || warp == kTc5PvWarp) && lane == 0) {
+    if ((warp == kTc5QkWarp || warp == kTc5PvWarp) && elect_one()) {
       const uint32_t bar = drain_bar + (warp == kTc5PvWarp ? 8 : 0);
       tc5_commit(bar);
       mbar_drain(bar, 0);
