@@ -390,7 +390,8 @@ __device__ __forceinline__ uint32_t prefix_word(int w, int P) {   // word w of t
 // One CTA of kSelThreads per (sequence, head, share of the active slots).  Per query: tau = lower edge
 // of the histogram bin that holds the k-th largest LOWER bound; every page whose UPPER bound reaches
 // tau is a candidate (a superset of the exact top-k, ties included: the exact score lies between the
-// bounds); exact scores in the fixed order for the candidates (four lanes each), sort, emit.  More
+// bounds); the candidates by descending lower bound; exact scores in the fixed order (four lanes each) only
+// for those that lie so close to a neighbour that the bounds leave their order open; emit.  More
 // than kSelCap candidates (possible only when most pages nearly tie): exact scores for every page
 // into the score row, then the plain threshold search.
 // POOLED (one list per KV head, Section 4.2's selector with the group's maximum as the page score):
@@ -402,19 +403,25 @@ constexpr int kMaxPool = 16;     // heads per KV head the interface admits
 template <int D, bool POOLED>
 struct RefineSmem {
   float qs[(POOLED ? kMaxPool : 1) * 2 * D];
-  unsigned long long ckey[kSelCap];
-  int cpage[kSelCap], cphys[kSelCap];
-  int hist[kSelBins];
+  unsigned long long ckey[kSelCap];              // candidates: exact score and page (RUNS: first, as found, lower bound and page)
+  union {
+    struct { int cpage[kSelCap], cphys[kSelCap]; };
+    unsigned long long skey[kSelCap];            // RUNS: by descending lower bound
+  };
+  union { int hist[kSelBins]; uint16_t close[kSelCap]; };   // (close: once tau is known)
+  uint32_t run[kSelCap / 32];                    // bit r: a run of close candidates starts at position r
   uint32_t red[2][kSelThreads / 32];
-  int ncand, bstar;
+  uint32_t width;                                // the widest pair of bounds, rounded up: the bits of a float
+  int ncand, nclose, bstar;
 };
+static_assert(kSelBins * sizeof(int) >= kSelCap * sizeof(uint16_t), "positions");
 
 // In a whole step the grid ends with the row tiles of the in-block attention (BK: its padded key
 // count).  It needs only the step's inputs, and these CTAs fill the gaps of a kernel that is bound by
 // latency.  On a second stream it was hidden as well, but the join in front of the step's last kernel
 // cost that kernel its early launch (4 us of idle GPU per step); in stage 1's launch it delayed stage
 // 2 (eight sequences: bounds from 12 us on instead of 7).
-template <int D, bool POOLED, int BK>
+template <int D, bool POOLED, int BK, bool RUNS>
 __global__ void __launch_bounds__(kSelThreads, POOLED ? 4 : 6)
 topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
   static_assert(kSelThreads == kMmaThreads, "one CTA size");
@@ -509,6 +516,7 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
       }
     }
     uint32_t lbc[kSelPerThread], ubc[kSelPerThread];
+    float width = 0.f;                                     // of the widest pair of bounds, rounded up
     if (cached) {
       float2 bv[kSelPerThread];
 #pragma unroll
@@ -533,6 +541,7 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
       }
 #pragma unroll
       for (int i = 0; i < kSelPerThread; ++i) {
+        if (RUNS) width = fmaxf(width, __fsub_ru(bv[i].y, bv[i].x));
         lbc[i] = order_bits(bv[i].x);
         ubc[i] = order_bits(bv[i].y);
       }
@@ -558,7 +567,7 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
       qs[gi * 2 * D + d] = fmaxf(v, 0.f);
       qs[gi * 2 * D + D + d] = fminf(v, 0.f);
     }
-    if (tid == 0) s_ncand = 0;
+    if (tid == 0) { s_ncand = 0; sm.r.nclose = 0; sm.r.width = 0u; }
     for (int b = tid; b < kSelBins; b += kSelThreads) hist[b] = 0;
     // ---- tau
     uint32_t tau = 0u;
@@ -572,8 +581,8 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
 #pragma unroll
       for (int w = 0; w < kSelThreads / 32; ++w) { lo = min(lo, s_red[0][w]); hi = max(hi, s_red[1][w]); }
       if (lo < hi) {
-        const int width = 32 - __clz(hi - lo);
-        const int shift = width > 8 ? width - 8 : 0;
+        const int bits_of = 32 - __clz(hi - lo);
+        const int shift = bits_of > 8 ? bits_of - 8 : 0;
         for_each_page([&](uint32_t lb, uint32_t, int) { atomicAdd(&hist[(lb - lo) >> shift], 1); });
         __syncthreads();
         if (warp == 0) {
@@ -621,14 +630,21 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
 #pragma unroll
       for (int i = 0; i < kSelPerThread; ++i) {
         const int mine = at + __popc(hit[i] & ((1u << lane) - 1u));
-        if (((hit[i] >> lane) & 1u) && mine < kSelCap) cpage[mine] = tid + kSelThreads * i;
+        if (((hit[i] >> lane) & 1u) && mine < kSelCap) {
+          if (RUNS) ckey[mine] = make_key(lbc[i], tid + kSelThreads * i);
+          else cpage[mine] = tid + kSelThreads * i;
+        }
         at += __popc(hit[i]);
       }
     } else {
-      for_each_page([&](uint32_t, uint32_t ub, int pg) {
+      for_each_page([&](uint32_t lb, uint32_t ub, int pg) {
         if (ub >= tau) {
           const int i = atomicAdd(&s_ncand, 1);
-          if (i < kSelCap) cpage[i] = pg;
+          if (i < kSelCap) {
+            if (RUNS) ckey[i] = make_key(lb, pg);
+            else cpage[i] = pg;
+          }
+          if (RUNS) width = fmaxf(width, __fsub_ru(unorder_bits(ub), unorder_bits(lb)));
         }
       });
     }
@@ -662,35 +678,113 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
       __syncthreads();
       continue;
     }
-    // a group of four lanes per candidate, 32 candidates per round, all physical page ids in one round trip
-    // (through shared memory: with four rounds' ids in registers the loop was unrolled, spilled, and a whole step
-    // took 1 us longer with one 8K sequence, 2 us with eight of 32K)
-    int* cphys = sm.r.cphys;
-    for (int i = tid; i < ncand; i += kSelThreads) cphys[i] = phys_of(cpage[i]);
-    __syncthreads();
-    constexpr int kPer = kSelThreads / 4;
-#pragma unroll 1
-    for (int i0 = 0; i0 < ncand; i0 += kPer) {           // uniform over the CTA
-      const int i = i0 + tid / 4, ic = min(i, ncand - 1);
-      const float e = exact_at(cphys[ic]);
-      if (u == 0 && i < ncand) ckey[i] = make_key(order_bits(e), cpage[i]);
-    }
-    // ---- order the candidates (descending) and emit the first kk
-    __syncthreads();
-    if (ncand <= kSelThreads) {
-      // few candidates (the usual case): a candidate's position is the number of larger keys (all
-      // keys differ); one candidate per thread, the keys are read as broadcasts, four at a time
-      if ((tid & ~31) < ncand) {                       // whole warps without a candidate skip the count
-        const unsigned long long mine = tid < ncand ? ckey[tid] : ~0ull;
-        int rank = 0;
-        const int n4 = ncand & ~3;
-        for (int i = 0; i < n4; i += 4) {
-          const ulonglong2 k01 = *reinterpret_cast<const ulonglong2*>(&ckey[i]);
-          const ulonglong2 k23 = *reinterpret_cast<const ulonglong2*>(&ckey[i + 2]);
-          rank += (k01.x > mine ? 1 : 0) + (k01.y > mine ? 1 : 0) + (k23.x > mine ? 1 : 0) + (k23.y > mine ? 1 : 0);
+    if constexpr (RUNS) {
+      // The candidates in descending order of their lower bounds.  No pair of bounds is wider than `width`: where a lower bound
+      // lies more than that below the one before it, everything from there on scores below everything before.  Only within a run
+      // of closer ones does the order need exact scores: 20 of 67 candidates at 64 pages per list (see refine_runs).
+      constexpr int kPer = kSelThreads / 4;
+      const bool all_exact = ncand <= kPer;                  // a single round is not worth the sorting
+      const unsigned long long* by_bound = all_exact ? ckey : sm.r.skey;
+      unsigned long long* exact = all_exact ? sm.r.skey : ckey;
+      int nclose = ncand;
+      if (!all_exact) {
+        const uint32_t wide = __reduce_max_sync(0xffffffffu, __float_as_uint(width));        // (not negative: ordered like its bits)
+        if (lane == 0) atomicMax(&sm.r.width, wide);
+        if (ncand <= kSelThreads) {
+          // a candidate's position is the number of larger keys (all differ); one candidate per thread, the keys are read as
+          // broadcasts, four at a time
+          if ((tid & ~31) < ncand) {                         // whole warps without a candidate skip the count
+            const unsigned long long mine = tid < ncand ? ckey[tid] : ~0ull;
+            int rank = 0;
+            const int n4 = ncand & ~3;
+            for (int i = 0; i < n4; i += 4) {
+              const ulonglong2 k01 = *reinterpret_cast<const ulonglong2*>(&ckey[i]);
+              const ulonglong2 k23 = *reinterpret_cast<const ulonglong2*>(&ckey[i + 2]);
+              rank += (k01.x > mine ? 1 : 0) + (k01.y > mine ? 1 : 0) + (k23.x > mine ? 1 : 0) + (k23.y > mine ? 1 : 0);
+            }
+            for (int i = n4; i < ncand; ++i) rank += ckey[i] > mine ? 1 : 0;
+            if (tid < ncand) sm.r.skey[rank] = mine;
+          }
+        } else {
+          int n2 = 2;
+          while (n2 < ncand) n2 <<= 1;
+          for (int i = ncand + tid; i < n2; i += kSelThreads) ckey[i] = 0ull;
+          __syncthreads();
+          for (int k2 = 2; k2 <= n2; k2 <<= 1) {
+            for (int j = k2 >> 1; j > 0; j >>= 1) {
+              for (int t = tid; t < (n2 >> 1); t += kSelThreads) {
+                const int i = ((t & ~(j - 1)) << 1) | (t & (j - 1));
+                const int x = i | j;
+                const unsigned long long ka = ckey[i], kb = ckey[x];
+                if ((ka < kb) == ((i & k2) == 0)) { ckey[i] = kb; ckey[x] = ka; }
+              }
+              __syncthreads();
+            }
+          }
+          for (int i = tid; i < ncand; i += kSelThreads) sm.r.skey[i] = ckey[i];
         }
-        for (int i = n4; i < ncand; ++i) rank += ckey[i] > mine ? 1 : 0;
-        if (tid < ncand && rank < kk) {
+        __syncthreads();
+        width = __uint_as_float(sm.r.width);
+        for (int r0 = warp * 32; r0 < ncand; r0 += kSelThreads) {
+          const int r = r0 + lane;
+          auto lower = [&](int i) { return unorder_bits(static_cast<uint32_t>(by_bound[i] >> 32)); };
+          auto starts = [&](int i) { return i == 0 || lower(i - 1) > __fadd_ru(lower(i), width); };
+          const bool in = r < ncand, first = in && starts(r), last = in && (r + 1 == ncand || starts(r + 1));
+          const bool open = in && (out_scores || !(first && last));
+          const uint32_t runs = __ballot_sync(0xffffffffu, first), opens = __ballot_sync(0xffffffffu, open);
+          int at = 0;
+          if (lane == 0) {
+            sm.r.run[r0 / 32] = runs;
+            if (opens) at = atomicAdd(&sm.r.nclose, __popc(opens));
+          }
+          at = __shfl_sync(0xffffffffu, at, 0) + __popc(opens & ((1u << lane) - 1u));
+          if (open) sm.r.close[at] = static_cast<uint16_t>(r);
+        }
+        __syncthreads();
+        nclose = sm.r.nclose;
+      }
+      auto position = [&](int i) { return all_exact ? i : static_cast<int>(sm.r.close[i]); };
+      auto page_at = [&](int r) { return static_cast<int>(~reinterpret_cast<const uint32_t*>(by_bound)[2 * r]); };     // (a key's low word)
+      int r_next = 0, pg_next = 0, ph_next = 0;
+      if (nclose > 0) {
+        r_next = position(min(tid / 4, nclose - 1));
+        pg_next = page_at(r_next);
+        ph_next = phys_of(pg_next);
+      }
+#pragma unroll 1
+      for (int i = tid / 4; i - tid / 4 < nclose; i += kPer) {      // uniform over the CTA
+        const int r = r_next, pg = pg_next, ph = ph_next;
+        if (i - tid / 4 + kPer < nclose) {                  // (the next round's pages are looked up beside this one's scores)
+          r_next = position(min(i + kPer, nclose - 1));
+          pg_next = page_at(r_next);
+          ph_next = phys_of(pg_next);
+        }
+        const float e = exact_at(ph);
+        if (u == 0 && i < nclose) exact[r] = make_key(order_bits(e), pg);
+      }
+      __syncthreads();
+      // ---- a candidate's position: its run's, and the number of larger keys in the run (all differ); emit the first kk
+      for (int r = tid; r < ncand; r += kSelThreads) {
+        int start = 0, end = ncand;
+        if (!all_exact) {
+          int w = r >> 5;
+          uint32_t b = sm.r.run[w] & (0xffffffffu >> (31 - (r & 31)));
+          while (b == 0u) b = sm.r.run[--w];
+          start = w * 32 + 31 - __clz(b);
+          if (start >= kk) continue;
+          w = r >> 5;
+          b = sm.r.run[w] & (0xfffffffeu << (r & 31));
+          const int nw = (ncand + 31) >> 5;
+          while (b == 0u && ++w < nw) b = sm.r.run[w];
+          if (b) end = w * 32 + __ffs(b) - 1;
+        }
+        unsigned long long mine = by_bound[r];
+        int rank = start;
+        if (all_exact || end - start > 1 || out_scores) {
+          mine = exact[r];
+          for (int i = start; i < end; ++i) rank += exact[i] > mine ? 1 : 0;
+        }
+        if (rank < kk) {
           const int pg = static_cast<int32_t>(0xffffffffu - static_cast<uint32_t>(mine));
           for (int gi = 0; gi < pool; ++gi) {
             out_pages[gi * p.k + rank] = pg;
@@ -702,30 +796,71 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
       for (int gi = 0; gi < pool; ++gi)
         for (int j = kk + tid; j < p.k; j += kSelThreads) out_pages[gi * p.k + j] = -1;
     } else {
-      int n2 = 2;
-      while (n2 < ncand) n2 <<= 1;
-      for (int i = ncand + tid; i < n2; i += kSelThreads) ckey[i] = 0ull;
+      // a group of four lanes per candidate, 32 candidates per round, all physical page ids in one round trip
+      // (through shared memory: with four rounds' ids in registers the loop was unrolled, spilled, and a whole step
+      // took 1 us longer with one 8K sequence, 2 us with eight of 32K)
+      int* cphys = sm.r.cphys;
+      for (int i = tid; i < ncand; i += kSelThreads) cphys[i] = phys_of(cpage[i]);
       __syncthreads();
-      for (int k2 = 2; k2 <= n2; k2 <<= 1) {
-        for (int j = k2 >> 1; j > 0; j >>= 1) {
-          for (int t = tid; t < (n2 >> 1); t += kSelThreads) {
-            const int i = ((t & ~(j - 1)) << 1) | (t & (j - 1));
-            const int x = i | j;
-            const unsigned long long ka = ckey[i], kb = ckey[x];
-            if ((ka < kb) == ((i & k2) == 0)) { ckey[i] = kb; ckey[x] = ka; }
-          }
-          __syncthreads();
-        }
+      constexpr int kPer = kSelThreads / 4;
+#pragma unroll 1
+      for (int i0 = 0; i0 < ncand; i0 += kPer) {           // uniform over the CTA
+        const int i = i0 + tid / 4, ic = min(i, ncand - 1);
+        const float e = exact_at(cphys[ic]);
+        if (u == 0 && i < ncand) ckey[i] = make_key(order_bits(e), cpage[i]);
       }
-      for (int gi = 0; gi < pool; ++gi) {
-        for (int j = tid; j < p.k; j += kSelThreads) {
-          if (j < kk) {
-            const unsigned long long key = ckey[j];
-            out_pages[gi * p.k + j] = static_cast<int32_t>(0xffffffffu - static_cast<uint32_t>(key));
-            if (out_scores) out_scores[gi * p.k + j] = unorder_bits(static_cast<uint32_t>(key >> 32));
-            if (gi == 0) mark(static_cast<int32_t>(0xffffffffu - static_cast<uint32_t>(key)));
-          } else {
-            out_pages[gi * p.k + j] = -1;
+      // ---- order the candidates (descending) and emit the first kk
+      __syncthreads();
+      if (ncand <= kSelThreads) {
+        // few candidates (the usual case): a candidate's position is the number of larger keys (all
+        // keys differ); one candidate per thread, the keys are read as broadcasts, four at a time
+        if ((tid & ~31) < ncand) {                       // whole warps without a candidate skip the count
+          const unsigned long long mine = tid < ncand ? ckey[tid] : ~0ull;
+          int rank = 0;
+          const int n4 = ncand & ~3;
+          for (int i = 0; i < n4; i += 4) {
+            const ulonglong2 k01 = *reinterpret_cast<const ulonglong2*>(&ckey[i]);
+            const ulonglong2 k23 = *reinterpret_cast<const ulonglong2*>(&ckey[i + 2]);
+            rank += (k01.x > mine ? 1 : 0) + (k01.y > mine ? 1 : 0) + (k23.x > mine ? 1 : 0) + (k23.y > mine ? 1 : 0);
+          }
+          for (int i = n4; i < ncand; ++i) rank += ckey[i] > mine ? 1 : 0;
+          if (tid < ncand && rank < kk) {
+            const int pg = static_cast<int32_t>(0xffffffffu - static_cast<uint32_t>(mine));
+            for (int gi = 0; gi < pool; ++gi) {
+              out_pages[gi * p.k + rank] = pg;
+              if (out_scores) out_scores[gi * p.k + rank] = unorder_bits(static_cast<uint32_t>(mine >> 32));
+            }
+            mark(pg);
+          }
+        }
+        for (int gi = 0; gi < pool; ++gi)
+          for (int j = kk + tid; j < p.k; j += kSelThreads) out_pages[gi * p.k + j] = -1;
+      } else {
+        int n2 = 2;
+        while (n2 < ncand) n2 <<= 1;
+        for (int i = ncand + tid; i < n2; i += kSelThreads) ckey[i] = 0ull;
+        __syncthreads();
+        for (int k2 = 2; k2 <= n2; k2 <<= 1) {
+          for (int j = k2 >> 1; j > 0; j >>= 1) {
+            for (int t = tid; t < (n2 >> 1); t += kSelThreads) {
+              const int i = ((t & ~(j - 1)) << 1) | (t & (j - 1));
+              const int x = i | j;
+              const unsigned long long ka = ckey[i], kb = ckey[x];
+              if ((ka < kb) == ((i & k2) == 0)) { ckey[i] = kb; ckey[x] = ka; }
+            }
+            __syncthreads();
+          }
+        }
+        for (int gi = 0; gi < pool; ++gi) {
+          for (int j = tid; j < p.k; j += kSelThreads) {
+            if (j < kk) {
+              const unsigned long long key = ckey[j];
+              out_pages[gi * p.k + j] = static_cast<int32_t>(0xffffffffu - static_cast<uint32_t>(key));
+              if (out_scores) out_scores[gi * p.k + j] = unorder_bits(static_cast<uint32_t>(key >> 32));
+              if (gi == 0) mark(static_cast<int32_t>(0xffffffffu - static_cast<uint32_t>(key)));
+            } else {
+              out_pages[gi * p.k + j] = -1;
+            }
           }
         }
       }
@@ -897,6 +1032,13 @@ int refine_slots(int lists, int resident, int block_size) {
   return std::min(slots, block_size);
 }
 
+// Exact scores only where the bounds leave the order open (RUNS), or for every candidate.  The former saves two rounds of
+// gathers out of three at 64 pages per list (eight 32K prompts: 29 MB of summaries out of L2, 4.6 us of a list's 11.7; 20 of 67
+// candidates are close) and costs a sort on the bounds.  It pays where many lists share L2's bandwidth, or a score is the largest of a
+// group's.  Whole step, us, without and with it: 256 lists of 64 pages 108.3 / 105.9, 32 pooled lists of 64 71.4 / 70.8; 32 lists of 32
+// pages 35.7 / 36.2, 32 lists of 64 out of 2,048 pages 47.4 / 48.7.
+bool refine_runs(int lists, int pool, int k) { return k >= 48 && (pool > 1 || lists >= 128); }
+
 bool selects_by_refinement(const losa_ctx* c, int32_t k, int selector) {
   return c->shape.dtype == LOSA_BF16 && (selector == kSelectorExact || selector == kSelectorPooled) && k <= kSelCap &&
          c->shape.max_pages_per_seq > 0;
@@ -954,8 +1096,10 @@ int32_t launch_page_scores_topk(losa_ctx* c, const void* q, const losa_kv_t* kv,
     with_block_attn_shape(sh, [&](auto d, auto bk) {
       constexpr int D = decltype(d)::value, BK = decltype(bk)::value;
       const int split = in_step ? cudaSharedmemCarveoutMaxShared : cudaSharedmemCarveoutDefault;
-      if (pool > 1) launch_split(split, topk_refine_kernel<D, true, BK>, grid, kSelThreads, 0, st, rp, bp);
-      else launch_split(split, topk_refine_kernel<D, false, BK>, grid, kSelThreads, 0, st, rp, bp);
+      auto launch = [&](auto kernel) { launch_split(split, kernel, grid, kSelThreads, 0, st, rp, bp); };
+      const bool runs = refine_runs(lists, pool, k);
+      if (pool > 1) launch(runs ? topk_refine_kernel<D, true, BK, true> : topk_refine_kernel<D, true, BK, false>);
+      else launch(runs ? topk_refine_kernel<D, false, BK, true> : topk_refine_kernel<D, false, BK, false>);
     });
     return after_launch(c);
   }
