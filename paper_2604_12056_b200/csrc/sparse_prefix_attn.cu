@@ -418,7 +418,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
                                   CUtensorMapFloatOOBfill);
 
-int32_t encode_pool_map(losa_ctx* c, unsigned char* blob, const void* pool, const losa_kv_t* kv, bool is_v) {
+int32_t encode_pool_map(losa_ctx* c, unsigned char* blob, const void* pool, const losa_kv_t* kv, bool plain) {
   const losa_shape_t& sh = c->shape;
   if (!c->encode_fn) {
     void* fn = nullptr;
@@ -430,7 +430,7 @@ int32_t encode_pool_map(losa_ctx* c, unsigned char* blob, const void* pool, cons
   const cuuint64_t dims[4] = {static_cast<cuuint64_t>(sh.head_dim), static_cast<cuuint64_t>(sh.page_size),
                               static_cast<cuuint64_t>(sh.n_kv_heads), static_cast<cuuint64_t>(kv->n_phys_pages)};
   // bf16 pages: 64-element (128-byte) boxes with the 128-byte swizzle, as the MMA descriptors expect them;
-  // FP8 pages: whole rows of d bytes; K swizzled over the row (an MMA operand), V as it lies (the kernel converts it)
+  // FP8 pages: whole rows of d bytes; swizzled over the row (an MMA operand), or as they lie (V that the kernel converts)
   const bool fp8 = kv->kv_format == LOSA_KV_FP8_E4M3;
   const cuuint64_t es = fp8 ? 1 : 2;
   const cuuint64_t strides[3] = {static_cast<cuuint64_t>(kv->stride_tok) * es, static_cast<cuuint64_t>(kv->stride_head) * es,
@@ -440,7 +440,7 @@ int32_t encode_pool_map(losa_ctx* c, unsigned char* blob, const void* pool, cons
   const CUresult r = reinterpret_cast<EncodeTiledFn>(c->encode_fn)(
       reinterpret_cast<CUtensorMap*>(blob), fp8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4,
       const_cast<void*>(pool), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-      fp8 && is_v ? CU_TENSOR_MAP_SWIZZLE_NONE : (fp8 && sh.head_dim == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B),
+      fp8 && plain ? CU_TENSOR_MAP_SWIZZLE_NONE : (fp8 && sh.head_dim == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B),
       CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     c->last_cuda_error = static_cast<int32_t>(r);
@@ -458,6 +458,8 @@ int32_t ensure_tensor_maps(losa_ctx* c, const losa_kv_t* kv) {
   int32_t rc = encode_pool_map(c, c->tmap_k, kv->k_pages, kv, false);
   if (rc != LOSA_OK) return rc;
   rc = encode_pool_map(c, c->tmap_v, kv->v_pages, kv, true);
+  if (rc != LOSA_OK) return rc;
+  rc = encode_pool_map(c, c->tmap_vs, kv->v_pages, kv, false);
   if (rc != LOSA_OK) return rc;
   c->tmap_key_k = kv->k_pages;
   c->tmap_key_v = kv->v_pages;
@@ -488,11 +490,17 @@ int32_t prepare_tc5(losa_ctx* c) {
   static_assert(smem <= kSmemBudget, "shared memory of the stage-4 kernel");
   constexpr int bit = FP8 ? 2 : 1;  // a context has one shape on one device: one instantiation per cache format
   if (c->attn_attr_set & bit) return LOSA_OK;
-  LOSA_CUDA_TRY(c, cudaFuncSetAttribute(attn_tc5_kernel<D, GP, FP8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  // the kernel moves registers between its warps: a build that is launched with fewer than it deals out would wait for ever
-  cudaFuncAttributes fa;
-  LOSA_CUDA_TRY(c, cudaFuncGetAttributes(&fa, attn_tc5_kernel<D, GP, FP8>));
-  if (fa.numRegs < (FP8 ? kTc5LaunchRegs8 : kTc5LaunchRegs)) return LOSA_ERR_UNSUPPORTED;
+  auto set = [&](auto kernel) -> int32_t {
+    LOSA_CUDA_TRY(c, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    // the kernel moves registers between its warps: a build that is launched with fewer than it deals out would wait for ever
+    cudaFuncAttributes fa;
+    LOSA_CUDA_TRY(c, cudaFuncGetAttributes(&fa, kernel));
+    return fa.numRegs < (FP8 ? kTc5LaunchRegs8 : kTc5LaunchRegs) ? LOSA_ERR_UNSUPPORTED : LOSA_OK;
+  };
+  int32_t rc = set(attn_tc5_kernel<D, GP, FP8, false>);
+  if constexpr (FP8 && D == 128)
+    if (rc == LOSA_OK) rc = set(attn_tc5_kernel<D, GP, FP8, true>);
+  if (rc != LOSA_OK) return rc;
   c->attn_attr_set |= bit;
   return LOSA_OK;
 }
@@ -510,11 +518,20 @@ int32_t prepare_f32(losa_ctx* c) {
 
 template <int D, int GP, bool FP8>
 int32_t launch_tc5(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool with_combine) {
-  CUtensorMap mk, mv;
+  CUtensorMap mk, mv, mvs;
   memcpy(&mk, c->tmap_k, sizeof(mk));
   memcpy(&mv, c->tmap_v, sizeof(mv));
+  memcpy(&mvs, c->tmap_vs, sizeof(mvs));
   if (c->profile) LOSA_CUDA_TRY(c, cudaEventRecord(c->ev_begin, st));
-  launch_k(attn_tc5_kernel<D, GP, FP8>, ap.n_ctas, tc5_threads<FP8>(), tc5_smem_bytes<D, GP, FP8>(), st, mk, mv, ap);
+  // With the narrow path where shares of eight groups of 128 tokens, its least, are to be expected: a sparse step lists about a quarter of a
+  // cache.  The kernel that has it starts 1.5 us later on the other path (2,600 tokens, a step 63 us, 65 with it).
+  auto launch = [&](auto kernel) { launch_k(kernel, ap.n_ctas, tc5_threads<FP8>(), tc5_smem_bytes<D, GP, FP8>(), st, mk, mv, mvs, ap); };
+  bool narrow = false;
+  if constexpr (FP8 && D == 128) {
+    narrow = static_cast<int64_t>(ap.n_sk) * ap.Pmax * GP >= static_cast<int64_t>(ap.n_ctas) * 4 * 8 * kTc5Tok;
+    if (narrow) launch(attn_tc5_kernel<D, GP, FP8, true>);
+  }
+  if (!narrow) launch(attn_tc5_kernel<D, GP, FP8, false>);
   if (c->profile) LOSA_CUDA_TRY(c, cudaEventRecord(c->ev_end, st));
   int32_t rc = after_launch(c);
   if (rc != LOSA_OK || !with_combine) return rc;

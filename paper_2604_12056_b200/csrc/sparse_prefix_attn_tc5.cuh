@@ -22,19 +22,22 @@
 
 constexpr int kTc5Sets = 3, kTc5SetWarps = 4;    // sets of softmax warps: set h takes every third group, thread = one query row
 constexpr int kTc5SoftmaxWarps = kTc5Sets * kTc5SetWarps;
+constexpr int kTc5ScaleWarps = 2 * kTc5SetWarps; // FP8: softmax warps that look at the value scales before a share begins
 constexpr int kTc5QkWarp = 12, kTc5PvWarp = 13, kTc5KWarp = 14, kTc5VWarp = 15;
 constexpr int kTc5CvtWarp = 16, kTc5CvtWarps = 4; // FP8 pages: four warps that convert V
 template <bool FP8> constexpr int tc5_threads() { return FP8 ? 640 : 512; }
 // Registers per thread at the launch, and as they are dealt out to the softmax warps and the others:
-// 12 x 32 x 136 + 4 x 32 x 104 = 512 x 128; FP8 12 x 32 x 112 + 8 x 32 x 72 = 640 x 96.
+// 12 x 32 x 136 + 4 x 32 x 104 = 512 x 128; FP8 12 x 32 x 112 + 8 x 32 x 72 = 640 x 96;
+// with the narrow path, whose producers would spill at 72 and are then late with every copy, 104 and 80.
 constexpr int kTc5LaunchRegs = 128, kTc5SoftmaxRegs = 136, kTc5OtherRegs = 104;
-constexpr int kTc5LaunchRegs8 = 96, kTc5SoftmaxRegs8 = 112, kTc5OtherRegs8 = 72;
+constexpr int kTc5LaunchRegs8 = 96, kTc5SoftmaxRegs8 = 112, kTc5OtherRegs8 = 72, kTc5nSoftmaxRegs = 104, kTc5nOtherRegs = 80;
 static_assert(kTc5SoftmaxWarps * kTc5SoftmaxRegs + 4 * kTc5OtherRegs <= 16 * kTc5LaunchRegs, "registers");
 static_assert(kTc5SoftmaxWarps * kTc5SoftmaxRegs8 + 8 * kTc5OtherRegs8 <= 20 * kTc5LaunchRegs8, "registers, FP8");
+static_assert(kTc5SoftmaxWarps * kTc5nSoftmaxRegs + 8 * kTc5nOtherRegs <= 20 * kTc5LaunchRegs8, "registers, FP8 with the narrow path");
 constexpr int kTc5Tok = 128;                     // tokens per group = N of Q K^T = columns of one S buffer
 constexpr float kTc5Tau = 8.0f;                  // reference maximum moves only when it would grow by more than this (log2 units)
 // Reference maxima [set][row]; row sums and the references they are relative to [piece parity][set][row]
-constexpr int kTc5XchgBytes = 5 * kTc5Sets * kRowsPerGroup * 4;
+template <bool FP8> constexpr int tc5_xchg_bytes() { return (5 * kTc5Sets * kRowsPerGroup + (FP8 ? 512 : 0)) * 4; }     // (FP8: the narrow path's need more)
 // FP8 pages: binary places by which P is held above the reference maximum.  P stays below 2^(8 + 7) < 65504.
 constexpr float kTc5Fp8Lift = 7.0f;
 constexpr int kTc5StgMax = 20;                   // FP8 pages: staging slots of V, one page each, at most
@@ -49,9 +52,9 @@ constexpr int kTc5VmulRing = 64;
 // hence P V of group g - NRK - 3 has released its S buffer: group g - NRK - 2 may still be read.
 constexpr int kTc5MetaRing = 16;
 // Barriers, the segment prefix and index cache, the exchange arrays, the charged prefix, the staging
-// barriers (landed, emptied) and the value pages' multipliers, two words per page of the meta ring
-template <int GP> constexpr int tc5_tail_bytes() {
-  return kTailBytes + kTc5XchgBytes + (kMaxSegments + 2) * 4 + kTc5StgMax * (8 + 8) + kTc5VmulRing * 4 + kTc5MetaRing * (kTc5Tok / GP) * 8;
+// barriers (landed, emptied) and the value pages' multipliers, two words per page of the meta ring (FP8: three)
+template <int GP, bool FP8> constexpr int tc5_tail_bytes() {
+  return kTailBytes + tc5_xchg_bytes<FP8>() + (kMaxSegments + 2) * 4 + kTc5StgMax * (8 + 8) + kTc5VmulRing * 4 + kTc5MetaRing * (kTc5Tok / GP) * (FP8 ? 12 : 8) + (FP8 ? 2 * kTc5ScaleWarps * 4 : 0);
 }
 
 // Shared memory: the Q tile (FP8: one tile of codes per term), a ring of group-sized slots for K and one for V, FP8: a
@@ -59,23 +62,41 @@ template <int GP> constexpr int tc5_tail_bytes() {
 template <int D> constexpr int tc5_slot_bytes() { return kTc5Tok * D * 2; }                              // V, and bf16 K
 template <int D, bool FP8> constexpr int tc5_kslot_bytes() { return kTc5Tok * D * (FP8 ? 1 : 2); }
 constexpr int kTc5QTerms = 3;                    // FP8: E5M2 terms of a query
-template <int D, bool FP8> constexpr int tc5_q_bytes() { return kRowsPerGroup * D * (FP8 ? kTc5QTerms : 2); }
+constexpr int kTc5nRows = 16;                    // FP8: most query rows of a share on the narrow path (sparse_prefix_attn_tc5n.cuh)
+constexpr int kTc5nLanes = 32;                   // entries of its per-row arrays, one per lane
+constexpr int kTc5nP = kTc5Tok * 16;             // bytes of one term of 16 rows of its P'
+constexpr int kTc5PTerms = 3;                    // E5M2 terms of P'
+constexpr float kTc5nLift = 11.0f, kTc5nTop = 15.0f;   // binary places by which P' is held above the reference, and by which it may outgrow it
+constexpr int tc5n_p_bytes() { return kTc5PTerms * kTc5nP; }
+template <int D> constexpr int tc5n_q_bytes() { return kTc5nRows * D * kTc5QTerms; }
+// The Q tile; narrow: in its place a smaller one and a set of P' terms for each set of softmax warps
+template <int D, bool FP8> constexpr int tc5_q_bytes() {
+  if (!FP8) return kRowsPerGroup * D * 2;
+  static_assert(D == 64 || kRowsPerGroup * D * kTc5QTerms >= tc5n_q_bytes<D>() + kTc5Sets * tc5n_p_bytes(), "the narrow path's tiles (d = 128) fit");
+  return kRowsPerGroup * D * kTc5QTerms;
+}
 template <int D, int GP, bool FP8> constexpr int tc5_ring_slots(bool v) {
   if (FP8) return v ? 2 : (D == 128 ? 3 : 6);                   // the staging slots take the rest
-  const int n = (kSmemBudget - 1024 - tc5_tail_bytes<GP>() - tc5_q_bytes<D, false>()) / tc5_slot_bytes<D>();
+  const int n = (kSmemBudget - 1024 - tc5_tail_bytes<GP, FP8>() - tc5_q_bytes<D, false>()) / tc5_slot_bytes<D>();
   const int own = v ? n / 2 : (n + 1) / 2;                      // K is ahead of V by the S buffers
   return own > 6 ? 6 : own;
 }
 // FP8: pages of the staging ring of V: what the ring slots leave, up to five groups
 template <int D, int GP> constexpr int tc5_stg_slots() {
-  const int fit = (kSmemBudget - 1024 - tc5_tail_bytes<GP>() - tc5_q_bytes<D, true>() - tc5_ring_slots<D, GP, true>(false) * tc5_kslot_bytes<D, true>() -
+  const int fit = (kSmemBudget - 1024 - tc5_tail_bytes<GP, true>() - tc5_q_bytes<D, true>() - tc5_ring_slots<D, GP, true>(false) * tc5_kslot_bytes<D, true>() -
                    tc5_ring_slots<D, GP, true>(true) * tc5_slot_bytes<D>()) / (GP * D), five = 5 * (kTc5Tok / GP);
   const int n = fit < five ? fit : five;
   return n < kTc5StgMax ? n : kTc5StgMax;
 }
+// FP8, narrow: the same memory as slots of a group's codes, half of them for K and half for V
+template <int D, int GP> constexpr int tc5n_slots() {
+  const int n = (tc5_ring_slots<D, GP, true>(false) * tc5_kslot_bytes<D, true>() + tc5_ring_slots<D, GP, true>(true) * tc5_slot_bytes<D>() +
+                 tc5_stg_slots<D, GP>() * GP * D) / (2 * tc5_kslot_bytes<D, true>());
+  return n < 6 ? n : 6;
+}
 template <int D, int GP, bool FP8> constexpr int tc5_smem_bytes() {
   return 1024 + tc5_q_bytes<D, FP8>() + tc5_ring_slots<D, GP, FP8>(false) * tc5_kslot_bytes<D, FP8>() + tc5_ring_slots<D, GP, FP8>(true) * tc5_slot_bytes<D>() +
-         (FP8 ? tc5_stg_slots<D, GP>() * GP * D : 0) + tc5_tail_bytes<GP>();
+         (FP8 ? tc5_stg_slots<D, GP>() * GP * D : 0) + tc5_tail_bytes<GP, FP8>();
 }
 
 // Shared-memory matrix descriptor: 128-byte swizzle, 8-row groups 1024 bytes apart; lbo = distance
@@ -185,6 +206,8 @@ __device__ __forceinline__ void tc5_wait_st() { asm volatile("tcgen05.wait::st.s
 // byte offset of 16-byte chunk c (0..7) of row t in a [rows][128 B] tile with the 128-byte swizzle
 __device__ __forceinline__ uint32_t tc5_sw(int t, int c) { return static_cast<uint32_t>(t * 128 + ((c ^ (t & 7)) << 4)); }
 
+#include "sparse_prefix_attn_tc5n.cuh"
+
 // FP8: the K / V pools hold E4M3 bytes with one power-of-two scale per (page, KV head).  K is an operand as
 // it lies: Q goes to shared memory as three E5M2 tiles whose sum is the bf16 query under a power of two of the row, and each is
 // multiplied with the codes by kind::f8f6f4, at twice the 16-bit rate and with fp32 sums.  A term takes three significant bits and
@@ -192,8 +215,8 @@ __device__ __forceinline__ uint32_t tc5_sw(int t, int c) { return static_cast<ui
 // 2^15 .. 2^16 that is exact down to 2^-9, 2^-24 of the largest, and below to within 2^-17, 2^-32 of it - more than the fp16
 // value of an element keeps in a row below 256.  (Two E4M3 terms lose an element's low bits from 2^-9 of the row's largest
 // on: with them the block of eight 32K prompts takes 954 us, 976 with three.  That is the third product; the slot of K's ring that its
-// tile takes at d = 128 costs nothing: four slots and fewer staging pages are no faster.)  V cannot: P needs more than three terms.
-// Its codes land in a staging ring as they lie in memory; four converting warps, one per scheduler, turn a
+// tile takes at d = 128 costs nothing: four slots and fewer staging pages are no faster.)  V is one on the narrow path only (P costs three terms there as well).  Here
+// its codes land in a staging ring as they lie in memory; four converting warps, one per scheduler, turn a
 // landed page into fp16 (exact) in the group's ring slot, in the layout the tensor maps of the bf16 path
 // produce, and P is fp16.  The scales stay out of the conversion, which is bound by its instruction count: the
 // key scale joins the softmax scale of the page's columns, and the value scale 2^e is added to their
@@ -205,12 +228,15 @@ __device__ __forceinline__ uint32_t tc5_sw(int t, int c) { return static_cast<ui
 // the reference lies 2^7 below the maximum.  A weight is then subnormal only 2^-15 or more below its row's
 // largest, 2^-14 without scales.  Staging slots are single pages, so that one is refilled while its
 // neighbours are converted.
-template <int D, int GP, bool FP8>
+// NARROW: with the narrow path (chosen by launch_tc5 on the size of the cache).
+template <int D, int GP, bool FP8, bool NARROW>
 __global__ void __launch_bounds__(tc5_threads<FP8>(), 1)
-attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, AttnParams p) {
+attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmVs, AttnParams p) {
   constexpr int NRK = tc5_ring_slots<D, GP, FP8>(false), NRV = tc5_ring_slots<D, GP, FP8>(true);   // slots per ring
   constexpr int NSP = FP8 ? tc5_stg_slots<D, GP>() : 1, STG = GP * D;   // FP8: staging slots of V, bytes of a slot (one page of codes)
   constexpr int NT = tc5_threads<FP8>();
+  static_assert(!NARROW || (FP8 && D == 128), "the narrow path");   // (d = 64: a group's bytes are HBM's 675 cycles, less than that path's own)
+  constexpr int NN = NARROW ? tc5n_slots<D, GP>() : 1;   // narrow: slots of K, and of V
   constexpr int KSLOT = tc5_kslot_bytes<D, FP8>(), SLOT = tc5_slot_bytes<D>(), QB = tc5_q_bytes<D, FP8>();
   constexpr int PG = kTc5Tok / GP;              // pages per group
   constexpr int MR = kTc5MetaRing;              // groups of the meta ring
@@ -227,8 +253,9 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   // A converting warp waits on the parity of a staging slot whose page before, NSP pages back, another warp may have taken: that page
   // has to lie two groups back at least, where all four warps have finished (less than two groups lie between them).
   static_assert(!FP8 || (NSP >= 2 * PG && NSP <= kTc5StgMax), "staging ring");
-  static_assert(NRK + 2 < MR, "the producer's lead fits the meta ring");
-  constexpr int kBars = 4 * 6 + 3 * SB + 3 + 4 + 4 * SB + 2;
+  static_assert(NRK + 2 < MR && NN + 3 < MR, "the producer's lead fits the meta ring");   // (narrow: a set reads the ring until it leaves P')
+  static_assert(!NARROW || (NN >= 2 && NN * 2 * KSLOT <= NRK * KSLOT + NRV * SLOT + NSP * STG), "narrow: slots");
+  constexpr int kBars = 4 * 6 + 3 * SB + 3 + 4 + 4 * SB + 2 + 2 * SB + 2;
   static_assert(8 * kBars + 16 <= 512, "tail layout");
 
   extern __shared__ uint8_t smem_raw[];
@@ -239,10 +266,11 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   constexpr int TAIL = QB + NRK * KSLOT + NRV * SLOT + (FP8 ? NSP * STG : 0);
   uint8_t* tail = gen + TAIL;
   const uint32_t tail_s = base + TAIL;
-  const uint32_t kfull = tail_s, kfree = kfull + 8 * NRK, vfull = kfree + 8 * NRK, vfree = vfull + 8 * NRV;
-  const uint32_t s_full = vfree + 8 * NRV, s_free = s_full + 8 * SB, p_full = s_free + 8 * SB, q_full = p_full + 8 * SB, q_free = q_full + 8, o_free = q_free + 8;
+  const uint32_t kfull = tail_s, kfree = kfull + 8 * 6, vfull = kfree + 8 * 6, vfree = vfull + 8 * 6;     // (room for six slots each)
+  const uint32_t s_full = vfree + 8 * 6, s_free = s_full + 8 * SB, p_full = s_free + 8 * SB, q_full = p_full + 8 * SB, q_free = q_full + 8, o_free = q_free + 8;
   const uint32_t xbar = o_free + 8, mbar = xbar + 32;     // per lane quarter: the sets meet; [set][quarter]: a group's reference is published
   const uint32_t drain_bar = mbar + 32 * SB;            // two barriers: the issuing threads' last commit when the CTA gives up
+  const uint32_t s_read = drain_bar + 16, meet = s_read + 8 * SB, piece_meet = meet + 8 * SB, path_bar = piece_meet + 8;   // FP8, narrow path
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 8 * kBars);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(const_cast<int*>(abort_flag) + 1);
   int* pre = reinterpret_cast<int*>(tail + 512);
@@ -252,7 +280,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   float* mref = reinterpret_cast<float*>(len_s + kStageSeq);   // [set][128]
   float* xsum = mref + SB * kRowsPerGroup;                       // [piece parity][set][128]: row sums of a piece ...
   float* xref = xsum + 2 * SB * kRowsPerGroup;                   // ... and the references they are relative to
-  int* vpre = reinterpret_cast<int*>(xref + 2 * SB * kRowsPerGroup);  // prefix of the charged segment lengths (pages + pad)
+  int* vpre = reinterpret_cast<int*>(mref + tc5_xchg_bytes<FP8>() / 4);  // prefix of the charged segment lengths (pages + pad)
   // FP8: a staging slot's page has landed / has been converted
   const uint32_t vstg_full = smem_u32(vpre + kMaxSegments + 1) + 4;   // (kMaxSegments + 1 is odd)
   const uint32_t vstg_free = vstg_full + 8 * kTc5StgMax;
@@ -262,16 +290,17 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
   // per page of the groups in flight, [MR][PG]: valid tokens (FP8: and the exponent field of the value scale's part in P << 8), FP8: key scale
   volatile int* meta = vpre + kMaxSegments + 2 + 4 * kTc5StgMax + kTc5VmulRing;
   volatile float* kscale_meta = reinterpret_cast<volatile float*>(const_cast<int*>(meta) + MR * PG);
+  volatile float* vlog_meta = kscale_meta + MR * PG;           // narrow: the value scale's logarithm
   const bool staged = p.N * p.B <= kStageIdx && p.N <= kStageSeq;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = warp_uniform(tid >> 5);
   if (tid == 0) {
-    for (int i = 0; i < NRK; ++i) {
+    for (int i = 0; i < (NRK > NN ? NRK : NN); ++i) {
       mbar_init(kfull + 8 * i, 1);
       mbar_init(kfree + 8 * i, 1);
     }
-    for (int i = 0; i < NRV; ++i) {
-      mbar_init(vfull + 8 * i, FP8 ? kTc5CvtWarps : 1);   // the converting warps / the copies' bytes
+    for (int i = 0; i < (NRV > NN ? NRV : NN); ++i) {
+      mbar_init(vfull + 8 * i, FP8 ? kTc5CvtWarps : 1);   // the converting warps (narrow: as many arrivals by the producer) / the copies' bytes
       mbar_init(vfree + 8 * i, 1);
     }
     for (int b = 0; b < SB; ++b) {
@@ -284,6 +313,14 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     mbar_init(o_free, kTc5SoftmaxWarps);
     for (int i = 0; i < 4; ++i) mbar_init(xbar + 8 * i, kTc5Sets);
     for (int i = 0; i < 4 * SB; ++i) mbar_init(mbar + 8 * i, 1);
+    if (NARROW) {
+      for (int b = 0; b < SB; ++b) {
+        mbar_init(s_read + 8 * b, kTc5SetWarps);       // the set's scores have been read
+        mbar_init(meet + 8 * b, kTc5SetWarps);         // the set's warps meet
+      }
+      mbar_init(piece_meet, kTc5SoftmaxWarps);         // all of them, at the end of a piece
+      mbar_init(path_bar, kTc5ScaleWarps);           // the share's value scales have been looked at
+    }
     mbar_init(drain_bar, 1);
     mbar_init(drain_bar + 8, 1);
     if (FP8)
@@ -349,13 +386,38 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     return;
   }
   while (pre[sg0 + 1] <= lo) ++sg0;
-  auto n_active_of = [&](int s) { return staged ? na_s[s] : clamp_active(p.n_active[s], p.B); };
   auto kv_len_of = [&](int s) { return staged ? len_s[s] : p.kv_len[s]; };
-  auto token_of = [&](int s, int a) { return staged ? tok_s[s * p.B + a] : p.active_idx[s * p.B + a]; };
+
+  Tc5Cta cta;
+  cta.gen = gen; cta.base = base; cta.kring = kring; cta.vring = kring + NN * KSLOT;
+  cta.kfull = kfull; cta.kfree = kfree; cta.vfull = vfull; cta.vfree = vfree; cta.s_full = s_full; cta.s_free = s_free; cta.p_full = p_full;
+  cta.q_full = q_full; cta.q_free = q_free; cta.o_free = o_free; cta.s_read = s_read; cta.meet = meet; cta.piece_meet = piece_meet;
+  cta.abort_flag = abort_flag; cta.pre = pre; cta.tok_s = tok_s; cta.na_s = na_s; cta.staged = staged;
+  cta.scratch = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(mref) + 15) & ~static_cast<uintptr_t>(15));
+  cta.meta = meta; cta.kscale_meta = kscale_meta; cta.vlog_meta = vlog_meta; cta.tmem = tmem; cta.lo = lo; cta.hi = hi; cta.sg0 = sg0;
+  // A share of eight groups or more (a group costs 650 cycles less this way, the start 1.9 us more), few rows in all of
+  // its segments, and value scales (positive, of one size within a factor of four): tokens take the lanes (see the narrow path's
+  // header).  The scales are the last of three dependent reads, for the softmax warps, which look at them all, as for the
+  // producers, whose copies wait for the answer.
+  bool narrow = NARROW && hi - lo >= 8 * PG;
+  for (int sg = sg0; narrow && sg < p.n_seg && pre[sg] < hi; ++sg)
+    if (pre[sg + 1] > pre[sg]) narrow = cta.rows_of(p, sg) <= kTc5nRows;
+  const bool few_rows = narrow;
+  float* scale_lo = reinterpret_cast<float*>(const_cast<int*>(meta)) + 3 * MR * PG;      // [8] smallest and largest, per warp that looks
+  float* scale_hi = scale_lo + kTc5ScaleWarps;
+  auto choose_path = [&]() {                         // false: a wait has run out
+    if (!NARROW || !few_rows) return true;
+    if (!warp_mbar_wait(path_bar, 0, abort_flag, p.status, p.wait_cycles)) return false;
+    float a = INFINITY, b = 0.f;
+#pragma unroll
+    for (int w = 0; w < kTc5ScaleWarps; ++w) { a = fminf(a, scale_lo[w]); b = fmaxf(b, scale_hi[w]); }
+    narrow = a > 1e-18f && b < 1e18f && b <= 4.f * a;
+    return true;
+  };
 
   int issued = -1;                                   // producer warps: newest group (FP8: page) whose copies have been issued
   if (warp >= kTc5SoftmaxWarps) {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(FP8 ? kTc5OtherRegs8 : kTc5OtherRegs));   // whole warpgroups
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(NARROW ? kTc5nOtherRegs : FP8 ? kTc5OtherRegs8 : kTc5OtherRegs));   // whole warpgroups
   if (warp == kTc5KWarp || warp == kTc5VWarp) {
     // ------------------------------------------------------------------ producer warps: one for K, one for V
     // Lane j of a batch of 32 consecutive items resolves item -> logical page -> physical page (a
@@ -365,10 +427,19 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     // group's bytes, then every lane of the run issues its page.
     const bool is_v = warp == kTc5VWarp;
     const unsigned long long policy = l2_evict_first_policy();
-    const CUtensorMap* map = is_v ? &tmV : &tmK;
-    const uint32_t ring = is_v ? vring : kring, full0 = is_v ? vfull : kfull, free0 = is_v ? vfree : kfree;
-    auto slot_of = [&](int grp) { return is_v ? grp % NRV : grp % NRK; };
-    auto round_of = [&](int grp) { return is_v ? grp / NRV : grp / NRK; };
+    bool staging = false;                              // page by page, into the staging ring
+    const CUtensorMap* map = nullptr;
+    uint32_t ring = 0;
+    const uint32_t full0 = is_v ? vfull : kfull, free0 = is_v ? vfree : kfree;
+    auto start = [&]() {                               // before the first copies: which path, hence which slots
+      const bool ok = choose_path();
+      staging = FP8 && is_v && !narrow;
+      map = is_v ? (NARROW && narrow ? &tmVs : &tmV) : &tmK;
+      ring = is_v ? (NARROW && narrow ? cta.vring : vring) : kring;
+      return ok;
+    };
+    auto slot_of = [&](int grp) { return NARROW && narrow ? grp % NN : is_v ? grp % NRV : grp % NRK; };
+    auto round_of = [&](int grp) { return NARROW && narrow ? grp / NN : is_v ? grp / NRV : grp / NRK; };
     int cursor = sg0, gbase = 0, pstart = lo;       // segment of the lane's newest item, groups before its piece, the piece's first item
     struct Item { int page, sk, grp, j, ng; };
     struct Ready { int phys, kh, valid, grp, j, ng; float ks, vs; };
@@ -418,7 +489,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     // copies of the batch of items b0 .. b0 + 31 (one per lane); false when a wait has run out
     auto issue = [&](int b0, const Ready& b) {
       const int nb = min(32, hi - b0);
-      if (FP8 && is_v) {                              // page by page: every lane handles its own staging slot
+      if (FP8 && staging) {                           // page by page: every lane handles its own staging slot
         // the value scale: 2^-6 .. 2^0 of it go into P (as an exponent field), the rest onto the codes (also
         // what a caller's own scale has beside its power of two)
         const __half2 in_v = __float2half2_rn(b.vs * __int_as_float((254 - scale_in_p(b.vs)) << 23));
@@ -455,10 +526,16 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         if (!is_v && mine) {
           const int at = (grp % MR) * PG + b.j;
           meta[at] = FP8 ? b.valid | scale_in_p(b.vs) << 8 : b.valid;
-          if (FP8) kscale_meta[at] = b.ks;
+          if (FP8) {
+            kscale_meta[at] = b.ks;
+            if (NARROW && narrow) vlog_meta[at] = log2f(b.vs);
+          }
         }
         __syncwarp();
-        if (j0 == 0 && lane == 0) mbar_expect_tx(full0 + 8 * slot, ng * (FP8 ? STG : PAGE_BYTES));
+        if (j0 == 0 && lane == 0) {
+          if (FP8 && is_v) mbar_arrive(full0 + 8 * slot, kTc5CvtWarps - 1);
+          mbar_expect_tx(full0 + 8 * slot, ng * (FP8 ? STG : PAGE_BYTES));
+        }
         __syncwarp();
         if (mine) {
           if constexpr (FP8) {                        // K: a page of codes, swizzled by the copy, is an operand as it is
@@ -487,11 +564,13 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       if (b0 >= lo - 32 - DEEP) b_next = stage_b(b0 + lane + 32 + DEEP, a);
       if constexpr (FP8) {
         if (b0 >= lo - 32) stage_c(b0 + lane + 32, b1);
-        if (b0 >= lo) go = issue(b0, b);
+        if (b0 == lo) go = start();
+        if (b0 >= lo && go) go = issue(b0, b);
         b = b1;
         b1 = b_next;
       } else {
         if (b0 >= lo) {
+          if (b0 == lo) start();
           stage_c(b0 + lane, b);
           go = issue(b0, b);
         }
@@ -500,6 +579,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       a = a_next;
     }
   } else if (FP8 && warp >= kTc5CvtWarp) {
+    if (choose_path() && !narrow) {
     // ------------------------------------------------------------------ converting warps (FP8 pages): V
     // A warp takes every fourth run of UT tokens (a page, or half a page of 64) of a group: one wait and one arrival for
     // up to 64 conversions (a quarter of every page per warp had four of each; a block of eight 32K prompts 1,032 us, 968 so).
@@ -577,92 +657,130 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       ++sg;
       while (item < hi && pre[sg + 1] <= item) ++sg;
     }
+    }
   } else if (warp == kTc5QkWarp) {
     // ------------------------------------------------------------------ Q K^T issuer (a warp, one elected lane issues)
-    const uint32_t qt = warp_uniform(qtile), kr = warp_uniform(kring), s_col0 = warp_uniform(tmem) + COL_S;
-    const int end = warp_uniform(hi);
-    auto wait = [&](uint32_t bar, uint32_t parity) { return warp_mbar_wait(bar, parity, abort_flag, p.status, p.wait_cycles); };
-    int sg = sg0, item = warp_uniform(lo), piece = 0, g = 0;
-    bool ok = true;
-    while (item < end && ok) {
-      const int seg_end = warp_uniform(min(end, pre[sg + 1]));
-      ok = wait(q_full, piece & 1);
-      for (int first = item; first < seg_end && ok; first += PG, ++g) {
-        const int ng = min(PG, seg_end - first), b = g % SB, use = g / SB, slot = g % NRK;
-        ok = wait(kfull + 8 * slot, (g / NRK) & 1);
-        ok = ok && (use == 0 || wait(s_free + 8 * b, (use - 1) & 1));
-        if (!ok) break;
-        tc5_fence_after();
-        if (elect_one()) {
-          const uint32_t kt = kr + slot * KSLOT, s_col = s_col0 + b * kTc5Tok;
-          if constexpr (FP8) {                       // the terms of Q (E5M2) against the same codes (E4M3)
-            const uint32_t idesc = tc5_idesc(kRowsPerGroup, ng * GP, 0, 1u, 0u);
-            const uint64_t qd = tc5_desc8<D>(qt), kd = tc5_desc8<D>(kt);
+    if (!choose_path()) {
+    } else if (narrow) {
+      if constexpr (NARROW) tc5n_issue_qk<D, GP>(p, cta);
+    } else {
+      const uint32_t qt = warp_uniform(qtile), kr = warp_uniform(kring), s_col0 = warp_uniform(tmem) + COL_S;
+      const int end = warp_uniform(hi);
+      auto wait = [&](uint32_t bar, uint32_t parity) { return warp_mbar_wait(bar, parity, abort_flag, p.status, p.wait_cycles); };
+      int sg = sg0, item = warp_uniform(lo), piece = 0, g = 0;
+      bool ok = true;
+      while (item < end && ok) {
+        const int seg_end = warp_uniform(min(end, pre[sg + 1]));
+        ok = wait(q_full, piece & 1);
+        for (int first = item; first < seg_end && ok; first += PG, ++g) {
+          const int ng = min(PG, seg_end - first), b = g % SB, use = g / SB, slot = g % NRK;
+          ok = wait(kfull + 8 * slot, (g / NRK) & 1);
+          ok = ok && (use == 0 || wait(s_free + 8 * b, (use - 1) & 1));
+          if (!ok) break;
+          tc5_fence_after();
+          if (elect_one()) {
+            const uint32_t kt = kr + slot * KSLOT, s_col = s_col0 + b * kTc5Tok;
+            if constexpr (FP8) {                       // the terms of Q (E5M2) against the same codes (E4M3)
+              const uint32_t idesc = tc5_idesc(kRowsPerGroup, ng * GP, 0, 1u, 0u);
+              const uint64_t qd = tc5_desc8<D>(qt), kd = tc5_desc8<D>(kt);
 #pragma unroll
-            for (int ks = 0; ks < D / 32; ++ks)
+              for (int ks = 0; ks < D / 32; ++ks)
 #pragma unroll
-              for (int t = 0; t < kTc5QTerms; ++t)
-                tc5_mma_ss8(s_col, qd + (t * (kRowsPerGroup * D) + ks * 32) / 16, kd + ks * 2, idesc, ks + t > 0 ? 1u : 0u);
-          } else {
-            const uint32_t idesc = tc5_idesc(kRowsPerGroup, ng * GP, 0, 1u, 1u);
-            const uint64_t qd = tc5_desc(qt, 16), kd = tc5_desc(kt, 16);
+                for (int t = 0; t < kTc5QTerms; ++t)
+                  tc5_mma_ss8(s_col, qd + (t * (kRowsPerGroup * D) + ks * 32) / 16, kd + ks * 2, idesc, ks + t > 0 ? 1u : 0u);
+            } else {
+              const uint32_t idesc = tc5_idesc(kRowsPerGroup, ng * GP, 0, 1u, 1u);
+              const uint64_t qd = tc5_desc(qt, 16), kd = tc5_desc(kt, 16);
 #pragma unroll
-            for (int ks = 0; ks < D / 16; ++ks) {
-              const uint32_t at = ((ks >> 2) * HS + (ks & 3) * 32) / 16;
-              tc5_mma_ss(s_col, qd + at, kd + at, idesc, ks > 0 ? 1u : 0u);
+              for (int ks = 0; ks < D / 16; ++ks) {
+                const uint32_t at = ((ks >> 2) * HS + (ks & 3) * 32) / 16;
+                tc5_mma_ss(s_col, qd + at, kd + at, idesc, ks > 0 ? 1u : 0u);
+              }
             }
+            tc5_commit(s_full + 8 * b);
+            tc5_commit(kfree + 8 * slot);
+            if (first + PG >= seg_end) tc5_commit(q_free);        // Q may be replaced once the piece's last product has run
           }
-          tc5_commit(s_full + 8 * b);
-          tc5_commit(kfree + 8 * slot);
-          if (first + PG >= seg_end) tc5_commit(q_free);        // Q may be replaced once the piece's last product has run
+          __syncwarp();
         }
-        __syncwarp();
+        item = seg_end;
+        ++sg;
+        ++piece;
+        while (item < end && warp_uniform(pre[sg + 1]) <= item) ++sg;
       }
-      item = seg_end;
-      ++sg;
-      ++piece;
-      while (item < end && warp_uniform(pre[sg + 1]) <= item) ++sg;
     }
   } else if (warp == kTc5PvWarp) {
     // ------------------------------------------------------------------ P V issuer (a warp, one elected lane issues)
-    const uint32_t idesc = tc5_idesc(kRowsPerGroup, D, 1, FP8 ? 0u : 1u, FP8 ? 0u : 1u);
-    const uint32_t vr = warp_uniform(vring), tm = warp_uniform(tmem);
-    const int end = warp_uniform(hi);
-    auto wait = [&](uint32_t bar, uint32_t parity) { return warp_mbar_wait(bar, parity, abort_flag, p.status, p.wait_cycles); };
-    int sg = sg0, item = warp_uniform(lo), piece = 0, g = 0;
-    bool ok = true;
-    while (item < end && ok) {
-      const int seg_end = warp_uniform(min(end, pre[sg + 1]));
-      for (int first = item; first < seg_end && ok; first += PG, ++g) {
-        const int ng = min(PG, seg_end - first), b = g % SB, use = g / SB, slot = g % NRV;
-        ok = wait(vfull + 8 * slot, (g / NRV) & 1);
-        if (first == item && piece > 0) ok = ok && wait(o_free, (piece - 1) & 1);   // O has been read
-        ok = ok && wait(p_full + 8 * b, use & 1);
-        if (!ok) break;
-        tc5_fence_after();
-        if (elect_one()) {
-          const uint64_t vd = tc5_desc(vr + slot * SLOT, HS);
-          const uint32_t p_col = tm + COL_S + b * kTc5Tok, fresh = first == item ? 0u : 1u;
-          if (ng == PG) {
+    if (!choose_path()) {
+    } else if (narrow) {
+      if constexpr (NARROW) tc5n_issue_pv<D, GP>(p, cta);
+    } else {
+      const uint32_t idesc = tc5_idesc(kRowsPerGroup, D, 1, FP8 ? 0u : 1u, FP8 ? 0u : 1u);
+      const uint32_t vr = warp_uniform(vring), tm = warp_uniform(tmem);
+      const int end = warp_uniform(hi);
+      auto wait = [&](uint32_t bar, uint32_t parity) { return warp_mbar_wait(bar, parity, abort_flag, p.status, p.wait_cycles); };
+      int sg = sg0, item = warp_uniform(lo), piece = 0, g = 0;
+      bool ok = true;
+      while (item < end && ok) {
+        const int seg_end = warp_uniform(min(end, pre[sg + 1]));
+        for (int first = item; first < seg_end && ok; first += PG, ++g) {
+          const int ng = min(PG, seg_end - first), b = g % SB, use = g / SB, slot = g % NRV;
+          ok = wait(vfull + 8 * slot, (g / NRV) & 1);
+          if (first == item && piece > 0) ok = ok && wait(o_free, (piece - 1) & 1);   // O has been read
+          ok = ok && wait(p_full + 8 * b, use & 1);
+          if (!ok) break;
+          tc5_fence_after();
+          if (elect_one()) {
+            const uint64_t vd = tc5_desc(vr + slot * SLOT, HS);
+            const uint32_t p_col = tm + COL_S + b * kTc5Tok, fresh = first == item ? 0u : 1u;
+            if (ng == PG) {
 #pragma unroll
-            for (int ks = 0; ks < kTc5Tok / 16; ++ks) tc5_mma_ts(tm + COL_O, p_col + ks * 8, vd + ks * 128, idesc, ks == 0 ? fresh : 1u);
-          } else {
-            for (int ks = 0; ks < ng * GP / 16; ++ks) tc5_mma_ts(tm + COL_O, p_col + ks * 8, vd + ks * 128, idesc, ks == 0 ? fresh : 1u);
+              for (int ks = 0; ks < kTc5Tok / 16; ++ks) tc5_mma_ts(tm + COL_O, p_col + ks * 8, vd + ks * 128, idesc, ks == 0 ? fresh : 1u);
+            } else {
+              for (int ks = 0; ks < ng * GP / 16; ++ks) tc5_mma_ts(tm + COL_O, p_col + ks * 8, vd + ks * 128, idesc, ks == 0 ? fresh : 1u);
+            }
+            tc5_commit(vfree + 8 * slot);
+            tc5_commit(s_free + 8 * b);
           }
-          tc5_commit(vfree + 8 * slot);
-          tc5_commit(s_free + 8 * b);
+          __syncwarp();
         }
-        __syncwarp();
+        item = seg_end;
+        ++sg;
+        ++piece;
+        while (item < end && warp_uniform(pre[sg + 1]) <= item) ++sg;
       }
-      item = seg_end;
-      ++sg;
-      ++piece;
-      while (item < end && warp_uniform(pre[sg + 1]) <= item) ++sg;
     }
   }
   } else {
     // ------------------------------------------------------------------ softmax / epilogue warps
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(FP8 ? kTc5SoftmaxRegs8 : kTc5SoftmaxRegs));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(NARROW ? kTc5nSoftmaxRegs : FP8 ? kTc5SoftmaxRegs8 : kTc5SoftmaxRegs));
+    if (NARROW && few_rows && warp < kTc5ScaleWarps) {  // the share's value scales (the last set has its instructions to fetch)
+      float a = INFINITY, b = 0.f;
+      int sg = sg0;
+      for (int i = lo + tid; i < hi; i += kTc5ScaleWarps * 32) {
+        while (pre[sg + 1] <= i) ++sg;
+        const int sk = sg % p.n_sk, page = ld_nc_s32(p.union_pages + static_cast<size_t>(sk) * p.Pmax + (i - pre[sg]));
+        const int phys = page >= 0 && page < p.Pmax ? ld_nc_s32(p.page_table + static_cast<size_t>(sk / p.Hkv) * p.Pmax + page) : -1;
+        const float v = phys >= 0 && phys < p.n_phys ? __ldg(p.v_scale + static_cast<size_t>(phys) * p.Hkv + sk % p.Hkv) : -1.f;
+        a = fminf(a, v == v ? v : -1.f);             // (NaN: the wide path)
+        b = fmaxf(b, v);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        a = fminf(a, __shfl_xor_sync(0xffffffffu, a, o));
+        b = fmaxf(b, __shfl_xor_sync(0xffffffffu, b, o));
+      }
+      if (lane == 0) {
+        scale_lo[warp] = a;
+        scale_hi[warp] = b;
+        mbar_arrive(path_bar, 1);
+      }
+    }
+    if constexpr (NARROW) {
+      if (few_rows) tc5n_softmax<D, GP>(p, cta, [&]() { return choose_path() && narrow; });
+    }
+    if (few_rows && (narrow || *abort_flag)) {
+    } else {
     // Thread = query row (tensor-memory lane 32 * (warp % 4) + lane); set h = warp / 4 takes the groups
     // h, h + 3, ..., all columns, in S buffer h.  The three warps of a scheduler work on different groups, a
     // third of a period apart, so that one's exponentials (one special-function unit per scheduler) run while
@@ -685,7 +803,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     while (item < hi && ok) {
       const int seg_end = min(hi, pre[sg + 1]);
       const int rg = sg / p.n_sk, sk = sg % p.n_sk, s = sk / p.Hkv, kh = sk % p.Hkv;
-      const int rows = rows_in_group(n_active_of(s), p.G, rg);
+      const int rows = rows_in_group(cta.n_active_of(p, s), p.G, rg);
       const bool warp_has_rows = quarter * 32 < rows;          // the same for the warps of a quarter
       float scale2 = p.sm_scale * kLog2e;
       // ---- the piece's Q tile: sets 0 and 1 write half a row per thread
@@ -693,7 +811,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         const uint4* src = nullptr;
         if (r < rows) {
           const int row = rg * kRowsPerGroup + r, a = row / p.G, gi = row % p.G;
-          int tok = token_of(s, a);
+          int tok = cta.token_of(p, s, a);
           if (tok < 0 || tok >= p.B) { set_status(p.status, LOSA_ERR_BOUNDS); tok = 0; }
           src = reinterpret_cast<const uint4*>(q + ((static_cast<size_t>(s) * p.B + tok) * p.Hq + kh * p.G + gi) * D);
         }
@@ -970,6 +1088,7 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
       ++piece;
       while (item < hi && pre[sg + 1] <= item) ++sg;
     }
+    }
   }
   // ---- every thread that passed the allocation meets here; tensor memory is returned on all paths
   tc5_fence_before();
@@ -981,8 +1100,9 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     // producer loop only stops between groups), the issuing threads for the products they issued.
     if ((warp == kTc5KWarp || warp == kTc5VWarp) && lane == 0) {
       const bool is_v = warp == kTc5VWarp;
-      const uint32_t full0 = is_v ? (FP8 ? vstg_full : vfull) : kfull;
-      const int NSL = is_v ? (FP8 ? NSP : NRV) : NRK;
+      const bool staging = FP8 && is_v && !narrow;
+      const uint32_t full0 = is_v ? (staging ? vstg_full : vfull) : kfull;
+      const int NSL = NARROW && narrow ? NN : is_v ? (FP8 ? NSP : NRV) : NRK;
       for (int sl = 0; sl < NSL; ++sl) {
         if (issued < sl) continue;
         const int gl = issued - (issued - sl) % NSL;

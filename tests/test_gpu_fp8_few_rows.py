@@ -1,0 +1,65 @@
+"""Stage 4 on FP8 pages with few query rows (tokens on the tensor cores' lanes, values as an operand): rows about the limit
+of 16, value scales about the factor of four up to which that path is taken, groups of pages that end inside a
+product's 32 tokens, rising and falling scores, tails that hold NaN; against float64 over the listed pages."""
+import numpy as np
+import pytest
+
+from paper_2604_12056_b200 import workloads as wl
+from test_gpu_fp8 import assert_rows_exact_to_p
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("g,d", [(16, 128), (32, 128), (64, 128), (32, 64)])       # (d = 64: the other path)
+@pytest.mark.parametrize("m,G", [(1, 1), (5, 3), (4, 4), (17, 1)])               # 1, 15, 16 and 17 rows (17: the other path)
+@pytest.mark.parametrize("powers", [(0,), (0, 1, 2), (0, 3), (-9, -8)])            # of the pages' value scales
+def test_few_rows_against_float64(g, d, m, G, powers):
+    import torch
+    from paper_2604_12056_b200.layer import LosaLayer
+    N, Hkv = 4, 8
+    lens = (19000 // g * g + 5, 128 * 149, 20000 // (2 * g) * 2 * g + g, g - 1)   # shares of eight groups and more, which end anywhere
+    cfg = wl.config("c2", n_q_heads=Hkv * G, n_kv_heads=Hkv, head_dim=d, page_size=g, kv_lens=lens, block_size=m, steps=1, topk=1,
+                    m_active=1)
+    mp = cfg.max_pages_per_seq
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(g + d + 7 * m + G + len(powers))
+    rnd = lambda *shape: torch.randn(*shape, generator=gen, device="cuda")
+    u = torch.nn.functional.normalize(rnd(d), dim=-1)
+    kp, vp = 0.3 * rnd(N * mp, Hkv, g, d), rnd(N * mp, Hkv, g, d).clamp(-3.4, 3.4)
+    # the largest score of a page rises by up to 60 binary places over a prefix (0), falls (1) or jumps (2)
+    at = torch.arange(mp, device="cuda").float() / mp
+    level = torch.stack([60.0 * at, 60.0 * (1.0 - at), 60.0 * torch.rand(mp, generator=gen, device="cuda"), 0.0 * at]).reshape(-1)
+    kp[:, :, 3] += (level * float(np.log(2.0)) / (3.0 * cfg.sm_scale))[:, None, None] * u
+    vp[:, :, 0, 0] = 3.5                                    # (every page's largest value: its scale is known)
+    vp *= torch.exp2(torch.tensor(powers, device="cuda")[torch.arange(N * mp, device="cuda") % len(powers)].float())[:, None, None, None]
+    q = (3.0 * u * torch.rand(N, m, Hkv * G, 1, generator=gen, device="cuda") + 0.5 * rnd(N, m, Hkv * G, d)).bfloat16()
+    kb, vb = (rnd(N, m, Hkv, d).bfloat16() for _ in range(2))
+    table = torch.randperm(N * mp, generator=gen, device="cuda").int().view(N, mp)
+    layer = LosaLayer(cfg, kp.bfloat16(), vp.bfloat16(), table, torch.tensor(lens, dtype=torch.int32, device="cuda"), fp8_kv=True)
+    if powers == (-9, -8):                                  # a caller's own scales, below what the quantiser gives, no powers of two
+        layer.v_scale *= 0.013
+    for s, n in enumerate(lens):
+        if n % g:
+            for codes in (layer.k_codes, layer.v_codes):
+                codes[table[s, n // g].long(), :, n % g:] = 0x7f
+    layer.run_step(q, kb, vb, torch.ones(N, dtype=torch.int32, device="cuda"))
+    assert layer.ctx.poll_status() == 0
+    for s in range(N):
+        assert_rows_exact_to_p(layer, cfg, q, s, f"{m * G} rows")
+
+
+@pytest.mark.parametrize("odd", [0.0, -1.0, float("inf")])
+def test_value_scales_that_are_no_positive_numbers_take_the_other_path(odd):
+    import torch
+    from paper_2604_12056_b200.layer import LosaLayer
+    cfg = wl.config("c2", n_q_heads=32, n_kv_heads=8, kv_lens=(80000,), block_size=4, steps=1, topk=1, m_active=1)
+    w = wl.DeviceWorkload(cfg)
+    x = w.start_block()
+    layer = LosaLayer(cfg, w.k_pages, w.v_pages, w.page_table, w.kv_len, fp8_kv=True)
+    layer.v_scale[w.page_table[0, 5].long()] = odd
+    layer.run_step(x.q, x.k_blk, x.v_blk, x.m_per_seq)
+    assert layer.ctx.poll_status() == 0
+    if np.isfinite(odd):
+        assert_rows_exact_to_p(layer, cfg, x.q, 0, str(odd))
+    else:
+        assert not torch.isfinite(layer.o_p).all()
