@@ -37,7 +37,8 @@ static_assert(kTc5SoftmaxWarps * kTc5nSoftmaxRegs + 8 * kTc5nOtherRegs <= 20 * k
 constexpr int kTc5Tok = 128;                     // tokens per group = N of Q K^T = columns of one S buffer
 constexpr float kTc5Tau = 8.0f;                  // reference maximum moves only when it would grow by more than this (log2 units)
 // Reference maxima [set][row]; row sums and the references they are relative to [piece parity][set][row]
-template <bool FP8> constexpr int tc5_xchg_bytes() { return (5 * kTc5Sets * kRowsPerGroup + (FP8 ? 512 : 0)) * 4; }     // (FP8: the narrow path's need more)
+constexpr int kTc5Xchg = 5 * kTc5Sets * kRowsPerGroup;
+template <bool FP8> constexpr int tc5_xchg_bytes() { return (kTc5Xchg + (FP8 ? 512 : 0)) * 4; }     // (FP8: the narrow path's need more)
 // FP8 pages: binary places by which P is held above the reference maximum.  P stays below 2^(8 + 7) < 65504.
 constexpr float kTc5Fp8Lift = 7.0f;
 constexpr int kTc5StgMax = 20;                   // FP8 pages: staging slots of V, one page each, at most

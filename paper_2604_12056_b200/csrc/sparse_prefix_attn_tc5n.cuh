@@ -181,7 +181,8 @@ __device__ __forceinline__ bool tc5n_clear(const Tc5Cta& c, int g, int ng, int t
 // ---- softmax / epilogue warps
 // decide(): waits until the path is known, false if it is not this one (or the wait has run out).
 // The last set first takes a group that is not there, before the path is known: no waits for other roles, no arrivals, no token
-// live, so that nothing changes (of the exchange arrays it touches what the wide path uses only once this set is with it).  It fetches the loop's instructions while the producers still look for their first pages.  Behind
+// live, so that nothing changes.  The other sets may be on the wide path by then, at the end of a short first piece even: what
+// this set writes of the exchange arrays lies behind all that path has there.  It fetches the loop's instructions while the producers still look for their first pages.  Behind
 // the page copies every missed line of them takes 400 cycles and more: the first groups' maxima and weights took 7,300 cycles,
 // with the rings full and HBM idle (a block of eight 32K prompts 11 us longer).
 template <int D, int GP, typename Decide>
@@ -193,15 +194,23 @@ __device__ __forceinline__ void tc5n_softmax(const AttnParams& p, const Tc5Cta& 
   const uint32_t lane_addr = c.tmem + (static_cast<uint32_t>(quarter * 32) << 16);
   const uint32_t s_addr = lane_addr + kTc5nColS + h * kTc5nRows, o_addr = lane_addr + kTc5nColO + h * OC;
   uint8_t* ptile = c.gen + tc5n_q_bytes<D>() + h * tc5n_p_bytes();
+  // The exchange arrays, in entries from c.scratch on: those of the first two sets, of a piece, of the last set.  (c.scratch is at most three
+  // entries behind the wide path's first.)
+  constexpr int kSetRefs = 2 * kTc5SetWarps * kTc5nLanes, kSetMax = kTc5SetWarps * kTc5nLanes;     // of one set
+  constexpr int kMax0 = (SB - 1) * kSetRefs, kSums = kMax0 + (SB - 1) * kSetMax, kRefs = kSums + 2 * NW * kTc5nLanes;
+  constexpr int kScale = kRefs + 2 * SB * kTc5nLanes, kPieceEnd = kScale + 2 * kTc5nLanes;
+  constexpr int kLast = kTc5Xchg, kLastMax = kLast + kSetRefs, kFlags = kLastMax + kSetMax;        // written by the walk without a group
+  static_assert(kPieceEnd <= kLast && kLast >= kTc5Xchg, "the last set's entries: behind the others' and the wide path's");
+  static_assert(kFlags * 4 + SB * 8 + 3 * 4 <= tc5_xchg_bytes<true>(), "exchange arrays");
+  const bool last_set = h == SB - 1;
   // Per row, a copy per warp: minus the reference maximum, +inf while there is none; the same with 0 for none.
-  float* neg_m = c.scratch + warp * 2 * kTc5nLanes;              // [12][2][32]
+  float* neg_m = c.scratch + (last_set ? kLast : h * kSetRefs) + quarter * 2 * kTc5nLanes;         // [4][2][32]
   float* neg_use = neg_m + kTc5nLanes;
-  float* wmax = c.scratch + 2 * NW * kTc5nLanes;                 // [12][32] maxima over a warp's tokens
-  float* xsum = wmax + NW * kTc5nLanes;                          // [piece parity][12][32] row sums of a piece over a warp's tokens ...
-  float* xref = xsum + 2 * NW * kTc5nLanes;                      // [piece parity][3][32]  ... and the references they are relative to
-  float* qscale = xref + 2 * SB * kTc5nLanes;                    // [piece parity][32] softmax scale times what undoes the row's power of two
-  volatile uint8_t* flags = reinterpret_cast<volatile uint8_t*>(qscale + 2 * kTc5nLanes);   // [3][meeting parity][4]
-  static_assert(((3 + 2) * NW + 2 * SB + 2) * kTc5nLanes * 4 + SB * 8 + 16 <= tc5_xchg_bytes<true>(), "exchange arrays");
+  float* wmax = c.scratch + (last_set ? kLastMax : kMax0 + h * kSetMax);      // [4][32] maxima over a warp's tokens
+  float* xsum = c.scratch + kSums;                               // [piece parity][12][32] row sums of a piece over a warp's tokens ...
+  float* xref = c.scratch + kRefs;                               // [piece parity][3][32]  ... and the references they are relative to
+  float* qscale = c.scratch + kScale;                            // [piece parity][32] softmax scale times what undoes the row's power of two
+  volatile uint8_t* flags = reinterpret_cast<volatile uint8_t*>(c.scratch + kFlags);        // [3][meeting parity][4]
   auto warp_wait = [&](uint32_t bar, uint32_t parity) {         // one answer for the warp: tensor-memory instructions need all lanes
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, c.abort_flag, p.status, p.wait_cycles)) != 0;
   };
@@ -348,10 +357,10 @@ __device__ __forceinline__ void tc5n_softmax(const AttnParams& p, const Tc5Cta& 
             if (lane == n + e) mine = k;
           }
         }
-        wmax[warp * kTc5nLanes + lane] = mine;
+        wmax[quarter * kTc5nLanes + lane] = mine;
         ok = set_meets();
         if (!ok) break;
-        const float* wm = wmax + h * kTc5SetWarps * kTc5nLanes + lane;
+        const float* wm = wmax + lane;
         const float top = fmaxf(fmaxf(wm[0], wm[kTc5nLanes]), fmaxf(wm[2 * kTc5nLanes], wm[3 * kTc5nLanes]));
         const float m_old = -neg_m[lane];
         const float m_new = (top > m_old + kTc5nTop || (m_old == -INFINITY && top > -INFINITY)) ? top - kTc5nLift : m_old;

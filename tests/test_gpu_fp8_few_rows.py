@@ -63,3 +63,39 @@ def test_value_scales_that_are_no_positive_numbers_take_the_other_path(odd):
         assert_rows_exact_to_p(layer, cfg, x.q, 0, str(odd))
     else:
         assert not torch.isfinite(layer.o_p).all()
+
+
+@pytest.mark.parametrize("g", [16, 32, 64])
+@pytest.mark.parametrize("powers", [(0, 3), (0, 1)])                          # the other path, this one
+def test_few_rows_in_shares_of_short_pieces(g, powers):
+    """Shares of some 30 groups, but pieces of one to ten: a piece ends before the last set of softmax warps has had a group,
+    and the share's first one while that set may still be in its walk without a group, whichever path the others are on.
+    Against float64, and the same bits every time."""
+    import torch
+    from paper_2604_12056_b200 import binding as B
+    from paper_2604_12056_b200.layer import LosaLayer
+    N, Hkv, G, Bk, d = 64, 16, 4, 4, 128
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(g + len(powers) + powers[1])
+    rnd = lambda *shape: torch.randn(*shape, generator=gen, device="cuda")
+    lens = tuple(128 * (1 + 3 * s % 10) - (s % 3) * 7 for s in range(N - 1)) + (128 * 10,)
+    cfg = wl.config("c2", n_q_heads=Hkv * G, n_kv_heads=Hkv, head_dim=d, page_size=g, kv_lens=lens, block_size=Bk, steps=1, topk=1,
+                    m_active=1)
+    mp = cfg.max_pages_per_seq
+    kp, vp = 0.3 * rnd(N * mp, Hkv, g, d), rnd(N * mp, Hkv, g, d).clamp(-3.4, 3.4)
+    vp[:, :, 0, 0] = 3.5                                    # (every page's largest value: its scale is known)
+    vp *= torch.exp2(torch.tensor(powers, device="cuda")[torch.arange(N * mp, device="cuda") % 2].float())[:, None, None, None]
+    q = rnd(N, Bk, Hkv * G, d).bfloat16()
+    kb, vb = (rnd(N, Bk, Hkv, d).bfloat16() for _ in range(2))
+    table = torch.arange(N * mp, dtype=torch.int32, device="cuda").view(N, mp)
+    layer = LosaLayer(cfg, kp.bfloat16(), vp.bfloat16(), table, torch.tensor(lens, dtype=torch.int32, device="cuda"), fp8_kv=True)
+    layer.run_step(q, kb, vb, torch.ones(N, dtype=torch.int32, device="cuda"))
+    assert layer.ctx.poll_status() == 0
+    first = layer.o_p.clone(), layer.lse_p.clone()
+    for s in range(N):
+        assert_rows_exact_to_p(layer, cfg, q, s, f"scales {powers}")
+    for _ in range(20):
+        layer.o_p.zero_()
+        B.losa_sparse_prefix_attn(layer.ctx, q, layer.kv, layer.active_idx, layer.n_active, layer.union_pages, layer.union_count, layer.state)
+        assert layer.ctx.poll_status() == 0
+        assert torch.equal(layer.o_p, first[0]) and torch.equal(layer.lse_p, first[1])
