@@ -67,6 +67,7 @@ constexpr int kTc5nRows = 16;                    // FP8: most query rows of a sh
 constexpr int kTc5nLanes = 32;                   // entries of its per-row arrays, one per lane
 constexpr int kTc5nP = kTc5Tok * 16;             // bytes of one term of 16 rows of its P'
 constexpr int kTc5PTerms = 3;                    // E5M2 terms of P'
+constexpr float kTc5nTermStep = 0.0625f;         // a term's unit is this much of the one before's
 constexpr float kTc5nLift = 11.0f, kTc5nTop = 15.0f;   // binary places by which P' is held above the reference, and by which it may outgrow it
 constexpr int tc5n_p_bytes() { return kTc5PTerms * kTc5nP; }
 template <int D> constexpr int tc5n_q_bytes() { return kTc5nRows * D * kTc5QTerms; }

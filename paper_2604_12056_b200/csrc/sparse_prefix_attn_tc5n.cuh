@@ -8,13 +8,16 @@
 //   S[128 tokens x rows]  = K . Q^T     A = the group's codes, B = Q's three E5M2 terms (one after the other into the same columns)
 //   softmax               thread = token, 16 exponentials; P' = 2^(s - m) vs, vs the page's value scale, in fp16 precision
 //   P'                    as three E5M2 terms in shared memory: an E5M2 value is the upper byte of an fp16 one, and three of
-//                         them, each rounded to nearest, make up the eleven significant bits of P' exactly
+//                         them, each rounded to nearest, make up the eleven significant bits of P'
 //   O[D x 3 rows]        += V^T . P'    A = the group's codes (MN-major), B = the terms (MN-major), a column each
-// E5M2 ends at 2^-16: P' keeps all its bits down to 2^-6 and is off by at most 2^-17 below.  The reference is held 2^11 below the
+// E5M2 ends at 2^-16, fp16 at 2^-24: the second term is stored times 2^4, the third times 2^8, which their columns of O take back
+// when the piece ends.  A term leaves at most 2^-4 of what it was rounded from, so none exceeds 2^15, and the three are P' exactly,
+// for every fp16 value of at most 2^15 (the low bits of a subnormal one, too).  The reference is held 2^11 below the
 // maximum of the shifted exponents and moves when that grows by 2^4 (P' <= 2^15).  The path is taken where the share's value
-// scales are within a factor of four of one another, so a weight loses bits no earlier than 2^-15 of its row's largest, as in
-// the wide path.  (With all of a scale in P' and pages of any scale side by side, columns that only low-scale pages fill were
-// off by three times what the wide path's bound allows.)
+// scales are within a factor of four of one another, so a weight loses bits no earlier than 2^-23 of its row's largest; with
+// the wide path's 2^7 that is 2^-19 there.  (Terms without powers of two of their own kept the bits of weights down to 2^-15.  With
+// all of a scale in P' and pages of any scale side by side, columns that only low-scale pages fill were off by three times what
+// the wide path's bound allows.)
 // A block of eight 32K prompts takes 900 us the wide way and 804 this way: a group of 128 tokens every 1,350 cycles, which is
 // HBM's pace, instead of every 2,000.  With V converted to fp16 here as well (P' as fp16) it was hardly faster than the wide way:
 // the conversion and 160 KB per group through shared memory bound it.
@@ -196,17 +199,16 @@ __device__ __forceinline__ void tc5n_softmax(const AttnParams& p, const Tc5Cta& 
   uint8_t* ptile = c.gen + tc5n_q_bytes<D>() + h * tc5n_p_bytes();
   // The exchange arrays, in entries from c.scratch on: those of the first two sets, of a piece, of the last set.  (c.scratch is at most three
   // entries behind the wide path's first.)
-  constexpr int kSetRefs = 2 * kTc5SetWarps * kTc5nLanes, kSetMax = kTc5SetWarps * kTc5nLanes;     // of one set
-  constexpr int kMax0 = (SB - 1) * kSetRefs, kSums = kMax0 + (SB - 1) * kSetMax, kRefs = kSums + 2 * NW * kTc5nLanes;
-  constexpr int kScale = kRefs + 2 * SB * kTc5nLanes, kPieceEnd = kScale + 2 * kTc5nLanes;
-  constexpr int kLast = kTc5Xchg, kLastMax = kLast + kSetRefs, kFlags = kLastMax + kSetMax;        // written by the walk without a group
-  static_assert(kPieceEnd <= kLast && kLast >= kTc5Xchg, "the last set's entries: behind the others' and the wide path's");
+  constexpr int kSetRefs = 2 * kTc5SetWarps * kTc5nLanes, kSet = kSetRefs + kTc5SetWarps * kTc5nLanes;     // of one set
+  constexpr int kSums = (SB - 1) * kSet, kRefs = kSums + 2 * NW * kTc5nLanes, kScale = kRefs + 2 * SB * kTc5nLanes;
+  constexpr int kLast = kTc5Xchg, kFlags = kLast + kSet;         // written by the walk without a group
+  static_assert(kScale + 2 * kTc5nLanes <= kLast && kLast >= kTc5Xchg, "the last set's entries: behind the others' and the wide path's");
   static_assert(kFlags * 4 + SB * 8 + 3 * 4 <= tc5_xchg_bytes<true>(), "exchange arrays");
-  const bool last_set = h == SB - 1;
+  float* own = c.scratch + (h == SB - 1 ? kLast : h * kSet);
   // Per row, a copy per warp: minus the reference maximum, +inf while there is none; the same with 0 for none.
-  float* neg_m = c.scratch + (last_set ? kLast : h * kSetRefs) + quarter * 2 * kTc5nLanes;         // [4][2][32]
+  float* neg_m = own + quarter * 2 * kTc5nLanes;                 // [4][2][32]
   float* neg_use = neg_m + kTc5nLanes;
-  float* wmax = c.scratch + (last_set ? kLastMax : kMax0 + h * kSetMax);      // [4][32] maxima over a warp's tokens
+  float* wmax = own + kSetRefs;                                  // [4][32] maxima over a warp's tokens
   float* xsum = c.scratch + kSums;                               // [piece parity][12][32] row sums of a piece over a warp's tokens ...
   float* xref = c.scratch + kRefs;                               // [piece parity][3][32]  ... and the references they are relative to
   float* qscale = c.scratch + kScale;                            // [piece parity][32] softmax scale times what undoes the row's power of two
@@ -290,7 +292,6 @@ __device__ __forceinline__ void tc5n_softmax(const AttnParams& p, const Tc5Cta& 
       __syncwarp();
       if (lane == 0) mbar_arrive(c.q_full, h == 0 ? 2 : 1);            // (the last set's arrivals with the first's)
     }
-    const int n_groups = (seg_end - item + PG - 1) / PG;
     const int parity = piece & 1;                               // of the exchange buffers
     float l[kTc5nRows];                                       // this thread's weights
 #pragma unroll
@@ -386,12 +387,12 @@ __device__ __forceinline__ void tc5n_softmax(const AttnParams& p, const Tc5Cta& 
       // ---- P' = 2^(s + vlog - m), its sum without the value scale, its three terms
       const float unscale = ex2(-vlog);
       {
-        uint32_t v[16], w[kTc5PTerms][4];
-        tc5_ld16(s_at, v);
+        uint32_t v[8], w[kTc5PTerms][4];                          // (the scores in two halves: all 16 spill registers)
 #pragma unroll
         for (int e = 0; e < 16; e += 4) {
+          if (e % 8 == 0) tc5_ld8(s_at + e, v);
           float2 y[2];
-          exponents(neg_use, e, v + e, y);
+          exponents(neg_use, e, v + e % 8, y);
           y[0] = make_float2(ex2(y[0].x), ex2(y[0].y));
           y[1] = make_float2(ex2(y[1].x), ex2(y[1].y));
           if (live) {                                           // (a lane without a token holds anything)
@@ -401,13 +402,14 @@ __device__ __forceinline__ void tc5n_softmax(const AttnParams& p, const Tc5Cta& 
           }
           uint32_t p0 = live ? pack_f16(y[0].x, y[0].y) : 0u, p1 = live ? pack_f16(y[1].x, y[1].y) : 0u;
 #pragma unroll
-          for (int k = 0; k < kTc5PTerms; ++k) {                // the nearest multiple of the upper byte's last place, ties away from zero
+          for (int k = 0; k < kTc5PTerms; ++k) {                // the nearest multiple of the upper byte's last place, ties away from zero; the rest, times 2^4
             const uint32_t r0 = p0 + 0x00800080u, r1 = p1 + 0x00800080u;
             w[k][e / 4] = __byte_perm(r0, r1, 0x7531);
             if (k + 1 < kTc5PTerms) {
               const uint32_t t0 = r0 & 0xff00ff00u, t1 = r1 & 0xff00ff00u;
-              const __half2 d0 = __hsub2(*reinterpret_cast<const __half2*>(&p0), *reinterpret_cast<const __half2*>(&t0));
-              const __half2 d1 = __hsub2(*reinterpret_cast<const __half2*>(&p1), *reinterpret_cast<const __half2*>(&t1));
+              const __half2 up = __float2half2_rn(1.f / kTc5nTermStep);
+              const __half2 d0 = __hmul2(__hsub2(*reinterpret_cast<const __half2*>(&p0), *reinterpret_cast<const __half2*>(&t0)), up);
+              const __half2 d1 = __hmul2(__hsub2(*reinterpret_cast<const __half2*>(&p1), *reinterpret_cast<const __half2*>(&t1)), up);
               p0 = *reinterpret_cast<const uint32_t*>(&d0);
               p1 = *reinterpret_cast<const uint32_t*>(&d1);
             }
@@ -436,6 +438,7 @@ __device__ __forceinline__ void tc5n_softmax(const AttnParams& p, const Tc5Cta& 
       ok = decide();
       continue;
     }
+    const int n_groups = (seg_end - item + PG - 1) / PG;
     g = g0 + n_groups;
     // the row sums over the warp's tokens, lane n left with row n (every step halves the rows a lane still adds for)
 #pragma unroll
@@ -498,7 +501,8 @@ __device__ __forceinline__ void tc5n_softmax(const AttnParams& p, const Tc5Cta& 
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           const float wx = __shfl_sync(0xffffffffu, w[x], n0 + e);
-          if (wx > 0.f) acc[e] = fmaf((__uint_as_float(o[2][e]) + __uint_as_float(o[1][e])) + __uint_as_float(o[0][e]), wx, acc[e]);
+          const float sum = fmaf(fmaf(__uint_as_float(o[2][e]), kTc5nTermStep, __uint_as_float(o[1][e])), kTc5nTermStep, __uint_as_float(o[0][e]));
+          if (wx > 0.f) acc[e] = fmaf(sum, wx, acc[e]);
         }
       }
       {

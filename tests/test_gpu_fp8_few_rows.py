@@ -5,14 +5,14 @@ import numpy as np
 import pytest
 
 from paper_2604_12056_b200 import workloads as wl
-from test_gpu_fp8 import assert_rows_exact_to_p
+from test_gpu_fp8 import assert_rows_exact_to_p, listed_prefix
 
 pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("g,d", [(16, 128), (32, 128), (64, 128), (32, 64)])       # (d = 64: the other path)
 @pytest.mark.parametrize("m,G", [(1, 1), (5, 3), (4, 4), (17, 1)])               # 1, 15, 16 and 17 rows (17: the other path)
-@pytest.mark.parametrize("powers", [(0,), (0, 1, 2), (0, 3), (-9, -8)])            # of the pages' value scales
+@pytest.mark.parametrize("powers", [(0,), (0, 1, 2), (0, 3), (1, 4), (-9, -8)])    # of the pages' values (a scale is 2^-6 at least: 0 and 3 are four apart)
 def test_few_rows_against_float64(g, d, m, G, powers):
     import torch
     from paper_2604_12056_b200.layer import LosaLayer
@@ -66,7 +66,7 @@ def test_value_scales_that_are_no_positive_numbers_take_the_other_path(odd):
 
 
 @pytest.mark.parametrize("g", [16, 32, 64])
-@pytest.mark.parametrize("powers", [(0, 3), (0, 1)])                          # the other path, this one
+@pytest.mark.parametrize("powers", [(1, 4), (0, 1)])                          # the other path (scales eight apart), this one
 def test_few_rows_in_shares_of_short_pieces(g, powers):
     """Shares of some 30 groups, but pieces of one to ten: a piece ends before the last set of softmax warps has had a group,
     and the share's first one while that set may still be in its walk without a group, whichever path the others are on.
@@ -99,3 +99,66 @@ def test_few_rows_in_shares_of_short_pieces(g, powers):
         B.losa_sparse_prefix_attn(layer.ctx, q, layer.kv, layer.active_idx, layer.n_active, layer.union_pages, layer.union_count, layer.state)
         assert layer.ctx.poll_status() == 0
         assert torch.equal(layer.o_p, first[0]) and torch.equal(layer.lse_p, first[1])
+
+
+def hot_token_per_prompt(g, m, G, powers, above):
+    """Prompts whose first page holds one token with a score `above` (log2 units) over all others, which are about equal, and in whose
+    column 5 only that page's other tokens have values: the column is theirs alone, beside a weight of one.  Long enough for
+    twice the shares of eight groups that are this path's least, whatever the number of SMs."""
+    import torch
+    from paper_2604_12056_b200.layer import LosaLayer
+    N, Hkv, d = 2, 8, 128
+    n_sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n_tok = n_sms * 4096 * 2 // (N * Hkv) // g * g + 5
+    cfg = wl.config("c2", n_q_heads=Hkv * G, n_kv_heads=Hkv, head_dim=d, page_size=g, kv_lens=(n_tok,) * N, block_size=m, steps=1, topk=1,
+                    m_active=1)
+    mp = cfg.max_pages_per_seq
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(g + m + G + int(above))
+    rnd = lambda *shape: torch.randn(*shape, generator=gen, device="cuda")
+    u = torch.nn.functional.normalize(rnd(d), dim=-1)
+    kp = 0.05 * rnd(N * mp, Hkv, g, d)
+    kp -= (kp @ u)[..., None] * u                           # orthogonal to the queries' direction
+    vp = rnd(N * mp, Hkv, g, d).clamp(-3.4, 3.4)
+    vp[..., 5] = 0.0
+    vp[:, :, 0, 0] = 3.5                                    # (every page's largest value: its scale is known)
+    vp[0::mp, :, :, 5] = 1.0 + rnd(N, Hkv, g).abs().clamp_max(2.0)
+    vp[0::mp, :, 3, 5] = 0.0
+    kp[0::mp, :, 3] = u * (above * float(np.log(2.0)) / (4.0 * cfg.sm_scale))
+    vp *= torch.exp2(torch.tensor(powers, device="cuda")[torch.arange(N * mp, device="cuda") % len(powers)].float())[:, None, None, None]
+    q = (4.0 * u + 0.02 * rnd(N, m, Hkv * G, d)).bfloat16()
+    kb, vb = (rnd(N, m, Hkv, d).bfloat16() for _ in range(2))
+    table = torch.arange(N * mp, dtype=torch.int32, device="cuda").view(N, mp)
+    layer = LosaLayer(cfg, kp.bfloat16(), vp.bfloat16(), table, torch.full((N,), n_tok, dtype=torch.int32, device="cuda"), fp8_kv=True)
+    layer.run_step(q, kb, vb, torch.ones(N, dtype=torch.int32, device="cuda"))
+    assert layer.ctx.poll_status() == 0
+    return layer, cfg, q
+
+
+@pytest.mark.parametrize("g", [16, 32, 64])
+@pytest.mark.parametrize("m,G", [(1, 1), (4, 4)])
+@pytest.mark.parametrize("above", [12, 18, 21, 24])
+def test_small_weights_beside_a_large_one_keep_their_bits(g, m, G, above):
+    """The reference lies 2^11 below a row's largest weight and P' is an fp16 value: weights keep all eleven bits down to 2^-25
+    of it.  So a column that only weights of about 2^-above fill is off by half a unit of each, 2^-11 sum p |v|, and as much
+    again for the sums in fp32 and 2^x; nothing is lost on the grid of 2^-24 that fp16 ends with."""
+    import torch
+    layer, cfg, q = hot_token_per_prompt(g, m, G, (0,), above)
+    for s in range(cfg.batch):
+        for h in range(cfg.n_kv_heads):
+            k, v = listed_prefix(layer, cfg, s, h)
+            heads = slice(h * G, (h + 1) * G)
+            p = torch.softmax(q[s, :, heads].double() @ k.T * cfg.sm_scale, -1)
+            want = p @ v[:, 5]                              # (no value of the column is negative)
+            assert (want < 2.0 ** (10 - above)).all() and (want > 2.0 ** (-2 - above)).all()
+            assert ((layer.o_p[s, :, heads, 5].double() - want).abs() <= 2.0 ** -10 * want).all(), (s, h)
+
+
+@pytest.mark.parametrize("g", [16, 32, 64])
+@pytest.mark.parametrize("m,G,powers,few", [(1, 1, (0,), True), (4, 4, (1, 2, 3), True), (16, 1, (3, 1), True), (17, 1, (1,), False),
+                                            (4, 4, (1, 4), False), (1, 1, (4, 2, 1), False)])
+def test_which_path_a_share_takes(g, m, G, powers, few):
+    """A weight of 2^-34 of its row's largest is 2^-23 under this path's reference, a value fp16 has, and 2^-27 under the other
+    path's, less than half of its smallest: the column tells which one the share took."""
+    layer, cfg, _ = hot_token_per_prompt(g, m, G, powers, 34)
+    assert ((layer.o_p[..., 5] != 0) == few).all()
