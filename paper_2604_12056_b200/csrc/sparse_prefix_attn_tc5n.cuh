@@ -479,7 +479,7 @@ __device__ __forceinline__ void tc5n_softmax(const AttnParams& p, const Tc5Cta& 
       w[x] = w[x] == -INFINITY ? 0.f : ex2(w[x] - M);
       const float* xs = xsum + (parity * NW + x * kTc5SetWarps) * kTc5nLanes + lane;
       const float sum = (xs[0] + xs[kTc5nLanes]) + (xs[2 * kTc5nLanes] + xs[3 * kTc5nLanes]);
-      if (w[x] > 0.f) L = fmaf(sum, w[x], L);
+      if (w[x] > 0.f || sum != sum) L = fmaf(sum, w[x], L);
     }
     if (warp == 0 && lane < rows) {
       float* rec = record_base(p.partials, blockIdx.x + sg, lane / kTileRows, D);
@@ -506,10 +506,13 @@ __device__ __forceinline__ void tc5n_softmax(const AttnParams& p, const Tc5Cta& 
         }
       }
       {
+        // a weight that is no number has no term (its rounding ends at zero), but spoils the row's sum: that goes into the outputs
         float* rec = record_base(p.partials, blockIdx.x + sg, n0 / kTileRows, D) + 2 * kTileRows + d;
 #pragma unroll
-        for (int e = 0; e < 8; ++e)
-          if (n0 + e < rows) rec[(n0 % kTileRows + e) * D] = acc[e];
+        for (int e = 0; e < 8; ++e) {
+          const float row_l = __shfl_sync(0xffffffffu, L, n0 + e);
+          if (n0 + e < rows) rec[(n0 % kTileRows + e) * D] = row_l == row_l ? acc[e] : row_l;
+        }
       }
     }
     tc5_fence_before();

@@ -162,3 +162,30 @@ def test_which_path_a_share_takes(g, m, G, powers, few):
     path's, less than half of its smallest: the column tells which one the share took."""
     layer, cfg, _ = hot_token_per_prompt(g, m, G, powers, 34)
     assert ((layer.o_p[..., 5] != 0) == few).all()
+
+
+@pytest.mark.parametrize("g", [16, 32, 64])
+@pytest.mark.parametrize("powers", [(1,), (1, 4)])                            # this path, the other one
+@pytest.mark.parametrize("where", ["key scale", "key code", "query"])
+def test_values_that_are_no_numbers_stay_in_the_cached_state(g, powers, where):
+    """A listed page whose key scale or one of whose key codes is NaN leaves NaN in o_p of all rows of its KV head, and a query
+    with an infinity in o_p of its row; no others."""
+    import torch
+    from paper_2604_12056_b200 import binding as B
+    G, m, page = 4, 4, 901
+    layer, cfg, q = hot_token_per_prompt(g, m, G, powers, 12)
+    bad = torch.zeros(cfg.batch, m, cfg.n_q_heads, dtype=torch.bool, device="cuda")
+    phys = int(layer.page_table[1, page])
+    if where == "query":
+        q[1, 2, 9, 7] = float("inf")
+        bad[1, 2, 9] = True
+    else:
+        bad[1, :, 2 * G:3 * G] = True
+        if where == "key scale":
+            layer.k_scale[phys, 2] = float("nan")
+        else:
+            layer.k_codes[phys, 2, 5, 77] = 0x7f
+    B.losa_sparse_prefix_attn(layer.ctx, q, layer.kv, layer.active_idx, layer.n_active, layer.union_pages, layer.union_count, layer.state)
+    assert layer.ctx.poll_status() == 0
+    assert torch.isnan(layer.o_p[bad]).all() and torch.isfinite(layer.o_p[~bad]).all()
+    assert not torch.isfinite(layer.lse_p[bad]).any() and torch.isfinite(layer.lse_p[~bad]).all()
