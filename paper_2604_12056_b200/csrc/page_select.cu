@@ -114,6 +114,7 @@ __device__ __forceinline__ unsigned long long make_key(uint32_t ob, int p) {
 // (P <= kSelThreads * kSelPerThread) their order bits stay in registers for the whole selection.
 constexpr int kSelThreads = 128;
 constexpr int kSelPerThread = 8;
+constexpr int kCrowd = 32;          // lists whose candidates crowd more than that into one bin take exact scores for all of them
 constexpr int kSelSlots = 8;        // CTAs per (sequence, head), at most: active slots are dealt out round-robin
 
 template <bool CACHED, typename Row, typename F>
@@ -387,6 +388,19 @@ __device__ __forceinline__ uint32_t prefix_word(int w, int P) {   // word w of t
   return (P >= lo + 32) ? 0xffffffffu : (P > lo ? ((1u << (P - lo)) - 1u) : 0u);
 }
 
+// How many of n keys (all different) are larger than `mine`: read as broadcasts, four at a time.
+__device__ __forceinline__ int larger_keys(const unsigned long long* keys, int n, unsigned long long mine) {
+  int rank = 0;
+  const int n4 = n & ~3;
+  for (int i = 0; i < n4; i += 4) {
+    const ulonglong2 k01 = *reinterpret_cast<const ulonglong2*>(&keys[i]);
+    const ulonglong2 k23 = *reinterpret_cast<const ulonglong2*>(&keys[i + 2]);
+    rank += (k01.x > mine ? 1 : 0) + (k01.y > mine ? 1 : 0) + (k23.x > mine ? 1 : 0) + (k23.y > mine ? 1 : 0);
+  }
+  for (int i = n4; i < n; ++i) rank += keys[i] > mine ? 1 : 0;
+  return rank;
+}
+
 // One CTA of kSelThreads per (sequence, head, share of the active slots).  Per query: tau = lower edge
 // of the histogram bin that holds the k-th largest LOWER bound; every page whose UPPER bound reaches
 // tau is a candidate (a superset of the exact top-k, ties included: the exact score lies between the
@@ -408,13 +422,13 @@ struct RefineSmem {
     struct { int cpage[kSelCap], cphys[kSelCap]; };
     unsigned long long skey[kSelCap];            // RUNS: by descending lower bound
   };
-  union { int hist[kSelBins]; uint16_t close[kSelCap]; };   // (close: once tau is known)
+  union { alignas(8) int hist[kSelBins]; uint16_t close[kSelCap]; };   // (close: once tau is known)
   uint32_t run[kSelCap / 32];                    // bit r: a run of close candidates starts at position r
   uint32_t red[2][kSelThreads / 32];
   uint32_t width;                                // the widest pair of bounds, rounded up: the bits of a float
   int ncand, nclose, bstar;
 };
-static_assert(kSelBins * sizeof(int) >= kSelCap * sizeof(uint16_t), "positions");
+static_assert(kSelBins * sizeof(int) >= kSelCap * sizeof(uint16_t) && kSelBins == 2 * kSelThreads, "positions; two bins per thread");
 
 // In a whole step the grid ends with the row tiles of the in-block attention (BK: its padded key
 // count).  It needs only the step's inputs, and these CTAs fill the gaps of a kernel that is bound by
@@ -571,6 +585,7 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
     for (int b = tid; b < kSelBins; b += kSelThreads) hist[b] = 0;
     // ---- tau
     uint32_t tau = 0u;
+    bool crowded = false;                          // RUNS: all bounds the same, or more than kCrowd pages in one of this thread's bins that reach the list
     if (kk < P) {
       uint32_t lo = 0xffffffffu, hi = 0u;
       for_each_page([&](uint32_t lb, uint32_t, int) { lo = min(lo, lb); hi = max(hi, lb); });
@@ -606,9 +621,15 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
           }
         }
         __syncthreads();
-        tau = lo + (static_cast<uint32_t>(s_bstar) << shift);
+        const int bstar = s_bstar;
+        tau = lo + (static_cast<uint32_t>(bstar) << shift);
+        if (RUNS) {
+          const int2 c = *reinterpret_cast<const int2*>(&hist[2 * tid]);
+          crowded = (2 * tid >= bstar && c.x > kCrowd) || (2 * tid + 1 >= bstar && c.y > kCrowd);
+        }
       } else {
         tau = lo;
+        crowded = true;
       }
     } else {
       __syncthreads();
@@ -648,7 +669,8 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
         }
       });
     }
-    __syncthreads();
+    if constexpr (RUNS) crowded = __syncthreads_or(crowded) != 0;
+    else __syncthreads();
     const int ncand = s_ncand;
     auto phys_of = [&](int pg) {
       int ph = __ldg(p.page_table + static_cast<size_t>(s) * p.Pmax + pg);
@@ -665,6 +687,14 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
       }
       return e;
     };
+    auto emit = [&](int rank, unsigned long long key) {      // entry `rank` of the list
+      const int pg = static_cast<int32_t>(0xffffffffu - static_cast<uint32_t>(key));
+      for (int gi = 0; gi < pool; ++gi) {
+        out_pages[gi * p.k + rank] = pg;
+        if (out_scores) out_scores[gi * p.k + rank] = unorder_bits(static_cast<uint32_t>(key >> 32));
+      }
+      mark(pg);
+    };
     if (ncand > kSelCap) {
       float* row = reinterpret_cast<float*>(row2);             // the bounds are not needed any more
       for (int p0 = 0; p0 < P; p0 += kSelThreads / 4) {          // whole warps: the shuffles need all lanes
@@ -678,50 +708,27 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
       __syncthreads();
       continue;
     }
-    if constexpr (RUNS) {
+    // RUNS: every candidate takes its exact score where one round of scores is enough for all, and where the pages crowd (most are close
+    // then: 300 pages of one score, 256 lists, bounds included, 72 us by bounds, 55 so); a list per head stays in the same code (beside
+    // the other way's it takes 1.1 us longer in a step with 256 lists), a pooled one, whose scores take longer, takes the other way's.
+    const bool all_exact = !RUNS || ncand <= kSelThreads / 4 || crowded;
+    if (RUNS && (!POOLED || !all_exact)) {
       // The candidates in descending order of their lower bounds.  No pair of bounds is wider than `width`: where a lower bound
       // lies more than that below the one before it, everything from there on scores below everything before.  Only within a run
       // of closer ones does the order need exact scores: 20 of 67 candidates at 64 pages per list (see refine_runs).
       constexpr int kPer = kSelThreads / 4;
-      const bool all_exact = ncand <= kPer;                  // a single round is not worth the sorting
-      const unsigned long long* by_bound = all_exact ? ckey : sm.r.skey;
-      unsigned long long* exact = all_exact ? sm.r.skey : ckey;
+      const bool every = !POOLED && all_exact;
+      const unsigned long long* by_bound = every ? ckey : sm.r.skey;
+      unsigned long long* exact = every ? sm.r.skey : ckey;
       int nclose = ncand;
-      if (!all_exact) {
+      if (!every) {
         const uint32_t wide = __reduce_max_sync(0xffffffffu, __float_as_uint(width));        // (not negative: ordered like its bits)
         if (lane == 0) atomicMax(&sm.r.width, wide);
-        if (ncand <= kSelThreads) {
-          // a candidate's position is the number of larger keys (all differ); one candidate per thread, the keys are read as
-          // broadcasts, four at a time
-          if ((tid & ~31) < ncand) {                         // whole warps without a candidate skip the count
-            const unsigned long long mine = tid < ncand ? ckey[tid] : ~0ull;
-            int rank = 0;
-            const int n4 = ncand & ~3;
-            for (int i = 0; i < n4; i += 4) {
-              const ulonglong2 k01 = *reinterpret_cast<const ulonglong2*>(&ckey[i]);
-              const ulonglong2 k23 = *reinterpret_cast<const ulonglong2*>(&ckey[i + 2]);
-              rank += (k01.x > mine ? 1 : 0) + (k01.y > mine ? 1 : 0) + (k23.x > mine ? 1 : 0) + (k23.y > mine ? 1 : 0);
-            }
-            for (int i = n4; i < ncand; ++i) rank += ckey[i] > mine ? 1 : 0;
-            if (tid < ncand) sm.r.skey[rank] = mine;
-          }
-        } else {
-          int n2 = 2;
-          while (n2 < ncand) n2 <<= 1;
-          for (int i = ncand + tid; i < n2; i += kSelThreads) ckey[i] = 0ull;
-          __syncthreads();
-          for (int k2 = 2; k2 <= n2; k2 <<= 1) {
-            for (int j = k2 >> 1; j > 0; j >>= 1) {
-              for (int t = tid; t < (n2 >> 1); t += kSelThreads) {
-                const int i = ((t & ~(j - 1)) << 1) | (t & (j - 1));
-                const int x = i | j;
-                const unsigned long long ka = ckey[i], kb = ckey[x];
-                if ((ka < kb) == ((i & k2) == 0)) { ckey[i] = kb; ckey[x] = ka; }
-              }
-              __syncthreads();
-            }
-          }
-          for (int i = tid; i < ncand; i += kSelThreads) sm.r.skey[i] = ckey[i];
+#pragma unroll 1
+        for (int i = tid; (i & ~31) < ncand; i += kSelThreads) {    // (whole warps without a candidate skip the count)
+          const unsigned long long mine = i < ncand ? ckey[i] : ~0ull;
+          const int rank = larger_keys(ckey, ncand, mine);
+          if (i < ncand) sm.r.skey[rank] = mine;
         }
         __syncthreads();
         width = __uint_as_float(sm.r.width);
@@ -730,7 +737,7 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
           auto lower = [&](int i) { return unorder_bits(static_cast<uint32_t>(by_bound[i] >> 32)); };
           auto starts = [&](int i) { return i == 0 || lower(i - 1) > __fadd_ru(lower(i), width); };
           const bool in = r < ncand, first = in && starts(r), last = in && (r + 1 == ncand || starts(r + 1));
-          const bool open = in && (out_scores || !(first && last));
+          const bool open = in && !(first && last);
           const uint32_t runs = __ballot_sync(0xffffffffu, first), opens = __ballot_sync(0xffffffffu, open);
           int at = 0;
           if (lane == 0) {
@@ -743,7 +750,7 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
         __syncthreads();
         nclose = sm.r.nclose;
       }
-      auto position = [&](int i) { return all_exact ? i : static_cast<int>(sm.r.close[i]); };
+      auto position = [&](int i) { return every ? i : static_cast<int>(sm.r.close[i]); };
       auto page_at = [&](int r) { return static_cast<int>(~reinterpret_cast<const uint32_t*>(by_bound)[2 * r]); };     // (a key's low word)
       int r_next = 0, pg_next = 0, ph_next = 0;
       if (nclose > 0) {
@@ -765,33 +772,30 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
       __syncthreads();
       // ---- a candidate's position: its run's, and the number of larger keys in the run (all differ); emit the first kk
       for (int r = tid; r < ncand; r += kSelThreads) {
-        int start = 0, end = ncand;
-        if (!all_exact) {
-          int w = r >> 5;
+        unsigned long long mine;
+        int rank;
+        if (every) {
+          mine = exact[r];
+          rank = larger_keys(exact, ncand, mine);
+        } else {
+          int w = r >> 5, end = ncand;
           uint32_t b = sm.r.run[w] & (0xffffffffu >> (31 - (r & 31)));
           while (b == 0u) b = sm.r.run[--w];
-          start = w * 32 + 31 - __clz(b);
+          const int start = w * 32 + 31 - __clz(b);
           if (start >= kk) continue;
           w = r >> 5;
           b = sm.r.run[w] & (0xfffffffeu << (r & 31));
           const int nw = (ncand + 31) >> 5;
           while (b == 0u && ++w < nw) b = sm.r.run[w];
           if (b) end = w * 32 + __ffs(b) - 1;
-        }
-        unsigned long long mine = by_bound[r];
-        int rank = start;
-        if (all_exact || end - start > 1 || out_scores) {
-          mine = exact[r];
-          for (int i = start; i < end; ++i) rank += exact[i] > mine ? 1 : 0;
-        }
-        if (rank < kk) {
-          const int pg = static_cast<int32_t>(0xffffffffu - static_cast<uint32_t>(mine));
-          for (int gi = 0; gi < pool; ++gi) {
-            out_pages[gi * p.k + rank] = pg;
-            if (out_scores) out_scores[gi * p.k + rank] = unorder_bits(static_cast<uint32_t>(mine >> 32));
+          mine = by_bound[r];
+          rank = start;
+          if (end - start > 1) {
+            mine = exact[r];
+            for (int i = start; i < end; ++i) rank += exact[i] > mine ? 1 : 0;
           }
-          mark(pg);
         }
+        if (rank < kk) emit(rank, mine);
       }
       for (int gi = 0; gi < pool; ++gi)
         for (int j = kk + tid; j < p.k; j += kSelThreads) out_pages[gi * p.k + j] = -1;
@@ -800,7 +804,10 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
       // (through shared memory: with four rounds' ids in registers the loop was unrolled, spilled, and a whole step
       // took 1 us longer with one 8K sequence, 2 us with eight of 32K)
       int* cphys = sm.r.cphys;
-      for (int i = tid; i < ncand; i += kSelThreads) cphys[i] = phys_of(cpage[i]);
+      for (int i = tid; i < ncand; i += kSelThreads) {
+        if (RUNS) cpage[i] = static_cast<int>(~static_cast<uint32_t>(ckey[i]));
+        cphys[i] = phys_of(cpage[i]);
+      }
       __syncthreads();
       constexpr int kPer = kSelThreads / 4;
 #pragma unroll 1
@@ -812,26 +819,11 @@ topk_refine_kernel(RefineParams p, BlockAttnParams bp) {
       // ---- order the candidates (descending) and emit the first kk
       __syncthreads();
       if (ncand <= kSelThreads) {
-        // few candidates (the usual case): a candidate's position is the number of larger keys (all
-        // keys differ); one candidate per thread, the keys are read as broadcasts, four at a time
+        // few candidates (the usual case): a candidate's position is the number of larger keys
         if ((tid & ~31) < ncand) {                       // whole warps without a candidate skip the count
           const unsigned long long mine = tid < ncand ? ckey[tid] : ~0ull;
-          int rank = 0;
-          const int n4 = ncand & ~3;
-          for (int i = 0; i < n4; i += 4) {
-            const ulonglong2 k01 = *reinterpret_cast<const ulonglong2*>(&ckey[i]);
-            const ulonglong2 k23 = *reinterpret_cast<const ulonglong2*>(&ckey[i + 2]);
-            rank += (k01.x > mine ? 1 : 0) + (k01.y > mine ? 1 : 0) + (k23.x > mine ? 1 : 0) + (k23.y > mine ? 1 : 0);
-          }
-          for (int i = n4; i < ncand; ++i) rank += ckey[i] > mine ? 1 : 0;
-          if (tid < ncand && rank < kk) {
-            const int pg = static_cast<int32_t>(0xffffffffu - static_cast<uint32_t>(mine));
-            for (int gi = 0; gi < pool; ++gi) {
-              out_pages[gi * p.k + rank] = pg;
-              if (out_scores) out_scores[gi * p.k + rank] = unorder_bits(static_cast<uint32_t>(mine >> 32));
-            }
-            mark(pg);
-          }
+          const int rank = larger_keys(ckey, ncand, mine);
+          if (tid < ncand && rank < kk) emit(rank, mine);
         }
         for (int gi = 0; gi < pool; ++gi)
           for (int j = kk + tid; j < p.k; j += kSelThreads) out_pages[gi * p.k + j] = -1;
@@ -1035,9 +1027,17 @@ int refine_slots(int lists, int resident, int block_size) {
 // Exact scores only where the bounds leave the order open (RUNS), or for every candidate.  The former saves two rounds of
 // gathers out of three at 64 pages per list (eight 32K prompts: 29 MB of summaries out of L2, 4.6 us of a list's 11.7; 20 of 67
 // candidates are close) and costs a sort on the bounds.  It pays where many lists share L2's bandwidth, or a score is the largest of a
-// group's.  Whole step, us, without and with it: 256 lists of 64 pages 108.3 / 105.9, 32 pooled lists of 64 71.4 / 70.8; 32 lists of 32
-// pages 35.7 / 36.2, 32 lists of 64 out of 2,048 pages 47.4 / 48.7.
-bool refine_runs(int lists, int pool, int k) { return k >= 48 && (pool > 1 || lists >= 128); }
+// group's and more than two rounds of scores are saved.  Not where the scores are asked for: all candidates need them then.
+// Whole step, us, without and with it, at 48 / 64 / 100 / 128 pages per list:
+//   256 lists (8 x 32K tokens)             95.1 / 106.1 / 125.8 / 143.1,  93.5 / 103.2 / 122.9 / 137.7
+//   128 lists (4 x 24K)                    58.0 / 62.3 / 71.1 / 79.9,  57.5 / 61.5 / 69.8 / 76.9
+//   128 lists (4 x 64K)                    70.1 / 76.8 / 92.2 / 103.9,  70.0 / 76.4 / 91.2 / 101.0
+//   96 lists (3 x 32K)                     52.3 / 56.3 / 64.1 / 71.8,  51.8 / 55.2 / 63.8 / 69.8
+//   32 lists (1 x 32K)                     37.5 / 39.0 / 42.5 / 47.1,  38.8 / 39.9 / 43.2 / 46.4
+//   8 pooled lists (8K)                    36.0 / 37.6 / 40.3 / 45.6,  36.4 / 36.4 / 39.6 / 41.4
+//   8 pooled lists (64K)                   42.9 / 45.5 / 48.7 / 55.4,  43.2 / 45.5 / 49.0 / 53.2
+//   64 pooled lists (8 x 16K, 8 active)    87.2 / 96.1 / 110.0 / 123.0,  85.7 / 92.1 / 105.5 / 114.6
+bool refine_runs(int lists, int pool, int k) { return pool > 1 ? k >= 60 : k >= 48 && lists >= 128; }
 
 bool selects_by_refinement(const losa_ctx* c, int32_t k, int selector) {
   return c->shape.dtype == LOSA_BF16 && (selector == kSelectorExact || selector == kSelectorPooled) && k <= kSelCap &&
@@ -1097,7 +1097,7 @@ int32_t launch_page_scores_topk(losa_ctx* c, const void* q, const losa_kv_t* kv,
       constexpr int D = decltype(d)::value, BK = decltype(bk)::value;
       const int split = in_step ? cudaSharedmemCarveoutMaxShared : cudaSharedmemCarveoutDefault;
       auto launch = [&](auto kernel) { launch_split(split, kernel, grid, kSelThreads, 0, st, rp, bp); };
-      const bool runs = refine_runs(lists, pool, k);
+      const bool runs = refine_runs(lists, pool, k) && !topk_scores_opt;
       if (pool > 1) launch(runs ? topk_refine_kernel<D, true, BK, true> : topk_refine_kernel<D, true, BK, false>);
       else launch(runs ? topk_refine_kernel<D, false, BK, true> : topk_refine_kernel<D, false, BK, false>);
     });

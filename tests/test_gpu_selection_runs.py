@@ -1,6 +1,6 @@
-"""Selection where only close candidates take exact scores (lists of 48 pages and more, many lists or pooled ones), against the
-oracle's lists: pages that tie exactly or differ in one bit of one key, lists shorter than the budget, more candidates than a
-CTA has threads, bounds kept in registers and read again, prefixes that tie as a whole."""
+"""Selection where only close candidates take exact scores (many lists of 48 pages and more, pooled ones of 60 and more), against the
+oracle's lists: pages that tie exactly or differ in one bit of one key, pages that crowd, lists shorter than the budget, more
+candidates than a CTA has threads, bounds kept in registers and read again, prefixes that tie as a whole."""
 import numpy as np
 import pytest
 
@@ -14,12 +14,14 @@ HEADS = dict(n_q_heads=32, n_kv_heads=4, head_dim=64, page_size=16)      # 4 seq
 
 
 @pytest.mark.parametrize("pooled", [False, True])
-@pytest.mark.parametrize("same", ["few", "pairs", "all"])
+@pytest.mark.parametrize("same", ["few", "pairs", "crowd", "all"])
 @pytest.mark.parametrize("kw", [
     dict(kv_lens=(16 * 100, 16 * 60 + 3, 16 * 48, 16 * 49), topk=48),            # 49 pages: every candidate but one is listed
     dict(kv_lens=(16 * 300, 16 * 129 + 1, 700, 0), topk=127),                    # 128 candidates and more: sorted as a whole
     dict(kv_lens=(16 * 1024, 16 * 1025 + 7, 16 * 64, 16 * 33), topk=64, m_active=1),
     dict(kv_lens=(32 * 90, 32 * 130 + 5, 32 * 70, 31), topk=50, page_size=32, head_dim=128, n_q_heads=32, n_kv_heads=8),
+    dict(kv_lens=(32 * 600, 32 * 130 + 5, 32 * 70, 32 * 61), topk=60, page_size=32, head_dim=128, n_q_heads=32, n_kv_heads=8),
+    dict(kv_lens=(16 * 700, 16 * 500, 16 * 401, 16 * 1100), topk=400, m_active=1),       # up to 512 candidates
 ])
 def test_lists_where_only_close_candidates_take_exact_scores(kw, same, pooled):
     import torch
@@ -34,6 +36,8 @@ def test_lists_where_only_close_candidates_take_exact_scores(kw, same, pooled):
                 w.k_pages[b] = w.k_pages[a]
                 if i % 3 == 0:
                     w.k_pages[b, :, i % g, i % cfg.head_dim] ^= 1        # the last bit of one key element per head
+            elif same == "crowd" and i < 20:             # 40 pages of one score: the other way, unless few pages are candidates
+                w.k_pages[a] = w.k_pages[b] = w.k_pages[w.page_table[s, 0]]
             elif same == "all":
                 w.k_pages[a] = w.k_pages[b] = w.k_pages[w.page_table[s, 0]]
     layers = [LosaLayer(cfg, w.k_pages, w.v_pages, w.page_table, w.kv_len, pooled=pooled) for _ in range(2)]
