@@ -51,7 +51,7 @@ struct losa_ctx {
   // cached TMA descriptors of the K / V pools (opaque 128-byte blobs, see sparse_prefix_attn.cu)
   alignas(64) unsigned char tmap_k[128];
   alignas(64) unsigned char tmap_v[128];
-  alignas(64) unsigned char tmap_vs[128];   // V once more, FP8: swizzled like K
+  alignas(64) unsigned char tmap_vs[128];   // FP8, d = 128: V once more, swizzled like K
   const void* tmap_key_k;
   const void* tmap_key_v;
   int64_t tmap_strides[3];

@@ -455,12 +455,16 @@ int32_t ensure_tensor_maps(losa_ctx* c, const losa_kv_t* kv) {
                     c->tmap_strides[2] == kv->stride_tok && c->tmap_n_phys == kv->n_phys_pages &&
                     c->tmap_format == kv->kv_format;
   if (same) return LOSA_OK;
-  int32_t rc = encode_pool_map(c, c->tmap_k, kv->k_pages, kv, false);
+  // (taken over together: a map of a new pool must not stay beside an old key when a later one cannot be encoded)
+  alignas(64) unsigned char k[128], v[128], vs[128];
+  const bool with_vs = kv->kv_format == LOSA_KV_FP8_E4M3 && c->shape.head_dim == 128;      // the kernel that has the narrow path
+  int32_t rc = encode_pool_map(c, k, kv->k_pages, kv, false);
+  if (rc == LOSA_OK) rc = encode_pool_map(c, v, kv->v_pages, kv, true);
+  if (rc == LOSA_OK && with_vs) rc = encode_pool_map(c, vs, kv->v_pages, kv, false);
   if (rc != LOSA_OK) return rc;
-  rc = encode_pool_map(c, c->tmap_v, kv->v_pages, kv, true);
-  if (rc != LOSA_OK) return rc;
-  rc = encode_pool_map(c, c->tmap_vs, kv->v_pages, kv, false);
-  if (rc != LOSA_OK) return rc;
+  memcpy(c->tmap_k, k, sizeof(k));
+  memcpy(c->tmap_v, v, sizeof(v));
+  if (with_vs) memcpy(c->tmap_vs, vs, sizeof(vs));
   c->tmap_key_k = kv->k_pages;
   c->tmap_key_v = kv->v_pages;
   c->tmap_strides[0] = kv->stride_page;
@@ -518,20 +522,22 @@ int32_t prepare_f32(losa_ctx* c) {
 
 template <int D, int GP, bool FP8>
 int32_t launch_tc5(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool with_combine) {
-  CUtensorMap mk, mv, mvs;
-  memcpy(&mk, c->tmap_k, sizeof(mk));
-  memcpy(&mv, c->tmap_v, sizeof(mv));
-  memcpy(&mvs, c->tmap_vs, sizeof(mvs));
   if (c->profile) LOSA_CUDA_TRY(c, cudaEventRecord(c->ev_begin, st));
   // With the narrow path where shares of eight groups of 128 tokens, its least, are to be expected: a sparse step lists about a quarter of a
   // cache.  The kernel that has it starts 1.5 us later on the other path (2,600 tokens, a step 63 us, 65 with it).
-  auto launch = [&](auto kernel) { launch_k(kernel, ap.n_ctas, tc5_threads<FP8>(), tc5_smem_bytes<D, GP, FP8>(), st, mk, mv, mvs, ap); };
+  auto launch = [&](auto kernel, const auto& maps) { launch_k(kernel, ap.n_ctas, tc5_threads<FP8>(), tc5_smem_bytes<D, GP, FP8>(), st, maps, ap); };
+  auto map_of = [](const unsigned char* blob) {
+    CUtensorMap m;
+    memcpy(&m, blob, sizeof(m));
+    return m;
+  };
+  const CUtensorMap mk = map_of(c->tmap_k), mv = map_of(c->tmap_v);
   bool narrow = false;
   if constexpr (FP8 && D == 128) {
     narrow = static_cast<int64_t>(ap.n_sk) * ap.Pmax * GP >= static_cast<int64_t>(ap.n_ctas) * 4 * 8 * kTc5Tok;
-    if (narrow) launch(attn_tc5_kernel<D, GP, FP8, true>);
+    if (narrow) launch(attn_tc5_kernel<D, GP, FP8, true>, Tc5Maps<true>{mk, mv, map_of(c->tmap_vs)});
   }
-  if (!narrow) launch(attn_tc5_kernel<D, GP, FP8, false>);
+  if (!narrow) launch(attn_tc5_kernel<D, GP, FP8, false>, Tc5Maps<false>{mk, mv});
   if (c->profile) LOSA_CUDA_TRY(c, cudaEventRecord(c->ev_end, st));
   int32_t rc = after_launch(c);
   if (rc != LOSA_OK || !with_combine) return rc;

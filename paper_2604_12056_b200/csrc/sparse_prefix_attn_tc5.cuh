@@ -231,9 +231,11 @@ __device__ __forceinline__ uint32_t tc5_sw(int t, int c) { return static_cast<ui
 // largest, 2^-14 without scales.  Staging slots are single pages, so that one is refilled while its
 // neighbours are converted.
 // NARROW: with the narrow path (chosen by launch_tc5 on the size of the cache).
+template <bool NARROW> struct Tc5Maps { CUtensorMap k, v; };
+template <> struct Tc5Maps<true> { CUtensorMap k, v, vs; };      // vs: V once more, swizzled like K
 template <int D, int GP, bool FP8, bool NARROW>
 __global__ void __launch_bounds__(tc5_threads<FP8>(), 1)
-attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmVs, AttnParams p) {
+attn_tc5_kernel(const __grid_constant__ Tc5Maps<NARROW> maps, AttnParams p) {
   constexpr int NRK = tc5_ring_slots<D, GP, FP8>(false), NRV = tc5_ring_slots<D, GP, FP8>(true);   // slots per ring
   constexpr int NSP = FP8 ? tc5_stg_slots<D, GP>() : 1, STG = GP * D;   // FP8: staging slots of V, bytes of a slot (one page of codes)
   constexpr int NT = tc5_threads<FP8>();
@@ -436,7 +438,9 @@ attn_tc5_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     auto start = [&]() {                               // before the first copies: which path, hence which slots
       const bool ok = choose_path();
       staging = FP8 && is_v && !narrow;
-      map = is_v ? (NARROW && narrow ? &tmVs : &tmV) : &tmK;
+      map = is_v ? &maps.v : &maps.k;
+      if constexpr (NARROW)
+        if (is_v && narrow) map = &maps.vs;
       ring = is_v ? (NARROW && narrow ? cta.vring : vring) : kring;
       return ok;
     };
