@@ -523,8 +523,6 @@ int32_t prepare_f32(losa_ctx* c) {
 template <int D, int GP, bool FP8>
 int32_t launch_tc5(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool with_combine) {
   if (c->profile) LOSA_CUDA_TRY(c, cudaEventRecord(c->ev_begin, st));
-  // With the narrow path where shares of eight groups of 128 tokens, its least, are to be expected: a sparse step lists about a quarter of a
-  // cache.  The kernel that has it starts 1.5 us later on the other path (2,600 tokens, a step 63 us, 65 with it).
   auto launch = [&](auto kernel, const auto& maps) { launch_k(kernel, ap.n_ctas, tc5_threads<FP8>(), tc5_smem_bytes<D, GP, FP8>(), st, maps, ap); };
   auto map_of = [](const unsigned char* blob) {
     CUtensorMap m;
@@ -532,12 +530,15 @@ int32_t launch_tc5(losa_ctx* c, const AttnParams& ap, cudaStream_t st, bool with
     return m;
   };
   const CUtensorMap mk = map_of(c->tmap_k), mv = map_of(c->tmap_v);
-  bool narrow = false;
+  // With the narrow path from 32 groups of 128 tokens per CTA in the whole table on.  How much of it the prompts fill, and whether a
+  // step has few rows, is known on the device only: in the kernel that has both paths a step that takes the other one is 0.5 us
+  // longer, in a large cache 1 % and less (64 segments, shares of 2 / 8 / 32 groups 18.0 / 27.6 / 55.9 us, 18.6 / 28.1 / 56.3).
+  bool both = false;
   if constexpr (FP8 && D == 128) {
-    narrow = static_cast<int64_t>(ap.n_sk) * ap.Pmax * GP >= static_cast<int64_t>(ap.n_ctas) * 4 * 8 * kTc5Tok;
-    if (narrow) launch(attn_tc5_kernel<D, GP, FP8, true>, Tc5Maps<true>{mk, mv, map_of(c->tmap_vs)});
+    both = static_cast<int64_t>(ap.n_sk) * ap.Pmax * GP >= static_cast<int64_t>(ap.n_ctas) * 32 * kTc5Tok;
+    if (both) launch(attn_tc5_kernel<D, GP, FP8, true>, Tc5Maps<true>{mk, mv, map_of(c->tmap_vs)});
   }
-  if (!narrow) launch(attn_tc5_kernel<D, GP, FP8, false>, Tc5Maps<false>{mk, mv});
+  if (!both) launch(attn_tc5_kernel<D, GP, FP8, false>, Tc5Maps<false>{mk, mv});
   if (c->profile) LOSA_CUDA_TRY(c, cudaEventRecord(c->ev_end, st));
   int32_t rc = after_launch(c);
   if (rc != LOSA_OK || !with_combine) return rc;

@@ -28,7 +28,8 @@ constexpr int kTc5CvtWarp = 16, kTc5CvtWarps = 4; // FP8 pages: four warps that 
 template <bool FP8> constexpr int tc5_threads() { return FP8 ? 640 : 512; }
 // Registers per thread at the launch, and as they are dealt out to the softmax warps and the others:
 // 12 x 32 x 136 + 4 x 32 x 104 = 512 x 128; FP8 12 x 32 x 112 + 8 x 32 x 72 = 640 x 96;
-// with the narrow path, whose producers would spill at 72 and are then late with every copy, 104 and 80.
+// with the narrow path in the kernel, whose producers would spill at 72 and are then late with every copy, 104 and 80 (one deal for
+// both paths: with two in a kernel the compiler spills everywhere).
 constexpr int kTc5LaunchRegs = 128, kTc5SoftmaxRegs = 136, kTc5OtherRegs = 104;
 constexpr int kTc5LaunchRegs8 = 96, kTc5SoftmaxRegs8 = 112, kTc5OtherRegs8 = 72, kTc5nSoftmaxRegs = 104, kTc5nOtherRegs = 80;
 static_assert(kTc5SoftmaxWarps * kTc5SoftmaxRegs + 4 * kTc5OtherRegs <= 16 * kTc5LaunchRegs, "registers");
@@ -63,7 +64,7 @@ template <int GP, bool FP8> constexpr int tc5_tail_bytes() {
 template <int D> constexpr int tc5_slot_bytes() { return kTc5Tok * D * 2; }                              // V, and bf16 K
 template <int D, bool FP8> constexpr int tc5_kslot_bytes() { return kTc5Tok * D * (FP8 ? 1 : 2); }
 constexpr int kTc5QTerms = 3;                    // FP8: E5M2 terms of a query
-constexpr int kTc5nRows = 16;                    // FP8: most query rows of a share on the narrow path (sparse_prefix_attn_tc5n.cuh)
+constexpr int kTc5nRows = 16;                    // FP8: most query rows of a segment on the narrow path (sparse_prefix_attn_tc5n.cuh)
 constexpr int kTc5nLanes = 32;                   // entries of its per-row arrays, one per lane
 constexpr int kTc5nP = kTc5Tok * 16;             // bytes of one term of 16 rows of its P'
 constexpr int kTc5PTerms = 3;                    // E5M2 terms of P'
@@ -230,17 +231,17 @@ __device__ __forceinline__ uint32_t tc5_sw(int t, int c) { return static_cast<ui
 // the reference lies 2^7 below the maximum.  A weight is then subnormal only 2^-15 or more below its row's
 // largest, 2^-14 without scales.  Staging slots are single pages, so that one is refilled while its
 // neighbours are converted.
-// NARROW: with the narrow path (chosen by launch_tc5 on the size of the cache).
-template <bool NARROW> struct Tc5Maps { CUtensorMap k, v; };
+// BOTH: with the narrow path (chosen by launch_tc5 on the size of the cache).
+template <bool BOTH> struct Tc5Maps { CUtensorMap k, v; };
 template <> struct Tc5Maps<true> { CUtensorMap k, v, vs; };      // vs: V once more, swizzled like K
-template <int D, int GP, bool FP8, bool NARROW>
+template <int D, int GP, bool FP8, bool BOTH>
 __global__ void __launch_bounds__(tc5_threads<FP8>(), 1)
-attn_tc5_kernel(const __grid_constant__ Tc5Maps<NARROW> maps, AttnParams p) {
+attn_tc5_kernel(const __grid_constant__ Tc5Maps<BOTH> maps, AttnParams p) {
+  static_assert(!BOTH || (FP8 && D == 128), "the narrow path");   // (d = 64: a group's bytes are HBM's 675 cycles, less than that path's own)
   constexpr int NRK = tc5_ring_slots<D, GP, FP8>(false), NRV = tc5_ring_slots<D, GP, FP8>(true);   // slots per ring
   constexpr int NSP = FP8 ? tc5_stg_slots<D, GP>() : 1, STG = GP * D;   // FP8: staging slots of V, bytes of a slot (one page of codes)
   constexpr int NT = tc5_threads<FP8>();
-  static_assert(!NARROW || (FP8 && D == 128), "the narrow path");   // (d = 64: a group's bytes are HBM's 675 cycles, less than that path's own)
-  constexpr int NN = NARROW ? tc5n_slots<D, GP>() : 1;   // narrow: slots of K, and of V
+  constexpr int NN = BOTH ? tc5n_slots<D, GP>() : 1;   // narrow: slots of K, and of V
   constexpr int KSLOT = tc5_kslot_bytes<D, FP8>(), SLOT = tc5_slot_bytes<D>(), QB = tc5_q_bytes<D, FP8>();
   constexpr int PG = kTc5Tok / GP;              // pages per group
   constexpr int MR = kTc5MetaRing;              // groups of the meta ring
@@ -258,7 +259,7 @@ attn_tc5_kernel(const __grid_constant__ Tc5Maps<NARROW> maps, AttnParams p) {
   // has to lie two groups back at least, where all four warps have finished (less than two groups lie between them).
   static_assert(!FP8 || (NSP >= 2 * PG && NSP <= kTc5StgMax), "staging ring");
   static_assert(NRK + 2 < MR && NN + 3 < MR, "the producer's lead fits the meta ring");   // (narrow: a set reads the ring until it leaves P')
-  static_assert(!NARROW || (NN >= 2 && NN * 2 * KSLOT <= NRK * KSLOT + NRV * SLOT + NSP * STG), "narrow: slots");
+  static_assert(!BOTH || (NN >= 2 && NN * 2 * KSLOT <= NRK * KSLOT + NRV * SLOT + NSP * STG), "narrow: slots");
   constexpr int kBars = 4 * 6 + 3 * SB + 3 + 4 + 4 * SB + 2 + 2 * SB + 2;
   static_assert(8 * kBars + 16 <= 512, "tail layout");
 
@@ -317,7 +318,7 @@ attn_tc5_kernel(const __grid_constant__ Tc5Maps<NARROW> maps, AttnParams p) {
     mbar_init(o_free, kTc5SoftmaxWarps);
     for (int i = 0; i < 4; ++i) mbar_init(xbar + 8 * i, kTc5Sets);
     for (int i = 0; i < 4 * SB; ++i) mbar_init(mbar + 8 * i, 1);
-    if (NARROW) {
+    if (BOTH) {
       for (int b = 0; b < SB; ++b) {
         mbar_init(s_read + 8 * b, kTc5SetWarps);       // the set's scores have been read
         mbar_init(meet + 8 * b, kTc5SetWarps);         // the set's warps meet
@@ -355,8 +356,12 @@ attn_tc5_kernel(const __grid_constant__ Tc5Maps<NARROW> maps, AttnParams p) {
       if (!p.early) len_s[i] = p.kv_len[i];
     }
   }
+  bool many_rows = false;                          // for the narrow path, in any sequence
+  if (BOTH && warp > 0)
+    for (int i = tid - 32; i < p.N; i += NT - 32) many_rows |= clamp_active(p.n_active[i], p.B) * p.G > kTc5nRows;
   tc5_fence_before();
-  __syncthreads();
+  if constexpr (BOTH) many_rows = __syncthreads_or(many_rows) != 0;
+  else __syncthreads();
   tc5_fence_after();
   const uint32_t tmem = *tmem_slot;
   // this CTA's share of the charged list, mapped back to pages: the first page at or after a charged position
@@ -399,29 +404,28 @@ attn_tc5_kernel(const __grid_constant__ Tc5Maps<NARROW> maps, AttnParams p) {
   cta.abort_flag = abort_flag; cta.pre = pre; cta.tok_s = tok_s; cta.na_s = na_s; cta.staged = staged;
   cta.scratch = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(mref) + 15) & ~static_cast<uintptr_t>(15));
   cta.meta = meta; cta.kscale_meta = kscale_meta; cta.vlog_meta = vlog_meta; cta.tmem = tmem; cta.lo = lo; cta.hi = hi; cta.sg0 = sg0;
-  // A share of eight groups or more (a group costs 650 cycles less this way, the start 1.9 us more), few rows in all of
-  // its segments, and value scales (positive, of one size within a factor of four): tokens take the lanes (see the narrow path's
-  // header).  The scales are the last of three dependent reads, for the softmax warps, which look at them all, as for the
-  // producers, whose copies wait for the answer.
-  bool narrow = NARROW && hi - lo >= 8 * PG;
-  for (int sg = sg0; narrow && sg < p.n_seg && pre[sg] < hi; ++sg)
-    if (pre[sg + 1] > pre[sg]) narrow = cta.rows_of(p, sg) <= kTc5nRows;
-  const bool few_rows = narrow;
+  // The roles, once with the narrow path and once without: wide code that asks which path it is on is a tenth slower (shares of 32
+  // groups 55.9 us, 61.7).
+  auto roles = [&](auto narrow_too) {
+  constexpr bool NARROW = decltype(narrow_too)::value;
+  // Narrow: the share's value scales (positive, of one size within a factor of four) have the last word.  They are the last of three
+  // dependent reads, for the softmax warps, which look at them all, as for the producers, whose copies wait for the answer.
+  bool narrow = NARROW;
   float* scale_lo = reinterpret_cast<float*>(const_cast<int*>(meta)) + 3 * MR * PG;      // [8] smallest and largest, per warp that looks
   float* scale_hi = scale_lo + kTc5ScaleWarps;
   auto choose_path = [&]() {                         // false: a wait has run out
-    if (!NARROW || !few_rows) return true;
+    if (!NARROW) return true;
     if (!warp_mbar_wait(path_bar, 0, abort_flag, p.status, p.wait_cycles)) return false;
     float a = INFINITY, b = 0.f;
 #pragma unroll
     for (int w = 0; w < kTc5ScaleWarps; ++w) { a = fminf(a, scale_lo[w]); b = fmaxf(b, scale_hi[w]); }
-    narrow = a > 1e-18f && b < 1e18f && b <= 4.f * a;
+    narrow = warp_uniform(a > 1e-18f && b < 1e18f && b <= 4.f * a ? 1 : 0) != 0;
     return true;
   };
 
   int issued = -1;                                   // producer warps: newest group (FP8: page) whose copies have been issued
   if (warp >= kTc5SoftmaxWarps) {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(NARROW ? kTc5nOtherRegs : FP8 ? kTc5OtherRegs8 : kTc5OtherRegs));   // whole warpgroups
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(BOTH ? kTc5nOtherRegs : FP8 ? kTc5OtherRegs8 : kTc5OtherRegs));   // whole warpgroups
   if (warp == kTc5KWarp || warp == kTc5VWarp) {
     // ------------------------------------------------------------------ producer warps: one for K, one for V
     // Lane j of a batch of 32 consecutive items resolves item -> logical page -> physical page (a
@@ -439,7 +443,7 @@ attn_tc5_kernel(const __grid_constant__ Tc5Maps<NARROW> maps, AttnParams p) {
       const bool ok = choose_path();
       staging = FP8 && is_v && !narrow;
       map = is_v ? &maps.v : &maps.k;
-      if constexpr (NARROW)
+      if constexpr (BOTH)
         if (is_v && narrow) map = &maps.vs;
       ring = is_v ? (NARROW && narrow ? cta.vring : vring) : kring;
       return ok;
@@ -759,8 +763,8 @@ attn_tc5_kernel(const __grid_constant__ Tc5Maps<NARROW> maps, AttnParams p) {
   }
   } else {
     // ------------------------------------------------------------------ softmax / epilogue warps
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(NARROW ? kTc5nSoftmaxRegs : FP8 ? kTc5SoftmaxRegs8 : kTc5SoftmaxRegs));
-    if (NARROW && few_rows && warp < kTc5ScaleWarps) {  // the share's value scales (the last set has its instructions to fetch)
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(BOTH ? kTc5nSoftmaxRegs : FP8 ? kTc5SoftmaxRegs8 : kTc5SoftmaxRegs));
+    if (NARROW && warp < kTc5ScaleWarps) {  // the share's value scales (the last set has its instructions to fetch)
       float a = INFINITY, b = 0.f;
       int sg = sg0;
       for (int i = lo + tid; i < hi; i += kTc5ScaleWarps * 32) {
@@ -783,9 +787,9 @@ attn_tc5_kernel(const __grid_constant__ Tc5Maps<NARROW> maps, AttnParams p) {
       }
     }
     if constexpr (NARROW) {
-      if (few_rows) tc5n_softmax<D, GP>(p, cta, [&]() { return choose_path() && narrow; });
+      tc5n_softmax<D, GP>(p, cta, [&]() { return choose_path() && narrow; });
     }
-    if (few_rows && (narrow || *abort_flag)) {
+    if (NARROW && (narrow || *abort_flag)) {
     } else {
     // Thread = query row (tensor-memory lane 32 * (warp % 4) + lane); set h = warp / 4 takes the groups
     // h, h + 3, ..., all columns, in S buffer h.  The three warps of a scheduler work on different groups, a
@@ -1137,6 +1141,19 @@ attn_tc5_kernel(const __grid_constant__ Tc5Maps<NARROW> maps, AttnParams p) {
       mbar_drain(bar, 0);
     }
     __syncthreads();
+  }
+  };
+  // Few rows in all sequences and shares of a group or more: tokens take the lanes (see the narrow path's header).  Every CTA comes to
+  // the same answer: with CTAs of both kinds in one grid, which fetch both paths' instructions behind each other's page
+  // copies, a grid takes longer than either way alone (shares of eight groups, 64 segments: 27.6 us wide, 22.9 narrow, 36.7 where
+  // every other share was a page too short).  Shares of 1 / 3 / 5 / 16 groups, one sequence of 12 rows per KV head: 17.0 / 19.7 /
+  // 22.4 / 34.8 us wide, 16.4 / 18.0 / 19.4 / 27.7 narrow.  (warp_uniform: under a branch that might diverge the products take
+  // no uniform operands, and the wide path 60.2 us for shares of 32 groups, 56.3 so.)
+  if constexpr (BOTH) {
+    if (warp_uniform(!many_rows && pre[p.n_seg] >= PG * n_share ? 1 : 0) != 0) roles(std::true_type{});
+    else roles(std::false_type{});
+  } else {
+    roles(std::false_type{});
   }
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(TMEM_COLS) : "memory");
 }

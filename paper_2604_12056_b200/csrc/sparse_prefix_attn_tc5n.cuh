@@ -1,5 +1,6 @@
 // Stage 4 on FP8 pages, shares of few query rows (sparse steps): the other way round.  Included by
-// sparse_prefix_attn_tc5.cuh (same namespace); part of attn_tc5_kernel, which decides per CTA.
+// sparse_prefix_attn_tc5.cuh (same namespace); part of attn_tc5_kernel, which decides for the whole grid, and once more per CTA on
+// the value scales.
 //
 // A sparse step has m active tokens x G heads, 4 to 32 rows for the most part, where the tile of sparse_prefix_attn_tc5.cuh has 128: there the
 // softmax is one warp's work per group (128 exponentials per thread, one after the other) while the others of its set idle,
@@ -25,7 +26,7 @@
 // so nothing passes from group to group; they meet at the end of a piece, where their outputs are merged.  The four warps of a
 // set agree on a reference in two steps: one flag per warp, and only if one is raised the maxima over the tokens.
 // Same producers and records as the wide path; K and V have rings of group-sized slots; the converting warps have nothing to do.
-// Only for d = 128 and shares of eight groups or more (see attn_tc5_kernel); 32 rows as two blocks of columns spill registers and took
+// Only for d = 128 and shares of a group or more (see attn_tc5_kernel); 32 rows as two blocks of columns spill registers and took
 // 852 us for the block where one takes 804.  bf16 pages stay with the wide path: it waits for HBM on sparse steps, and its first group has less code to fetch behind the
 // page copies (four steps of eight 32K prompts 435 us wide, 441 this way; eight of one 8K sequence 285 and 284).
 #pragma once
