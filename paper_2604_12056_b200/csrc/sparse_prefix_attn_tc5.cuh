@@ -408,8 +408,12 @@ attn_tc5_kernel(const __grid_constant__ Tc5Maps<BOTH> maps, AttnParams p) {
   // groups 55.9 us, 61.7).
   auto roles = [&](auto narrow_too) {
   constexpr bool NARROW = decltype(narrow_too)::value;
-  // Narrow: the share's value scales (positive, of one size within a factor of four) have the last word.  They are the last of three
-  // dependent reads, for the softmax warps, which look at them all, as for the producers, whose copies wait for the answer.
+  // Narrow: the share's value scales have the last word.  They must be positive, and so close to one another that no weight keeps fewer
+  // bits than on the other path: P' holds a page's whole scale here, under a reference 2^4 higher, the part from 2^-6 to 2^0
+  // there.  (Values up to 448 have no larger scales, and always pass.  With a limit of four, a hundredth of the pages eight times the
+  // others' scale sent half of the CTAs the other way: a step of eight 32K prompts 120 us, 108 with all of them on it, 83 so.)
+  // They are the last of three dependent reads, for the softmax warps, which look at them all, as for the producers, whose copies
+  // wait for the answer.
   bool narrow = NARROW;
   float* scale_lo = reinterpret_cast<float*>(const_cast<int*>(meta)) + 3 * MR * PG;      // [8] smallest and largest, per warp that looks
   float* scale_hi = scale_lo + kTc5ScaleWarps;
@@ -419,7 +423,8 @@ attn_tc5_kernel(const __grid_constant__ Tc5Maps<BOTH> maps, AttnParams p) {
     float a = INFINITY, b = 0.f;
 #pragma unroll
     for (int w = 0; w < kTc5ScaleWarps; ++w) { a = fminf(a, scale_lo[w]); b = fmaxf(b, scale_hi[w]); }
-    narrow = warp_uniform(a > 1e-18f && b < 1e18f && b <= 4.f * a ? 1 : 0) != 0;
+    auto in_p = [](float v) { return fminf(fmaxf(v, 0.015625f), 1.f); };
+    narrow = warp_uniform(a > 1e-18f && b < 1e18f && b * in_p(a) <= 16.f * a * in_p(b) ? 1 : 0) != 0;
     return true;
   };
 

@@ -1,5 +1,5 @@
 """Stage 4 on FP8 pages with few query rows (tokens on the tensor cores' lanes, values as an operand): rows about the limit
-of 16, value scales about the factor of four up to which that path is taken, groups of pages that end inside a
+of 16, value scales about the spread up to which that path is taken, groups of pages that end inside a
 product's 32 tokens, rising and falling scores, tails that hold NaN; against float64 over the listed pages."""
 import numpy as np
 import pytest
@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("g,d", [(16, 128), (32, 128), (64, 128), (32, 64)])       # (d = 64: the other path)
 @pytest.mark.parametrize("m,G", [(1, 1), (5, 3), (4, 4), (17, 1)])               # 1, 15, 16 and 17 rows (17: the other path)
-@pytest.mark.parametrize("powers", [(0,), (0, 1, 2), (0, 3), (1, 4), (-9, -8)])    # of the pages' values (a scale is 2^-6 at least: 0 and 3 are four apart)
+@pytest.mark.parametrize("powers", [(0,), (0, 1, 2), (0, 3), (1, 7), (1, 11), (1, 12), (-9, -8)])    # of the pages' values (a scale is 2^-6 at least)
 def test_few_rows_against_float64(g, d, m, G, powers):
     import torch
     from paper_2604_12056_b200.layer import LosaLayer
@@ -66,7 +66,7 @@ def test_value_scales_that_are_no_positive_numbers_take_the_other_path(odd):
 
 
 @pytest.mark.parametrize("g", [16, 32, 64])
-@pytest.mark.parametrize("powers", [(1, 4), (0, 1)])                          # the other path (scales eight apart), this one
+@pytest.mark.parametrize("powers", [(1, 12), (0, 1)])                         # the other path (scales 2^11 apart), this one
 def test_few_rows_in_shares_of_short_pieces(g, powers):
     """Shares of some 30 groups, but pieces of one to ten: a piece ends before the last set of softmax warps has had a group,
     and the share's first one while that set may still be in its walk without a group, whichever path the others are on.
@@ -101,9 +101,9 @@ def test_few_rows_in_shares_of_short_pieces(g, powers):
         assert torch.equal(layer.o_p, first[0]) and torch.equal(layer.lse_p, first[1])
 
 
-def hot_token_per_prompt(g, m, G, powers, above):
+def hot_token_per_prompt(g, m, G, powers, above, faint=0):
     """Prompts whose first page holds one token with a score `above` (log2 units) over all others, which are about equal, and in whose
-    column 5 only that page's other tokens have values: the column is theirs alone, beside a weight of one.  Long enough for
+    column 5 only the tokens of page `faint` have values: the column is theirs alone, beside a weight of one.  Long enough for
     twice the shares of eight groups that are this path's least, whatever the number of SMs."""
     import torch
     from paper_2604_12056_b200.layer import LosaLayer
@@ -122,7 +122,7 @@ def hot_token_per_prompt(g, m, G, powers, above):
     vp = rnd(N * mp, Hkv, g, d).clamp(-3.4, 3.4)
     vp[..., 5] = 0.0
     vp[:, :, 0, 0] = 3.5                                    # (every page's largest value: its scale is known)
-    vp[0::mp, :, :, 5] = 1.0 + rnd(N, Hkv, g).abs().clamp_max(2.0)
+    vp[faint::mp, :, :, 5] = 1.0 + rnd(N, Hkv, g).abs().clamp_max(2.0)
     vp[0::mp, :, 3, 5] = 0.0
     kp[0::mp, :, 3] = u * (above * float(np.log(2.0)) / (4.0 * cfg.sm_scale))
     vp *= torch.exp2(torch.tensor(powers, device="cuda")[torch.arange(N * mp, device="cuda") % len(powers)].float())[:, None, None, None]
@@ -155,8 +155,24 @@ def test_small_weights_beside_a_large_one_keep_their_bits(g, m, G, above):
 
 
 @pytest.mark.parametrize("g", [16, 32, 64])
-@pytest.mark.parametrize("m,G,powers,few", [(1, 1, (0,), True), (4, 4, (1, 2, 3), True), (16, 1, (3, 1), True), (17, 1, (1,), False),
-                                            (4, 4, (1, 4), False), (1, 1, (4, 2, 1), False)])
+@pytest.mark.parametrize("powers,above", [((7, 1), 12), ((7, 1), 18), ((4, 1), 21), ((11, 1), 14)])
+def test_small_weights_on_pages_of_small_scale_keep_their_bits(g, powers, above):
+    """As above, the large weight on a page whose values are 2^(p0 - p1) as large: a weight's P' carries its page's scale, so it
+    keeps eleven bits down to 2^(p0 - p1 - 25) of the row's largest."""
+    import torch
+    layer, cfg, q = hot_token_per_prompt(g, 4, 4, powers, above, faint=1)
+    for s in range(cfg.batch):
+        for h in range(cfg.n_kv_heads):
+            k, v = listed_prefix(layer, cfg, s, h)
+            heads = slice(4 * h, 4 * h + 4)
+            p = torch.softmax(q[s, :, heads].double() @ k.T * cfg.sm_scale, -1)
+            want = p @ v[:, 5]
+            assert ((layer.o_p[s, :, heads, 5].double() - want).abs() <= 2.0 ** -10 * want).all(), (s, h)
+
+
+@pytest.mark.parametrize("g", [16, 32, 64])
+@pytest.mark.parametrize("m,G,powers,few", [(1, 1, (0,), True), (4, 4, (1, 7), True), (16, 1, (11, 1), True), (17, 1, (1,), False),
+                                            (4, 4, (1, 12), False), (1, 1, (7, 11, 7), True), (1, 1, (7, 12, 7), False)])
 def test_which_path_a_share_takes(g, m, G, powers, few):
     """A weight of 2^-34 of its row's largest is 2^-23 under this path's reference, a value fp16 has, and 2^-27 under the other
     path's, less than half of its smallest: the column tells which one the share took."""
@@ -165,7 +181,7 @@ def test_which_path_a_share_takes(g, m, G, powers, few):
 
 
 @pytest.mark.parametrize("g", [16, 32, 64])
-@pytest.mark.parametrize("powers", [(1,), (1, 4)])                            # this path, the other one
+@pytest.mark.parametrize("powers", [(1,), (1, 12)])                           # this path, the other one
 @pytest.mark.parametrize("where", ["key scale", "key code", "query"])
 def test_values_that_are_no_numbers_stay_in_the_cached_state(g, powers, where):
     """A listed page whose key scale or one of whose key codes is NaN leaves NaN in o_p of all rows of its KV head, and a query
