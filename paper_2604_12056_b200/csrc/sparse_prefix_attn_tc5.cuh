@@ -899,9 +899,11 @@ attn_tc5_kernel(const __grid_constant__ Tc5Maps<BOTH> maps, AttnParams p) {
       float m_ref = -INFINITY, l = 0.f;                         // l: the groups of this set, relative to m_ref
       // The last set, which has time until the share's third group, first takes one that is not there: no waits, no arrivals, nothing
       // written.  It fetches the loop's instructions while the producers still look for their pages; the first group's set
-      // would wait for every line of them behind the page copies (a step of one 64K sequence 42.5 us, 41.9 so, of one of 128K 47.7 and
-      // 47.2).  Longer shares wait for HBM from the start: eight 32K prompts, 36 groups, 105.2 us without it and 105.5 with it.
-      int dry = piece == 0 && h == kTc5Sets - 1 && hi - lo < 24 * PG ? 1 : 0;
+      // would wait for every line of them behind the page copies (two steps of one 64K sequence in two layers 164.8 us, 163.8 so, of one of
+      // 128K 188.0 and 186.8, of pooled lists 282.3 and 280.0).  Not where a first piece of one or two groups ends before others of the
+      // share: the sets meet there, and this one would come late (64 segments, shares of one group 14.0 us, 15.0 with the walk).
+      // Longer shares wait for HBM from the start: eight 32K prompts, 36 groups, 420.3 us without it and 420.9 with it.
+      int dry = piece == 0 && h == kTc5Sets - 1 && hi - lo < 24 * PG && (seg_end == hi || seg_end - item >= 3 * PG) ? 1 : 0;
       for (int first = item; first < seg_end && ok;) {
         asm volatile("" : "+r"(dry));                           // (one copy of the code)
         const int turn = g % kTc5Sets;
