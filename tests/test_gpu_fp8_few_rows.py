@@ -205,3 +205,66 @@ def test_values_that_are_no_numbers_stay_in_the_cached_state(g, powers, where):
     assert layer.ctx.poll_status() == 0
     assert torch.isnan(layer.o_p[bad]).all() and torch.isfinite(layer.o_p[~bad]).all()
     assert not torch.isfinite(layer.lse_p[bad]).any() and torch.isfinite(layer.lse_p[~bad]).all()
+
+
+def assert_this_path(layer, cfg, rows):
+    """What launch and kernel decide by: the table's length, the rows, the pages listed."""
+    import torch
+    n_sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert layer.union_count.numel() * cfg.max_pages_per_seq * cfg.page_size >= n_sms * 32 * 128
+    assert rows <= 16 and int(layer.union_count.sum()) >= n_sms * 128 // cfg.page_size
+
+
+@pytest.mark.parametrize("state_bf16", [False, True])
+@pytest.mark.parametrize("pooled", [False, True])
+def test_few_rows_of_whole_steps(pooled, state_bf16):
+    """Short prompts in a table for long ones: sparse steps through the whole-step call, both selectors and state formats,
+    against the six calls' bits and float64 over the listed pages; the first step, with all rows, beside them."""
+    import torch
+    from paper_2604_12056_b200.layer import LosaLayer
+    N, m, lens = 4, 3, (2500, 3000, 1801, 2200)
+    n_sms = torch.cuda.get_device_properties(0).multi_processor_count
+    cfg = wl.config("c2", kv_lens=(n_sms * 32 * 128 // (N * 8) + 64,) * N, block_size=16, steps=4, topk=24, m_active=m)
+    w = wl.DeviceWorkload(cfg)
+    layers = [LosaLayer(cfg, w.k_pages, w.v_pages, w.page_table, w.kv_len, fp8_kv=True, pooled=pooled, state_bf16=state_bf16) for _ in range(2)]
+    exact = LosaLayer(cfg, w.k_pages, w.v_pages, w.page_table, w.kv_len, fp8_kv=True, pooled=pooled)
+    for layer in layers + [exact]:
+        layer.kv_len.copy_(torch.tensor(lens, dtype=torch.int32))
+    for t in range(4):
+        x = w.start_block() if t == 0 else w.next_step()
+        args = (x.q, x.k_blk, x.v_blk, torch.full((N,), m, dtype=torch.int32, device="cuda"))
+        layers[0].run_step_fused(*args)
+        layers[1].run_step(*args)
+        exact.run_step_fused(*args)
+        assert all(layer.ctx.poll_status() == 0 for layer in layers + [exact])
+        if t > 0:
+            assert_this_path(layers[0], cfg, m * 4)
+        for name in ("active_idx", "n_active", "union_count", "o_p", "lse_p"):
+            assert torch.equal(getattr(layers[0], name), getattr(layers[1], name)), (t, name)
+        assert torch.equal(layers[0].o_p.bfloat16(), exact.o_p.bfloat16())
+        for s in range(N):
+            assert_rows_exact_to_p(exact, cfg, x.q, s, f"step {t}")
+
+
+@pytest.mark.parametrize("g", [16, 32, 64])
+def test_few_rows_of_one_page_prompts(g):
+    """Some thousand segments of one or two pages, partial ones among them: every group is a piece of its own."""
+    import torch
+    from paper_2604_12056_b200.layer import LosaLayer
+    N, Hkv, G, Bk, d = 64, 16, 4, 4, 128
+    n_sms = torch.cuda.get_device_properties(0).multi_processor_count
+    lens = tuple((1 + (s % 2) * (g < 32)) * g - s % 5 for s in range(N - 1)) + (n_sms * 32 * 128 // (N * Hkv) + g,)
+    cfg = wl.config("c2", n_q_heads=Hkv * G, n_kv_heads=Hkv, head_dim=d, page_size=g, kv_lens=lens, block_size=Bk, steps=1, topk=1,
+                    m_active=1)
+    mp = cfg.max_pages_per_seq
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(g)
+    rnd = lambda *shape: torch.randn(*shape, generator=gen, device="cuda").bfloat16()
+    table = torch.arange(N * mp, dtype=torch.int32, device="cuda").view(N, mp)
+    layer = LosaLayer(cfg, rnd(N * mp, Hkv, g, d), rnd(N * mp, Hkv, g, d), table, torch.tensor(lens, dtype=torch.int32, device="cuda"), fp8_kv=True)
+    q, kb, vb = rnd(N, Bk, Hkv * G, d), rnd(N, Bk, Hkv, d), rnd(N, Bk, Hkv, d)
+    layer.run_step(q, kb, vb, torch.ones(N, dtype=torch.int32, device="cuda"))
+    assert layer.ctx.poll_status() == 0
+    assert_this_path(layer, cfg, Bk * G)
+    for s in range(N):
+        assert_rows_exact_to_p(layer, cfg, q, s, f"prompt {s}")
