@@ -794,8 +794,7 @@ attn_tc5_kernel(const __grid_constant__ Tc5Maps<BOTH> maps, AttnParams p) {
     if constexpr (NARROW) {
       tc5n_softmax<D, GP>(p, cta, [&]() { return choose_path() && narrow; });
     }
-    if (NARROW && (narrow || *abort_flag)) {
-    } else {
+    if (!narrow) {                                     // (still set where a wait has run out)
     // Thread = query row (tensor-memory lane 32 * (warp % 4) + lane); set h = warp / 4 takes the groups
     // h, h + 3, ..., all columns, in S buffer h.  The three warps of a scheduler work on different groups, a
     // third of a period apart, so that one's exponentials (one special-function unit per scheduler) run while

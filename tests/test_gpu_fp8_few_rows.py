@@ -268,3 +268,21 @@ def test_few_rows_of_one_page_prompts(g):
     assert_this_path(layer, cfg, Bk * G)
     for s in range(N):
         assert_rows_exact_to_p(layer, cfg, q, s, f"prompt {s}")
+
+
+def test_few_rows_expired_wait_is_reported_and_the_context_stays_usable():
+    """With the bound of its waits set to a few cycles every CTA gives up at the first one that is not satisfied at once, on this path
+    before or behind the choice of it: the call reports it and ends, and the next one, with the default bound, is right."""
+    import torch
+    from paper_2604_12056_b200 import binding as B
+    layer, cfg, q = hot_token_per_prompt(32, 4, 4, (1,), 12)
+    want = layer.o_p.clone(), layer.lse_p.clone()
+    call = lambda: B.losa_sparse_prefix_attn(layer.ctx, q, layer.kv, layer.active_idx, layer.n_active, layer.union_pages, layer.union_count, layer.state)
+    layer.ctx.set_wait_limit(1)
+    call()
+    assert layer.ctx.poll_status() == B.LOSA_ERR_TIMEOUT
+    layer.ctx.set_wait_limit(0)
+    layer.o_p.zero_()
+    call()
+    assert layer.ctx.poll_status() == 0
+    assert torch.equal(layer.o_p, want[0]) and torch.equal(layer.lse_p, want[1])
