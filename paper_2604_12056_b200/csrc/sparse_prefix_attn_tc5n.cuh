@@ -12,13 +12,13 @@
 //                         them, each rounded to nearest, make up the eleven significant bits of P'
 //   O[D x 3 rows]        += V^T . P'    A = the group's codes (MN-major), B = the terms (MN-major), a column each
 // E5M2 ends at 2^-16, fp16 at 2^-24: the second term is stored times 2^4, the third times 2^8, which their columns of O take back
-// when the piece ends.  A term leaves at most 2^-4 of what it was rounded from, so none exceeds 2^15, and the three are P' exactly,
+// when the piece ends.  What rounding a value below 2^15 leaves is at most 2^11, so no term exceeds 2^15, and the three are P' exactly,
 // for every fp16 value of at most 2^15 (the low bits of a subnormal one, too).  The reference is held 2^11 below the
 // maximum of the shifted exponents and moves when that grows by 2^4 (P' <= 2^15): a weight loses bits no earlier than 2^-25 of its
 // row's largest, with the wide path's 2^7 2^-21; where a page's scale is 1 / r of the largest's, 2^-25 r here, and 2^-21 r for what
 // of the scales is in P' there.  (Terms without powers of two of their own kept the bits of weights down to 2^-17: pages of
 // different scales side by side were off by three times what the wide path's bound allows.)
-// A block of eight 32K prompts takes 900 us the wide way and 804 this way: a group of 128 tokens every 1,350 cycles, which is
+// A block of eight 32K prompts takes 900 us the wide way and 797 this way: a group of 128 tokens every 1,350 cycles, which is
 // HBM's pace, instead of every 2,000.  With V converted to fp16 here as well (P' as fp16) it was hardly faster than the wide way:
 // the conversion and 160 KB per group through shared memory bound it.
 // The three sets of softmax warps take every third group as in the wide path, but each has its own O and its own references,
